@@ -28,9 +28,11 @@ struct InstDesc {
 cudaError_t launch_b_load(const double *x, const double *v, int64_t m, int64_t base,
                           const InstDesc *desc, const long long *p0, int n_inst, double dt,
                           Ctrl *ctrl, cudaStream_t st);
-cudaError_t launch_b_unload(int64_t o0, int64_t m, const int32_t *inv, const InstDesc *desc,
-                            const long long *p0, int n_inst, double dt, const Ctrl *ctrl,
-                            double *x, double *v, cudaStream_t st);
+// after launch_unload_records over all particles; c0 (one entry per instance,
+// its first particle in the caller's order) or null: see k_b_unload
+cudaError_t launch_b_unload(int64_t o0, int64_t m, const InstDesc *desc, const long long *p0,
+                            int n_inst, const long long *c0, double dt, const Ctrl *ctrl, double *x,
+                            double *v, cudaStream_t st);
 cudaError_t launch_b_sort(int64_t n, const InstDesc *desc, const long long *p0, int n_inst,
                           int ntiles, int chunk, Ctrl *ctrl, int32_t *bins, int32_t *scan_tmp,
                           int32_t *tile_items, int2 *tile_range, int4 *items, cudaStream_t st);

@@ -63,7 +63,7 @@ struct pic_batch {
     int64_t staging;
     // arena layout
     size_t o_ctrl, o_desc, o_p0, o_g0, o_tinst, o_sets, set_stride, o_rho, o_rho64, o_E4, o_E8, o_rhoh,
-        o_Eh, o_Epl, o_bins, o_scan, o_titems, o_trange, o_items, o_fpart, o_ppart, o_modes, o_ring, o_inv,
+        o_Eh, o_Epl, o_bins, o_scan, o_titems, o_trange, o_items, o_fpart, o_ppart, o_modes, o_ring, o_c0,
         o_sx, o_sv, o_fft, total;
     char *arena;
     cudaStream_t st;
@@ -161,7 +161,7 @@ void batch_layout(pic_batch *b) {
     b->o_ppart = take((size_t)b->max_items * 4 * 8);
     b->o_modes = take((size_t)b->n_inst * 2 * 8);
     b->o_ring = take((size_t)b->prm.diag_capacity * b->n_inst * sizeof(pic_diag_t));
-    b->o_inv = take((size_t)capn * 4);
+    b->o_c0 = take(sizeof(long long) * b->n_inst);
     b->o_sx = take((size_t)b->staging * 24);
     b->o_sv = take((size_t)b->staging * 24);
     b->o_fft = take(b->fft_reserve);
@@ -460,6 +460,13 @@ int pic_batch_bind_workspace(pic_batch_t b, void *arena, size_t bytes, void *str
                            cudaMemcpyHostToDevice, b->st));
     B_CUDA(cudaMemcpyAsync(b->at<long long>(b->o_g0), b->g0.data(), sizeof(long long) * (b->n_inst + 1),
                            cudaMemcpyHostToDevice, b->st));
+    std::vector<long long> c0(b->n_inst);   // internal order -> first particle in the caller's order
+    for (int i = 0, j; i < b->n_inst; ++i) {
+        j = b->where[i];
+        c0[j] = i > 0 ? c0[b->where[i - 1]] + b->inst[i - 1].n_particles : 0;
+    }
+    B_CUDA(cudaMemcpyAsync(b->at<long long>(b->o_c0), c0.data(), sizeof(long long) * b->n_inst,
+                           cudaMemcpyHostToDevice, b->st));
     B_CUDA(cudaMemcpyAsync(b->at<int32_t>(b->o_tinst), b->tile_inst.data(), sizeof(int32_t) * b->ntiles,
                            cudaMemcpyHostToDevice, b->st));
     B_CUDA(cudaMemsetAsync(b->at<char>(b->o_E4), 0, (size_t)b->ng * 16, b->st));
@@ -570,10 +577,14 @@ int pic_batch_get_particles(pic_batch_t b, double *x, double *v, int dst_is_devi
     int r = b_loaded(b);
     if (r) return r;
     if (b->np > 0 && (!x || !v)) return record_error(PIC_ERR_ARG, "null output array");
-    int32_t *inv = b->at<int32_t>(b->o_inv);
-    B_CUDA(launch_invperm(b->np, b->ctrl(), inv, b->st));
+    B_CUDA(launch_unload_records(b->np, b->ctrl(), b->st));
     const InstDesc *desc = b->at<InstDesc>(b->o_desc);
     const long long *p0 = b->at<long long>(b->o_p0);
+    if (dst_is_device) {
+        B_CUDA(launch_b_unload(0, b->np, desc, p0, b->n_inst, b->at<long long>(b->o_c0), b->prm.dt,
+                               b->ctrl(), x, v, b->st));
+        return PIC_OK;
+    }
     double *sx = b->at<double>(b->o_sx), *sv = b->at<double>(b->o_sv);
     int64_t dst = 0;   // caller-order offset
     for (int i = 0; i < b->n_inst; ++i) {
@@ -581,19 +592,14 @@ int pic_batch_get_particles(pic_batch_t b, double *x, double *v, int dst_is_devi
         const int64_t n = b->inst[i].n_particles, src = b->p0[j];
         for (int64_t o = 0; o < n; o += b->staging) {
             const int64_t m = std::min<int64_t>(b->staging, n - o);
-            if (dst_is_device) {
-                B_CUDA(launch_b_unload(src + o, m, inv, desc, p0, b->n_inst, b->prm.dt, b->ctrl(),
-                                       x + 3 * (dst + o), v + 3 * (dst + o), b->st));
-            } else {
-                B_CUDA(launch_b_unload(src + o, m, inv, desc, p0, b->n_inst, b->prm.dt, b->ctrl(), sx,
-                                       sv, b->st));
-                B_CUDA(cudaMemcpyAsync(x + 3 * (dst + o), sx, (size_t)m * 24, cudaMemcpyDeviceToHost, b->st));
-                B_CUDA(cudaMemcpyAsync(v + 3 * (dst + o), sv, (size_t)m * 24, cudaMemcpyDeviceToHost, b->st));
-            }
+            B_CUDA(launch_b_unload(src + o, m, desc, p0, b->n_inst, nullptr, b->prm.dt, b->ctrl(),
+                                   sx, sv, b->st));
+            B_CUDA(cudaMemcpyAsync(x + 3 * (dst + o), sx, (size_t)m * 24, cudaMemcpyDeviceToHost, b->st));
+            B_CUDA(cudaMemcpyAsync(v + 3 * (dst + o), sv, (size_t)m * 24, cudaMemcpyDeviceToHost, b->st));
         }
         dst += n;
     }
-    if (!dst_is_device) B_CUDA(cudaStreamSynchronize(b->st));
+    B_CUDA(cudaStreamSynchronize(b->st));
     return PIC_OK;
 }
 

@@ -22,6 +22,7 @@
 #include "cic.cuh"
 #include "push.cuh"
 #include "pic_internal.cuh"
+#include "records.cuh"
 
 namespace pic {
 
@@ -441,20 +442,49 @@ __global__ void k_adj_zero(int64_t n, const Ctrl *__restrict__ ctrl) {
     }
 }
 
-// dJ/dx0 = ly_0, dJ/dv0 = lv_0 + dt/2 ly_0 (y_0 = x_0 + dt/2 v_0), in load
-// order, scaled by the caller's upstream gradient
-__global__ void k_adj_unload(int64_t o0, int64_t m, const int32_t *__restrict__ inv,
-                             const Ctrl *__restrict__ ctrl, double half_dt, double scale,
-                             double *__restrict__ gx, double *__restrict__ gv) {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= m) return;
-    const ParticleSet lam = ctrl->sets[1 - ctrl->cur];
-    const int64_t p = inv[o0 + q];
+// The gradients in load order, through 32-byte records like the particle
+// readback: scattered full-sector writes by pid, then a streaming pass.
+__global__ void __launch_bounds__(256) k_adj_unload_records(int64_t n,
+                                                            const Ctrl *__restrict__ ctrl,
+                                                            float4 *__restrict__ rec) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const int cur = ctrl->cur;
+    const int32_t q = ctrl->sets[cur].pid[p];
+    if ((uint64_t)(int64_t)q >= (uint64_t)n) return;   // only after a sort that gave up
+    const ParticleSet lam = ctrl->sets[1 - cur];
+    st_record(rec, q, make_float4(lam.o[0][p], lam.o[1][p], lam.o[2][p], 0.0f),
+              make_float4(lam.v[0][p], lam.v[1][p], lam.v[2][p], 0.0f));
+}
+
+// dJ/dx0 = ly_0, dJ/dv0 = lv_0 + dt/2 ly_0 (y_0 = x_0 + dt/2 v_0), scaled by
+// the caller's upstream gradient
+__global__ void __launch_bounds__(256) k_adj_unload(int64_t o0, int64_t m,
+                                                    const float4 *__restrict__ rec, double half_dt,
+                                                    double scale, double *__restrict__ gx,
+                                                    double *__restrict__ gv) {
+    __shared__ double sx[3 * 256], sv[3 * 256];
+    const int64_t q0 = (int64_t)blockIdx.x * 256;
+    const int cnt = (int)(m - q0 < 256 ? m - q0 : 256);
+    if ((int)threadIdx.x < cnt) {
+        float4 a, b;
+        ld_record(rec, o0 + q0 + threadIdx.x, a, b);
+        const float y[3] = {a.x, a.y, a.z}, w[3] = {b.x, b.y, b.z};
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        const double ly = lam.o[d][p], lv = lam.v[d][p];
-        gx[3 * q + d] = scale * ly;
-        gv[3 * q + d] = scale * (lv + half_dt * ly);
+        for (int d = 0; d < 3; ++d) {
+            const double ly = widen(y[d]), lv = widen(w[d]);
+            sx[3 * threadIdx.x + d] = scale * ly;
+            sv[3 * threadIdx.x + d] = scale * fma(half_dt, ly, lv);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const int j = r * 256 + threadIdx.x;
+        if (j < 3 * cnt) {
+            gx[3 * q0 + j] = sx[j];
+            gv[3 * q0 + j] = sv[j];
+        }
     }
 }
 
@@ -639,12 +669,16 @@ cudaError_t launch_adj_reorder(int64_t n, const int32_t *pos, const int32_t *pid
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_unload(int64_t o0, int64_t m, const int32_t *inv, const Ctrl *ctrl,
-                              double half_dt, double scale, double *gx, double *gv,
-                              cudaStream_t st) {
+cudaError_t launch_adj_unload_records(int64_t n, const Ctrl *ctrl, float4 *rec, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    k_adj_unload_records<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ctrl, rec);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_adj_unload(int64_t o0, int64_t m, const float4 *rec, double half_dt,
+                              double scale, double *gx, double *gv, cudaStream_t st) {
     if (m <= 0) return cudaSuccess;
-    k_adj_unload<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(o0, m, inv, ctrl, half_dt, scale,
-                                                              gx, gv);
+    k_adj_unload<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(o0, m, rec, half_dt, scale, gx, gv);
     return cudaGetLastError();
 }
 

@@ -18,6 +18,7 @@
 #include "batch.cuh"
 #include "cic.cuh"
 #include "push.cuh"
+#include "records.cuh"
 #include "sort_staged.cuh"
 
 namespace pic {
@@ -74,25 +75,49 @@ __global__ void k_b_load(const double *__restrict__ x, const double *__restrict_
     ps.pid[p] = (int32_t)p;
 }
 
-__global__ void k_b_unload(int64_t o0, int64_t m, const int32_t *__restrict__ inv,
-                           const InstDesc *__restrict__ desc, const long long *__restrict__ p0,
-                           int n_inst, double dt, const Ctrl *ctrl, double *__restrict__ x,
-                           double *__restrict__ v) {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= m) return;
-    const ParticleSet ps = ctrl->sets[ctrl->cur];
-    const int64_t p = inv[o0 + q];
-    const InstDesc &D = desc[inst_of_particle(p0, n_inst, p)];
-    const int32_t c = ps.cell[p];
-    const int idx[3] = {cell_i(c), cell_j(c), cell_k(c)};
-    for (int d = 0; d < 3; ++d) {
-        const double vd = (double)ps.v[d][p];
-        double xd = ((double)idx[d] + 0.5 + (double)ps.o[d][p]) * D.h_d[d] - 0.5 * dt * vd;
-        xd -= D.L_d[d] * floor(xd / D.L_d[d]);
-        if (xd >= D.L_d[d]) xd -= D.L_d[d];
-        if (xd < 0.0) xd = 0.0;
-        x[3 * q + d] = xd;
-        v[3 * q + d] = vd;
+// Records [o0, o0 + m) (launch_unload_records over the whole store: pids are
+// store slots, instances in internal order) -> x, v.  With c0 the whole store
+// goes out in one launch, each instance to its place c0 in the caller's order;
+// without, one instance's records go out contiguously.
+__global__ void __launch_bounds__(256) k_b_unload(int64_t o0, int64_t m,
+                                                  const InstDesc *__restrict__ desc,
+                                                  const long long *__restrict__ p0, int n_inst,
+                                                  const long long *__restrict__ c0, double half_dt,
+                                                  const Ctrl *ctrl, double *__restrict__ x,
+                                                  double *__restrict__ v) {
+    const float4 *rec = reinterpret_cast<const float4 *>(ctrl->sets[1 - ctrl->cur].cell);
+    __shared__ double sx[3 * 256], sv[3 * 256];
+    __shared__ long long dst[256];
+    const int64_t q0 = (int64_t)blockIdx.x * 256;
+    const int cnt = (int)(m - q0 < 256 ? m - q0 : 256);
+    if ((int)threadIdx.x < cnt) {
+        const int64_t p = o0 + q0 + threadIdx.x;
+        const int inst = inst_of_particle(p0, n_inst, p);
+        const InstDesc &D = desc[inst];
+        dst[threadIdx.x] = c0 ? c0[inst] + (p - p0[inst]) : p - o0;
+        float4 a, b;
+        ld_record(rec, p, a, b);
+        const int32_t c = __float_as_int(a.x);
+        const int idx[3] = {cell_i(c), cell_j(c), cell_k(c)};
+        const float o[3] = {a.y, a.z, a.w}, w[3] = {b.x, b.y, b.z};
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const double vd = widen(w[d]);
+            const double pos = (half_node(idx[d]) + widen(o[d])) * D.h_d[d];
+            sx[3 * threadIdx.x + d] = wrap_position(fma(-half_dt, vd, pos), D.L_d[d]);
+            sv[3 * threadIdx.x + d] = vd;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        const int j = r * 256 + threadIdx.x;
+        if (j < 3 * cnt) {
+            const int t = j / 3;
+            const int64_t k = 3 * dst[t] + (j - 3 * t);
+            x[k] = sx[j];
+            v[k] = sv[j];
+        }
     }
 }
 
@@ -421,12 +446,12 @@ cudaError_t launch_b_load(const double *x, const double *v, int64_t m, int64_t b
     return cudaGetLastError();
 }
 
-cudaError_t launch_b_unload(int64_t o0, int64_t m, const int32_t *inv, const InstDesc *desc,
-                            const long long *p0, int n_inst, double dt, const Ctrl *ctrl,
-                            double *x, double *v, cudaStream_t st) {
+cudaError_t launch_b_unload(int64_t o0, int64_t m, const InstDesc *desc, const long long *p0,
+                            int n_inst, const long long *c0, double dt, const Ctrl *ctrl, double *x,
+                            double *v, cudaStream_t st) {
     if (m <= 0) return cudaSuccess;
-    k_b_unload<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(o0, m, inv, desc, p0, n_inst, dt, ctrl,
-                                                            x, v);
+    k_b_unload<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(o0, m, desc, p0, n_inst, c0,
+                                                            0.5 * dt, ctrl, x, v);
     return cudaGetLastError();
 }
 

@@ -13,6 +13,7 @@
 
 #include "cic.cuh"
 #include "push.cuh"
+#include "records.cuh"
 
 namespace pic {
 
@@ -117,19 +118,58 @@ __global__ void __launch_bounds__(kLoadThreads) k_load(const double *__restrict_
     if (any_bad) raise_flag(ctrl, PIC_FLAG_NONFINITE);
 }
 
+// ---------------------------------------------------------------------------
+// synchronised readback x_n = x_{n+1/2} - dt/2 v_n in load order, in two
+// passes through 32-byte records in the other particle set (its contents are
+// dead between two re-binnings): k_unload_records reads the store in its own
+// order and writes record pid, one full sector each; k_unload streams the
+// records out as FP64 triples.
+//
+// Both are bound by DRAM (the first by its scattered sector writes).  Read
+// through an inverse permutation, seven scattered 4-byte loads per particle,
+// each fetching a 32-byte sector, took 24.1 ms at 134M particles; the two
+// passes take 5.3 ms.  Writing the FP64 triples scattered in one pass
+// (partial sectors) measured 12.3 ms.
+//
+// To host memory the link is the bound (193 GB/s, 4 particles per ns, which the
+// scattered loads reach), so there the inverse permutation stays: it is the
+// shorter pass to wait for (58 against 141 us at 8M particles).
+// ---------------------------------------------------------------------------
 __global__ void k_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv) {
     int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const ParticleSet ps = ctrl->sets[ctrl->cur];
-    inv[ps.pid[p]] = (int32_t)p;
+    const int32_t q = ps.pid[p];
+    if ((uint64_t)(int64_t)q < (uint64_t)n) inv[q] = (int32_t)p;   // else: a sort gave up
 }
 
-// synchronised readback: x_n = x_{n+1/2} - dt/2 v_n, in load order
+__global__ void __launch_bounds__(256) k_unload_records(int64_t n, const Ctrl *__restrict__ ctrl) {
+    const int cur = ctrl->cur;
+    const ParticleSet ps = ctrl->sets[cur];
+    float4 *rec = reinterpret_cast<float4 *>(ctrl->sets[1 - cur].cell);
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const int32_t q = __ldcs(ps.pid + p);
+    if ((uint64_t)(int64_t)q >= (uint64_t)n) return;   // only after a sort that gave up
+    st_record(rec, q,
+              make_float4(__int_as_float(__ldcs(ps.cell + p)), __ldcs(ps.o[0] + p),
+                          __ldcs(ps.o[1] + p), __ldcs(ps.o[2] + p)),
+              make_float4(__ldcs(ps.v[0] + p), __ldcs(ps.v[1] + p), __ldcs(ps.v[2] + p), 0.0f));
+}
+
+// Particles [o0, o0 + m) of the load order -> x, v, from their records or
+// (GATHER) from the store through inv.  FP64 instructions run at about two lanes
+// per clock and SM on this part, so each component costs two: the node positions
+// come from a table, floats are widened and the wrap is tested on the bits (with
+// conversions and divisions the FP64 pipe was 85% busy: 5.0 ms at 134M).
+template <bool GATHER>
 __global__ void __launch_bounds__(kLoadThreads) k_unload(int64_t o0, int64_t m,
-                                                        const int32_t *__restrict__ inv, Geom g,
+                                                        const int32_t *__restrict__ inv,
+                                                        const double *__restrict__ node_pos,
                                                         double h0, double h1, double h2,
-                                                        double L0, double L1, double L2, double dt,
-                                                        const Ctrl *ctrl, double *__restrict__ x,
+                                                        double L0, double L1, double L2,
+                                                        double half_dt, const Ctrl *ctrl,
+                                                        double *__restrict__ x,
                                                         double *__restrict__ v) {
     // results are staged in shared memory and written as contiguous runs (the
     // destination may be host memory written over the chip-to-chip link)
@@ -137,22 +177,26 @@ __global__ void __launch_bounds__(kLoadThreads) k_unload(int64_t o0, int64_t m,
     const int64_t q0 = (int64_t)blockIdx.x * kLoadThreads;
     const int cnt = (int)(m - q0 < kLoadThreads ? m - q0 : kLoadThreads);
     if ((int)threadIdx.x < cnt) {
-        const ParticleSet ps = ctrl->sets[ctrl->cur];
-        const int64_t p = inv[o0 + q0 + threadIdx.x];
-        const int32_t c = ps.cell[p];
+        float4 a, b;
+        if (GATHER) {
+            const ParticleSet ps = ctrl->sets[ctrl->cur];
+            const int64_t p = inv[o0 + q0 + threadIdx.x];
+            a = make_float4(__int_as_float(ps.cell[p]), ps.o[0][p], ps.o[1][p], ps.o[2][p]);
+            b = make_float4(ps.v[0][p], ps.v[1][p], ps.v[2][p], 0.0f);
+        } else {
+            ld_record(reinterpret_cast<const float4 *>(ctrl->sets[1 - ctrl->cur].cell),
+                      o0 + q0 + threadIdx.x, a, b);
+        }
+        const int32_t c = __float_as_int(a.x);
         const int idx[3] = {cell_i(c), cell_j(c), cell_k(c)};
+        const float o[3] = {a.y, a.z, a.w}, w[3] = {b.x, b.y, b.z};
         const double h[3] = {h0, h1, h2};
         const double L[3] = {L0, L1, L2};
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const double vd = (double)ps.v[d][p];
-            double xd = ((double)idx[d] + 0.5 + (double)ps.o[d][p]) * h[d] - 0.5 * dt * vd;
-            if (xd < 0.0 || xd >= L[d]) {   // wrap (the FP64 division only when needed)
-                xd -= L[d] * floor(xd / L[d]);
-                if (xd >= L[d]) xd -= L[d];
-                if (xd < 0.0) xd = 0.0;
-            }
-            sx[3 * threadIdx.x + d] = xd;
+            const double vd = widen(w[d]);
+            const double pos = fma(widen(o[d]), h[d], __ldg(node_pos + d * kMaxN + idx[d]));
+            sx[3 * threadIdx.x + d] = wrap_position(fma(-half_dt, vd, pos), L[d]);
             sv[3 * threadIdx.x + d] = vd;
         }
     }
@@ -478,20 +522,34 @@ cudaError_t launch_pid_positions(int64_t n, const int32_t *pid, int32_t *pos, cu
     return cudaGetLastError();
 }
 
-cudaError_t launch_invperm(int64_t n, Ctrl *ctrl, int32_t *inv, cudaStream_t st) {
+cudaError_t launch_unload_records(int64_t n, const Ctrl *ctrl, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
-    const int T = 256;
-    k_invperm<<<(unsigned)((n + T - 1) / T), T, 0, st>>>(n, ctrl, inv);
+    k_unload_records<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ctrl);
     return cudaGetLastError();
 }
 
-cudaError_t launch_unload(int64_t o0, int64_t m, const int32_t *inv, const Geom &g,
+cudaError_t launch_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    k_invperm<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ctrl, inv);
+    return cudaGetLastError();
+}
+
+void node_positions(const double *h_d, double *node_pos) {
+    for (int d = 0; d < 3; ++d)
+        for (int i = 0; i < kMaxN; ++i) node_pos[d * kMaxN + i] = ((double)i + 0.5) * h_d[d];
+}
+
+cudaError_t launch_unload(int64_t o0, int64_t m, const int32_t *inv, const double *node_pos,
                           const double *h_d, const double *L_d, double dt, const Ctrl *ctrl,
                           double *x, double *v, cudaStream_t st) {
     if (m <= 0) return cudaSuccess;
-    const int T = kLoadThreads;
-    k_unload<<<(unsigned)((m + T - 1) / T), T, 0, st>>>(o0, m, inv, g, h_d[0], h_d[1], h_d[2],
-                                                        L_d[0], L_d[1], L_d[2], dt, ctrl, x, v);
+    const unsigned blocks = (unsigned)((m + kLoadThreads - 1) / kLoadThreads);
+#define PIC_UL(G)                                                                            \
+    k_unload<G><<<blocks, kLoadThreads, 0, st>>>(o0, m, inv, node_pos, h_d[0], h_d[1], h_d[2], \
+                                                 L_d[0], L_d[1], L_d[2], 0.5 * dt, ctrl, x, v)
+    if (inv) PIC_UL(true);
+    else PIC_UL(false);
+#undef PIC_UL
     return cudaGetLastError();
 }
 

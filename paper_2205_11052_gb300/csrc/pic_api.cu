@@ -49,7 +49,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // Byte offsets of every device buffer inside the caller's arena.
 struct Layout {
     size_t ctrl, sets, rho, rho64, rho_hat, E_hat, E4, E8, lrho2, bins, scan_tmp, tile_items, tile_range,
-        items, fpart, ppart, ring, inv, stage_x, stage_v, adjE4, ktab, fft, total;
+        items, fpart, ppart, ring, inv, stage_x, stage_v, adjE4, ktab, node_pos, fft, total;
     size_t set_stride;   // bytes of one per-particle array
 };
 
@@ -222,6 +222,7 @@ void compute_layout(pic_ctx *c) {
     L.adjE4 = take((size_t)c->ng * 16);
     L.lrho2 = take((size_t)c->ng * 8);
     L.ktab = take((size_t)(c->geom.nh + c->grid.n[1] + c->grid.n[2]) * 4);
+    L.node_pos = take((size_t)3 * kMaxN * 8);
     L.fft = take(c->fft_reserve);
     L.total = o;
 }
@@ -963,6 +964,10 @@ int pic_bind_workspace(pic_handle_t c, void *arena, size_t bytes, void *stream) 
     green_table(c->geom, c->L, ktab.data());
     PIC_CUDA(cudaMemcpyAsync(c->at<float>(c->lay.ktab), ktab.data(), ktab.size() * 4,
                              cudaMemcpyHostToDevice, c->st));
+    std::vector<double> npos((size_t)3 * kMaxN);
+    node_positions(c->h, npos.data());
+    PIC_CUDA(cudaMemcpyAsync(c->at<double>(c->lay.node_pos), npos.data(), npos.size() * 8,
+                             cudaMemcpyHostToDevice, c->st));
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.E4), 0, (size_t)c->ng * 16, c->st));
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.rho), 0, (size_t)c->ng * 4, c->st));
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.rho64), 0, (size_t)c->ng * 8, c->st));
@@ -1091,26 +1096,28 @@ int pic_get_particles(pic_handle_t c, double *x, double *v, int dst_is_device) {
     int r = check_loaded(c);
     if (r) return r;
     if (c->np > 0 && (!x || !v)) return fail(PIC_ERR_ARG, "null output array");
-    int32_t *inv = c->at<int32_t>(c->lay.inv);
-    PIC_CUDA(launch_invperm(c->np, c->ctrl(), inv, c->st));
+    const double *npos = c->at<double>(c->lay.node_pos);
     if (dst_is_device) {
-        PIC_CUDA(launch_unload(0, c->np, inv, c->geom, c->h, c->L, c->prm.dt, c->ctrl(), x, v, c->st));
+        PIC_CUDA(launch_unload_records(c->np, c->ctrl(), c->st));
+        PIC_CUDA(launch_unload(0, c->np, nullptr, npos, c->h, c->L, c->prm.dt, c->ctrl(), x, v, c->st));
         return PIC_OK;
     }
+    // host destinations: the host link is slower than the scattered reads
+    int32_t *inv = c->at<int32_t>(c->lay.inv);
+    PIC_CUDA(launch_invperm(c->np, c->ctrl(), inv, c->st));
     double *mx = static_cast<double *>(const_cast<void *>(mapped_host(x, (size_t)c->np * 24)));
     double *mv = mx ? static_cast<double *>(const_cast<void *>(mapped_host(v, (size_t)c->np * 24)))
                     : nullptr;
     if (mx && mv) {
         // page-locked host arrays: written in place by the unload kernel
-        PIC_CUDA(launch_unload(0, c->np, inv, c->geom, c->h, c->L, c->prm.dt, c->ctrl(), mx, mv,
-                               c->st));
+        PIC_CUDA(launch_unload(0, c->np, inv, npos, c->h, c->L, c->prm.dt, c->ctrl(), mx, mv, c->st));
         PIC_CUDA(cudaStreamSynchronize(c->st));
         return PIC_OK;
     }
     double *sx = c->at<double>(c->lay.stage_x), *sv = c->at<double>(c->lay.stage_v);
     for (int64_t o = 0; o < c->np; o += c->staging) {
         const int64_t m = std::min<int64_t>(c->staging, c->np - o);
-        PIC_CUDA(launch_unload(o, m, inv, c->geom, c->h, c->L, c->prm.dt, c->ctrl(), sx, sv, c->st));
+        PIC_CUDA(launch_unload(o, m, inv, npos, c->h, c->L, c->prm.dt, c->ctrl(), sx, sv, c->st));
         PIC_CUDA(cudaMemcpyAsync(x + 3 * o, sx, (size_t)m * 24, cudaMemcpyDeviceToHost, c->st));
         PIC_CUDA(cudaMemcpyAsync(v + 3 * o, sv, (size_t)m * 24, cudaMemcpyDeviceToHost, c->st));
     }
@@ -1435,16 +1442,18 @@ int pic_adjoint_backward(pic_handle_t c, double scale, double *gx, double *gv, i
     // state the forward sweep started from, re-binned, with its work items).
     if ((r = adj_restore(c, L, 0, cur))) return r;
 
-    // gradients in load order: dJ/dx0 = ly, dJ/dv0 = lv + dt/2 ly
-    int32_t *inv = c->at<int32_t>(c->lay.inv);
-    PIC_CUDA(launch_invperm(c->np, c->ctrl(), inv, c->st));
+    // gradients in load order: dJ/dx0 = ly, dJ/dv0 = lv + dt/2 ly; the records
+    // take the place of the checkpoint that was just restored (eight arrays of
+    // 4 bytes per particle, the last one read of this sweep)
+    float4 *rec = reinterpret_cast<float4 *>(c->adj.buf);
+    PIC_CUDA(launch_adj_unload_records(c->np, c->ctrl(), rec, c->st));
     if (dst_is_device) {
-        PIC_CUDA(launch_adj_unload(0, c->np, inv, c->ctrl(), 0.5 * c->prm.dt, scale, gx, gv, c->st));
+        PIC_CUDA(launch_adj_unload(0, c->np, rec, 0.5 * c->prm.dt, scale, gx, gv, c->st));
     } else {
         double *sx = c->at<double>(c->lay.stage_x), *sv = c->at<double>(c->lay.stage_v);
         for (int64_t o = 0; o < c->np; o += c->staging) {
             const int64_t m = std::min<int64_t>(c->staging, c->np - o);
-            PIC_CUDA(launch_adj_unload(o, m, inv, c->ctrl(), 0.5 * c->prm.dt, scale, sx, sv, c->st));
+            PIC_CUDA(launch_adj_unload(o, m, rec, 0.5 * c->prm.dt, scale, sx, sv, c->st));
             PIC_CUDA(cudaMemcpyAsync(gx + 3 * o, sx, (size_t)m * 24, cudaMemcpyDeviceToHost, c->st));
             PIC_CUDA(cudaMemcpyAsync(gv + 3 * o, sv, (size_t)m * 24, cudaMemcpyDeviceToHost, c->st));
         }

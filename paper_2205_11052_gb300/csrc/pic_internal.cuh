@@ -194,8 +194,14 @@ __device__ __forceinline__ void item_run(const int4 *__restrict__ items, int n_i
 cudaError_t launch_load(const double *x, const double *v, int64_t m, int64_t base,
                         const Geom &g, const double *inv_h_d, double dt, Ctrl *ctrl,
                         cudaStream_t st, int max_blocks = 0);
-cudaError_t launch_invperm(int64_t n, Ctrl *ctrl, int32_t *inv, cudaStream_t st);
-cudaError_t launch_unload(int64_t o0, int64_t m, const int32_t *inv, const Geom &g,
+// readback in load order: the current set's particles as 32-byte records (by
+// pid) in the other set, or the inverse of the store's order (inv[pid]); then
+// particles [o0, o0 + m) as FP64 triples from the records (inv null) or through
+// inv; node_pos: kMaxN node positions (i + 1/2) h per axis
+cudaError_t launch_unload_records(int64_t n, const Ctrl *ctrl, cudaStream_t st);
+cudaError_t launch_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv, cudaStream_t st);
+void node_positions(const double *h_d, double *node_pos);
+cudaError_t launch_unload(int64_t o0, int64_t m, const int32_t *inv, const double *node_pos,
                           const double *h_d, const double *L_d, double dt, const Ctrl *ctrl,
                           double *x, double *v, cudaStream_t st);
 
@@ -354,9 +360,11 @@ cudaError_t launch_adj_reorder(int64_t n, const int32_t *pos, const int32_t *pid
                                float *const out_o[3], float *const out_v[3], cudaStream_t st);
 // pos[pid[j]] = j for j < n (the inverse of a particle order)
 cudaError_t launch_pid_positions(int64_t n, const int32_t *pid, int32_t *pos, cudaStream_t st);
-cudaError_t launch_adj_unload(int64_t o0, int64_t m, const int32_t *inv, const Ctrl *ctrl,
-                              double half_dt, double scale, double *gx, double *gv,
-                              cudaStream_t st);
+// the multipliers in load order: records (by pid) in `rec` (32 bytes per
+// particle, caller's scratch), then records [o0, o0 + m) as the gradients
+cudaError_t launch_adj_unload_records(int64_t n, const Ctrl *ctrl, float4 *rec, cudaStream_t st);
+cudaError_t launch_adj_unload(int64_t o0, int64_t m, const float4 *rec, double half_dt,
+                              double scale, double *gx, double *gv, cudaStream_t st);
 cudaError_t launch_objective(const double *fpart, int nb, double dV, const double *w,
                              double *out, cudaStream_t st);
 cudaError_t launch_dot(int64_t n, const double *a, const double *b, double *part, int max_part,

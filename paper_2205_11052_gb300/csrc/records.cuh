@@ -1,0 +1,62 @@
+// 32-byte particle records: the readback's scratch between the store's order
+// and load order (one aligned sector per particle), and the FP64 helpers of
+// the readback kernels.
+#pragma once
+
+#include "pic_internal.cuh"
+
+namespace pic {
+
+__device__ __forceinline__ void st_record(float4 *rec, int64_t q, const float4 &a, const float4 &b) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(rec + 2 * q),
+                 "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+__device__ __forceinline__ void ld_record(const float4 *rec, int64_t q, float4 &a, float4 &b) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z),
+                   "=f"(b.w)
+                 : "l"(rec + 2 * q));
+}
+
+// (double)f by integer instructions: the exponent is rebiased and the mantissa
+// shifted; subnormals are scaled by 2^64 first, infinities and NaNs get the
+// top exponent (the FP64 pipe, which conversions also use, runs at about two
+// lanes per clock and SM on this part)
+__device__ __forceinline__ double widen(float f) {
+    const unsigned sign = __float_as_uint(f) & 0x80000000u;
+    unsigned b = __float_as_uint(f) & 0x7fffffffu;
+    unsigned bias = 0x38000000u;   // (1023 - 127) << 20
+    if (b < 0x00800000u) {         // zero or subnormal
+        b = __float_as_uint(__uint_as_float(b) * 18446744073709551616.0f);
+        bias = b ? 0x34000000u : 0u;   // 2^-64 more
+    }
+    if (b >= 0x7f800000u) bias = 0x70000000u;   // infinity, NaN
+    return __hiloint2double((int)(((b >> 3) + bias) | sign), (int)(b << 29));
+}
+
+// i + 1/2 in FP64 for 0 <= i < 2^31: 2^51 + (2 i + 1) / 2 built from its bits
+__device__ __forceinline__ double half_node(int i) {
+    return __hiloint2double(0x43200000, 2 * i + 1) - 2251799813685248.0;
+}
+
+// whether x lies in [0, L), on the bits: non-negative doubles order like their
+// bit patterns, a set sign bit or a NaN compares above
+__device__ __forceinline__ bool in_box(double x, double L) {
+    return (unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(L);
+}
+
+// x folded into [0, L); the FP64 division is for positions more than a box away
+__device__ __forceinline__ double wrap_position(double x, double L) {
+    if (!in_box(x, L)) {
+        x += __double_as_longlong(x) < 0 ? L : -L;
+        if (!in_box(x, L)) {
+            x -= L * floor(x / L);
+            if (x >= L) x -= L;
+            if (x < 0.0) x = 0.0;
+        }
+    }
+    return x;
+}
+
+}  // namespace pic
