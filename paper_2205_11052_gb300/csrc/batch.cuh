@@ -55,8 +55,12 @@ cudaError_t launch_b_rho_finish(int64_t ng, const InstDesc *desc, const long lon
                                 unsigned long long *rho64, float *rho, cudaStream_t st);
 cudaError_t launch_b_green(const InstDesc *desc, int first, int m, int64_t nhalf,
                            const float2 *rho_hat, float2 *E_hat, double *modes, cudaStream_t st);
-cudaError_t launch_b_diag(const InstDesc *desc, int n_inst, const float *rho, const float4 *E4,
-                          double *fpart, cudaStream_t st);
+// partial field sums per instance (fpart: kBatchDiagBlocks x 4 doubles each);
+// max_blocks: the largest batch_diag_blocks of any instance
+constexpr int kBatchDiagBlocks = 64;
+int batch_diag_blocks(const Geom &g);
+cudaError_t launch_b_diag(const InstDesc *desc, int n_inst, int max_blocks, const float *rho,
+                          const float4 *E4, double *fpart, cudaStream_t st);
 cudaError_t launch_b_diag_finalize(const InstDesc *desc, int n_inst, const int32_t *item_off,
                                    const double *fpart, const double *ppart, const double *modes,
                                    Ctrl *ctrl, double dt, pic_diag_t *ring, int ring_cap,

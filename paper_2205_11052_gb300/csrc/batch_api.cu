@@ -58,6 +58,7 @@ struct pic_batch {
     int64_t np, ng, nhalf_tot;
     int ntiles, max_items, chunk, sparse_below, fused_blocks, block;
     bool stage_E;   // the push stages each tile's box of E in shared memory
+    int diag_blocks;           // field-diagnostic blocks of the largest instance
     int max_S;                 // largest tile (plus guard) of any instance, in nodes
     size_t fft_reserve;
     int64_t staging;
@@ -157,7 +158,7 @@ void batch_layout(pic_batch *b) {
     b->o_titems = take((size_t)(b->ntiles + 1) * 4);
     b->o_trange = take((size_t)b->ntiles * 8);
     b->o_items = take((size_t)b->max_items * 16);
-    b->o_fpart = take((size_t)b->n_inst * 4 * 8);
+    b->o_fpart = take((size_t)b->n_inst * kBatchDiagBlocks * 4 * 8);
     b->o_ppart = take((size_t)b->max_items * 4 * 8);
     b->o_modes = take((size_t)b->n_inst * 2 * 8);
     b->o_ring = take((size_t)b->prm.diag_capacity * b->n_inst * sizeof(pic_diag_t));
@@ -387,6 +388,8 @@ int pic_batch_create(const pic_instance_t *inst, int n_inst, double q_over_m,
     b->ntiles = tile0;
     b->max_items = (int)std::min<int64_t>(max_items, 2147483647LL);
     b->max_S = max_S;
+    b->diag_blocks = 1;
+    for (const InstDesc &D : b->desc) b->diag_blocks = std::max(b->diag_blocks, batch_diag_blocks(D.g));
     if (batch_push_smem(max_S) > (size_t)kMaxSmemPerBlock) {
         delete b;
         return record_error(PIC_ERR_ARG, "deposit tile plus guard too large for shared memory");
@@ -528,7 +531,7 @@ int pic_batch_step(pic_batch_t b, int n) {
         if ((r = b_solve(b))) return r;
         const bool diag = b->prm.diag_every > 0 && ((b->step + 1) % b->prm.diag_every == 0);
         if (diag)
-            B_CUDA(launch_b_diag(b->at<InstDesc>(b->o_desc), b->n_inst, b->at<float>(b->o_rho),
+            B_CUDA(launch_b_diag(b->at<InstDesc>(b->o_desc), b->n_inst, b->diag_blocks, b->at<float>(b->o_rho),
                                  b->at<float4>(b->o_E4), b->at<double>(b->o_fpart), b->st));
         if ((r = b_deposit_pass(b, true, diag))) return r;
         if (diag)

@@ -14,6 +14,7 @@
 // accumulated in FP64 per block in a fixed order, then summed by one block.
 #include <math.h>
 
+#include "ffsum.cuh"
 #include "pic_internal.cuh"
 
 namespace pic {
@@ -56,26 +57,6 @@ __global__ void __launch_bounds__(128) k_green(int nx, int ny, int nz, int nh,
         ctrl->mode[0] = (double)m.x;
         ctrl->mode[1] = mode_conj ? -(double)m.y : (double)m.y;
     }
-}
-
-// (hi, lo) += a, with the rounding error of the FP32 sum (Knuth's TwoSum,
-// exact in round-to-nearest) carried in lo.
-__device__ __forceinline__ void ff_add(float &hi, float &lo, float a) {
-    const float s = __fadd_rn(hi, a);
-    const float bb = __fsub_rn(s, hi);
-    const float err = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(a, bb));
-    lo = __fadd_rn(lo, err);
-    hi = s;
-}
-
-// (hi, lo) += x^2: the product x*x is split exactly into its rounded value
-// and the FMA residual x*x - fl(x*x) (an FP32 product of FP32 inputs is exact
-// in 48 bits)
-__device__ __forceinline__ void ff_add_sq(float &hi, float &lo, float x) {
-    const float p = __fmul_rn(x, x);
-    const float e = __fmaf_rn(x, x, -p);
-    ff_add(hi, lo, p);
-    lo = __fadd_rn(lo, e);
 }
 
 // Per-block partial sums of Ex^2, Ey^2, Ez^2 and rho.  Each thread keeps FP32
