@@ -196,7 +196,8 @@ int b_deposit_pass(pic_batch *b, bool push, bool diag) {
                                  b->stage_E ? b->at<float4>(b->o_E4) : nullptr,
                                  b->at<float4>(b->o_E8),
                                  b->at<float>(b->o_rho), b->at<unsigned long long>(b->o_rho64),
-                                 b->sparse_below, b->at<double>(b->o_ppart), b->st));
+                                 b->sparse_below, std::max(1, b->chunk / 4), b->at<double>(b->o_ppart),
+                                 b->st));
     if (b_fixed(b))
         B_CUDA(launch_b_rho_finish(b->ng, b->at<InstDesc>(b->o_desc), b->at<long long>(b->o_g0),
                                    b->n_inst, b->at<unsigned long long>(b->o_rho64),

@@ -122,7 +122,8 @@ __global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, co
                                                       const float4 *__restrict__ E8,
                                                       float4 *__restrict__ lE4, float c_kick,
                                                       float dt, float wz2, AdjRhoTerm rt,
-                                                      AdjBound ab, PGrad pg, Ctrl *ctrl_w) {
+                                                      AdjBound ab, PGrad pg, int item_cost,
+                                                      Ctrl *ctrl_w) {
     // 3 * S integer accumulators (x, y, z components) in units of 1 / qs
     extern __shared__ int acc[];
     const int cur = ctrl->cur;
@@ -160,168 +161,177 @@ __global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, co
     float pa[kPGradTerms];
 #pragma unroll
     for (int q = 0; q < kPGradTerms; ++q) pa[q] = 0.0f;
-    for (int it = blockIdx.x; it < n_items; it += gridDim.x) {
-        const int4 item = items[it];
-        const int tile = item.x;
-        const int tx = tile % g.ntile[0];
-        const int ty = (tile / g.ntile[0]) % g.ntile[1];
-        const int tz = tile / (g.ntile[0] * g.ntile[1]);
-        const int ox = tx * g.tile[0], oy = ty * g.tile[1], oz = tz * g.tile[2];
-        const cic::Tile tb = cic::tile_of(g, tile);
-        for (int q = threadIdx.x; q < 3 * S; q += blockDim.x) acc[q] = 0;
-        __syncthreads();
+    Segments run = run_segments(items, n_items, item_cost);
+    for (int q = threadIdx.x; q < 3 * S; q += blockDim.x) acc[q] = 0;
+    cic::Tile tb = cic::tile_of(g, 0);
+    // adds the block's tile to lE4 and clears it
+    auto flush = [&]() {
+        for (int q = threadIdx.x; q < S; q += blockDim.x) {
+            const int ix = acc[q], iy = acc[S + q], iz = acc[2 * S + q];
+            if (ix != 0 || iy != 0 || iz != 0) {
+                acc[q] = 0;
+                acc[S + q] = 0;
+                acc[2 * S + q] = 0;
+                const float ax = (float)ix * inv_qs, ay = (float)iy * inv_qs, az = (float)iz * inv_qs;
+                atomicAdd(lE4 + cic::slot_node(tb, g, q), make_float4(ax, ay, az, 0.0f));
+            }
+        }
+    };
+    // the run's particles tile by tile; the tile goes to the grid when the run
+    // leaves it and after 4095 particles at most (the int32 bound above)
+    int tile, begin, end;
+    while (next_segment(run, tile, begin, end)) {
         // the next particle's position and multipliers are loaded before the
         // current one is reversed
-        int p = item.y + threadIdx.x;
+        int p = begin + threadIdx.x;
         int32_t nyc = 0;
         float nly0 = 0.f, nly1 = 0.f, nly2 = 0.f, nfx = 0.f, nfy = 0.f, nfz = 0.f;
         float nlv0 = 0.f, nlv1 = 0.f, nlv2 = 0.f;
-        if (p < item.z) {
+        if (p < end) {
             nyc = ycell[p];
             nly0 = lam.o[0][p]; nly1 = lam.o[1][p]; nly2 = lam.o[2][p];
             nfx = yo0[p]; nfy = yo1[p]; nfz = yo2[p];
             nlv0 = lam.v[0][p]; nlv1 = lam.v[1][p]; nlv2 = lam.v[2][p];
         }
-        for (; p < item.z; p += blockDim.x) {
-            int i, j, k;
-            if (!decode(nyc, g, i, j, k)) bad = 1;
-            float ly0 = nly0, ly1 = nly1, ly2 = nly2;
-            const float fx = nfx, fy = nfy, fz = nfz;
-            const float plv0 = nlv0, plv1 = nlv1, plv2 = nlv2;
-            {
-                const int pn = p + (int)blockDim.x;
-                if (pn < item.z) {
-                    nyc = ycell[pn];
-                    nly0 = lam.o[0][pn]; nly1 = lam.o[1][pn]; nly2 = lam.o[2][pn];
-                    nfx = yo0[pn]; nfy = yo1[pn]; nfz = yo2[pn];
-                    nlv0 = lam.v[0][pn]; nlv1 = lam.v[1][pn]; nlv2 = lam.v[2][pn];
+        __syncthreads();
+        flush();
+        tb = cic::tile_of(g, tile);
+        const int ox = tb.ox, oy = tb.oy, oz = tb.oz;
+        __syncthreads();
+        for (int done = begin;;) {
+            done += min(end - done, cic::fill_limit() * (int)blockDim.x);
+            for (; p < done; p += blockDim.x) {
+                int i, j, k;
+                if (!decode(nyc, g, i, j, k)) bad = 1;
+                float ly0 = nly0, ly1 = nly1, ly2 = nly2;
+                const float fx = nfx, fy = nfy, fz = nfz;
+                const float plv0 = nlv0, plv1 = nlv1, plv2 = nlv2;
+                {
+                    const int pn = p + (int)blockDim.x;
+                    if (pn < end) {
+                        nyc = ycell[pn];
+                        nly0 = lam.o[0][pn]; nly1 = lam.o[1][pn]; nly2 = lam.o[2][pn];
+                        nfx = yo0[pn]; nfy = yo1[pn]; nfz = yo2[pn];
+                        nlv0 = lam.v[0][pn]; nlv1 = lam.v[1][pn]; nlv2 = lam.v[2][pn];
+                    }
                 }
-            }
-            if (rt.cell) {
-                // the deposit term (dD/dy)^T lrho of the step after this one
-                int ri, rj, rk;
-                decode(rt.cell[p], g, ri, rj, rk);
-                float rs[8];
-                corners_from_pairs(rt.lrho2, ri, rj, rk, nx, ny, nz, rs);
-                float rx, ry, rz;
-                interp_grad(rt.o[0][p], rt.o[1][p], rt.o[2][p], rs, rx, ry, rz);
-                ly0 += rt.sx * rx;
-                ly1 += rt.sy * ry;
-                ly2 += rt.sz * rz;
-            }
-            float lv0 = plv0 + dt * ly0;
-            float lv1 = plv1 + dt * ly1;
-            float lv2 = plv2 + dt * ly2;
-            const float lt0 = lv0, lt1 = lv1, lt2 = lv2;   // lv_tot (for PG)
-            float le0, le1, le2;
-            if (ab.mag) {
-                // lv <- R^T lv_tot, le = (c/2)(R^T lv_tot + lv_tot)
-                const float r0 = ab.R[0] * lv0 + ab.R[3] * lv1 + ab.R[6] * lv2;
-                const float r1 = ab.R[1] * lv0 + ab.R[4] * lv1 + ab.R[7] * lv2;
-                const float r2 = ab.R[2] * lv0 + ab.R[5] * lv1 + ab.R[8] * lv2;
-                const float hc = 0.5f * c_kick;
-                le0 = hc * (r0 + lv0);
-                le1 = hc * (r1 + lv1);
-                le2 = hc * (r2 + lv2);
-                lv0 = r0;
-                lv1 = r1;
-                lv2 = r2;
-            } else {
-                le0 = c_kick * lv0;
-                le1 = c_kick * lv1;
-                le2 = c_kick * lv2;
-            }
-            int nd[8];
-            corners(i, j, k, nx, ny, nz, nd);
-            float sc[8];
-            float ex = 0.0f, ey = 0.0f, ez = 0.0f;   // E at y (PG)
+                if (rt.cell) {
+                    // the deposit term (dD/dy)^T lrho of the step after this one
+                    int ri, rj, rk;
+                    decode(rt.cell[p], g, ri, rj, rk);
+                    float rs[8];
+                    corners_from_pairs(rt.lrho2, ri, rj, rk, nx, ny, nz, rs);
+                    float rx, ry, rz;
+                    interp_grad(rt.o[0][p], rt.o[1][p], rt.o[2][p], rs, rx, ry, rz);
+                    ly0 += rt.sx * rx;
+                    ly1 += rt.sy * ry;
+                    ly2 += rt.sz * rz;
+                }
+                float lv0 = plv0 + dt * ly0;
+                float lv1 = plv1 + dt * ly1;
+                float lv2 = plv2 + dt * ly2;
+                const float lt0 = lv0, lt1 = lv1, lt2 = lv2;   // lv_tot (for PG)
+                float le0, le1, le2;
+                if (ab.mag) {
+                    // lv <- R^T lv_tot, le = (c/2)(R^T lv_tot + lv_tot)
+                    const float r0 = ab.R[0] * lv0 + ab.R[3] * lv1 + ab.R[6] * lv2;
+                    const float r1 = ab.R[1] * lv0 + ab.R[4] * lv1 + ab.R[7] * lv2;
+                    const float r2 = ab.R[2] * lv0 + ab.R[5] * lv1 + ab.R[8] * lv2;
+                    const float hc = 0.5f * c_kick;
+                    le0 = hc * (r0 + lv0);
+                    le1 = hc * (r1 + lv1);
+                    le2 = hc * (r2 + lv2);
+                    lv0 = r0;
+                    lv1 = r1;
+                    lv2 = r2;
+                } else {
+                    le0 = c_kick * lv0;
+                    le1 = c_kick * lv1;
+                    le2 = c_kick * lv2;
+                }
+                int nd[8];
+                corners(i, j, k, nx, ny, nz, nd);
+                float sc[8];
+                float ex = 0.0f, ey = 0.0f, ez = 0.0f;   // E at y (PG)
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                float4 e0, e1;
-                ld_pair(E8 + 2 * nd[2 * r], e0, e1);
-                sc[2 * r] = le0 * e0.x + le1 * e0.y + le2 * e0.z;
-                sc[2 * r + 1] = le0 * e1.x + le1 * e1.y + le2 * e1.z;
+                for (int r = 0; r < 4; ++r) {
+                    float4 e0, e1;
+                    ld_pair(E8 + 2 * nd[2 * r], e0, e1);
+                    sc[2 * r] = le0 * e0.x + le1 * e0.y + le2 * e0.z;
+                    sc[2 * r + 1] = le0 * e1.x + le1 * e1.y + le2 * e1.z;
+                    if (PG) {
+                        // corners 2r, 2r + 1 share the (y, z) factor of their weights
+                        const float wyz = ((r & 1) ? fy : 1.0f - fy) * ((r & 2) ? fz : 1.0f - fz);
+                        const float w0 = (1.0f - fx) * wyz, w1 = fx * wyz;
+                        ex += w0 * e0.x + w1 * e1.x;
+                        ey += w0 * e0.y + w1 * e1.y;
+                        ez += w0 * e0.z + w1 * e1.z;
+                    }
+                }
                 if (PG) {
-                    // corners 2r, 2r + 1 share the (y, z) factor of their weights
-                    const float wyz = ((r & 1) ? fy : 1.0f - fy) * ((r & 2) ? fz : 1.0f - fz);
-                    const float w0 = (1.0f - fx) * wyz, w1 = fx * wyz;
-                    ex += w0 * e0.x + w1 * e1.x;
-                    ey += w0 * e0.y + w1 * e1.y;
-                    ez += w0 * e0.z + w1 * e1.z;
+                    // the quadrupole direction Q(y) = (-(x-c)/2, -(y-c)/2, (z-c)) as in
+                    // the forward kick, vm = v + (c_kick / 2) (e + wz2 Q); sums of
+                    // lv_tot_i vm_j and le . Q
+                    float ux = (float)i - pg.half_n[0] + 0.5f + fx;
+                    float uy = (float)j - pg.half_n[1] + 0.5f + fy;
+                    float uz = (float)k - pg.half_n[2] + 0.5f + fz;
+                    if (ux >= pg.half_n[0]) ux -= (float)nx;
+                    if (uy >= pg.half_n[1]) uy -= (float)ny;
+                    if (uz >= pg.half_n[2]) uz -= (float)nz;
+                    const float Q0 = -0.5f * ux * pg.h[0], Q1 = -0.5f * uy * pg.h[1], Q2 = uz * pg.h[2];
+                    const float hc = 0.5f * c_kick;
+                    const float vm0 = pg.yv[0][p] + hc * (ex + wz2 * Q0);
+                    const float vm1 = pg.yv[1][p] + hc * (ey + wz2 * Q1);
+                    const float vm2 = pg.yv[2][p] + hc * (ez + wz2 * Q2);
+                    pa[0] += lt0 * vm0; pa[1] += lt0 * vm1; pa[2] += lt0 * vm2;
+                    pa[3] += lt1 * vm0; pa[4] += lt1 * vm1; pa[5] += lt1 * vm2;
+                    pa[6] += lt2 * vm0; pa[7] += lt2 * vm1; pa[8] += lt2 * vm2;
+                    pa[9] += le0 * Q0 + le1 * Q1 + le2 * Q2;
+                }
+                float dx, dy, dz;
+                interp_grad(fx, fy, fz, sc, dx, dy, dz);
+                ly0 += g.inv_h[0] * dx - 0.5f * wz2 * le0;
+                ly1 += g.inv_h[1] * dy - 0.5f * wz2 * le1;
+                ly2 += g.inv_h[2] * dz + wz2 * le2;
+                lam.o[0][p] = ly0;
+                lam.o[1][p] = ly1;
+                lam.o[2][p] = ly2;
+                lam.v[0][p] = lv0;
+                lam.v[1][p] = lv1;
+                lam.v[2][p] = lv2;
+                mly = fmaxf(mly, fmaxf(fabsf(ly0), fmaxf(fabsf(ly1), fabsf(ly2))));
+                mlv = fmaxf(mlv, fmaxf(fabsf(lv0), fmaxf(fabsf(lv1), fabsf(lv2))));
+                // G^T le
+                const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
+                const float w[8] = {gx * gy * gz, fx * gy * gz, gx * fy * gz, fx * fy * gz,
+                                    gx * gy * fz, fx * gy * fz, gx * fy * fz, fx * fy * fz};
+                const int si = tile_slot(i, ox, nx, g.tile[0], G);
+                const int sj = tile_slot(j, oy, ny, g.tile[1], G);
+                const int sk = tile_slot(k, oz, nz, g.tile[2], G);
+                if (si >= 0 && sj >= 0 && sk >= 0) {
+                    const int s = si + S0 * sj + S01 * sk;
+                    const int off[8] = {0, 1, S0, S0 + 1, S01, S01 + 1, S01 + S0, S01 + S0 + 1};
+                    const float q0 = qs * le0, q1 = qs * le1, q2 = qs * le2;
+#pragma unroll
+                    for (int cc = 0; cc < 8; ++cc) {
+                        atomicAdd(acc + s + off[cc], __float2int_rn(w[cc] * q0));
+                        atomicAdd(acc + S + s + off[cc], __float2int_rn(w[cc] * q1));
+                        atomicAdd(acc + 2 * S + s + off[cc], __float2int_rn(w[cc] * q2));
+                    }
+                } else {
+#pragma unroll
+                    for (int cc = 0; cc < 8; ++cc)
+                        atomicAdd(lE4 + nd[cc], make_float4(w[cc] * le0, w[cc] * le1, w[cc] * le2, 0.0f));
                 }
             }
-            if (PG) {
-                // the quadrupole direction Q(y) = (-(x-c)/2, -(y-c)/2, (z-c)) as in
-                // the forward kick, vm = v + (c_kick / 2) (e + wz2 Q); sums of
-                // lv_tot_i vm_j and le . Q
-                float ux = (float)i - pg.half_n[0] + 0.5f + fx;
-                float uy = (float)j - pg.half_n[1] + 0.5f + fy;
-                float uz = (float)k - pg.half_n[2] + 0.5f + fz;
-                if (ux >= pg.half_n[0]) ux -= (float)nx;
-                if (uy >= pg.half_n[1]) uy -= (float)ny;
-                if (uz >= pg.half_n[2]) uz -= (float)nz;
-                const float Q0 = -0.5f * ux * pg.h[0], Q1 = -0.5f * uy * pg.h[1], Q2 = uz * pg.h[2];
-                const float hc = 0.5f * c_kick;
-                const float vm0 = pg.yv[0][p] + hc * (ex + wz2 * Q0);
-                const float vm1 = pg.yv[1][p] + hc * (ey + wz2 * Q1);
-                const float vm2 = pg.yv[2][p] + hc * (ez + wz2 * Q2);
-                pa[0] += lt0 * vm0; pa[1] += lt0 * vm1; pa[2] += lt0 * vm2;
-                pa[3] += lt1 * vm0; pa[4] += lt1 * vm1; pa[5] += lt1 * vm2;
-                pa[6] += lt2 * vm0; pa[7] += lt2 * vm1; pa[8] += lt2 * vm2;
-                pa[9] += le0 * Q0 + le1 * Q1 + le2 * Q2;
-            }
-            float dx, dy, dz;
-            interp_grad(fx, fy, fz, sc, dx, dy, dz);
-            ly0 += g.inv_h[0] * dx - 0.5f * wz2 * le0;
-            ly1 += g.inv_h[1] * dy - 0.5f * wz2 * le1;
-            ly2 += g.inv_h[2] * dz + wz2 * le2;
-            lam.o[0][p] = ly0;
-            lam.o[1][p] = ly1;
-            lam.o[2][p] = ly2;
-            lam.v[0][p] = lv0;
-            lam.v[1][p] = lv1;
-            lam.v[2][p] = lv2;
-            mly = fmaxf(mly, fmaxf(fabsf(ly0), fmaxf(fabsf(ly1), fabsf(ly2))));
-            mlv = fmaxf(mlv, fmaxf(fabsf(lv0), fmaxf(fabsf(lv1), fabsf(lv2))));
-            // G^T le
-            const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
-            const float w[8] = {gx * gy * gz, fx * gy * gz, gx * fy * gz, fx * fy * gz,
-                                gx * gy * fz, fx * gy * fz, gx * fy * fz, fx * fy * fz};
-            const int si = tile_slot(i, ox, nx, g.tile[0], G);
-            const int sj = tile_slot(j, oy, ny, g.tile[1], G);
-            const int sk = tile_slot(k, oz, nz, g.tile[2], G);
-            if (si >= 0 && sj >= 0 && sk >= 0) {
-                const int s = si + S0 * sj + S01 * sk;
-                const int off[8] = {0, 1, S0, S0 + 1, S01, S01 + 1, S01 + S0, S01 + S0 + 1};
-                const float q0 = qs * le0, q1 = qs * le1, q2 = qs * le2;
-#pragma unroll
-                for (int cc = 0; cc < 8; ++cc) {
-                    atomicAdd(acc + s + off[cc], __float2int_rn(w[cc] * q0));
-                    atomicAdd(acc + S + s + off[cc], __float2int_rn(w[cc] * q1));
-                    atomicAdd(acc + 2 * S + s + off[cc], __float2int_rn(w[cc] * q2));
-                }
-            } else {
-#pragma unroll
-                for (int cc = 0; cc < 8; ++cc)
-                    atomicAdd(lE4 + nd[cc], make_float4(w[cc] * le0, w[cc] * le1, w[cc] * le2, 0.0f));
-            }
+            if (done == end) break;
+            __syncthreads();
+            flush();
+            __syncthreads();
         }
-        __syncthreads();
-        for (int q = threadIdx.x; q < S; q += blockDim.x) {
-            const int ix = acc[q], iy = acc[S + q], iz = acc[2 * S + q];
-            if (ix != 0 || iy != 0 || iz != 0) {
-                const float ax = (float)ix * inv_qs, ay = (float)iy * inv_qs, az = (float)iz * inv_qs;
-                int a, b, cz;
-                cic::tile_pos(tb, q, a, b, cz);
-                const int gi = cic::wrap_index(ox - G + a, nx);
-                const int gj = cic::wrap_index(oy - G + b, ny);
-                const int gk = cic::wrap_index(oz - G + cz, nz);
-                atomicAdd(lE4 + gi + (int64_t)nx * (gj + (int64_t)ny * gk),
-                          make_float4(ax, ay, az, 0.0f));
-            }
-        }
-        __syncthreads();
     }
+    __syncthreads();
+    flush();
     max_to(&ctrl_w->adj_ly[ab.par], mly);
     max_to(&ctrl_w->adj_lv[ab.par], mlv);
     if (bad) atomicOr(&ctrl_w->flags, PIC_FLAG_BAD_CELL);
@@ -562,7 +572,7 @@ cudaError_t launch_adj_seed(int64_t ng, const float4 *E4, float4 *lE4, const dou
 }
 
 cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, int max_items,
-                            const int32_t *ycell, const float *const yo[3], const float4 *E8,
+                            int item_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
                             float4 *lE4, float c_kick, float dt, float wz2, const AdjRhoTerm &rt,
                             const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, cudaStream_t st) {
     const int S = (g.tile[0] + 2 * g.guard + 1) * (g.tile[1] + 2 * g.guard + 1) *
@@ -579,7 +589,7 @@ cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, 
         }                                                                                       \
         k_adj_push<PGV><<<blocks, 256, smem, st>>>(g, ctrl, items, ycell, yo[0], yo[1], yo[2],  \
                                                    E8, lE4, c_kick, dt, wz2, rt, ab, pg,        \
-                                                   ctrl_w);                                     \
+                                                   item_cost, ctrl_w);                                     \
     } while (0)
     if (pg.part) PIC_ADJ(true);
     else PIC_ADJ(false);

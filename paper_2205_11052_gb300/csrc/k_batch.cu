@@ -161,16 +161,16 @@ struct BatchKey {
 
 // Work items (instance tile, particle range) in contiguous runs per block:
 // the deposit of the instance's tile and (PUSH) the gather + push before it.
-// Each item's tile accumulates in shared memory (u32 fixed point, or FP32
-// bits) and is folded into a 64-bit per-tile sum after the item; the sum is
-// flushed to the instance's grid when the block moves to another tile, so
-// consecutive items of one tile cost one flush.  With DIAG each item leaves
+// The tile accumulates in shared memory (u32 fixed point, or FP32 bits), is
+// folded into 64-bit per-tile sums before an item that would take it past 4095
+// particles, and flushed to the instance's grid when the block moves to another
+// tile, so consecutive items of one tile cost one flush.  With DIAG each item leaves
 // its FP32 particle moments, summed in FP64 in a fixed order, in part[item].
 template <bool PUSH, bool DIAG, bool EXT, bool MAG, bool FIXED>
 __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit(
     const InstDesc *__restrict__ desc, const int32_t *__restrict__ tile_inst, Ctrl *ctrl,
     const int4 *__restrict__ items, const float4 *__restrict__ E4, const float4 *__restrict__ E8,
-    float *rho, unsigned long long *rho64, int sparse_below, int max_S,
+    float *rho, unsigned long long *rho64, int sparse_below, int item_cost, int max_S,
     double *__restrict__ part) {
     extern __shared__ __align__(16) uint32_t acc[];
     __shared__ double red[4][8];
@@ -179,19 +179,20 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
     int it0, it1;
-    item_run(items, n_items, it0, it1);
+    item_run(items, n_items, item_cost, it0, it1);
     for (int s = threadIdx.x; s < max_S; s += blockDim.x) {
         acc[s] = 0u;
         if (FIXED) reinterpret_cast<unsigned long long *>(sum)[s] = 0ull;
         else reinterpret_cast<float *>(sum)[s] = 0.0f;
     }
-    __syncthreads();
     int bad = 0;
-    int cur_tile = -1;
+    int cur_tile = -1, filled = 0;
+    bool folded = false;
     const InstDesc *Dc = desc;
-    cic::Tile tc{};
+    cic::Tile t{};   // the tile of the dense items
     for (int it = it0; it < it1; ++it) {
-        const int4 item = items[it];
+        int4 item = items[it];   // z: end of its tile
+        if (it + 1 < item.w) item.z = items[it + 1].y;
         const InstDesc &D = desc[tile_inst[item.x]];
         const Geom g = D.g;
         const PushConst pc = D.pc;
@@ -200,18 +201,28 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
         unsigned long long *rho64i = rho64 + D.g0;
         const float qscale = D.qscale;
         const bool sparse = item.z - item.y < sparse_below;
-        const cic::Tile t = cic::tile_of(g, item.x - D.tile0);
-        if (!sparse && item.x != cur_tile) {
-            if (cur_tile >= 0)
-                cic::tile_flush_sum<FIXED>(sum, tc, Dc->g, rho + Dc->g0, rho64 + Dc->g0, Dc->qscale);
-            cur_tile = item.x;
-            tc = t;
-            Dc = &D;
-            if (PUSH && E4 != nullptr) {
-                // every read of the previous box ended at the item's last barrier
-                cic::stage_box(sE, E4 + D.g0, t, g);
+        if (!sparse) {
+            if (item.x != cur_tile) {
+                __syncthreads();   // every add to the tile and read of its box is done
+                if (cur_tile >= 0)
+                    cic::tile_flush<FIXED>(acc, sum, folded, t, Dc->g, rho + Dc->g0, rho64 + Dc->g0,
+                                           Dc->qscale);
+                cur_tile = item.x;
+                filled = 0;
+                folded = false;
+                t = cic::tile_of(g, item.x - D.tile0);
+                Dc = &D;
+                if (PUSH && E4 != nullptr) cic::stage_box(sE, E4 + D.g0, t, g);
+                cic::stage_wait();
                 __syncthreads();
+            } else if (filled + (item.z - item.y) > kMaxChunk) {
+                __syncthreads();
+                cic::tile_fold<FIXED>(acc, sum, t.S);
+                __syncthreads();
+                filled = 0;
+                folded = true;
             }
+            filled += item.z - item.y;
         }
         const float4 *sEi = (PUSH && E4 != nullptr && !sparse) ? sE : nullptr;
         float a[4] = {0.f, 0.f, 0.f, 0.f};
@@ -269,11 +280,6 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
                 cic::tile_add<FIXED>(acc, t, g, i, j, k, fx, fy, fz, rhoi, rho64i, qscale);
             }
         }
-        if (!sparse) {
-            __syncthreads();
-            cic::tile_fold<FIXED>(acc, sum, t.S);
-            __syncthreads();
-        }
         if (DIAG) {
             const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
             for (int q = 0; q < 4; ++q) {
@@ -290,8 +296,9 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
             __syncthreads();
         }
     }
+    __syncthreads();
     if (cur_tile >= 0)
-        cic::tile_flush_sum<FIXED>(sum, tc, Dc->g, rho + Dc->g0, rho64 + Dc->g0, Dc->qscale);
+        cic::tile_flush<FIXED>(acc, sum, folded, t, Dc->g, rho + Dc->g0, rho64 + Dc->g0, Dc->qscale);
     if (bad) atomicOr(&ctrl->flags, bad);
 }
 
@@ -521,7 +528,7 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
                                   const int4 *items, int blocks, int threads, int max_S,
                                   const float4 *E4, const float4 *E8,
                                   float *rho, unsigned long long *rho64, int sparse_below,
-                                  double *part, cudaStream_t st) {
+                                  int item_cost, double *part, cudaStream_t st) {
     const size_t smem = batch_push_smem(max_S, E4 != nullptr && push);
     cudaError_t e = cudaSuccess;
 #define PIC_BPD(P, D, X, M, F)                                                                  \
@@ -532,7 +539,8 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
                                       (int)smem)) != cudaSuccess)                               \
             return e;                                                                           \
         kern<<<blocks, threads, smem, st>>>(desc, tile_inst, ctrl, items, push ? E4 : nullptr, \
-                                            E8, rho, rho64, sparse_below, max_S, part);         \
+                                            E8, rho, rho64, sparse_below, item_cost, max_S,     \
+                                            part);                                              \
     } while (0)
 #define PIC_BPD_F(P, D, X, M) \
     do { if (fixed) PIC_BPD(P, D, X, M, true); else PIC_BPD(P, D, X, M, false); } while (0)

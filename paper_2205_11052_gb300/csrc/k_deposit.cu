@@ -9,9 +9,9 @@
 // binned particles whose stencil base was inside one tile at the last sort;
 // consecutive items share tiles) and accumulates the unscaled weights in a
 // shared-memory copy of the tile plus `guard` cells on each side (plus the +1
-// stencil layer).  After each item the tile is folded into per-tile sums
-// that go to the grid with one global atomic per touched node when the run
-// moves to another tile.  Particles that drifted beyond the guard since the
+// stencil layer), folded into per-tile sums every 4095 particles at most; both
+// go to the grid with one global atomic per touched node when the run moves to
+// another tile.  Particles that drifted beyond the guard since the
 // last sort go straight to the grid with global atomics, so the result never
 // depends on the sort cadence.  Each thread loads its next particle before
 // depositing the current one.
@@ -41,14 +41,13 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
                                                            const int4 *__restrict__ items,
                                                            float qscale, float *rho,
                                                            unsigned long long *rho64, Ctrl *ctrl_w,
-                                                           int sparse_below) {
+                                                           int sparse_below, int item_cost) {
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
     unsigned long long strays = 0;
     int bad = 0;
-    int it0, it1;
-    item_run(items, n_items, it0, it1);
+    Segments run = run_segments(items, n_items, item_cost);
     const int S = tile_of(g, 0).S;
     void *sum = reinterpret_cast<char *>(acc) + sum_offset(S);
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
@@ -56,15 +55,14 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
         if (FIXED) reinterpret_cast<unsigned long long *>(sum)[s] = 0ull;
         else reinterpret_cast<float *>(sum)[s] = 0.0f;
     }
-    __syncthreads();
-    // t: the tile of the dense items (sparse items go straight to the grid)
-    int cur_tile = -1;
+    // t: the tile of the dense segments (sparse ones go straight to the grid)
+    bool any = false, folded = false;
     Tile t = tile_of(g, 0);
-    for (int it = it0; it < it1; ++it) {
-        const int4 item = items[it];
-        if (item.z - item.y < sparse_below) {
+    int tile, begin, end;
+    while (next_segment(run, tile, begin, end)) {
+        if (end - begin < sparse_below) {
             // few particles: skip the shared tile, add straight to the grid
-            for (int p = item.y + threadIdx.x; p < item.z; p += blockDim.x) {
+            for (int p = begin + threadIdx.x; p < end; p += blockDim.x) {
                 int i, j, k;
                 if (!decode_cell(ps.cell[p], g, i, j, k)) bad = 1;
                 const float fx = ps.o[0][p], fy = ps.o[1][p], fz = ps.o[2][p];
@@ -74,39 +72,46 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
             }
             continue;
         }
-        if (item.x != cur_tile) {
-            if (cur_tile >= 0) tile_flush_sum<FIXED>(sum, t, g, rho, rho64, qscale);
-            cur_tile = item.x;
-            t = tile_of(g, item.x);
-        }
-        int p = item.y + threadIdx.x;
+        int p = begin + threadIdx.x;
         int32_t nc = 0;
         float nfx = 0.f, nfy = 0.f, nfz = 0.f;
-        if (p < item.z) {
+        if (p < end) {
             nc = __ldcs(ps.cell + p);
             nfx = __ldcs(ps.o[0] + p);
             nfy = __ldcs(ps.o[1] + p);
             nfz = __ldcs(ps.o[2] + p);
         }
-        for (; p < item.z; p += blockDim.x) {
-            const int32_t c = nc;
-            const float fx = nfx, fy = nfy, fz = nfz;
-            const int pn = p + (int)blockDim.x;
-            if (pn < item.z) {
-                nc = __ldcs(ps.cell + pn);
-                nfx = __ldcs(ps.o[0] + pn);
-                nfy = __ldcs(ps.o[1] + pn);
-                nfz = __ldcs(ps.o[2] + pn);
+        __syncthreads();   // every add to the tile is done
+        if (any) tile_flush<FIXED>(acc, sum, folded, t, g, rho, rho64, qscale);
+        any = true;
+        folded = false;
+        t = tile_of(g, tile);
+        __syncthreads();
+        for (int done = begin;;) {
+            done += min(end - done, fill_limit() * (int)blockDim.x);
+            for (; p < done; p += blockDim.x) {
+                const int32_t c = nc;
+                const float fx = nfx, fy = nfy, fz = nfz;
+                const int pn = p + (int)blockDim.x;
+                if (pn < end) {
+                    nc = __ldcs(ps.cell + pn);
+                    nfx = __ldcs(ps.o[0] + pn);
+                    nfy = __ldcs(ps.o[1] + pn);
+                    nfz = __ldcs(ps.o[2] + pn);
+                }
+                int i, j, k;
+                if (!decode_cell(c, g, i, j, k)) bad = 1;
+                if (!tile_add<FIXED, B>(acc, t, g, i, j, k, fx, fy, fz, rho, rho64, qscale)) ++strays;
             }
-            int i, j, k;
-            if (!decode_cell(c, g, i, j, k)) bad = 1;
-            if (!tile_add<FIXED, B>(acc, t, g, i, j, k, fx, fy, fz, rho, rho64, qscale)) ++strays;
+            if (done == end) break;
+            __syncthreads();
+            tile_fold<FIXED>(acc, sum, S);
+            __syncthreads();
+            folded = true;
         }
-        __syncthreads();
-        tile_fold<FIXED>(acc, sum, S);
-        __syncthreads();
     }
-    if (cur_tile >= 0) tile_flush_sum<FIXED>(sum, t, g, rho, rho64, qscale);
+    __syncthreads();
+    if (any) tile_flush<FIXED>(acc, sum, folded, t, g, rho, rho64, qscale);
     if (bad) atomicOr(&ctrl_w->flags, PIC_FLAG_BAD_CELL);
     if (strays) atomicAdd(&ctrl_w->stray, strays);
 }
@@ -146,7 +151,7 @@ cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *r
 cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int4 *items,
                            int max_items, double qscale_d, float *rho, unsigned long long *rho64,
                            bool fixed, Ctrl *ctrl_w, int grid_blocks, int sparse_below,
-                           cudaStream_t st) {
+                           int item_cost, cudaStream_t st) {
     (void)n;
     const float qscale = (float)qscale_d;
     const size_t smem = tile_deposit_smem(g);   // item tile + the block's tile sums
@@ -163,7 +168,7 @@ cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int
                                       (int)smem)) != cudaSuccess)                              \
             return e;                                                                          \
         k_deposit_tiles<F, B><<<blocks, 256, smem, st>>>(g, ctrl, items, qscale, rho, rho64,   \
-                                                         ctrl_w, sparse_below);                \
+                                                         ctrl_w, sparse_below, item_cost);                \
     } while (0)
     if (fixed) {
         if (cbox) PIC_DT(true, 13);

@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(PIC_PD_THREADS, PIC_PD_MIN_BLOCKS) k_push_depo
                                                           const float4 *__restrict__ E4,
                                                           const float4 *__restrict__ E8,
                                                           float *rho, unsigned long long *rho64,
-                                                          float qscale, int sparse_below,
+                                                          float qscale, int sparse_below, int item_cost,
                                                           double *__restrict__ part,
                                                           SaveY save) {
     extern __shared__ __align__(16) uint32_t acc[];
@@ -363,9 +363,8 @@ __global__ void __launch_bounds__(PIC_PD_THREADS, PIC_PD_MIN_BLOCKS) k_push_depo
     double dm[4] = {0.0, 0.0, 0.0, 0.0};
     int bad = 0;
     unsigned long long strays = 0;
-    // a contiguous run of work items per block (consecutive items share tiles)
-    int it0, it1;
-    item_run(items, n_items, it0, it1);
+    // a contiguous run of work items per block, walked tile by tile
+    Segments run = run_segments(items, n_items, item_cost);
     const int S = cic::tile_of(g, 0).S;
     void *sum = reinterpret_cast<char *>(acc) + cic::sum_offset(S);
     float4 *sE = reinterpret_cast<float4 *>(reinterpret_cast<char *>(acc) + cic::stage_offset(S));
@@ -374,72 +373,77 @@ __global__ void __launch_bounds__(PIC_PD_THREADS, PIC_PD_MIN_BLOCKS) k_push_depo
         if (FIXED) reinterpret_cast<unsigned long long *>(sum)[s] = 0ull;
         else reinterpret_cast<float *>(sum)[s] = 0.0f;
     }
-    __syncthreads();
-    // t: the tile of the dense items (sparse items deposit and gather globally)
-    int cur_tile = -1;
+    // t: the tile of the dense segments (sparse ones deposit and gather globally)
+    bool any = false, folded = false;
     cic::Tile t = cic::tile_of(g, 0);
-    for (int it = it0; it < it1; ++it) {
-        const int4 item = items[it];
-        const bool sparse = item.z - item.y < sparse_below;
-        if (!sparse && item.x != cur_tile) {
-            if (cur_tile >= 0) cic::tile_flush_sum<FIXED>(sum, t, g, rho, rho64, qscale);
-            cur_tile = item.x;
-            t = cic::tile_of(g, item.x);
-            if (E4 != nullptr) {
-                // every read of the previous box ended at the item's last barrier
-                cic::stage_box(sE, E4, t, g);
-                __syncthreads();
-            }
-        }
-        const float4 *sEi = (E4 != nullptr && !sparse) ? sE : nullptr;
+    int tile, begin, end;
+    while (next_segment(run, tile, begin, end)) {
+        const bool sparse = end - begin < sparse_below;
         // one particle per thread and iteration (coalesced 4-byte streams);
         // the next iteration's particle is loaded before this one is pushed
-        int p = item.y + threadIdx.x;
+        int p = begin + threadIdx.x;
         int32_t nc = 0;
         float nfx = 0.f, nfy = 0.f, nfz = 0.f, nvx = 0.f, nvy = 0.f, nvz = 0.f;
-        if (p < item.z) {
+        if (p < end) {
             nc = __ldcs(ps.cell + p);
             nfx = __ldcs(ps.o[0] + p); nfy = __ldcs(ps.o[1] + p); nfz = __ldcs(ps.o[2] + p);
             nvx = __ldcs(ps.v[0] + p); nvy = __ldcs(ps.v[1] + p); nvz = __ldcs(ps.v[2] + p);
         }
-        for (; p < item.z; p += blockDim.x) {
-            int32_t c = nc;
-            float fx = nfx, fy = nfy, fz = nfz, vx = nvx, vy = nvy, vz = nvz;
-            const int pn = p + (int)blockDim.x;
-            if (pn < item.z) {
-                nc = __ldcs(ps.cell + pn);
-                nfx = __ldcs(ps.o[0] + pn); nfy = __ldcs(ps.o[1] + pn); nfz = __ldcs(ps.o[2] + pn);
-                nvx = __ldcs(ps.v[0] + pn); nvy = __ldcs(ps.v[1] + pn); nvz = __ldcs(ps.v[2] + pn);
-            }
-            if (save.cell) {
-                __stcs(save.cell + p, c);
-                __stcs(save.o[0] + p, fx);
-                __stcs(save.o[1] + p, fy);
-                __stcs(save.o[2] + p, fz);
-                if (save.v[0]) {
-                    __stcs(save.v[0] + p, vx);
-                    __stcs(save.v[1] + p, vy);
-                    __stcs(save.v[2] + p, vz);
-                }
-            }
-            pd_one<DIAG, EXT, MAG, FIXED, B>(g, pc, E8, sEi, sparse, acc, t, rho, rho64, qscale, c,
-                                          fx, fy, fz, vx, vy, vz, bad, strays, a);
-            __stcs(ps.cell + p, c);
-            __stcs(ps.o[0] + p, fx);
-            __stcs(ps.o[1] + p, fy);
-            __stcs(ps.o[2] + p, fz);
-            __stcs(ps.v[0] + p, vx);
-            __stcs(ps.v[1] + p, vy);
-            __stcs(ps.v[2] + p, vz);
-        }
-        if (DIAG) fold_moments(a, dm);
         if (!sparse) {
+            __syncthreads();   // every add to the tile and read of its box is done
+            const cic::Tile tn = cic::tile_of(g, tile);
+            if (E4 != nullptr) cic::stage_box(sE, E4, tn, g);
+            if (any) cic::tile_flush<FIXED>(acc, sum, folded, t, g, rho, rho64, qscale);
+            any = true;
+            folded = false;
+            t = tn;
+            cic::stage_wait();
+            __syncthreads();
+        }
+        const float4 *sEi = (E4 != nullptr && !sparse) ? sE : nullptr;
+        for (int done = begin;;) {
+            // as many particles as the tile takes without a fold
+            done += min(end - done, cic::fill_limit() * (int)blockDim.x);
+            for (; p < done; p += blockDim.x) {
+                int32_t c = nc;
+                float fx = nfx, fy = nfy, fz = nfz, vx = nvx, vy = nvy, vz = nvz;
+                const int pn = p + (int)blockDim.x;
+                if (pn < end) {
+                    nc = __ldcs(ps.cell + pn);
+                    nfx = __ldcs(ps.o[0] + pn); nfy = __ldcs(ps.o[1] + pn); nfz = __ldcs(ps.o[2] + pn);
+                    nvx = __ldcs(ps.v[0] + pn); nvy = __ldcs(ps.v[1] + pn); nvz = __ldcs(ps.v[2] + pn);
+                }
+                if (save.cell) {
+                    __stcs(save.cell + p, c);
+                    __stcs(save.o[0] + p, fx);
+                    __stcs(save.o[1] + p, fy);
+                    __stcs(save.o[2] + p, fz);
+                    if (save.v[0]) {
+                        __stcs(save.v[0] + p, vx);
+                        __stcs(save.v[1] + p, vy);
+                        __stcs(save.v[2] + p, vz);
+                    }
+                }
+                pd_one<DIAG, EXT, MAG, FIXED, B>(g, pc, E8, sEi, sparse, acc, t, rho, rho64, qscale, c,
+                                              fx, fy, fz, vx, vy, vz, bad, strays, a);
+                __stcs(ps.cell + p, c);
+                __stcs(ps.o[0] + p, fx);
+                __stcs(ps.o[1] + p, fy);
+                __stcs(ps.o[2] + p, fz);
+                __stcs(ps.v[0] + p, vx);
+                __stcs(ps.v[1] + p, vy);
+                __stcs(ps.v[2] + p, vz);
+            }
+            if (DIAG) fold_moments(a, dm);
+            if (done == end) break;
             __syncthreads();
             cic::tile_fold<FIXED>(acc, sum, S);
             __syncthreads();
+            folded = true;
         }
     }
-    if (cur_tile >= 0) cic::tile_flush_sum<FIXED>(sum, t, g, rho, rho64, qscale);
+    __syncthreads();
+    if (any) cic::tile_flush<FIXED>(acc, sum, folded, t, g, rho, rho64, qscale);
     if (bad) raise_flag(ctrl, bad);
     if (strays) {
         atomicAdd(&ctrl->stray, strays);
@@ -626,7 +630,8 @@ __device__ __forceinline__ void block_moments(const double (&d)[4], double *part
 template <bool DIAG, bool FIXED, int B>
 __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
     Geom g, uint64_t seed, Ctrl *ctrl, const int4 *__restrict__ items, float *rho,
-    unsigned long long *rho64, float qscale, int sparse_below, double *__restrict__ part) {
+    unsigned long long *rho64, float qscale, int sparse_below, int item_cost,
+    double *__restrict__ part) {
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
@@ -635,8 +640,7 @@ __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
     double dm[4] = {0.0, 0.0, 0.0, 0.0};
     int bad = 0;
     unsigned long long strays = 0;
-    int it0, it1;
-    item_run(items, n_items, it0, it1);
+    Segments run = run_segments(items, n_items, item_cost);
     const int S = cic::tile_of(g, 0).S;
     void *sum = reinterpret_cast<char *>(acc) + cic::sum_offset(S);
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
@@ -644,66 +648,72 @@ __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
         if (FIXED) reinterpret_cast<unsigned long long *>(sum)[s] = 0ull;
         else reinterpret_cast<float *>(sum)[s] = 0.0f;
     }
-    __syncthreads();
-    // t: the tile of the dense items (sparse items deposit globally)
-    int cur_tile = -1;
+    // t: the tile of the dense segments (sparse ones deposit globally)
+    bool any = false, folded = false;
     cic::Tile t = cic::tile_of(g, 0);
-    for (int it = it0; it < it1; ++it) {
-        const int4 item = items[it];
-        const bool sparse = item.z - item.y < sparse_below;
-        if (!sparse && item.x != cur_tile) {
-            if (cur_tile >= 0) cic::tile_flush_sum<FIXED>(sum, t, g, rho, rho64, qscale);
-            cur_tile = item.x;
-            t = cic::tile_of(g, item.x);
-        }
+    int tile, begin, end;
+    while (next_segment(run, tile, begin, end)) {
+        const bool sparse = end - begin < sparse_below;
         // the next particle's streams are loaded before the current one moves
-        int p = item.y + threadIdx.x;
+        int p = begin + threadIdx.x;
         int32_t nc = 0, npid = 0;
         float nfx = 0.f, nfy = 0.f, nfz = 0.f;
-        if (p < item.z) {
+        if (p < end) {
             nc = __ldcs(ps.cell + p);
             nfx = __ldcs(ps.o[0] + p); nfy = __ldcs(ps.o[1] + p); nfz = __ldcs(ps.o[2] + p);
             npid = ps.pid[p];
         }
-        for (; p < item.z; p += blockDim.x) {
-            int32_t c = nc;
-            float fx = nfx, fy = nfy, fz = nfz;
-            const int32_t pid = npid;
-            const int pn = p + (int)blockDim.x;
-            if (pn < item.z) {
-                nc = __ldcs(ps.cell + pn);
-                nfx = __ldcs(ps.o[0] + pn); nfy = __ldcs(ps.o[1] + pn); nfz = __ldcs(ps.o[2] + pn);
-                npid = ps.pid[pn];
-            }
-            move_one(g, seed, n, pid, c, fx, fy, fz, bad);
-            const int i = cell_i(c), j = cell_j(c), k = cell_k(c);
-            if (sparse) {
-                float w[8];
-                cic::weights(fx, fy, fz, w);
-                cic::deposit_global<FIXED>(rho, rho64, g, i, j, k, w, fx, fy, fz, qscale);
-            } else if (!cic::tile_add<FIXED, B>(acc, t, g, i, j, k, fx, fy, fz, rho, rho64, qscale)) {
-                ++strays;
-            }
-            if (DIAG) {
-                const float vx = ps.v[0][p], vy = ps.v[1][p], vz = ps.v[2][p];
-                a[0] += vx;
-                a[1] += vy;
-                a[2] += vz;
-                a[3] += vx * vx + vy * vy + vz * vz;
-            }
-            __stcs(ps.cell + p, c);
-            __stcs(ps.o[0] + p, fx);
-            __stcs(ps.o[1] + p, fy);
-            __stcs(ps.o[2] + p, fz);
-        }
-        if (DIAG) fold_moments(a, dm);
         if (!sparse) {
+            __syncthreads();   // every add to the tile is done
+            if (any) cic::tile_flush<FIXED>(acc, sum, folded, t, g, rho, rho64, qscale);
+            any = true;
+            folded = false;
+            t = cic::tile_of(g, tile);
+            __syncthreads();
+        }
+        for (int done = begin;;) {
+            done += min(end - done, cic::fill_limit() * (int)blockDim.x);
+            for (; p < done; p += blockDim.x) {
+                int32_t c = nc;
+                float fx = nfx, fy = nfy, fz = nfz;
+                const int32_t pid = npid;
+                const int pn = p + (int)blockDim.x;
+                if (pn < end) {
+                    nc = __ldcs(ps.cell + pn);
+                    nfx = __ldcs(ps.o[0] + pn); nfy = __ldcs(ps.o[1] + pn); nfz = __ldcs(ps.o[2] + pn);
+                    npid = ps.pid[pn];
+                }
+                move_one(g, seed, n, pid, c, fx, fy, fz, bad);
+                const int i = cell_i(c), j = cell_j(c), k = cell_k(c);
+                if (sparse) {
+                    float w[8];
+                    cic::weights(fx, fy, fz, w);
+                    cic::deposit_global<FIXED>(rho, rho64, g, i, j, k, w, fx, fy, fz, qscale);
+                } else if (!cic::tile_add<FIXED, B>(acc, t, g, i, j, k, fx, fy, fz, rho, rho64, qscale)) {
+                    ++strays;
+                }
+                if (DIAG) {
+                    const float vx = ps.v[0][p], vy = ps.v[1][p], vz = ps.v[2][p];
+                    a[0] += vx;
+                    a[1] += vy;
+                    a[2] += vz;
+                    a[3] += vx * vx + vy * vy + vz * vz;
+                }
+                __stcs(ps.cell + p, c);
+                __stcs(ps.o[0] + p, fx);
+                __stcs(ps.o[1] + p, fy);
+                __stcs(ps.o[2] + p, fz);
+            }
+            if (DIAG) fold_moments(a, dm);
+            if (done == end) break;
             __syncthreads();
             cic::tile_fold<FIXED>(acc, sum, S);
             __syncthreads();
+            folded = true;
         }
     }
-    if (cur_tile >= 0) cic::tile_flush_sum<FIXED>(sum, t, g, rho, rho64, qscale);
+    __syncthreads();
+    if (any) cic::tile_flush<FIXED>(acc, sum, folded, t, g, rho, rho64, qscale);
     if (bad) raise_flag(ctrl, bad);
     if (strays) {
         atomicAdd(&ctrl->stray, strays);
@@ -759,15 +769,16 @@ bool const_box(const Geom &g) {
 
 cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, bool fixed, bool deposit,
                         Ctrl *ctrl, const int4 *items, int max_items, float *rho,
-                        unsigned long long *rho64, double qscale, int sparse_below, double *part,
-                        int blocks, cudaStream_t st) {
+                        unsigned long long *rho64, double qscale, int sparse_below, int item_cost,
+                        double *part, int blocks, cudaStream_t st) {
     const int nb = std::max(1, std::min(blocks, deposit ? max_items : blocks));
     if (deposit) {
         const size_t smem = tile_deposit_smem(g);
         const float qs = (float)qscale;
         const bool cbox = const_box(g);
 #define PIC_MV(D, F, B) \
-    k_move_deposit<D, F, B><<<nb, 256, smem, st>>>(g, seed, ctrl, items, rho, rho64, qs, sparse_below, part)
+    k_move_deposit<D, F, B><<<nb, 256, smem, st>>>(g, seed, ctrl, items, rho, rho64, qs, sparse_below, \
+                                                   item_cost, part)
         if (diag) {
             if (!fixed) PIC_MV(true, false, 0);
             else if (cbox) PIC_MV(true, true, kConstBox);
@@ -847,8 +858,8 @@ cudaError_t push_deposit_prepare(const Geom &g) {
 cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, bool fixed,
                                 Ctrl *ctrl, const int4 *items, int max_items, const float4 *E4,
                                 const float4 *E8, float *rho, unsigned long long *rho64,
-                                double qscale, int sparse_below, double *part, int blocks,
-                                const SaveY &save, cudaStream_t st) {
+                                double qscale, int sparse_below, int item_cost, double *part,
+                                int blocks, const SaveY &save, cudaStream_t st) {
     const bool ext = pc.wz2 != 0.0f;
     const bool mag = pc.t[0] != 0.0f || pc.t[1] != 0.0f || pc.t[2] != 0.0f;
     const size_t smem = push_deposit_smem(g);
@@ -860,7 +871,7 @@ cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, b
 #define PIC_PD(D, X, M, F, B)                                                                   \
     k_push_deposit<D, X, M, F, B><<<nb, PIC_PD_THREADS, smem, st>>>(g, pc, ctrl, items, E4s, E8, \
                                                                     rho, rho64, qs,             \
-                                                                    sparse_below, part, save)
+                                                                    sparse_below, item_cost, part, save)
 #define PIC_PD_F(D, X, M)                                  \
     do {                                                   \
         if (!fixed) PIC_PD(D, X, M, false, 0);             \

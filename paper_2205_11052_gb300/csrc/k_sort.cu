@@ -176,10 +176,10 @@ __global__ void k_fill_items(int ntiles, int chunk, const int32_t *__restrict__ 
     }
     if (t >= ntiles) return;
     const int2 r = tile_range[t];
-    int o = item_off[t];
-    for (int s = r.x; s < r.y; s += chunk) {
-        items[o++] = make_int4(t, s, min(r.y, s + chunk), 0);
-    }
+    const int o = item_off[t], cnt = r.y - r.x;
+    const int k = (cnt + chunk - 1) / chunk;
+    for (int i = 0; i < k; ++i)
+        items[o + i] = make_int4(t, r.x + (int)((long long)cnt * i / k), r.y, o + k);
 }
 
 __global__ void k_flip(Ctrl *ctrl) { ctrl->cur = 1 - ctrl->cur; }

@@ -306,11 +306,21 @@ int timer_end(pic_ctx *c, int ph, int kernels) {
     return PIC_OK;
 }
 
+// particles per work item: the caller's, or so many that the blocks of one wave
+// get kItemsPerBlock items each
+constexpr int64_t kItemTarget = (int64_t)kNumSMs * PIC_PD_MIN_BLOCKS * kItemsPerBlock;
+int chunk_of(const pic_ctx *c) {
+    if (c->chunk) return c->chunk;
+    const int64_t per = (c->np + kItemTarget - 1) / kItemTarget;
+    return (int)std::max<int64_t>(kMinChunk, std::min<int64_t>(per, kMaxChunk));
+}
+int item_cost_of(const pic_ctx *c) { return std::max(1, chunk_of(c) / 4); }
+
 // presort: the store is in arbitrary order (right after a load)
 int do_sort(pic_ctx *c, bool presort = false) {
     int r = timer_begin(c, PIC_PHASE_SORT);
     if (r) return r;
-    PIC_CUDA(launch_sort(c->np, c->geom, c->chunk, c->ctrl(), c->at<int32_t>(c->lay.bins),
+    PIC_CUDA(launch_sort(c->np, c->geom, chunk_of(c), c->ctrl(), c->at<int32_t>(c->lay.bins),
                          c->nbins, c->at<int32_t>(c->lay.scan_tmp),
                          c->at<int32_t>(c->lay.tile_items), c->at<int2>(c->lay.tile_range),
                          c->at<int4>(c->lay.items), presort, c->st));
@@ -325,7 +335,7 @@ int do_sort_gated(pic_ctx *c) {
     if (r) return r;
     const long long max_strays = (long long)floor(c->prm.stray_rebin * (double)c->np);
     PIC_CUDA(launch_rebin_decide(c->ctrl(), max_strays, c->prm.sort_period, c->st));
-    PIC_CUDA(launch_sort(c->np, c->geom, c->chunk, c->ctrl(), c->at<int32_t>(c->lay.bins),
+    PIC_CUDA(launch_sort(c->np, c->geom, chunk_of(c), c->ctrl(), c->at<int32_t>(c->lay.bins),
                          c->nbins, c->at<int32_t>(c->lay.scan_tmp),
                          c->at<int32_t>(c->lay.tile_items), c->at<int2>(c->lay.tile_range),
                          c->at<int4>(c->lay.items), false, c->st, &c->ctrl()->rebin));
@@ -344,7 +354,7 @@ int do_deposit(pic_ctx *c) {
         PIC_CUDA(launch_deposit(c->np, c->geom, c->ctrl(), c->at<int4>(c->lay.items),
                                 (int)c->max_items, qscale_of(c), c->at<float>(c->lay.rho),
                                 c->at<unsigned long long>(c->lay.rho64), fixed, c->ctrl(),
-                                c->deposit_blocks, c->sparse_below, c->st));
+                                c->deposit_blocks, c->sparse_below, item_cost_of(c), c->st));
         c->rho_current = true;
         return timer_end(c, PIC_PHASE_DEPOSIT, fixed ? 2 : 1);
     }
@@ -371,7 +381,7 @@ int do_gather_push(pic_ctx *c, bool diag) {
     if (r) return r;
     if (uniform_move(c) && c->np > 0) {
         PIC_CUDA(launch_move(c->np, c->geom, c->prm.seed, diag, false, false, c->ctrl(), nullptr, 0,
-                             nullptr, nullptr, 0.0, 0, c->at<double>(c->lay.ppart),
+                             nullptr, nullptr, 0.0, 0, 0, c->at<double>(c->lay.ppart),
                              push_blocks_of(c), c->st));
     } else {
         PIC_CUDA(launch_gather_push(c->np, c->geom, push_const(c), diag, c->ctrl(),
@@ -426,15 +436,15 @@ int do_push_deposit(pic_ctx *c, bool diag, const SaveY &save = SaveY{}) {
         PIC_CUDA(launch_move(c->np, c->geom, c->prm.seed, diag, fixed, true, c->ctrl(),
                              c->at<int4>(c->lay.items), (int)c->max_items, c->at<float>(c->lay.rho),
                              c->at<unsigned long long>(c->lay.rho64), qscale_of(c),
-                             c->sparse_below, c->at<double>(c->lay.ppart), fused_blocks_of(c),
-                             c->st));
+                             c->sparse_below, item_cost_of(c), c->at<double>(c->lay.ppart),
+                             fused_blocks_of(c), c->st));
     } else if (c->np > 0) {
         PIC_CUDA(launch_push_deposit(c->geom, push_const(c), diag, fixed, c->ctrl(),
                                      c->at<int4>(c->lay.items), (int)c->max_items,
                                      c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8),
                                      c->at<float>(c->lay.rho),
                                      c->at<unsigned long long>(c->lay.rho64), qscale_of(c),
-                                     c->sparse_below, c->at<double>(c->lay.ppart),
+                                     c->sparse_below, item_cost_of(c), c->at<double>(c->lay.ppart),
                                      fused_blocks_of(c), save, c->st));
     } else {
         // nothing to push: the plain kernel still records zero moments and the step
@@ -844,7 +854,7 @@ int pic_create(const pic_grid_t *grid, const pic_species_t *species, const pic_p
     if (p.diag_capacity == 0) p.diag_capacity = 1024;
     if (p.guard == 0) p.guard = 2;
     c->block = p.block ? p.block : 256;
-    c->chunk = p.chunk ? p.chunk : kMaxChunk;
+    c->chunk = p.chunk;
 
     Geom &g = c->geom;
     int64_t nt = 1;
@@ -881,7 +891,10 @@ int pic_create(const pic_grid_t *grid, const pic_species_t *species, const pic_p
     c->cap = species->n_particles;
     c->ng = (int64_t)grid->n[0] * grid->n[1] * grid->n[2];
     c->nhalf = (int64_t)g.nh * grid->n[1] * grid->n[2];
-    c->max_items = c->ntiles + (c->cap + c->chunk - 1) / c->chunk + 1;
+    // bounds the items of any load up to the capacity (see chunk_of)
+    c->max_items = c->ntiles + 1 +
+                   (c->chunk ? (c->cap + c->chunk - 1) / c->chunk
+                             : std::max<int64_t>(kItemTarget, (c->cap + kMaxChunk - 1) / kMaxChunk));
     c->staging = std::max<int64_t>(1, std::min<int64_t>(c->cap, (int64_t)1 << 22));
     c->sparse_below = 64;
     c->deposit_blocks = 152 * PIC_DEP_MIN_BLOCKS * PIC_DEP_WAVES;   // waves of the resident blocks
@@ -1404,7 +1417,7 @@ int pic_adjoint_backward(pic_handle_t c, double scale, double *gx, double *gv, i
                 pg.part = pg_part;
             }
             PIC_CUDA(launch_adj_push(c->geom, c->ctrl(), c->at<int4>(c->lay.items),
-                                     (int)c->max_items, ycell, yo, En, lE4, c_kick, dt, wz2, rt,
+                                     (int)c->max_items, item_cost_of(c), ycell, yo, En, lE4, c_kick, dt, wz2, rt,
                                      step_bound(ab, n & 1), pg, c->ctrl(), c->st));
             if (pgrad) PIC_CUDA(launch_pgrad_acc(pg_part, (int)c->max_items, pg_acc, c->st));
             if ((r = adj_solve(c, n & 1))) return r;

@@ -137,21 +137,29 @@ constexpr int kMaxChunk = 4095;   // fixed-point tile slots stay below 2^32
 // Set the thread-local message returned by pic_last_error(); returns `code`.
 int record_error(int code, const char *fmt, ...);
 
+// Work items: int4 (tile, begin, end of its tile, first item of the next tile).  A tile of
+// cnt particles is split into ceil(cnt / chunk) items of equal size; items only
+// say where a block's run may begin and end, and a block walks the particles of
+// its run tile by tile (next_segment), so small items cost it nothing.
+//
 // The run of work items [it0, it1) of this block.  Items cover the particles
-// [0, P) in order; item i costs its particles plus a fixed kItemCost for its
-// tile's fold and flush, so the cost before item i is y_i + kItemCost i, and
-// the block takes the items that start within its equal share of the total
+// [0, P) in order; item i costs its particles plus item_cost for its share of
+// the tile's staging and flush, so the cost before item i is y_i + item_cost i,
+// and the block takes the items that start within its equal share of the total
 // (with fewer items than blocks, block b takes item b).
-#ifndef PIC_ITEM_COST
-#define PIC_ITEM_COST 1024
-#endif
-constexpr long long kItemCost = PIC_ITEM_COST;
+//
+// With at most 4095 particles an item, 4.2M particles on 512 tiles of 8192 gave
+// a block two or three items (9200 particles), and 33k particles on 8 tiles kept
+// 9 of 456 blocks busy; sixteen items a block (256..4095 particles) keep the
+// shares within a few percent (push 110 -> 101 us and 40.6 -> 17.4 us).
+constexpr int kItemsPerBlock = 16;
+constexpr int kMinChunk = 256;
 // Called by every thread of the block (it synchronises): the two item
 // indices are found by a two-level search in which each thread tests one
 // sample per round, so a block start costs a few dependent loads (two while
 // n_items <= blockDim^2), not log2(n_items).
-__device__ __forceinline__ void item_run(const int4 *__restrict__ items, int n_items, int &it0,
-                                         int &it1) {
+__device__ __forceinline__ void item_run(const int4 *__restrict__ items, int n_items,
+                                         long long item_cost, int &it0, int &it1) {
     if (n_items <= (int)gridDim.x) {
         // at most one item per block: consecutive blocks (spread over the SMs)
         // take consecutive items, however large
@@ -160,10 +168,10 @@ __device__ __forceinline__ void item_run(const int4 *__restrict__ items, int n_i
         return;
     }
     const long long total =
-        n_items > 0 ? (long long)items[n_items - 1].z + kItemCost * n_items : 0;
+        n_items > 0 ? (long long)items[n_items - 1].z + item_cost * n_items : 0;
     const long long c0 = total * blockIdx.x / gridDim.x;
     const long long c1 = total * (blockIdx.x + 1) / gridDim.x;
-    auto cost = [&](int i) { return (long long)items[i].y + kItemCost * i; };
+    auto cost = [&](int i) { return (long long)items[i].y + item_cost * i; };
     // level 1: sample i_t = (t + 1) * step - 1; the first index with cost >= c lies
     // in the step-wide bucket after the last sample below c
     const int nt = (int)blockDim.x;
@@ -185,6 +193,37 @@ __device__ __forceinline__ void item_run(const int4 *__restrict__ items, int n_i
     }
     it0 = min(n_items, lo0 + r0);
     it1 = blockIdx.x + 1 == gridDim.x ? n_items : min(n_items, lo1 + r1);
+}
+
+// The particles [begin, end) of one tile, of a block's run [it, it1) of items;
+// next_segment moves on to the next tile.  `next` holds the item it will start
+// from, loaded while the segment before is worked on.
+struct Segments {
+    const int4 *items;
+    int it, it1, pb;   // pb: the run's last particle + 1
+    int4 next;
+};
+__device__ __forceinline__ Segments run_segments(const int4 *__restrict__ items, int n_items,
+                                                 long long item_cost) {
+    Segments r;
+    r.items = items;
+    item_run(items, n_items, item_cost, r.it, r.it1);
+    r.next = make_int4(0, 0, 0, 0);
+    r.pb = 0;
+    if (r.it < r.it1) {
+        r.next = items[r.it];
+        r.pb = r.it1 < n_items ? items[r.it1].y : items[n_items - 1].z;
+    }
+    return r;
+}
+__device__ __forceinline__ bool next_segment(Segments &r, int &tile, int &begin, int &end) {
+    if (r.it >= r.it1) return false;
+    tile = r.next.x;
+    begin = r.next.y;
+    end = min(r.next.z, r.pb);
+    r.it = r.next.w;
+    if (r.it < r.it1) r.next = r.items[r.it];
+    return true;
 }
 
 // ----------------------------------------------------------------------------
@@ -236,7 +275,7 @@ cudaError_t launch_timeout_selftest(Ctrl *ctrl, cudaStream_t st);
 cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int4 *items,
                            int max_items, double qscale, float *rho, unsigned long long *rho64,
                            bool fixed, Ctrl *ctrl_w, int grid_blocks, int sparse_below,
-                           cudaStream_t st);
+                           int item_cost, cudaStream_t st);
 
 cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *rho, double qscale,
                               cudaStream_t st);
@@ -245,8 +284,8 @@ cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *r
 // items, like launch_push_deposit); advances the device step counter
 cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, bool fixed, bool deposit,
                         Ctrl *ctrl, const int4 *items, int max_items, float *rho,
-                        unsigned long long *rho64, double qscale, int sparse_below, double *part,
-                        int blocks, cudaStream_t st);
+                        unsigned long long *rho64, double qscale, int sparse_below, int item_cost,
+                        double *part, int blocks, cudaStream_t st);
 // dynamic shared memory of the fused push + deposit kernel for geometry g,
 // whether it stages E in shared memory, and the one-time attribute setting it
 // needs above 48 KiB
@@ -266,8 +305,8 @@ struct SaveY {
 cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, bool fixed,
                                 Ctrl *ctrl, const int4 *items, int max_items, const float4 *E4,
                                 const float4 *E8, float *rho, unsigned long long *rho64, double qscale,
-                                int sparse_below, double *part, int blocks, const SaveY &save,
-                                cudaStream_t st);
+                                int sparse_below, int item_cost, double *part, int blocks,
+                                const SaveY &save, cudaStream_t st);
 cudaError_t launch_gather_push(int64_t n, const Geom &g, const PushConst &pc, bool diag,
                                Ctrl *ctrl, const float4 *E8, double *part, int blocks,
                                int threads, cudaStream_t st);
@@ -329,7 +368,7 @@ struct PGrad {
 constexpr int kPGradTerms = 10;
 constexpr int kAdjPushMaxBlocks = kNumSMs * PIC_ADJ_MIN_BLOCKS * 2;
 cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, int max_items,
-                            const int32_t *ycell, const float *const yo[3], const float4 *E8,
+                            int item_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
                             float4 *lE4, float c_kick, float dt, float wz2, const AdjRhoTerm &rt,
                             const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, cudaStream_t st);
 // acc[q] += the fixed-order sum of the kPGradTerms partials of the blocks the
