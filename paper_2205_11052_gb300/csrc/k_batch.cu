@@ -496,8 +496,9 @@ cudaError_t launch_b_unload(int64_t o0, int64_t m, const InstDesc *desc, const l
 cudaError_t launch_b_sort(int64_t n, const InstDesc *desc, const long long *p0, int n_inst,
                           int ntiles, int chunk, Ctrl *ctrl, int32_t *bins, int32_t *scan_tmp,
                           int32_t *tile_items, int2 *tile_range, int4 *items, cudaStream_t st) {
-    cudaError_t e = staged_pass(n, BatchKey{desc, p0, n_inst}, ntiles, ctrl, bins, scan_tmp, st);
-    if (e != cudaSuccess) return e;
+    const PassEnd pe{n > 0 && ntiles <= kFusedBins, true, chunk, tile_items, tile_range, items};
+    cudaError_t e = staged_pass(n, BatchKey{desc, p0, n_inst}, ntiles, ctrl, bins, scan_tmp, pe, st);
+    if (e != cudaSuccess || pe.fused) return e;
     return launch_worklist(bins, ntiles, chunk, tile_items, tile_range, items, scan_tmp, ctrl,
                            n > 0 ? 1 : 0, st);
 }

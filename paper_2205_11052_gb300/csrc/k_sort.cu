@@ -25,7 +25,6 @@ namespace pic {
 
 namespace {
 
-constexpr int kScanThreads = 256;
 constexpr int kScanItems = 16;
 constexpr int kScanSeg = kScanThreads * kScanItems;   // 4096 elements per block
 
@@ -50,32 +49,6 @@ struct TileKey {
 };
 
 // ---- exclusive scan of int32 (in place), total written to data[n] -------------
-
-__device__ __forceinline__ int block_exclusive_scan(int val, int *total) {
-    __shared__ int warp_tot[kScanThreads / 32];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    int inc = val;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += t;
-    }
-    if (lane == 31) warp_tot[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-        int w = (lane < kScanThreads / 32) ? warp_tot[lane] : 0;
-        int wi = w;
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, wi, o);
-            if (lane >= o) wi += t;
-        }
-        if (lane < kScanThreads / 32) warp_tot[lane] = wi - w;   // exclusive warp offsets
-        if (lane == kScanThreads / 32 - 1) *total = wi;
-    }
-    __syncthreads();
-    const int r = warp_tot[wid] + inc - val;
-    __syncthreads();
-    return r;
-}
 
 __global__ void k_scan_reduce(const int32_t *__restrict__ data, int64_t n, int32_t *sums,
                               const int32_t *gate) {
@@ -158,7 +131,7 @@ __global__ void k_tile_ranges(const int32_t *__restrict__ bin_end, int ntiles, i
     const int s = (t == 0) ? 0 : bin_end[t - 1];
     const int e = bin_end[t];
     tile_range[t] = make_int2(s, e);
-    tile_items[t] = (e - s + chunk - 1) / chunk;
+    tile_items[t] = items_of(e - s, chunk);
 }
 
 __global__ void k_fill_items(int ntiles, int chunk, const int32_t *__restrict__ item_off,
@@ -168,18 +141,10 @@ __global__ void k_fill_items(int ntiles, int chunk, const int32_t *__restrict__ 
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t == 0) {
         ctrl->n_items = item_off[ntiles];
-        if (flip) ctrl->cur = 1 - ctrl->cur;    // particles now live in the other set
-        // a re-binning: every particle is back inside its tile
-        ctrl->rebins += 1;
-        ctrl->since_sort = 0;
-        ctrl->stray_step = 0ull;
+        rebinned(ctrl, flip != 0);
     }
     if (t >= ntiles) return;
-    const int2 r = tile_range[t];
-    const int o = item_off[t], cnt = r.y - r.x;
-    const int k = (cnt + chunk - 1) / chunk;
-    for (int i = 0; i < k; ++i)
-        items[o + i] = make_int4(t, r.x + (int)((long long)cnt * i / k), r.y, o + k);
+    fill_tile(t, tile_range[t], item_off[t], chunk, items);
 }
 
 __global__ void k_flip(Ctrl *ctrl) { ctrl->cur = 1 - ctrl->cur; }
@@ -205,31 +170,32 @@ cudaError_t launch_rebin_decide(Ctrl *ctrl, long long max_strays, int period, cu
     return cudaGetLastError();
 }
 
+namespace {
 // per-tile ranges from the bin ends left by a scatter, then the work items
+cudaError_t worklist(const int32_t *bin_end, int ntiles, int chunk, int32_t *tile_items,
+                     int2 *tile_range, int4 *items, int32_t *scan_tmp, Ctrl *ctrl, int flip,
+                     cudaStream_t st, const int32_t *gate) {
+    const int T = 256;
+    const int tb = (ntiles + T - 1) / T;
+    k_tile_ranges<<<tb, T, 0, st>>>(bin_end, ntiles, chunk, tile_items, tile_range, gate);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    if ((e = exclusive_scan_impl(tile_items, ntiles, scan_tmp, st, gate)) != cudaSuccess) return e;
+    k_fill_items<<<tb, T, 0, st>>>(ntiles, chunk, tile_items, tile_range, items, ctrl, flip, gate);
+    return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_worklist(const int32_t *bin_end, int ntiles, int chunk, int32_t *tile_items,
                             int2 *tile_range, int4 *items, int32_t *scan_tmp, Ctrl *ctrl, int flip,
                             cudaStream_t st) {
-    const int T = 256;
-    const int tb = (ntiles + T - 1) / T;
-    k_tile_ranges<<<tb, T, 0, st>>>(bin_end, ntiles, chunk, tile_items, tile_range, nullptr);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if ((e = exclusive_scan_impl(tile_items, ntiles, scan_tmp, st)) != cudaSuccess) return e;
-    k_fill_items<<<tb, T, 0, st>>>(ntiles, chunk, tile_items, tile_range, items, ctrl, flip,
-                                   nullptr);
-    return cudaGetLastError();
+    return worklist(bin_end, ntiles, chunk, tile_items, tile_range, items, scan_tmp, ctrl, flip, st,
+                    nullptr);
 }
 
 // One-time set-up outside any stream capture: the staged scatter's shared memory.
 cudaError_t sort_prepare() {
     return staged_prepare<TileKey>();
-}
-
-// histogram, scan and staged scatter by tile key >> shift (nb keys)
-cudaError_t sort_pass(int64_t n, const Geom &g, int shift, int64_t nb, Ctrl *ctrl, int32_t *bins,
-                      int32_t *scan_tmp, cudaStream_t st, SortRange rg = SortRange{0, 0},
-                      const int32_t *gate = nullptr) {
-    return staged_pass(n, TileKey{g, shift}, nb, ctrl, bins, scan_tmp, st, rg, gate);
 }
 
 // Shifts of the coarse passes that precede the full-key pass for particles in
@@ -253,9 +219,14 @@ int coarse_shifts(int ntiles, int *shifts) {
     return k;
 }
 
-int sort_launches(int64_t n, int ntiles, bool presort) {
+int presort_passes(int64_t ntiles) {
     int sh[32];
-    const int passes = (presort && n > 0) ? coarse_shifts(ntiles, sh) : 0;
+    return coarse_shifts((int)ntiles, sh);
+}
+
+int sort_launches(int64_t n, int64_t ntiles, bool presort) {
+    const int passes = (presort && n > 0) ? presort_passes(ntiles) : 0;
+    if (n > 0 && ntiles <= kFusedBins) return (passes + 1) * 2;   // histogram, scatter
     // per coarse pass: histogram, 3 scan, scatter, flip; then the full-key pass
     // (histogram, 3 scan, scatter) and the work list (ranges, 3 scan, fill)
     return passes * 6 + (n > 0 ? 10 : 8);
@@ -266,29 +237,28 @@ cudaError_t launch_sort(int64_t n, const Geom &g, int chunk, Ctrl *ctrl, int32_t
                         int2 *tile_range, int4 *items, bool presort, cudaStream_t st,
                         const int32_t *gate) {
     cudaError_t e;
+    const int nt = g.ntile[0] * g.ntile[1] * g.ntile[2];
+    const bool fused = n > 0 && nt <= kFusedBins;
     if (presort && n > 0) {
-        const int nt = g.ntile[0] * g.ntile[1] * g.ntile[2];
         int sh[32];
         const int passes = coarse_shifts(nt, sh);
         for (int p = 0; p < passes; ++p) {
-            if ((e = sort_pass(n, g, sh[p], ((nt - 1) >> sh[p]) + 1, ctrl, bins, scan_tmp, st)))
+            const PassEnd pe{fused, true, 0, nullptr, nullptr, nullptr};
+            if ((e = staged_pass(n, TileKey{g, sh[p]}, ((nt - 1) >> sh[p]) + 1, ctrl, bins, scan_tmp,
+                                 pe, st)))
                 return e;
+            if (fused) continue;
             k_flip<<<1, 1, 0, st>>>(ctrl);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     }
-    if ((e = sort_pass(n, g, 0, nbins, ctrl, bins, scan_tmp, st, SortRange{0, 0}, gate)) !=
-        cudaSuccess)
+    const PassEnd pe{fused, true, chunk, tile_items, tile_range, items};
+    if ((e = staged_pass(n, TileKey{g, 0}, nbins, ctrl, bins, scan_tmp, pe, st, SortRange{0, 0},
+                         gate)) != cudaSuccess)
         return e;
-    const int T = 256;
-    const int ntiles = g.ntile[0] * g.ntile[1] * g.ntile[2];
-    const int tb = (ntiles + T - 1) / T;
-    k_tile_ranges<<<tb, T, 0, st>>>(bins, ntiles, chunk, tile_items, tile_range, gate);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = exclusive_scan_impl(tile_items, ntiles, scan_tmp, st, gate)) != cudaSuccess) return e;
-    k_fill_items<<<tb, T, 0, st>>>(ntiles, chunk, tile_items, tile_range, items, ctrl,
-                                   n > 0 ? 1 : 0, gate);
-    return cudaGetLastError();
+    if (fused) return cudaSuccess;
+    return worklist(bins, nt, chunk, tile_items, tile_range, items, scan_tmp, ctrl, n > 0 ? 1 : 0,
+                    st, gate);
 }
 
 // Coarse passes and the full-key pass over particles [o, o + n) alone, set
@@ -309,9 +279,11 @@ cudaError_t launch_sort_range(int64_t n, int64_t o, const Geom &g, Ctrl *ctrl, i
     cudaError_t e;
     for (int p = 0; p <= k; ++p) {
         const int64_t nb = p < k ? ((nt - 1) >> sh[p]) + 1 : nbins;
-        if ((e = sort_pass(n, g, sh[p], nb, ctrl, bins, scan_tmp, st, SortRange{o, p & 1})))
+        const PassEnd pe{nt <= kFusedBins, false, 0, nullptr, nullptr, nullptr};
+        if ((e = staged_pass(n, TileKey{g, sh[p]}, nb, ctrl, bins, scan_tmp, pe, st,
+                             SortRange{o, p & 1})))
             return e;
-        *kernels += 5;
+        *kernels += pe.fused ? 2 : 5;
     }
     *passes = k + 1;
     return cudaSuccess;

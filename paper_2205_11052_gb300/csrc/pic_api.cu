@@ -325,7 +325,7 @@ int do_sort(pic_ctx *c, bool presort = false) {
                          c->at<int32_t>(c->lay.tile_items), c->at<int2>(c->lay.tile_range),
                          c->at<int4>(c->lay.items), presort, c->st));
     c->since_sort = 0;
-    return timer_end(c, PIC_PHASE_SORT, sort_launches(c->np, (int)c->ntiles, presort));
+    return timer_end(c, PIC_PHASE_SORT, sort_launches(c->np, c->ntiles, presort));
 }
 
 // stray-triggered re-binning: the device decides (from the last push's strays
@@ -339,7 +339,7 @@ int do_sort_gated(pic_ctx *c) {
                          c->nbins, c->at<int32_t>(c->lay.scan_tmp),
                          c->at<int32_t>(c->lay.tile_items), c->at<int2>(c->lay.tile_range),
                          c->at<int4>(c->lay.items), false, c->st, &c->ctrl()->rebin));
-    return timer_end(c, PIC_PHASE_SORT, 1 + sort_launches(c->np, (int)c->ntiles, false));
+    return timer_end(c, PIC_PHASE_SORT, 1 + sort_launches(c->np, c->ntiles, false));
 }
 
 int do_deposit(pic_ctx *c) {
@@ -1018,11 +1018,6 @@ void pic_destroy(pic_handle_t c) {
 
 namespace {
 
-// coarse passes the first binning of particles in arbitrary order needs
-int presort_passes(const pic_ctx *c) {
-    return (sort_launches(1, (int)c->ntiles, true) - sort_launches(1, (int)c->ntiles, false)) / 6;
-}
-
 int load_overlapped(pic_ctx *c, const double *mx, const double *mv, int64_t n) {
     if (!c->side_made) {
         PIC_CUDA(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
@@ -1071,7 +1066,7 @@ int pic_load_particles(pic_handle_t c, const double *x, const double *v, int64_t
     const double *mv = mx ? static_cast<const double *>(mapped_host(v, (size_t)n * 24)) : nullptr;
     if (src_is_device) {
         PIC_CUDA(launch_load(x, v, n, 0, c->geom, c->inv_h, c->prm.dt, c->ctrl(), c->st));
-    } else if (mx && mv && n >= kOverlapMin && presort_passes(c) > 0) {
+    } else if (mx && mv && n >= kOverlapMin && presort_passes(c->ntiles) > 0) {
         // page-locked host arrays, read in place by the load kernel one range
         // at a time on one block per SM (the host link, not the SMs, bounds
         // it); each loaded range is binned on the side stream meanwhile, so

@@ -49,6 +49,7 @@ struct Ctrl {
     long long rebins;
     int32_t since_sort;
     int32_t rebin;
+    unsigned int done[2];   // blocks done, of the histogram and the scatter (0 between launches)
     int32_t cur;            // which ParticleSet holds the particles
     int32_t pad0;
     ParticleSet sets[2];
@@ -262,7 +263,8 @@ cudaError_t launch_sort(int64_t n, const Geom &g, int chunk, Ctrl *ctrl, int32_t
 // ctrl->stray_step > max_strays; clears ctrl->stray_step
 cudaError_t launch_rebin_decide(Ctrl *ctrl, long long max_strays, int period, cudaStream_t st);
 // kernels launch_sort issues
-int sort_launches(int64_t n, int ntiles, bool presort);
+int sort_launches(int64_t n, int64_t ntiles, bool presort);
+int presort_passes(int64_t ntiles);   // coarse passes of a presort
 // coarse passes + full-key pass over particles [o, o + n) of the current set
 // (which stays unchanged); the range ends in set cur ^ (*passes & 1)
 cudaError_t launch_sort_range(int64_t n, int64_t o, const Geom &g, Ctrl *ctrl, int32_t *bins,

@@ -16,6 +16,111 @@ namespace pic {
 
 namespace {
 
+constexpr int kScanThreads = 256;
+
+__device__ __forceinline__ int block_exclusive_scan(int val, int *total) {
+    __shared__ int warp_tot[kScanThreads / 32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int inc = val;
+    for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += t;
+    }
+    if (lane == 31) warp_tot[wid] = inc;
+    __syncthreads();
+    if (wid == 0) {
+        int w = (lane < kScanThreads / 32) ? warp_tot[lane] : 0;
+        int wi = w;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, wi, o);
+            if (lane >= o) wi += t;
+        }
+        if (lane < kScanThreads / 32) warp_tot[lane] = wi - w;   // exclusive warp offsets
+        if (lane == kScanThreads / 32 - 1) *total = wi;
+    }
+    __syncthreads();
+    const int r = warp_tot[wid] + inc - val;
+    __syncthreads();
+    return r;
+}
+
+// What the last block of a pass does besides: the histogram's scans its counts
+// into bin starts (and, for the full-key pass, lays out the work items), the
+// scatter's flips the current set.  One launch each instead of eleven per
+// re-binning (three of a scan twice, ranges, items): those took 30 of 38 us a
+// re-binning of 33k particles.  One block walks the bins, so passes of more than
+// kFusedBins keys keep the separate kernels (fused = false).  A step of 33k
+// particles that re-bins: 131 -> 97 us.
+constexpr int kFusedBins = 1 << 15;
+struct PassEnd {
+    bool fused;
+    bool flip;             // the scatter's last block flips ctrl->cur
+    int chunk;             // > 0: build the work list (particles per item)
+    int32_t *tile_items;   // first item of each tile, total last
+    int2 *tile_range;      // particles of each tile
+    int4 *items;
+};
+
+// Whether this block is the last of its grid to get here (the same answer for
+// every thread); the counter wraps to zero for the next launch.
+__device__ __forceinline__ bool last_block(unsigned int *done) {
+    __shared__ int last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    __threadfence();
+    return last != 0;
+}
+
+__device__ __forceinline__ int items_of(int cnt, int chunk) { return (cnt + chunk - 1) / chunk; }
+
+// counts -> exclusive starts in place, ranges and first items per tile; one
+// block of kScanThreads, each thread a contiguous run of bins
+__device__ __forceinline__ void finish_bins(int32_t *bins, int nb, const PassEnd &pe, Ctrl *ctrl) {
+    __shared__ int tot;
+    const int per = ((nb + kScanThreads - 1) / kScanThreads + 3) & ~3;
+    const int t0 = threadIdx.x * per, t1 = min(nb, t0 + per);
+    int cnt = 0, it = 0;
+    for (int t = t0; t < t1; ++t) {
+        const int k = __ldcg(bins + t);
+        cnt += k;
+        if (pe.chunk > 0) it += items_of(k, pe.chunk);
+    }
+    int run = block_exclusive_scan(cnt, &tot);
+    int item = pe.chunk > 0 ? block_exclusive_scan(it, &tot) : 0;
+    for (int t = t0; t < t1; ++t) {
+        const int k = __ldcg(bins + t);
+        bins[t] = run;
+        if (pe.chunk > 0) {
+            pe.tile_range[t] = make_int2(run, run + k);
+            pe.tile_items[t] = item;
+            item += items_of(k, pe.chunk);
+        }
+        run += k;
+    }
+    if (pe.chunk > 0 && threadIdx.x == 0) {
+        pe.tile_items[nb] = tot;
+        ctrl->n_items = tot;
+    }
+}
+
+// tile t's items: begins of equal shares of its particles, the tile's end and
+// the next tile's first item
+__device__ __forceinline__ void fill_tile(int t, int2 r, int o, int chunk, int4 *items) {
+    const int cnt = r.y - r.x, k = items_of(cnt, chunk);
+    for (int i = 0; i < k; ++i)
+        items[o + i] = make_int4(t, r.x + (int)((long long)cnt * i / k), r.y, o + k);
+}
+
+// a re-binning is complete: the particles are in the other set, each inside its tile
+__device__ __forceinline__ void rebinned(Ctrl *ctrl, bool flip) {
+    if (flip) ctrl->cur = 1 - ctrl->cur;
+    ctrl->rebins += 1;
+    ctrl->since_sort = 0;
+    ctrl->stray_step = 0ull;
+}
+
 // Lanes of a warp whose keys form a contiguous run (consecutive lanes, equal
 // keys; binned particles arrive in such runs) share shared-table updates:
 // the run's first lane does one update for the whole run.
@@ -114,8 +219,8 @@ struct SortRange {
 
 template <class Key>
 __global__ void __launch_bounds__(256) k_scatter_staged(int64_t n, Key key_param, Ctrl *ctrl,
-                                                         int32_t *bins, SortRange rg,
-                                                         const int32_t *gate) {
+                                                         int32_t *bins, int nb, SortRange rg,
+                                                         PassEnd pe, const int32_t *gate) {
     if (gate && !*gate) return;
     Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
     extern __shared__ __align__(128) unsigned char smem[];
@@ -135,6 +240,16 @@ __global__ void __launch_bounds__(256) k_scatter_staged(int64_t n, Key key_param
     const ParticleSet dst = offset_set(ctrl->sets[1 - cur], rg.o);
     const int64_t nslices = (n + kStage - 1) / kStage;
     int bad = 0;
+    if (pe.fused && pe.chunk > 0)
+        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nb; t += gridDim.x * blockDim.x)
+            fill_tile(t, pe.tile_range[t], pe.tile_items[t], pe.chunk, pe.items);
+    // every block has read ctrl->cur by the time it gets here
+    auto finish = [&]() {
+        if (pe.fused && pe.flip && last_block(&ctrl->done[1]) && threadIdx.x == 0) {
+            if (pe.chunk > 0) rebinned(ctrl, true);
+            else ctrl->cur = 1 - ctrl->cur;
+        }
+    };
     if (threadIdx.x == 0) {
         mbar_init(&bar[0], 1);
         mbar_init(&bar[1], 1);
@@ -174,6 +289,7 @@ __global__ void __launch_bounds__(256) k_scatter_staged(int64_t n, Key key_param
             if (__syncthreads_or(!ok)) {
                 if (threadIdx.x == 0) atomicOr(&ctrl->flags, PIC_FLAG_TIMEOUT);
                 mbar_wait(&bar[b], phase[b] ^ 1u);   // one more bounded wait for the copies
+                finish();
                 return;
             }
         } else {
@@ -290,39 +406,41 @@ __global__ void __launch_bounds__(256) k_scatter_staged(int64_t n, Key key_param
         __syncthreads();   // buffer b and the table are free again
     }
     if (bad) atomicOr(&ctrl->flags, PIC_FLAG_BAD_CELL);
+    finish();
 }
 
 // Histogram with the same per-slice aggregation: counts of the slice's
 // distinct tiles in a shared hash table, one global atomic per tile and
 // slice (per-warp aggregated atomics when the table overflows).
-template <class Key>
+template <class Key, int PER>
 __global__ void __launch_bounds__(256) k_histogram_staged(int64_t n, Key key_param, Ctrl *ctrl,
-                                                           int32_t *bins, SortRange rg,
-                                                           const int32_t *gate) {
+                                                           int32_t *bins, int nb, SortRange rg,
+                                                           PassEnd pe, const int32_t *gate) {
     if (gate && !*gate) return;
     Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
     __shared__ int32_t hkey[kHash];
     __shared__ int32_t hcnt[kHash];
     const ParticleSet ps = offset_set(ctrl->sets[ctrl->cur ^ rg.rel], rg.o);
-    const int64_t nslices = (n + kHistStage - 1) / kHistStage;
+    constexpr int SL = 256 * PER;   // particles per slice
+    const int64_t nslices = (n + SL - 1) / SL;
     int bad = 0;
     for (int64_t sl = blockIdx.x; sl < nslices; sl += gridDim.x) {
-        const int64_t s0 = sl * kHistStage;
-        const int m = (int)(s0 + kHistStage <= n ? kHistStage : n - s0);
+        const int64_t s0 = sl * SL;
+        const int m = (int)(s0 + SL <= n ? SL : n - s0);
         for (int h = threadIdx.x; h < kHash; h += blockDim.x) {
             hkey[h] = -1;
             hcnt[h] = 0;
         }
         __syncthreads();
-        // the slice's cells first (kHistStage / 256 loads in flight per thread)
-        int32_t cv[kHistPer];
+        // the slice's cells first (PER loads in flight per thread)
+        int32_t cv[PER];
 #pragma unroll
-        for (int u = 0; u < kHistPer; ++u) {
+        for (int u = 0; u < PER; ++u) {
             const int j = u * 256 + threadIdx.x;
             cv[u] = j < m ? __ldcs(ps.cell + s0 + j) : 0;
         }
 #pragma unroll
-        for (int u = 0; u < kHistPer; ++u) {
+        for (int u = 0; u < PER; ++u) {
             const int j = u * 256 + threadIdx.x;
             const bool act = j < m;
             const int lane = threadIdx.x & 31;
@@ -340,6 +458,7 @@ __global__ void __launch_bounds__(256) k_histogram_staged(int64_t n, Key key_par
         __syncthreads();
     }
     if (bad) atomicOr(&ctrl->flags, PIC_FLAG_BAD_CELL);
+    if (pe.fused && last_block(&ctrl->done[0])) finish_bins(bins, nb, pe, ctrl);
 }
 
 
@@ -347,23 +466,28 @@ __global__ void __launch_bounds__(256) k_histogram_staged(int64_t n, Key key_par
 // into the same range of the other set; nb keys (bins holds nb + 1 ints).
 template <class Key>
 cudaError_t staged_pass(int64_t n, const Key &key_of, int64_t nb, Ctrl *ctrl, int32_t *bins,
-                        int32_t *scan_tmp, cudaStream_t st, SortRange rg = SortRange{0, 0},
-                        const int32_t *gate = nullptr) {
+                        int32_t *scan_tmp, const PassEnd &pe, cudaStream_t st,
+                        SortRange rg = SortRange{0, 0}, const int32_t *gate = nullptr) {
     cudaError_t e = cudaMemsetAsync(bins, 0, sizeof(int32_t) * (size_t)(nb + 1), st);
     if (e != cudaSuccess) return e;
     const int T = 256;
     if (n > 0) {
-        const int hblocks = (int)std::min<int64_t>((n + kHistStage - 1) / kHistStage, 152 * 8);
-        k_histogram_staged<Key><<<hblocks, T, 0, st>>>(n, key_of, ctrl, bins, rg, gate);
+        // short slices while long ones would leave SMs without one
+        const int per = n <= (int64_t)kNumSMs * kHistStage ? 4 : kHistPer;
+        const int64_t slice = 256 * per;
+        const int hblocks = (int)std::min<int64_t>((n + slice - 1) / slice, kNumSMs * 8);
+        if (per == 4) k_histogram_staged<Key, 4><<<hblocks, T, 0, st>>>(n, key_of, ctrl, bins, (int)nb, rg, pe, gate);
+        else k_histogram_staged<Key, kHistPer><<<hblocks, T, 0, st>>>(n, key_of, ctrl, bins, (int)nb, rg, pe, gate);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    if ((e = exclusive_scan(bins, nb, scan_tmp, st, gate)) != cudaSuccess) return e;
+    if (!(pe.fused && n > 0) && (e = exclusive_scan(bins, nb, scan_tmp, st, gate)) != cudaSuccess)
+        return e;
     if (n > 0) {
         // resident blocks per SM as the staging buffer allows (228 KB per SM)
         const int per_sm =
             (int)std::max<size_t>(1, std::min<size_t>(8, (228 * 1024) / (kStageSmem + 1024)));
         const int sblocks = (int)std::min<int64_t>((n + kStage - 1) / kStage, 152 * per_sm);
-        k_scatter_staged<Key><<<sblocks, T, kStageSmem, st>>>(n, key_of, ctrl, bins, rg, gate);
+        k_scatter_staged<Key><<<sblocks, T, kStageSmem, st>>>(n, key_of, ctrl, bins, (int)nb, rg, pe, gate);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
