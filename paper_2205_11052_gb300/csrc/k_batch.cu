@@ -386,19 +386,8 @@ __global__ void __launch_bounds__(256) k_b_diag_field(const InstDesc *__restrict
         ff_add_sq(hi[2], lo[2], e.z);
         ff_add(hi[3], lo[3], rho[q]);
     }
-    __shared__ double red[4][8];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int q = 0; q < 4; ++q) {
-        double t = (double)hi[q] + (double)lo[q];
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-        if (lane == 0) red[q][wid] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x < 4) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[threadIdx.x][w];
-        fpart[4 * ((int64_t)blockIdx.x * kBatchDiagBlocks + blockIdx.y) + threadIdx.x] = t;
-    }
+    block_field_sums<256>(hi, lo,
+                          fpart + 4 * ((int64_t)blockIdx.x * kBatchDiagBlocks + blockIdx.y));
 }
 
 // One record per instance, one block each: the instance's items are

@@ -1,0 +1,394 @@
+// Field solve (Section 3.1 step 2, Eq. potential; Section 3.2 of
+// arXiv 2205.11052) of grids whose three axes are at most kFftMaxN long, in
+// three kernels around the line transforms of fft.cuh:
+//   k_fft_x_forward   rows of rho -> spectra over x (two real rows per complex
+//                     line), stored by x frequency: rho_hat[kx][z][y]
+//   k_fft_yz          one (y, z) plane of one x frequency and one component per
+//                     block, in shared memory: forward over y and z, the Green
+//                     kernel of k_green, back over z and y
+//   k_fft_x_backward  rows of the three components -> E4, its x-paired copy E8
+//                     and, when asked, the block's partial field sums
+// The adjoint's solve runs the mirrored kernels (three components forward, the
+// conjugate symbol, one density backward).
+//
+// Around cuFFT the same solve took eleven launches: its transforms over one axis
+// each (six), the Green kernel, the interleaving, the pairing and the field sums,
+// each a pass over memory: 20 steps with records of 16^3 x 8 took 1.95 ms, now 1.47,
+// of 64^3 x 16 4.22, now 3.59.
+#include <math.h>
+
+#include <algorithm>
+
+#include "ffsum.cuh"
+#include "fft.cuh"
+#include "pic_internal.cuh"
+
+namespace pic {
+
+namespace {
+
+using fft::lines;
+
+constexpr int kRowsF = 32;   // rows of one plane per block of the forward x kernel
+constexpr int kRowsB = 16;   // of the backward one
+constexpr int kXThreads = 128;
+
+__device__ __forceinline__ void load_twiddles(float2 *tw, const FftTables *tab, int axis, int n) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) tw[i] = tab->tw[axis][i];
+}
+
+// The spectra of the two real rows packed in a complex line: Z = A + i B, with
+// A(k) = (Z(k) + Z*(n - k)) / 2 and B(k) = (Z(k) - Z*(n - k)) / (2 i).
+__device__ __forceinline__ void unpack_rows(float2 z, float2 m, float2 &a, float2 &b) {
+    a = make_float2(0.5f * (z.x + m.x), 0.5f * (z.y - m.y));
+    b = make_float2(0.5f * (z.y + m.y), 0.5f * (m.x - z.x));
+}
+
+// COMPS = 1: rows of rho (float).  COMPS = 3: rows of the three components of
+// lE4, which is cleared for the next reverse push.
+template <int COMPS>
+__global__ void __launch_bounds__(kXThreads) k_fft_x_forward(int ny, int nz, int nh, FftAxis ax,
+                                                             const FftTables *__restrict__ tab,
+                                                             const float *__restrict__ rho,
+                                                             float4 *__restrict__ lE4,
+                                                             float2 *__restrict__ out, int64_t nhalf) {
+    constexpr int ROWS = COMPS == 1 ? kRowsF : kRowsB;
+    constexpr int PAIRS = ROWS / 2;
+    extern __shared__ float2 sm[];
+    const int n = ax.n, pitch = n | 1;
+    float2 *s = sm, *tw = sm + COMPS * PAIRS * pitch;
+    const int z = blockIdx.y, y0 = blockIdx.x * ROWS, rows = min(ROWS, ny - y0);
+    load_twiddles(tw, tab, 0, n);
+    float *sf = reinterpret_cast<float *>(s);
+    for (int w = threadIdx.x; w < ROWS * n; w += kXThreads) {
+        const int r = w / n, x = w - r * n;
+        const int64_t g = ((int64_t)z * ny + y0 + r) * n + x;
+        float v[3] = {0.f, 0.f, 0.f};
+        if (r < rows) {
+            if (COMPS == 1) {
+                v[0] = rho[g];
+            } else {
+                const float4 e = lE4[g];
+                v[0] = e.x;
+                v[1] = e.y;
+                v[2] = e.z;
+                lE4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+#pragma unroll
+        for (int d = 0; d < COMPS; ++d) sf[2 * ((d * PAIRS + (r >> 1)) * pitch + x) + (r & 1)] = v[d];
+    }
+    __syncthreads();
+    lines<false>(s, COMPS * PAIRS, pitch, 1, ax, tw);
+    // lanes over the rows: runs of ROWS values at one frequency
+    for (int w = threadIdx.x; w < COMPS * nh * PAIRS; w += kXThreads) {
+        const int q = w % PAIRS, u = w / PAIRS;
+        const int d = u / nh, k = u - d * nh;
+        const float2 *line = s + (d * PAIRS + q) * pitch;
+        float2 a, b;
+        unpack_rows(line[tab->pos[0][k]], line[tab->pos[0][k == 0 ? 0 : n - k]], a, b);
+        float2 *o = out + d * nhalf + ((int64_t)k * nz + z) * ny + y0;
+        if (2 * q < rows) o[2 * q] = a;
+        if (2 * q + 1 < rows) o[2 * q + 1] = b;
+    }
+}
+
+// plane of one x frequency: [z][y] in global memory, pitch ny | 1 in shared
+__device__ __forceinline__ void load_plane(float2 *s, const float2 *__restrict__ in, int ny, int nz,
+                                           int pitch) {
+    for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
+        const int z = w / ny;
+        s[z * pitch + (w - z * ny)] = in[w];
+    }
+}
+
+// out_d = symbol_d(in) over one plane (blockIdx.x: x frequency, blockIdx.y: d)
+__global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, FftAxis ay, FftAxis az,
+                                                const FftTables *__restrict__ tab,
+                                                const float *__restrict__ ktab, float inv_ng,
+                                                const float2 *__restrict__ in,
+                                                float2 *__restrict__ out, int64_t nhalf, int mi, int mj,
+                                                int mk, int mode_comp, int mode_conj, Ctrl *ctrl) {
+    extern __shared__ float2 sm[];
+    const int pitch = ny | 1, a = blockIdx.x, d = blockIdx.y;
+    float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
+    load_twiddles(twy, tab, 1, ny);
+    load_twiddles(twz, tab, 2, nz);
+    load_plane(s, in + (int64_t)a * ny * nz, ny, nz, pitch);
+    __syncthreads();
+    lines<false>(s, nz, pitch, 1, ay, twy);
+    lines<false>(s, ny, 1, pitch, az, twz);
+    const float kx = ktab[a];
+    const float gx = ((nx & 1) == 0 && a == nx / 2) ? 0.0f : kx;
+    for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
+        const int pz = w / ny, py = w - pz * ny;
+        const int b = tab->freq[1][py], c = tab->freq[2][pz];
+        const float ky = ktab[nh + b], kz = ktab[nh + ny + c];
+        const float gy = ((ny & 1) == 0 && b == ny / 2) ? 0.0f : ky;
+        const float gz = ((nz & 1) == 0 && c == nz / 2) ? 0.0f : kz;
+        float2 &e = s[pz * pitch + py];
+        const float2 rh = e;
+        float2 v = make_float2(0.f, 0.f);
+        if ((a | b | c) != 0) {
+            const float sc = inv_ng / (kx * kx + ky * ky + kz * kz) * (d == 0 ? gx : (d == 1 ? gy : gz));
+            v = make_float2(sc * rh.y, -sc * rh.x);   // -i g rh
+        }
+        e = v;
+        if (d == mode_comp && a == mi && b == mj && c == mk) {
+            ctrl->mode[0] = (double)v.x;
+            ctrl->mode[1] = mode_conj ? -(double)v.y : (double)v.y;
+        }
+    }
+    __syncthreads();
+    lines<true>(s, ny, 1, pitch, az, twz);
+    lines<true>(s, nz, pitch, 1, ay, twy);
+    float2 *o = out + d * nhalf + (int64_t)a * ny * nz;
+    for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
+        const int z = w / ny;
+        o[w] = s[z * pitch + (w - z * ny)];
+    }
+}
+
+// lrho^ = sum_d (+i g_d / |k|^2) lE^_d / N_g of one x frequency: three planes
+// forward, summed in global memory (each element by one thread), one plane back
+__global__ void __launch_bounds__(512) k_fft_yz_adj(int nx, int ny, int nz, int nh, FftAxis ay,
+                                                    FftAxis az, const FftTables *__restrict__ tab,
+                                                    const float *__restrict__ ktab, float inv_ng,
+                                                    const float2 *__restrict__ in,
+                                                    float2 *__restrict__ out, int64_t nhalf) {
+    extern __shared__ float2 sm[];
+    const int pitch = ny | 1, a = blockIdx.x;
+    float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
+    load_twiddles(twy, tab, 1, ny);
+    load_twiddles(twz, tab, 2, nz);
+    float2 *o = out + (int64_t)a * ny * nz;
+    const float kx = ktab[a];
+    for (int d = 0; d < 3; ++d) {
+        __syncthreads();
+        load_plane(s, in + d * nhalf + (int64_t)a * ny * nz, ny, nz, pitch);
+        __syncthreads();
+        lines<false>(s, nz, pitch, 1, ay, twy);
+        lines<false>(s, ny, 1, pitch, az, twz);
+        for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
+            const int pz = w / ny, py = w - pz * ny;
+            const int b = tab->freq[1][py], c = tab->freq[2][pz];
+            const float ky = ktab[nh + b], kz = ktab[nh + ny + c];
+            float g = d == 0 ? kx : (d == 1 ? ky : kz);
+            const int m = d == 0 ? a : (d == 1 ? b : c), n = d == 0 ? nx : (d == 1 ? ny : nz);
+            if ((n & 1) == 0 && m == n / 2) g = 0.0f;
+            const float2 e = s[pz * pitch + py];
+            float2 v = make_float2(-g * e.y, g * e.x);   // +i g e
+            if (d > 0) v = fft::cadd(v, o[w]);
+            if (d == 2) {
+                const float sc = (a | b | c) != 0 ? inv_ng / (kx * kx + ky * ky + kz * kz) : 0.0f;
+                s[pz * pitch + py] = make_float2(sc * v.x, sc * v.y);
+            } else {
+                o[w] = v;
+            }
+        }
+    }
+    __syncthreads();
+    lines<true>(s, ny, 1, pitch, az, twz);
+    lines<true>(s, nz, pitch, 1, ay, twy);
+    for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
+        const int z = w / ny;
+        o[w] = s[z * pitch + (w - z * ny)];
+    }
+}
+
+// rows y0.. of plane z of COMPS components, from spectra by x frequency to two
+// real rows per complex line in shared memory
+template <int COMPS>
+__device__ __forceinline__ void rows_backward(float2 *s, float2 *tw, const float2 *__restrict__ in,
+                                              int64_t nhalf, int ny, int nz, int nh, int z, int y0,
+                                              int rows, const FftAxis &ax,
+                                              const FftTables *__restrict__ tab) {
+    constexpr int PAIRS = kRowsB / 2;
+    const int n = ax.n, pitch = n | 1;
+    load_twiddles(tw, tab, 0, n);
+    for (int w = threadIdx.x; w < COMPS * nh * PAIRS; w += kXThreads) {
+        const int q = w % PAIRS, u = w / PAIRS;
+        const int d = u / nh, k = u - d * nh;
+        const float2 *p = in + d * nhalf + ((int64_t)k * nz + z) * ny + y0;
+        float2 a = make_float2(0.f, 0.f), b = a;
+        if (2 * q < rows) a = p[2 * q];
+        if (2 * q + 1 < rows) b = p[2 * q + 1];
+        if (k == 0 || 2 * k == n) a.y = b.y = 0.0f;   // real for a real row
+        float2 *line = s + (d * PAIRS + q) * pitch;
+        line[tab->pos[0][k]] = make_float2(a.x - b.y, a.y + b.x);   // A + i B
+        if (k != 0 && 2 * k != n)
+            line[tab->pos[0][n - k]] = make_float2(a.x + b.y, b.x - a.y);   // A* + i B*
+    }
+    __syncthreads();
+    lines<true>(s, COMPS * PAIRS, pitch, 1, ax, tw);
+}
+
+__global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, int nh, FftAxis ax,
+                                                              const FftTables *__restrict__ tab,
+                                                              const float2 *__restrict__ in,
+                                                              int64_t nhalf, float4 *__restrict__ E4,
+                                                              float4 *__restrict__ E8,
+                                                              const float *__restrict__ rho,
+                                                              double *__restrict__ fpart) {
+    constexpr int PAIRS = kRowsB / 2;
+    extern __shared__ float2 sm[];
+    const int n = ax.n, pitch = n | 1;
+    const int z = blockIdx.y, y0 = blockIdx.x * kRowsB, rows = min(kRowsB, ny - y0);
+    rows_backward<3>(sm, sm + 3 * PAIRS * pitch, in, nhalf, ny, nz, nh, z, y0, rows, ax, tab);
+    const float *sf = reinterpret_cast<const float *>(sm);
+    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int w = threadIdx.x; w < rows * n; w += kXThreads) {
+        const int r = w / n, x = w - r * n, x1 = x + 1 == n ? 0 : x + 1;
+        const float *f0 = sf + 2 * ((r >> 1) * pitch) + (r & 1);
+        const float *f1 = f0 + 2 * PAIRS * pitch, *f2 = f1 + 2 * PAIRS * pitch;
+        const float4 e = make_float4(f0[2 * x], f1[2 * x], f2[2 * x], 0.0f);
+        const int64_t g = ((int64_t)z * ny + y0 + r) * n + x;
+        E4[g] = e;
+        E8[2 * g] = e;
+        E8[2 * g + 1] = make_float4(f0[2 * x1], f1[2 * x1], f2[2 * x1], 0.0f);
+        if (fpart) {
+            ff_add_sq(hi[0], lo[0], e.x);
+            ff_add_sq(hi[1], lo[1], e.y);
+            ff_add_sq(hi[2], lo[2], e.z);
+            ff_add(hi[3], lo[3], rho[g]);
+        }
+    }
+    if (fpart) block_field_sums<kXThreads>(hi, lo, fpart + 4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x));
+}
+
+// lrho rows -> the x-paired copy read by the deposit-term gathers; the largest
+// |lrho| goes to adj_lrho[par], and the slots of the next reverse push are cleared
+__global__ void __launch_bounds__(kXThreads) k_fft_x_backward_adj(int ny, int nz, int nh, FftAxis ax,
+                                                                  const FftTables *__restrict__ tab,
+                                                                  const float2 *__restrict__ in,
+                                                                  float2 *__restrict__ lrho2, Ctrl *ctrl,
+                                                                  int par) {
+    constexpr int PAIRS = kRowsB / 2;
+    extern __shared__ float2 sm[];
+    const int n = ax.n, pitch = n | 1;
+    const int z = blockIdx.y, y0 = blockIdx.x * kRowsB, rows = min(kRowsB, ny - y0);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+        ctrl->adj_ly[par ^ 1] = 0u;
+        ctrl->adj_lv[par ^ 1] = 0u;
+    }
+    rows_backward<1>(sm, sm + PAIRS * pitch, in, 0, ny, nz, nh, z, y0, rows, ax, tab);
+    const float *sf = reinterpret_cast<const float *>(sm);
+    float m = 0.0f;
+    for (int w = threadIdx.x; w < rows * n; w += kXThreads) {
+        const int r = w / n, x = w - r * n, x1 = x + 1 == n ? 0 : x + 1;
+        const float *f = sf + 2 * ((r >> 1) * pitch) + (r & 1);
+        lrho2[((int64_t)z * ny + y0 + r) * n + x] = make_float2(f[2 * x], f[2 * x1]);
+        m = fmaxf(m, fabsf(f[2 * x]));
+    }
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(&ctrl->adj_lrho[par], __float_as_uint(m));
+}
+
+// Split n into the radices of fft.cuh, fewest stages first, or one with a
+// larger prime up to kFftMaxPrime.
+void split(int m, int depth, int *cur, int &best, int &best_sum, FftAxis &a) {
+    if (m == 1) {
+        int sum = 0;
+        for (int i = 0; i < depth; ++i) sum += cur[i];
+        if (depth < best || (depth == best && sum < best_sum)) {
+            best = depth;
+            best_sum = sum;
+            a.stages = depth;
+            for (int i = 0; i < depth; ++i) a.radix[i] = cur[i];
+        }
+        return;
+    }
+    if (depth >= kFftMaxStages) return;
+    for (int r = std::min(m, kFftMaxPrime); r >= 2; --r) {
+        if (m % r != 0 || (depth > 0 && r > cur[depth - 1])) continue;
+        const bool prime = r != 4 && r != 6 && r != 9 && r % 2 != 0 && (r == 3 || r % 3 != 0) &&
+                           (r == 5 || r % 5 != 0);   // among r <= 31, none else is odd and composite
+        if (!(r <= 8 || r == 16 || prime)) continue;
+        cur[depth] = r;
+        split(m / r, depth + 1, cur, best, best_sum, a);
+    }
+}
+
+size_t yz_smem(const Geom &g) {
+    return sizeof(float2) * ((size_t)g.n[2] * (g.n[1] | 1) + g.n[1] + g.n[2]);
+}
+size_t x_smem(const Geom &g, int line_count) {
+    return sizeof(float2) * ((size_t)line_count * (g.n[0] | 1) + g.n[0]);
+}
+int yz_threads(const Geom &g) {
+    const int pts = g.n[1] * g.n[2];
+    return pts >= 2048 ? 512 : (pts >= 512 ? 256 : 128);
+}
+
+}  // namespace
+
+bool fft_axis(int n, FftAxis &a) {
+    a = FftAxis{};
+    a.n = n;
+    if (n < 1 || n > kFftMaxN) return false;
+    int best = kFftMaxStages + 1, best_sum = 0, cur[kFftMaxStages];
+    split(n, 0, cur, best, best_sum, a);
+    return best <= kFftMaxStages;
+}
+
+void fft_tables(const FftAxis ax[3], FftTables &t) {
+    for (int d = 0; d < 3; ++d) {
+        const int n = ax[d].n;
+        for (int k = 0; k < n; ++k) {
+            const double phi = -2.0 * 3.14159265358979323846 * k / n;
+            t.tw[d][k] = make_float2((float)cos(phi), (float)sin(phi));
+            int f = k, p = 0, m = n;
+            for (int i = 0; i < ax[d].stages; ++i) {
+                m /= ax[d].radix[i];
+                p += (f % ax[d].radix[i]) * m;
+                f /= ax[d].radix[i];
+            }
+            t.pos[d][k] = p;
+            t.freq[d][p] = k;
+        }
+    }
+}
+
+int fft_sum_blocks(const Geom &g) { return (g.n[1] + kRowsB - 1) / kRowsB * g.n[2]; }
+
+cudaError_t fft_prepare() {
+    cudaError_t e;
+    const int most = (int)(sizeof(float2) * (kFftMaxN * (kFftMaxN | 1) + 2 * kFftMaxN));
+    if ((e = cudaFuncSetAttribute(k_fft_yz, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess)
+        return e;
+    return cudaFuncSetAttribute(k_fft_yz_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
+cudaError_t launch_fft_solve(const Geom &g, const FftAxis ax[3], const FftTables *tab, const float *ktab,
+                             const float *rho, float2 *rho_hat, float2 *E_hat, int64_t nhalf,
+                             const int *mode_idx, int mode_comp, int mode_conj, Ctrl *ctrl, float4 *E4,
+                             float4 *E8, double *fpart, cudaStream_t st) {
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const float inv_ng = (float)(1.0 / ((double)nx * ny * nz));
+    k_fft_x_forward<1><<<dim3((ny + kRowsF - 1) / kRowsF, nz), kXThreads, x_smem(g, kRowsF / 2), st>>>(
+        ny, nz, g.nh, ax[0], tab, rho, nullptr, rho_hat, nhalf);
+    k_fft_yz<<<dim3(g.nh, 3), yz_threads(g), yz_smem(g), st>>>(nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab,
+                                                              inv_ng, rho_hat, E_hat, nhalf, mode_idx[0],
+                                                              mode_idx[1], mode_idx[2], mode_comp, mode_conj,
+                                                              ctrl);
+    k_fft_x_backward<<<dim3((ny + kRowsB - 1) / kRowsB, nz), kXThreads, x_smem(g, 3 * kRowsB / 2), st>>>(
+        ny, nz, g.nh, ax[0], tab, E_hat, nhalf, E4, E8, rho, fpart);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fft_adj_solve(const Geom &g, const FftAxis ax[3], const FftTables *tab,
+                                 const float *ktab, float4 *lE4, float2 *lE_hat, float2 *lrho_hat,
+                                 int64_t nhalf, float2 *lrho2, Ctrl *ctrl, int par, cudaStream_t st) {
+    const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
+    const float inv_ng = (float)(1.0 / ((double)nx * ny * nz));
+    const dim3 rows((ny + kRowsB - 1) / kRowsB, nz);
+    k_fft_x_forward<3><<<rows, kXThreads, x_smem(g, 3 * kRowsB / 2), st>>>(ny, nz, g.nh, ax[0], tab, nullptr,
+                                                                           lE4, lE_hat, nhalf);
+    k_fft_yz_adj<<<g.nh, yz_threads(g), yz_smem(g), st>>>(nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab, inv_ng,
+                                                          lE_hat, lrho_hat, nhalf);
+    k_fft_x_backward_adj<<<rows, kXThreads, x_smem(g, kRowsB / 2), st>>>(ny, nz, g.nh, ax[0], tab, lrho_hat,
+                                                                         lrho2, ctrl, par);
+    return cudaGetLastError();
+}
+
+}  // namespace pic

@@ -49,7 +49,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // Byte offsets of every device buffer inside the caller's arena.
 struct Layout {
     size_t ctrl, sets, rho, rho64, rho_hat, E_hat, E4, E8, lrho2, bins, scan_tmp, tile_items, tile_range,
-        items, fpart, ppart, ring, inv, stage_x, stage_v, adjE4, ktab, node_pos, fft, total;
+        items, fpart, ppart, ring, inv, stage_x, stage_v, adjE4, ktab, node_pos, fft_tab, fft, total;
     size_t set_stride;   // bytes of one per-particle array
 };
 
@@ -86,6 +86,8 @@ struct pic_ctx {
     cufftHandle r2c, c2r;     // rho -> rho^ ; 3 x E^ -> E4 (stride 4)
     cufftHandle r2c3, c2r1;   // adjoint: lE4 (stride 4) -> 3 x lE^ ; lrho^ -> lrho
     bool plans;
+    bool own_fft;             // the field solve runs on k_fft.cu instead of cuFFT
+    FftAxis ax[3];
     ParticleSet hsets[2];     // host copies of the device set descriptors
     // state of the last pic_adjoint_forward
     struct {
@@ -213,7 +215,7 @@ void compute_layout(pic_ctx *c) {
     L.tile_items = take((size_t)(c->ntiles + 1) * 4);
     L.tile_range = take((size_t)c->ntiles * 8);
     L.items = take((size_t)c->max_items * 16);
-    L.fpart = take((size_t)kDiagFieldBlocks * 4 * 8);
+    L.fpart = take((size_t)std::max(kDiagFieldBlocks, c->own_fft ? fft_sum_blocks(c->geom) : 0) * 4 * 8);
     L.ppart = take((size_t)kMaxPushBlocks * 4 * 8);
     L.ring = take((size_t)c->prm.diag_capacity * sizeof(pic_diag_t));
     L.inv = take(capb);
@@ -223,6 +225,7 @@ void compute_layout(pic_ctx *c) {
     L.lrho2 = take((size_t)c->ng * 8);
     L.ktab = take((size_t)(c->geom.nh + c->grid.n[1] + c->grid.n[2]) * 4);
     L.node_pos = take((size_t)3 * kMaxN * 8);
+    L.fft_tab = take(sizeof(FftTables));
     L.fft = take(c->fft_reserve);
     L.total = o;
 }
@@ -362,15 +365,34 @@ int do_deposit(pic_ctx *c) {
     return PIC_OK;
 }
 
-int do_solve(pic_ctx *c) {
+// blocks that leave partial field sums in fpart
+int field_blocks_of(const pic_ctx *c) {
+    return c->own_fft ? fft_sum_blocks(c->geom) : kDiagFieldBlocks;
+}
+
+// sums: also leave the partial field sums of the diagnostics
+int do_solve(pic_ctx *c, bool sums = false) {
     int r = timer_begin(c, PIC_PHASE_SOLVE);
     if (r) return r;
+    if (c->own_fft) {
+        PIC_CUDA(launch_fft_solve(c->geom, c->ax, c->at<FftTables>(c->lay.fft_tab),
+                                  c->at<float>(c->lay.ktab), c->at<float>(c->lay.rho),
+                                  c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat), c->nhalf,
+                                  c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl(),
+                                  c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8),
+                                  sums ? c->at<double>(c->lay.fpart) : nullptr, c->st));
+        return timer_end(c, PIC_PHASE_SOLVE, 3);
+    }
     PIC_CUFFT(cufftExecR2C(c->r2c, c->at<cufftReal>(c->lay.rho), c->at<cufftComplex>(c->lay.rho_hat)));
     PIC_CUDA(launch_green(c->geom, c->at<float>(c->lay.ktab), c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat),
                           c->nhalf, c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl(), c->st));
     PIC_CUFFT(cufftExecC2R(c->c2r, c->at<cufftComplex>(c->lay.E_hat), c->at<cufftReal>(c->lay.E4)));
     PIC_CUDA(launch_pair_E(c->geom, c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8), c->st));
-    return timer_end(c, PIC_PHASE_SOLVE, 2);
+    if ((r = timer_end(c, PIC_PHASE_SOLVE, 2)) || !sums) return r;
+    if ((r = timer_begin(c, PIC_PHASE_DIAG))) return r;
+    PIC_CUDA(launch_diag_field(c->geom, c->at<float>(c->lay.rho), c->at<float4>(c->lay.E4),
+                               c->at<double>(c->lay.fpart), c->st));
+    return timer_end(c, PIC_PHASE_DIAG, 1);
 }
 
 bool uniform_move(const pic_ctx *c) { return (c->prm.options & PIC_OPT_UNIFORM_MOVE) != 0; }
@@ -394,19 +416,11 @@ int do_gather_push(pic_ctx *c, bool diag) {
     return timer_end(c, PIC_PHASE_PUSH, 1);
 }
 
-int do_diag_field(pic_ctx *c) {
-    int r = timer_begin(c, PIC_PHASE_DIAG);
-    if (r) return r;
-    PIC_CUDA(launch_diag_field(c->geom, c->at<float>(c->lay.rho), c->at<float4>(c->lay.E4),
-                               c->at<double>(c->lay.fpart), c->st));
-    return timer_end(c, PIC_PHASE_DIAG, 1);
-}
-
 int do_diag_finalize(pic_ctx *c, int push_blocks) {
     int r = timer_begin(c, PIC_PHASE_DIAG);
     if (r) return r;
-    PIC_CUDA(launch_diag_finalize(c->at<double>(c->lay.fpart), c->at<double>(c->lay.ppart),
-                                  push_blocks, c->dV, mp_of(c), c->prm.dt, c->ctrl(),
+    PIC_CUDA(launch_diag_finalize(c->at<double>(c->lay.fpart), field_blocks_of(c),
+                                  c->at<double>(c->lay.ppart), push_blocks, c->dV, mp_of(c), c->prm.dt, c->ctrl(),
                                   c->at<pic_diag_t>(c->lay.ring), c->prm.diag_capacity, c->st));
     return timer_end(c, PIC_PHASE_DIAG, 1);
 }
@@ -741,6 +755,13 @@ int adj_keep_step(pic_ctx *c, const AdjLayout &L, int seg, int a0, int n, int *c
 
 // the adjoint field solve of step m (par = m & 1: its bound bookkeeping slot)
 int adj_solve(pic_ctx *c, int par) {
+    if (c->own_fft) {
+        PIC_CUDA(launch_fft_adj_solve(c->geom, c->ax, c->at<FftTables>(c->lay.fft_tab),
+                                      c->at<float>(c->lay.ktab), c->at<float4>(c->lay.adjE4),
+                                      c->at<float2>(c->lay.E_hat), c->at<float2>(c->lay.rho_hat), c->nhalf,
+                                      c->at<float2>(c->lay.lrho2), c->ctrl(), par, c->st));
+        return PIC_OK;
+    }
     PIC_CUFFT(cufftExecR2C(c->r2c3, c->at<cufftReal>(c->lay.adjE4), c->at<cufftComplex>(c->lay.E_hat)));
     PIC_CUDA(launch_green_adj(c->geom, c->L, c->at<float2>(c->lay.E_hat),
                               c->at<float2>(c->lay.rho_hat), c->nhalf, c->st));
@@ -909,12 +930,17 @@ int pic_create(const pic_grid_t *grid, const pic_species_t *species, const pic_p
     c->mode_idx[1] = ((m[1] % grid->n[1]) + grid->n[1]) % grid->n[1];
     c->mode_idx[2] = ((m[2] % grid->n[2]) + grid->n[2]) % grid->n[2];
 
-    // cuFFT work area: the library's own size query when it works here,
-    // never less than a conservative bound
-    size_t wmax = 0;
-    size_t bound = (size_t)c->nhalf * 8 * 3 + ((size_t)4 << 20);
-    if (make_plans(c, true, &wmax) == PIC_OK) bound = std::max(bound, wmax);
-    c->fft_reserve = bound;
+    c->own_fft = true;
+    for (int d = 0; d < 3; ++d) c->own_fft = fft_axis(g.n[d], c->ax[d]) && c->own_fft;
+    c->fft_reserve = 0;
+    if (!c->own_fft) {
+        // cuFFT work area: the library's own size query when it works here,
+        // never less than a conservative bound
+        size_t wmax = 0;
+        size_t bound = (size_t)c->nhalf * 8 * 3 + ((size_t)4 << 20);
+        if (make_plans(c, true, &wmax) == PIC_OK) bound = std::max(bound, wmax);
+        c->fft_reserve = bound;
+    }
     compute_layout(c);
     *out = c;
     snprintf(g_err, sizeof(g_err), "no error");
@@ -942,18 +968,27 @@ int pic_bind_workspace(pic_handle_t c, void *arena, size_t bytes, void *stream) 
     c->adj.ready = false;
     c->arena = static_cast<char *>(arena);
     c->st = static_cast<cudaStream_t>(stream);
-    size_t wmax = 0;
-    int r = make_plans(c, false, &wmax);
-    if (r) return r;
-    if (wmax > c->fft_reserve) {
-        destroy_plans(c);
-        return fail(PIC_ERR_CAPACITY, "cuFFT needs %zu work bytes, %zu reserved", wmax,
-                    c->fft_reserve);
-    }
-    void *work = c->arena + c->lay.fft;
-    for (cufftHandle p : {c->r2c, c->c2r, c->r2c3, c->c2r1}) {
-        PIC_CUFFT(cufftSetWorkArea(p, work));
-        PIC_CUFFT(cufftSetStream(p, c->st));
+    if (c->own_fft) {
+        FftTables tab{};
+        fft_tables(c->ax, tab);
+        PIC_CUDA(fft_prepare());
+        PIC_CUDA(cudaMemcpyAsync(c->at<FftTables>(c->lay.fft_tab), &tab, sizeof(tab),
+                                 cudaMemcpyHostToDevice, c->st));
+        PIC_CUDA(cudaStreamSynchronize(c->st));
+    } else {
+        size_t wmax = 0;
+        int r = make_plans(c, false, &wmax);
+        if (r) return r;
+        if (wmax > c->fft_reserve) {
+            destroy_plans(c);
+            return fail(PIC_ERR_CAPACITY, "cuFFT needs %zu work bytes, %zu reserved", wmax,
+                        c->fft_reserve);
+        }
+        void *work = c->arena + c->lay.fft;
+        for (cufftHandle p : {c->r2c, c->c2r, c->r2c3, c->c2r1}) {
+            PIC_CUFFT(cufftSetWorkArea(p, work));
+            PIC_CUFFT(cufftSetStream(p, c->st));
+        }
     }
 
     PIC_CUDA(sort_prepare());
@@ -998,7 +1033,8 @@ int pic_set_stream(pic_handle_t c, void *stream) {
     int r = check_ready(c);
     if (r) return r;
     c->st = static_cast<cudaStream_t>(stream);
-    for (cufftHandle p : {c->r2c, c->c2r, c->r2c3, c->c2r1}) PIC_CUFFT(cufftSetStream(p, c->st));
+    if (c->plans)
+        for (cufftHandle p : {c->r2c, c->c2r, c->r2c3, c->c2r1}) PIC_CUFFT(cufftSetStream(p, c->st));
     return PIC_OK;
 }
 
@@ -1199,9 +1235,8 @@ int pic_step(pic_handle_t c, int n) {
             if ((r = do_sort(c))) return r;
         }
         if (!c->rho_current && (r = do_deposit(c))) return r;
-        if ((r = do_solve(c))) return r;
         const bool diag = c->prm.diag_every > 0 && ((c->step + 1) % c->prm.diag_every == 0);
-        if (diag && (r = do_diag_field(c))) return r;
+        if ((r = do_solve(c, diag))) return r;
         if ((r = do_push_deposit(c, diag))) return r;
         if (diag && (r = do_diag_finalize(c, c->np > 0 ? fused_blocks_of(c) : 1))) return r;
     }
@@ -1318,10 +1353,8 @@ int pic_adjoint_forward(pic_handle_t c, int n_steps, int K, const double *w, voi
     }
     c->adj.cur_end = cur;
     if (!c->rho_current && (r = do_deposit(c))) return r;
-    if ((r = do_solve(c))) return r;
-    PIC_CUDA(launch_diag_field(c->geom, c->at<float>(c->lay.rho), c->at<float4>(c->lay.E4),
-                               c->at<double>(c->lay.fpart), c->st));
-    PIC_CUDA(launch_objective(c->at<double>(c->lay.fpart), kDiagFieldBlocks, c->dV, c->adj.w,
+    if ((r = do_solve(c, true))) return r;
+    PIC_CUDA(launch_objective(c->at<double>(c->lay.fpart), field_blocks_of(c), c->dV, c->adj.w,
                               &c->ctrl()->scalar[0], c->st));
     PIC_CUDA(cudaMemcpyAsync(J, &c->ctrl()->scalar[0], sizeof(double), cudaMemcpyDeviceToHost, c->st));
     PIC_CUDA(cudaStreamSynchronize(c->st));

@@ -322,9 +322,40 @@ cudaError_t launch_green(const Geom &g, const float *ktab, const float2 *rho_hat
                          int mode_conj, Ctrl *ctrl, cudaStream_t st);
 cudaError_t launch_diag_field(const Geom &g, const float *rho, const float4 *E4,
                               double *part, cudaStream_t st);
-cudaError_t launch_diag_finalize(const double *field_part, const double *push_part,
-                                 int push_blocks, double dV, double mp, double dt,
+cudaError_t launch_diag_finalize(const double *field_part, int field_blocks,
+                                 const double *push_part, int push_blocks, double dV, double mp, double dt,
                                  Ctrl *ctrl, pic_diag_t *ring, int ring_cap, cudaStream_t st);
+
+// Field solve by the library's own line transforms (k_fft.cu), for grids whose
+// axes are at most kFftMaxN long with no prime factor above kFftMaxPrime (one
+// (y, z) plane of a spectrum then fits a block's shared memory); others go
+// through cuFFT.
+constexpr int kFftMaxN = 128;
+constexpr int kFftMaxPrime = 31;
+constexpr int kFftMaxStages = 4;
+struct FftAxis {
+    int n, stages;
+    int radix[kFftMaxStages];   // forward order
+};
+// per axis: exp(-2 pi i k / n), the position of frequency k after a forward
+// transform and the frequency at a position
+struct FftTables {
+    float2 tw[3][kFftMaxN];
+    int pos[3][kFftMaxN], freq[3][kFftMaxN];
+};
+bool fft_axis(int n, FftAxis &a);   // false: not supported
+void fft_tables(const FftAxis ax[3], FftTables &t);
+int fft_sum_blocks(const Geom &g);   // blocks that leave partial field sums
+cudaError_t fft_prepare();           // kernel attributes; outside any stream capture
+// rho -> E4 and E8 (and fpart, 4 doubles per block, unless null)
+cudaError_t launch_fft_solve(const Geom &g, const FftAxis ax[3], const FftTables *tab, const float *ktab,
+                             const float *rho, float2 *rho_hat, float2 *E_hat, int64_t nhalf,
+                             const int *mode_idx, int mode_comp, int mode_conj, Ctrl *ctrl, float4 *E4,
+                             float4 *E8, double *fpart, cudaStream_t st);
+// lE4 (cleared) -> lrho2, with the bound bookkeeping of launch_adj_pair_rho
+cudaError_t launch_fft_adj_solve(const Geom &g, const FftAxis ax[3], const FftTables *tab,
+                                 const float *ktab, float4 *lE4, float2 *lE_hat, float2 *lrho_hat,
+                                 int64_t nhalf, float2 *lrho2, Ctrl *ctrl, int par, cudaStream_t st);
 
 // adjoint (k_adjoint.cu)
 cudaError_t launch_adj_seed(int64_t ng, const float4 *E4, float4 *lE4, const double *scale3,
