@@ -7,8 +7,8 @@
 // with |k|^2 over the continuous wavenumbers (m_d in [-N_d/2, N_d/2)), the
 // k = 0 mode (the uniform ion background) set to zero and each axis' Nyquist
 // component of the gradient set to zero so E stays real.  The 1/N_g of the
-// inverse transform is folded in here.  The C2R writes E interleaved as
-// float4 (Ex, Ey, Ez, 0) so the gather reads one 16-byte vector per node.
+// inverse transform is folded in here.  k_pack_E interleaves the three planar
+// components as float4 (Ex, Ey, Ez, 0) so the gather reads 16-byte vectors.
 //
 // Diagnostics (figures of Section 4): W_d = h^3 sum_g E_d^2, Q = h^3 sum_g rho,
 // accumulated in FP64 per block in a fixed order, then summed by one block.
@@ -59,38 +59,6 @@ __global__ void __launch_bounds__(128) k_green(int nx, int ny, int nz, int nh,
     }
 }
 
-// Per-block partial sums of Ex^2, Ey^2, Ez^2 and rho.  Each thread keeps FP32
-// (hi, lo) pairs whose error is that of ~48-bit arithmetic (FP64 instructions
-// run at a small fraction of the FP32 rate on this part); the pairs are
-// combined in FP64 across threads and blocks in a fixed order.
-__global__ void __launch_bounds__(256) k_diag_field(int64_t ng, const float *__restrict__ rho,
-                                                     const float4 *__restrict__ E4, double *part) {
-    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // two nodes per iteration, both loaded before either is summed
-    int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; g + stride < ng; g += 2 * stride) {
-        const float4 e = __ldcs(E4 + g), e2 = __ldcs(E4 + g + stride);
-        const float r = __ldcs(rho + g), r2 = __ldcs(rho + g + stride);
-        ff_add_sq(hi[0], lo[0], e.x);
-        ff_add_sq(hi[1], lo[1], e.y);
-        ff_add_sq(hi[2], lo[2], e.z);
-        ff_add(hi[3], lo[3], r);
-        ff_add_sq(hi[0], lo[0], e2.x);
-        ff_add_sq(hi[1], lo[1], e2.y);
-        ff_add_sq(hi[2], lo[2], e2.z);
-        ff_add(hi[3], lo[3], r2);
-    }
-    if (g < ng) {
-        const float4 e = E4[g];
-        ff_add_sq(hi[0], lo[0], e.x);
-        ff_add_sq(hi[1], lo[1], e.y);
-        ff_add_sq(hi[2], lo[2], e.z);
-        ff_add(hi[3], lo[3], rho[g]);
-    }
-    block_field_sums<256>(hi, lo, part + 4 * (int64_t)blockIdx.x);
-}
-
 __global__ void k_diag_finalize(const double *__restrict__ fpart, int fblocks,
                                 const double *__restrict__ ppart, int pblocks, double dV,
                                 double mp, double dt, Ctrl *ctrl, pic_diag_t *ring,
@@ -130,21 +98,49 @@ __global__ void k_diag_finalize(const double *__restrict__ fpart, int fblocks,
 
 }  // namespace
 
-// The push kernels read E through 256-bit loads of x-adjacent node pairs:
-// E8[2q] = E at node q, E8[2q + 1] = E at its +x neighbour (periodic).
-__global__ void k_pair_E(int nx, int64_t ng, const float4 *__restrict__ E4, float4 *__restrict__ E8) {
-    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= ng) return;
-    const int64_t row = q / nx;
-    const int i = (int)(q - row * nx);
-    const int64_t q1 = (i + 1 == nx) ? row * nx : q + 1;
-    E8[2 * q] = E4[q];
-    E8[2 * q + 1] = E4[q1];
+namespace {
+// Planar field rows (component d of row r at planar + d * dist + r * pitch) ->
+// E4, the x-paired E8 read by 256-bit loads (E8[2q] = E at q, E8[2q + 1] = E at
+// its +x neighbour, periodic) and, with SUMS, the block's partial sums of
+// Ex^2, Ey^2, Ez^2 and rho.  Bound by DRAM: 12 bytes read and 48 written per
+// node (16.8M nodes: 246 us).  With the interleaving left to the inverse
+// transform (output stride 4: 407 us against 92 planar), a pairing pass (120)
+// and a pass for the sums (81), a 256^3 solve with sums took 0.85 ms, now 0.54.
+template <bool SUMS>
+__global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pitch, int64_t dist,
+                                                const float *__restrict__ planar,
+                                                float4 *__restrict__ E4, float4 *__restrict__ E8,
+                                                const float *__restrict__ rho,
+                                                double *__restrict__ part) {
+    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+        const float *p0 = planar + r * pitch, *p1 = p0 + dist, *p2 = p1 + dist;
+        for (int x = threadIdx.x; x < nx; x += 256) {
+            const int x1 = x + 1 == nx ? 0 : x + 1;
+            const int64_t q = r * nx + x;
+            const float4 e = make_float4(p0[x], p1[x], p2[x], 0.0f);
+            E4[q] = e;
+            E8[2 * q] = e;
+            E8[2 * q + 1] = make_float4(p0[x1], p1[x1], p2[x1], 0.0f);
+            if (SUMS) {
+                ff_add_sq(hi[0], lo[0], e.x);
+                ff_add_sq(hi[1], lo[1], e.y);
+                ff_add_sq(hi[2], lo[2], e.z);
+                ff_add(hi[3], lo[3], rho[q]);
+            }
+        }
+    }
+    if (SUMS) block_field_sums<256>(hi, lo, part + 4 * (int64_t)blockIdx.x);
 }
+}  // namespace
 
-cudaError_t launch_pair_E(const Geom &g, const float4 *E4, float4 *E8, cudaStream_t st) {
-    const int64_t ng = (int64_t)g.n[0] * g.n[1] * g.n[2];
-    k_pair_E<<<(unsigned)((ng + 255) / 256), 256, 0, st>>>(g.n[0], ng, E4, E8);
+cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E4,
+                          float4 *E8, const float *rho, double *part, cudaStream_t st) {
+    const int64_t rows = (int64_t)g.n[1] * g.n[2];
+    if (part)
+        k_pack_E<true><<<kDiagFieldBlocks, 256, 0, st>>>(g.n[0], rows, pitch, dist, planar, E4, E8, rho, part);
+    else
+        k_pack_E<false><<<kDiagFieldBlocks, 256, 0, st>>>(g.n[0], rows, pitch, dist, planar, E4, E8, rho, part);
     return cudaGetLastError();
 }
 
@@ -171,13 +167,6 @@ cudaError_t launch_green(const Geom &g, const float *ktab, const float2 *rho_hat
     k_green<<<grid, T, 0, st>>>(g.n[0], g.n[1], g.n[2], g.nh, ktab, (float)(1.0 / ng), rho_hat,
                                 E_hat, nhalf, mode_idx[0], mode_idx[1], mode_idx[2], mode_comp,
                                 mode_conj, ctrl);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_diag_field(const Geom &g, const float *rho, const float4 *E4, double *part,
-                              cudaStream_t st) {
-    const int64_t ng = (int64_t)g.n[0] * g.n[1] * g.n[2];
-    k_diag_field<<<kDiagFieldBlocks, 256, 0, st>>>(ng, rho, E4, part);
     return cudaGetLastError();
 }
 

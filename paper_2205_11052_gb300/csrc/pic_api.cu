@@ -83,7 +83,7 @@ struct pic_ctx {
     bool bound;
     char *arena;
     cudaStream_t st;
-    cufftHandle r2c, c2r;     // rho -> rho^ ; 3 x E^ -> E4 (stride 4)
+    cufftHandle r2c, c2r;     // rho -> rho^ ; 3 x E^ -> planar E, in place
     cufftHandle r2c3, c2r1;   // adjoint: lE4 (stride 4) -> 3 x lE^ ; lrho^ -> lrho
     bool plans;
     bool own_fft;             // the field solve runs on k_fft.cu instead of cuFFT
@@ -128,22 +128,24 @@ namespace {
 
 bool finite_pos(double x) { return isfinite(x) && x > 0.0; }
 
-// Plan dimensions, slowest first, dropping unit y/z axes (x is the R2C axis).
-int fft_dims(const pic_ctx *c, long long *n, long long *nin) {
+// Plan dimensions, slowest first, dropping unit y/z axes (x is the R2C axis);
+// npad: those of real rows in the place of their half spectra.
+int fft_dims(const pic_ctx *c, long long *n, long long *nin, long long *npad) {
     int r = 0;
-    if (c->grid.n[2] > 1) { n[r] = c->grid.n[2]; nin[r] = c->grid.n[2]; ++r; }
-    if (c->grid.n[1] > 1) { n[r] = c->grid.n[1]; nin[r] = c->grid.n[1]; ++r; }
+    if (c->grid.n[2] > 1) { n[r] = c->grid.n[2]; nin[r] = npad[r] = c->grid.n[2]; ++r; }
+    if (c->grid.n[1] > 1) { n[r] = c->grid.n[1]; nin[r] = npad[r] = c->grid.n[1]; ++r; }
     n[r] = c->grid.n[0];
     nin[r] = c->grid.n[0] / 2 + 1;
+    npad[r] = 2 * nin[r];
     ++r;
     return r;
 }
 
-// The four transforms: rho -> rho^ (R2C), 3 x E^ -> E4 (C2R, batch 3, output
-// stride 4), lE4 -> 3 x lE^ (R2C, batch 3, input stride 4), lrho^ -> lrho (C2R).
+// The four transforms: rho -> rho^ (R2C), 3 x E^ -> planar E in its place (C2R,
+// batch 3, rows padded to their half spectra), lE4 -> 3 x lE^ (R2C, batch 3, input stride 4), lrho^ -> lrho (C2R).
 int make_plans(pic_ctx *c, bool estimate_only, size_t *ws_max) {
-    long long n[3], nh[3];
-    const int rank = fft_dims(c, n, nh);
+    long long n[3], nh[3], npad[3];
+    const int rank = fft_dims(c, n, nh, npad);
     cufftHandle p[4] = {0, 0, 0, 0};
     size_t ws[4] = {0, 0, 0, 0};
     cufftResult r = CUFFT_SUCCESS;
@@ -163,7 +165,7 @@ int make_plans(pic_ctx *c, bool estimate_only, size_t *ws_max) {
                                    t, batch, &ws[q]);
     };
     if (r == CUFFT_SUCCESS) r = plan(0, nullptr, 1, 0, nullptr, 1, 0, CUFFT_R2C, 1);
-    if (r == CUFFT_SUCCESS) r = plan(1, nh, 1, c->nhalf, n, 4, 1, CUFFT_C2R, 3);
+    if (r == CUFFT_SUCCESS) r = plan(1, nh, 1, c->nhalf, npad, 1, 2 * c->nhalf, CUFFT_C2R, 3);
     if (r == CUFFT_SUCCESS) r = plan(2, n, 4, 1, nh, 1, c->nhalf, CUFFT_R2C, 3);
     if (r == CUFFT_SUCCESS) r = plan(3, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 1);
     if (r != CUFFT_SUCCESS || estimate_only) {
@@ -386,13 +388,11 @@ int do_solve(pic_ctx *c, bool sums = false) {
     PIC_CUFFT(cufftExecR2C(c->r2c, c->at<cufftReal>(c->lay.rho), c->at<cufftComplex>(c->lay.rho_hat)));
     PIC_CUDA(launch_green(c->geom, c->at<float>(c->lay.ktab), c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat),
                           c->nhalf, c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl(), c->st));
-    PIC_CUFFT(cufftExecC2R(c->c2r, c->at<cufftComplex>(c->lay.E_hat), c->at<cufftReal>(c->lay.E4)));
-    PIC_CUDA(launch_pair_E(c->geom, c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8), c->st));
-    if ((r = timer_end(c, PIC_PHASE_SOLVE, 2)) || !sums) return r;
-    if ((r = timer_begin(c, PIC_PHASE_DIAG))) return r;
-    PIC_CUDA(launch_diag_field(c->geom, c->at<float>(c->lay.rho), c->at<float4>(c->lay.E4),
-                               c->at<double>(c->lay.fpart), c->st));
-    return timer_end(c, PIC_PHASE_DIAG, 1);
+    PIC_CUFFT(cufftExecC2R(c->c2r, c->at<cufftComplex>(c->lay.E_hat), c->at<cufftReal>(c->lay.E_hat)));
+    PIC_CUDA(launch_pack_E(c->geom, c->at<float>(c->lay.E_hat), 2 * (int64_t)c->geom.nh, 2 * c->nhalf,
+                           c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8), c->at<float>(c->lay.rho),
+                           sums ? c->at<double>(c->lay.fpart) : nullptr, c->st));
+    return timer_end(c, PIC_PHASE_SOLVE, 2);
 }
 
 bool uniform_move(const pic_ctx *c) { return (c->prm.options & PIC_OPT_UNIFORM_MOVE) != 0; }

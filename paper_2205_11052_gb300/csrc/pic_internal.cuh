@@ -96,7 +96,7 @@ struct PushConst {
 };
 
 // Diagnostic partial layout: 4 doubles per block.
-constexpr int kDiagFieldBlocks = 512;
+constexpr int kDiagFieldBlocks = 152 * 8;
 constexpr int kNumSMs = 152;   // streaming multiprocessors of the GPU (two dies of 76)
 constexpr int kMaxPushBlocks = kNumSMs * 8;
 constexpr int kMaxSmemPerBlock = 227 * 1024;   // opt-in shared memory per block
@@ -302,7 +302,7 @@ struct SaveY {
     float *o[3];
     float *v[3];   // also the velocities before the kick (null: not saved)
 };
-// E4: the field, one float4 per node; E8: the x-paired field (launch_pair_E),
+// E4: the field, one float4 per node; E8: the x-paired field (launch_pack_E),
 // 2 float4 per node
 cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, bool fixed,
                                 Ctrl *ctrl, const int4 *items, int max_items, const float4 *E4,
@@ -312,16 +312,17 @@ cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, b
 cudaError_t launch_gather_push(int64_t n, const Geom &g, const PushConst &pc, bool diag,
                                Ctrl *ctrl, const float4 *E8, double *part, int blocks,
                                int threads, cudaStream_t st);
-// E8[2q] = E4[q], E8[2q + 1] = E4[q + x (periodic)]
-cudaError_t launch_pair_E(const Geom &g, const float4 *E4, float4 *E8, cudaStream_t st);
+// planar E (component d of row r at planar + d * dist + r * pitch) -> E4, the
+// x-paired E8[2q] = E4[q], E8[2q + 1] = E4[q + x (periodic)], and unless null the
+// partial field sums of kDiagFieldBlocks blocks
+cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E4,
+                          float4 *E8, const float *rho, double *part, cudaStream_t st);
 
 // FP32 wavenumbers of every FFT index per axis (x: nh, y: ny, z: nz entries)
 void green_table(const Geom &g, const double *L_d, float *ktab);
 cudaError_t launch_green(const Geom &g, const float *ktab, const float2 *rho_hat,
                          float2 *E_hat, int64_t nhalf, const int *mode_idx, int mode_comp,
                          int mode_conj, Ctrl *ctrl, cudaStream_t st);
-cudaError_t launch_diag_field(const Geom &g, const float *rho, const float4 *E4,
-                              double *part, cudaStream_t st);
 cudaError_t launch_diag_finalize(const double *field_part, int field_blocks,
                                  const double *push_part, int push_blocks, double dV, double mp, double dt,
                                  Ctrl *ctrl, pic_diag_t *ring, int ring_cap, cudaStream_t st);
