@@ -299,6 +299,22 @@ __device__ __forceinline__ void stage_box(float4 *sE, const float4 *__restrict__
 }
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// The same box with x pairs, from E8: sA holds (Ex, Ey, Ez) of a slot and Ex of
+// its +x neighbour, sB the neighbour's Ey and Ez.
+__device__ __forceinline__ void stage_pairs(float4 *sA, float2 *sB, const float4 *__restrict__ E8,
+                                            const Tile &t, const Geom &g) {
+    const uint32_t da = (uint32_t)__cvta_generic_to_shared(sA);
+    const uint32_t db = (uint32_t)__cvta_generic_to_shared(sB);
+    for (int s = threadIdx.x; s < t.S; s += blockDim.x) {
+        const float4 *p = E8 + 2 * (int64_t)slot_node(t, g, s);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(da + 16u * (uint32_t)s), "l"(p)
+                     : "memory");
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(db + 8u * (uint32_t)s),
+                     "l"(p + 1)
+                     : "memory");
+    }
+}
+
 // byte offset of a staged box of S slots in the push kernels' shared memory,
 // after the item tile and the tile sums
 __host__ __device__ __forceinline__ size_t stage_offset(int S) {

@@ -453,8 +453,8 @@ __global__ void k_b_pack(int64_t mng, int nx, const float *__restrict__ planar,
         const int64_t q1 = (i + 1 == nx) ? q - i : q + 1;
         const float4 e = make_float4(planar[q], planar[q + mng], planar[q + 2 * mng], 0.0f);
         E4[q] = e;
-        E8[2 * q] = e;
-        E8[2 * q + 1] = make_float4(planar[q1], planar[q1 + mng], planar[q1 + 2 * mng], 0.0f);
+        E8[2 * q] = make_float4(e.x, e.y, e.z, planar[q1]);
+        E8[2 * q + 1] = make_float4(planar[q1 + mng], planar[q1 + 2 * mng], 0.0f, 0.0f);
     }
 }
 
@@ -502,15 +502,9 @@ size_t batch_push_smem(int max_S, bool staged) {
 }
 
 bool batch_stages_E(int max_S, int threads) {
-#if PIC_PD_STAGE_E
     const int64_t per_sm = std::max(1, PIC_BATCH_PD_MIN_BLOCKS * 256 / std::max(1, threads));
     const size_t per_block = batch_push_smem(max_S, true) + 256 + 1024;
     return (size_t)per_sm * per_block <= (size_t)228 * 1024;
-#else
-    (void)max_S;
-    (void)threads;
-    return false;
-#endif
 }
 
 cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool fixed,

@@ -244,8 +244,8 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
         const float4 e = make_float4(f0[2 * x], f1[2 * x], f2[2 * x], 0.0f);
         const int64_t g = ((int64_t)z * ny + y0 + r) * n + x;
         E4[g] = e;
-        E8[2 * g] = e;
-        E8[2 * g + 1] = make_float4(f0[2 * x1], f1[2 * x1], f2[2 * x1], 0.0f);
+        E8[2 * g] = make_float4(e.x, e.y, e.z, f0[2 * x1]);
+        E8[2 * g + 1] = make_float4(f1[2 * x1], f2[2 * x1], 0.0f, 0.0f);
         if (fpart) {
             ff_add_sq(hi[0], lo[0], e.x);
             ff_add_sq(hi[1], lo[1], e.y);

@@ -100,8 +100,8 @@ __global__ void k_diag_finalize(const double *__restrict__ fpart, int fblocks,
 
 namespace {
 // Planar field rows (component d of row r at planar + d * dist + r * pitch) ->
-// E4, the x-paired E8 read by 256-bit loads (E8[2q] = E at q, E8[2q + 1] = E at
-// its +x neighbour, periodic) and, with SUMS, the block's partial sums of
+// E4, the x-paired E8 read by 256-bit loads (the components at q, then those at
+// its +x neighbour, periodic: Ex Ey Ez Ex' | Ey' Ez' 0 0) and, with SUMS, the block's partial sums of
 // Ex^2, Ey^2, Ez^2 and rho.  Bound by DRAM: 12 bytes read and 48 written per
 // node (16.8M nodes: 246 us).  With the interleaving left to the inverse
 // transform (output stride 4: 407 us against 92 planar), a pairing pass (120)
@@ -120,8 +120,8 @@ __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pi
             const int64_t q = r * nx + x;
             const float4 e = make_float4(p0[x], p1[x], p2[x], 0.0f);
             E4[q] = e;
-            E8[2 * q] = e;
-            E8[2 * q + 1] = make_float4(p0[x1], p1[x1], p2[x1], 0.0f);
+            E8[2 * q] = make_float4(e.x, e.y, e.z, p0[x1]);
+            E8[2 * q + 1] = make_float4(p1[x1], p2[x1], 0.0f, 0.0f);
             if (SUMS) {
                 ff_add_sq(hi[0], lo[0], e.x);
                 ff_add_sq(hi[1], lo[1], e.y);

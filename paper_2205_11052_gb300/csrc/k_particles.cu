@@ -319,16 +319,17 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(int64_t n, Geom g, PushC
 // bytes per particle) instead of being read again by a separate deposit.
 // ---------------------------------------------------------------------------
 // E from the block's shared copy of its tile's box when it holds one (see
-// push_one_staged), else from the x-paired grid.
+// push_one_pair_box), else from the x-paired grid.
 template <bool DIAG, bool EXT, bool MAG, bool FIXED, int B>
 __device__ __forceinline__ void pd_one(const Geom &g, const PushConst &pc, const float4 *E8,
-                                       const float4 *sE, bool sparse, uint32_t *acc,
+                                       const float4 *sA, const float2 *sB, bool sparse,
+                                       uint32_t *acc,
                                        const cic::Tile &t, float *rho, unsigned long long *rho64,
                                        float qscale, int32_t &c, float &fx, float &fy, float &fz,
                                        float &vx, float &vy, float &vz, int &bad,
                                        unsigned long long &strays, float (&a)[4]) {
     int i, j, k;
-    push_one_staged<EXT, MAG, B>(g, pc, E8, sE, t, c, fx, fy, fz, vx, vy, vz, bad, i, j, k);
+    push_one_pair_box<EXT, MAG, B>(g, pc, E8, sA, sB, t, c, fx, fy, fz, vx, vy, vz, bad, i, j, k);
     if (sparse) {
         float w[8];
         cic::weights(fx, fy, fz, w);
@@ -344,13 +345,13 @@ __device__ __forceinline__ void pd_one(const Geom &g, const PushConst &pc, const
     }
 }
 
-// E4 not null: the block copies its tile's box of E4 to shared memory at
-// each change of tile and gathers there (see pd_one).  B > 0: every tile box
+// staged: the block copies its tile's box of E8 to shared memory at each change
+// of tile and gathers there (see pd_one).  B > 0: every tile box
 // is B slots long on each axis (see cic::box_row).
 template <bool DIAG, bool EXT, bool MAG, bool FIXED, int B>
-__global__ void __launch_bounds__(PIC_PD_THREADS, PIC_PD_MIN_BLOCKS) k_push_deposit(Geom g, PushConst pc, Ctrl *ctrl,
+__global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom g, PushConst pc, Ctrl *ctrl,
                                                           const int4 *__restrict__ items,
-                                                          const float4 *__restrict__ E4,
+                                                          bool staged,
                                                           const float4 *__restrict__ E8,
                                                           float *rho, unsigned long long *rho64,
                                                           float qscale, int sparse_below, int item_cost,
@@ -367,7 +368,8 @@ __global__ void __launch_bounds__(PIC_PD_THREADS, PIC_PD_MIN_BLOCKS) k_push_depo
     Segments run = run_segments(items, n_items, item_cost);
     const int S = cic::tile_of(g, 0).S;
     void *sum = reinterpret_cast<char *>(acc) + cic::sum_offset(S);
-    float4 *sE = reinterpret_cast<float4 *>(reinterpret_cast<char *>(acc) + cic::stage_offset(S));
+    float4 *sA = reinterpret_cast<float4 *>(reinterpret_cast<char *>(acc) + cic::stage_offset(S));
+    float2 *sB = reinterpret_cast<float2 *>(sA + S);
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
         acc[s] = 0u;
         if (FIXED) reinterpret_cast<unsigned long long *>(sum)[s] = 0ull;
@@ -392,7 +394,7 @@ __global__ void __launch_bounds__(PIC_PD_THREADS, PIC_PD_MIN_BLOCKS) k_push_depo
         if (!sparse) {
             __syncthreads();   // every add to the tile and read of its box is done
             const cic::Tile tn = cic::tile_of(g, tile);
-            if (E4 != nullptr) cic::stage_box(sE, E4, tn, g);
+            if (staged) cic::stage_pairs(sA, sB, E8, tn, g);
             if (any) cic::tile_flush<FIXED>(acc, sum, folded, t, g, rho, rho64, qscale);
             any = true;
             folded = false;
@@ -400,7 +402,7 @@ __global__ void __launch_bounds__(PIC_PD_THREADS, PIC_PD_MIN_BLOCKS) k_push_depo
             cic::stage_wait();
             __syncthreads();
         }
-        const float4 *sEi = (E4 != nullptr && !sparse) ? sE : nullptr;
+        const float4 *sAi = (staged && !sparse) ? sA : nullptr;
         for (int done = begin;;) {
             // as many particles as the tile takes without a fold
             done += min(end - done, cic::fill_limit() * (int)blockDim.x);
@@ -424,8 +426,8 @@ __global__ void __launch_bounds__(PIC_PD_THREADS, PIC_PD_MIN_BLOCKS) k_push_depo
                         __stcs(save.v[2] + p, vz);
                     }
                 }
-                pd_one<DIAG, EXT, MAG, FIXED, B>(g, pc, E8, sEi, sparse, acc, t, rho, rho64, qscale, c,
-                                              fx, fy, fz, vx, vy, vz, bad, strays, a);
+                pd_one<DIAG, EXT, MAG, FIXED, B>(g, pc, E8, sAi, sB, sparse, acc, t, rho, rho64, qscale,
+                                              c, fx, fy, fz, vx, vy, vz, bad, strays, a);
                 __stcs(ps.cell + p, c);
                 __stcs(ps.o[0] + p, fx);
                 __stcs(ps.o[1] + p, fy);
@@ -451,7 +453,7 @@ __global__ void __launch_bounds__(PIC_PD_THREADS, PIC_PD_MIN_BLOCKS) k_push_depo
     }
     if (DIAG) {
         const double *d = dm;
-        __shared__ double red[4][PIC_PD_THREADS / 32];
+        __shared__ double red[4][kPushThreadsPerSM / 64];
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
         for (int q = 0; q < 4; ++q) {
             double tt = d[q];
@@ -805,22 +807,19 @@ size_t tile_deposit_smem(const Geom &g) {
     const cic::Tile t0 = cic::tile_of(g, 0);
     return cic::sum_offset(t0.S) + 8 * (size_t)t0.S;
 }
-// staged field: the box's float4 slots after the deposit tiles, if
-// PIC_PD_MIN_BLOCKS such blocks (plus the kernel's static shared memory and
-// the runtime's 1 KiB per block) fit in an SM's 228 KiB
-bool push_stages_E(const Geom &g) {
-#if PIC_PD_STAGE_E
+// Blocks of the fused push + deposit: two of 384 threads per SM with the x-paired
+// box (24 bytes a slot after the deposit tiles' 12) while two fit in its 228 KiB
+// (plus the kernel's static shared memory and the runtime's 1 KiB per block), else
+// three of 256 that read the grid.  13^3 slots (8^3 tiles, two guard layers) take
+// the first: 20 steps of 128^3 x 64 64.1 ms, with whole nodes in the box (16 bytes
+// a slot, three blocks of 256) 66.9.  15^3 slots (three guard layers) take the
+// second: one block of 768 threads with the box made the Penning bunch's 10 steps
+// 53.7 ms instead of 50.7.
+PushShape push_shape(const Geom &g) {
     const int S = cic::tile_of(g, 0).S;
-    const size_t per_block = cic::stage_offset(S) + 16 * (size_t)S + 256 + 1024;
-    return per_block * PIC_PD_MIN_BLOCKS <= (size_t)228 * 1024;
-#else
-    (void)g;
-    return false;
-#endif
-}
-size_t push_deposit_smem(const Geom &g) {
-    const int S = cic::tile_of(g, 0).S;
-    return push_stages_E(g) ? cic::stage_offset(S) + 16 * (size_t)S : tile_deposit_smem(g);
+    const size_t box = cic::stage_offset(S) + 24 * (size_t)S;
+    if (2 * (box + 2048) <= (size_t)228 * 1024) return PushShape{kPushThreadsPerSM / 2, 2, true, box};
+    return PushShape{kPushThreadsPerSM / 3, 3, false, tile_deposit_smem(g)};
 }
 
 // Allow the fused kernels' shared memory (call outside any stream capture)
@@ -837,7 +836,7 @@ cudaError_t push_deposit_prepare(const Geom &g) {
         PIC_MVA(true, true, 0); PIC_MVA(false, true, kConstBox); PIC_MVA(true, true, kConstBox);
 #undef PIC_MVA
     }
-    const size_t smem = push_deposit_smem(g);
+    const size_t smem = push_shape(g).smem;
     if (smem <= 48 * 1024) return cudaSuccess;
 #define PIC_PDA(D, X, M, F, B)                                                                \
     if ((e = cudaFuncSetAttribute(k_push_deposit<D, X, M, F, B>,                              \
@@ -856,20 +855,19 @@ cudaError_t push_deposit_prepare(const Geom &g) {
 }
 
 cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, bool fixed,
-                                Ctrl *ctrl, const int4 *items, int max_items, const float4 *E4,
+                                Ctrl *ctrl, const int4 *items, int max_items,
                                 const float4 *E8, float *rho, unsigned long long *rho64,
                                 double qscale, int sparse_below, int item_cost, double *part,
                                 int blocks, const SaveY &save, cudaStream_t st) {
     const bool ext = pc.wz2 != 0.0f;
     const bool mag = pc.t[0] != 0.0f || pc.t[1] != 0.0f || pc.t[2] != 0.0f;
-    const size_t smem = push_deposit_smem(g);
-    const float4 *E4s = push_stages_E(g) ? E4 : nullptr;
+    const PushShape ps = push_shape(g);
     const int nb = std::max(1, std::min(blocks, max_items));
     const float qs = (float)qscale;
     cudaError_t e = cudaSuccess;
     const bool cbox = const_box(g);
 #define PIC_PD(D, X, M, F, B)                                                                   \
-    k_push_deposit<D, X, M, F, B><<<nb, PIC_PD_THREADS, smem, st>>>(g, pc, ctrl, items, E4s, E8, \
+    k_push_deposit<D, X, M, F, B><<<nb, ps.threads, ps.smem, st>>>(g, pc, ctrl, items, ps.staged, E8, \
                                                                     rho, rho64, qs,             \
                                                                     sparse_below, item_cost, part, save)
 #define PIC_PD_F(D, X, M)                                  \

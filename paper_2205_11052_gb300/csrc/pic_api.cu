@@ -313,7 +313,7 @@ int timer_end(pic_ctx *c, int ph, int kernels) {
 
 // particles per work item: the caller's, or so many that the blocks of one wave
 // get kItemsPerBlock items each
-constexpr int64_t kItemTarget = (int64_t)kNumSMs * PIC_PD_MIN_BLOCKS * kItemsPerBlock;
+constexpr int64_t kItemTarget = (int64_t)kNumSMs * 3 * kItemsPerBlock;
 int chunk_of(const pic_ctx *c) {
     if (c->chunk) return c->chunk;
     const int64_t per = (c->np + kItemTarget - 1) / kItemTarget;
@@ -435,7 +435,7 @@ int do_diag_finalize(pic_ctx *c, int push_blocks) {
 #endif
 
 int fused_blocks_of(const pic_ctx *c) {
-    const int per = uniform_move(c) ? PIC_MV_MIN_BLOCKS * PIC_MV_WAVES : PIC_PD_MIN_BLOCKS * PIC_PD_WAVES;
+    const int per = uniform_move(c) ? PIC_MV_MIN_BLOCKS * PIC_MV_WAVES : push_shape(c->geom).per_sm;
     return (int)std::max<int64_t>(1, std::min<int64_t>(c->max_items, std::min(kMaxPushBlocks, 152 * per)));
 }
 
@@ -455,8 +455,7 @@ int do_push_deposit(pic_ctx *c, bool diag, const SaveY &save = SaveY{}) {
     } else if (c->np > 0) {
         PIC_CUDA(launch_push_deposit(c->geom, push_const(c), diag, fixed, c->ctrl(),
                                      c->at<int4>(c->lay.items), (int)c->max_items,
-                                     c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8),
-                                     c->at<float>(c->lay.rho),
+                                     c->at<float4>(c->lay.E8), c->at<float>(c->lay.rho),
                                      c->at<unsigned long long>(c->lay.rho64), qscale_of(c),
                                      c->sparse_below, item_cost_of(c), c->at<double>(c->lay.ppart),
                                      fused_blocks_of(c), save, c->st));

@@ -100,23 +100,8 @@ constexpr int kDiagFieldBlocks = 152 * 8;
 constexpr int kNumSMs = 152;   // streaming multiprocessors of the GPU (two dies of 76)
 constexpr int kMaxPushBlocks = kNumSMs * 8;
 constexpr int kMaxSmemPerBlock = 227 * 1024;   // opt-in shared memory per block
-// resident blocks per SM the fused push + deposit kernel is compiled for
-#ifndef PIC_PD_MIN_BLOCKS
-#define PIC_PD_MIN_BLOCKS 3
-#endif
-// threads per block of the fused push + deposit, and its grid in waves of
-// PIC_PD_MIN_BLOCKS blocks per SM
-#ifndef PIC_PD_THREADS
-#define PIC_PD_THREADS 256
-#endif
-#ifndef PIC_PD_WAVES
-#define PIC_PD_WAVES 1
-#endif
-// the fused push + deposit gathers E from a shared-memory copy of its tile's
-// box when PIC_PD_MIN_BLOCKS blocks with that copy still fit on an SM
-#ifndef PIC_PD_STAGE_E
-#define PIC_PD_STAGE_E 1
-#endif
+// threads per SM the fused push + deposit kernel is compiled for (80 registers)
+constexpr int kPushThreadsPerSM = 768;
 // resident blocks per SM of the uniform-plasma move + deposit
 #ifndef PIC_MV_MIN_BLOCKS
 #define PIC_MV_MIN_BLOCKS 4
@@ -288,11 +273,15 @@ cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, boo
                         Ctrl *ctrl, const int4 *items, int max_items, float *rho,
                         unsigned long long *rho64, double qscale, int sparse_below, int item_cost,
                         double *part, int blocks, cudaStream_t st);
-// dynamic shared memory of the fused push + deposit kernel for geometry g,
-// whether it stages E in shared memory, and the one-time attribute setting it
-// needs above 48 KiB
-size_t push_deposit_smem(const Geom &g);
-bool push_stages_E(const Geom &g);
+// block size, blocks per SM, whether the blocks stage E, and the dynamic shared
+// memory of the fused push + deposit kernel for geometry g; the one-time
+// attribute setting it needs above 48 KiB
+struct PushShape {
+    int threads, per_sm;
+    bool staged;
+    size_t smem;
+};
+PushShape push_shape(const Geom &g);
 size_t tile_deposit_smem(const Geom &g);   // the deposit tiles alone (unstaged kernels)
 cudaError_t push_deposit_prepare(const Geom &g);
 // Optional copy of the positions a push starts from (cell, o[3]), written by
@@ -302,19 +291,18 @@ struct SaveY {
     float *o[3];
     float *v[3];   // also the velocities before the kick (null: not saved)
 };
-// E4: the field, one float4 per node; E8: the x-paired field (launch_pack_E),
-// 2 float4 per node
+// E8: the x-paired field (launch_pack_E), 2 float4 per node
 cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, bool fixed,
-                                Ctrl *ctrl, const int4 *items, int max_items, const float4 *E4,
-                                const float4 *E8, float *rho, unsigned long long *rho64, double qscale,
+                                Ctrl *ctrl, const int4 *items, int max_items, const float4 *E8,
+                                float *rho, unsigned long long *rho64, double qscale,
                                 int sparse_below, int item_cost, double *part, int blocks,
                                 const SaveY &save, cudaStream_t st);
 cudaError_t launch_gather_push(int64_t n, const Geom &g, const PushConst &pc, bool diag,
                                Ctrl *ctrl, const float4 *E8, double *part, int blocks,
                                int threads, cudaStream_t st);
 // planar E (component d of row r at planar + d * dist + r * pitch) -> E4, the
-// x-paired E8[2q] = E4[q], E8[2q + 1] = E4[q + x (periodic)], and unless null the
-// partial field sums of kDiagFieldBlocks blocks
+// x-paired E8 (six floats in 32 bytes per node: E at q, then E at q + x, periodic),
+// and unless null the partial field sums of kDiagFieldBlocks blocks
 cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E4,
                           float4 *E8, const float *rho, double *part, cudaStream_t st);
 

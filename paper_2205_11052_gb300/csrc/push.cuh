@@ -55,12 +55,12 @@ __device__ __forceinline__ void gather_E_global(const Geom &g, const float4 *__r
     interp_E(e, fx, fy, fz, ex, ey, ez);
 }
 
-// E8 holds, per node q, E at q and at its +x neighbour (periodic): 32 bytes,
-// so each of the four (y, z) corner rows of the stencil is one aligned
-// 256-bit read-only load
+// E8 holds, per node q, E at q and at its +x neighbour (periodic) as six
+// consecutive floats in 32 bytes, so each of the four (y, z) corner rows of the
+// stencil is one aligned 256-bit read-only load
 __device__ __forceinline__ void ld_pair(const float4 *p, float4 &a, float4 &b) {
     asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+        : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(a.w), "=f"(b.w)
         : "l"(p));
 }
 
@@ -219,6 +219,49 @@ __device__ __forceinline__ void push_one_pairs(const Geom &g, const PushConst &p
                                                float &vy, float &vz, int &bad) {
     int i, j, k;
     push_one_pairs<EXT, MAG>(g, pc, E8, c, fx, fy, fz, vx, vy, vz, bad, i, j, k);
+}
+
+// E at the particle from the x-paired copy of the box (cic::stage_pairs): the
+// four (y, z) rows of the stencil cost a 16-byte and an 8-byte shared load each,
+// 24 bytes a row against two 16-byte loads of whole nodes.  Lanes at random slots
+// collide in the banks, so the wavefronts go with the bytes: about 67 per warp and
+// gather, 85 with whole nodes.
+template <int B = 0>
+__device__ __forceinline__ void gather_E_pair_box(const float4 *sA, const float2 *sB, int s0, int S0r,
+                                                  int S01r, float fx, float fy, float fz, float &ex,
+                                                  float &ey, float &ez) {
+    const int S0 = B > 0 ? B : S0r, S01 = B > 0 ? B * B : S01r;   // B > 0: a constant box
+    const int off[4] = {0, S0, S01, S01 + S0};
+    float4 e[8];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const float4 a = sA[s0 + off[r]];
+        const float2 b = sB[s0 + off[r]];
+        e[2 * r] = a;
+        e[2 * r + 1] = make_float4(a.w, b.x, b.y, 0.0f);
+    }
+    interp_E(e, fx, fy, fz, ex, ey, ez);
+}
+
+// Gather + kick + drift with E read from (sA, sB), the block's shared-memory copy
+// of the box of tile t (cic::stage_pairs), when the particle's stencil lies in
+// that box.  Other particles, and every particle when sA is null, read the
+// x-paired grid E8.  (i, j, k) receives the new stencil base.
+template <bool EXT, bool MAG, int B = 0>
+__device__ __forceinline__ void push_one_pair_box(const Geom &g, const PushConst &pc,
+                                                  const float4 *__restrict__ E8, const float4 *sA,
+                                                  const float2 *sB, const cic::Tile &t, int32_t &c,
+                                                  float &fx, float &fy, float &fz, float &vx,
+                                                  float &vy, float &vz, int &bad, int &i, int &j,
+                                                  int &k) {
+    decode_base(g, c, i, j, k, bad);
+    float ex, ey, ez;
+    int s0;
+    if (sA != nullptr && cic::box_base<B>(t, g, i, j, k, s0))
+        gather_E_pair_box<B>(sA, sB, s0, t.S0, t.S01, fx, fy, fz, ex, ey, ez);
+    else
+        gather_E_pairs(g, E8, i, j, k, fx, fy, fz, ex, ey, ez);
+    kick_drift<EXT, MAG>(g, pc, ex, ey, ez, i, j, k, c, fx, fy, fz, vx, vy, vz, bad);
 }
 
 // Gather + kick + drift with E read from sE, the block's shared-memory copy
