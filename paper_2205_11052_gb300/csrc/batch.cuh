@@ -23,6 +23,8 @@ struct InstDesc {
     double inv_h_d[3], h_d[3], L_d[3], two_pi_over_L[3];
     double inv_ng;             // 1 / N_g (folded into the Green kernel)
     int mode_idx[3], mode_comp, mode_conj;
+    int sum_blocks;            // blocks that leave its partial field sums
+    bool own_fft;              // its size class is solved by k_fft.cu (sums included)
 };
 
 cudaError_t launch_b_load(const double *x, const double *v, int64_t m, int64_t base,
@@ -55,13 +57,13 @@ cudaError_t launch_b_rho_finish(int64_t ng, const InstDesc *desc, const long lon
                                 unsigned long long *rho64, float *rho, cudaStream_t st);
 cudaError_t launch_b_green(const InstDesc *desc, int first, int m, int64_t nhalf,
                            const float2 *rho_hat, float2 *E_hat, double *modes, cudaStream_t st);
-// partial field sums per instance (fpart: kBatchDiagBlocks x 4 doubles each);
-// max_blocks: the largest batch_diag_blocks of any instance
-constexpr int kBatchDiagBlocks = 64;
+// partial field sums of the instances whose solve leaves none (fpart: fstride x 4
+// doubles per instance); max_blocks: the largest sum_blocks of any of them
 int batch_diag_blocks(const Geom &g);
-cudaError_t launch_b_diag(const InstDesc *desc, int n_inst, int max_blocks, const float *rho,
-                          const float4 *E4, double *fpart, cudaStream_t st);
-cudaError_t launch_b_diag_finalize(const InstDesc *desc, int n_inst, const int32_t *item_off,
+cudaError_t launch_b_diag(const InstDesc *desc, int n_inst, int max_blocks, int fstride,
+                          const float *rho, const float4 *E4, double *fpart, cudaStream_t st);
+cudaError_t launch_b_diag_finalize(const InstDesc *desc, int n_inst, int fstride,
+                                   const int32_t *item_off,
                                    const double *fpart, const double *ppart, const double *modes,
                                    Ctrl *ctrl, double dt, pic_diag_t *ring, int ring_cap,
                                    cudaStream_t st);

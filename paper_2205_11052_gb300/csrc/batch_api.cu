@@ -39,6 +39,9 @@ struct SizeClass {
     int first, m;             // internal instances [first, first + m)
     int64_t ng, nhalf;        // per instance
     int64_t g0, h0;           // offsets of the class in the grid / half-spectrum arrays
+    bool own;                 // solved by k_fft.cu: axes, tables, wavenumber tables of its instances
+    FftAxis ax[3];
+    size_t o_tab, o_ktab;
     cufftHandle r2c, c2r;
 };
 
@@ -58,7 +61,8 @@ struct pic_batch {
     int64_t np, ng, nhalf_tot;
     int ntiles, max_items, chunk, sparse_below, fused_blocks, block;
     bool stage_E;   // the push stages each tile's box of E in shared memory
-    int diag_blocks;           // field-diagnostic blocks of the largest instance
+    int diag_blocks;           // field-diagnostic blocks of the largest instance solved by cuFFT
+    int sum_stride;            // most blocks with partial field sums of an instance
     int max_S;                 // largest tile (plus guard) of any instance, in nodes
     size_t fft_reserve;
     int64_t staging;
@@ -82,6 +86,7 @@ namespace {
 int batch_plans(pic_batch *b, bool estimate, size_t *ws_max) {
     *ws_max = 0;
     for (SizeClass &c : b->cls) {
+        if (c.own) continue;
         long long n[3], nh[3];
         int r = 0;
         if (c.n[2] > 1) { n[r] = c.n[2]; nh[r] = c.n[2]; ++r; }
@@ -125,6 +130,7 @@ int batch_plans(pic_batch *b, bool estimate, size_t *ws_max) {
 void batch_destroy_plans(pic_batch *b) {
     if (!b->plans) return;
     for (SizeClass &c : b->cls) {
+        if (c.own) continue;
         cufftDestroy(c.r2c);
         cufftDestroy(c.c2r);
     }
@@ -158,7 +164,11 @@ void batch_layout(pic_batch *b) {
     b->o_titems = take((size_t)(b->ntiles + 1) * 4);
     b->o_trange = take((size_t)b->ntiles * 8);
     b->o_items = take((size_t)b->max_items * 16);
-    b->o_fpart = take((size_t)b->n_inst * kBatchDiagBlocks * 4 * 8);
+    b->o_fpart = take((size_t)b->n_inst * b->sum_stride * 4 * 8);
+    for (SizeClass &c : b->cls) {
+        c.o_tab = take(sizeof(FftTables));
+        c.o_ktab = take((size_t)c.m * (c.n[0] / 2 + 1 + c.n[1] + c.n[2]) * 4);
+    }
     b->o_ppart = take((size_t)b->max_items * 4 * 8);
     b->o_modes = take((size_t)b->n_inst * 2 * 8);
     b->o_ring = take((size_t)b->prm.diag_capacity * b->n_inst * sizeof(pic_diag_t));
@@ -215,11 +225,30 @@ int b_sort(pic_batch *b) {
     return PIC_OK;
 }
 
-int b_solve(pic_batch *b) {
+// sums: also leave the partial field sums of the classes solved by k_fft.cu
+int b_solve(pic_batch *b, bool sums) {
     float *rho = b->at<float>(b->o_rho);
     float2 *rhoh = b->at<float2>(b->o_rhoh), *Eh = b->at<float2>(b->o_Eh);
     float *E = b->at<float>(b->o_E4);
     for (SizeClass &c : b->cls) {
+        if (c.own) {
+            const InstDesc &D = b->desc[c.first];   // same grid and mode indices for the class
+            const int64_t kt = c.n[0] / 2 + 1 + c.n[1] + c.n[2];
+            for (int j = 0; j < c.m; j += 65535) {   // grid.z
+                const int m = std::min(c.m - j, 65535);
+                const int64_t g0 = c.g0 + j * c.ng, h0 = c.h0 + j * c.nhalf;
+                B_CUDA(launch_fft_solve(D.g, m, c.ax, b->at<FftTables>(c.o_tab),
+                                        b->at<float>(c.o_ktab) + j * kt, rho + g0, rhoh + h0, Eh + 3 * h0,
+                                        c.nhalf, D.mode_idx, D.mode_comp, D.mode_conj,
+                                        b->at<double>(b->o_modes) + 2 * (c.first + j),
+                                        reinterpret_cast<float4 *>(E) + g0, b->at<float4>(b->o_E8) + 2 * g0,
+                                        sums ? b->at<double>(b->o_fpart) + 4 * (int64_t)b->sum_stride *
+                                                                               (c.first + j)
+                                             : nullptr,
+                                        b->sum_stride, b->st));
+            }
+            continue;
+        }
         B_CUFFT(cufftExecR2C(c.r2c, rho + c.g0, reinterpret_cast<cufftComplex *>(rhoh + c.h0)));
         B_CUDA(launch_b_green(b->at<InstDesc>(b->o_desc), c.first, c.m, c.nhalf, rhoh + c.h0,
                              Eh + 3 * c.h0, b->at<double>(b->o_modes), b->st));
@@ -389,8 +418,20 @@ int pic_batch_create(const pic_instance_t *inst, int n_inst, double q_over_m,
     b->ntiles = tile0;
     b->max_items = (int)std::min<int64_t>(max_items, 2147483647LL);
     b->max_S = max_S;
-    b->diag_blocks = 1;
-    for (const InstDesc &D : b->desc) b->diag_blocks = std::max(b->diag_blocks, batch_diag_blocks(D.g));
+    b->diag_blocks = 0;
+    b->sum_stride = 1;
+    for (SizeClass &c : b->cls) {
+        c.own = true;
+        for (int d = 0; d < 3; ++d) c.own = fft_axis(c.n[d], c.ax[d]) && c.own;
+        const Geom &g = b->desc[c.first].g;
+        const int blocks = c.own ? fft_sum_blocks(g) : batch_diag_blocks(g);
+        for (int j = c.first; j < c.first + c.m; ++j) {
+            b->desc[j].own_fft = c.own;
+            b->desc[j].sum_blocks = blocks;
+        }
+        if (!c.own) b->diag_blocks = std::max(b->diag_blocks, blocks);
+        b->sum_stride = std::max(b->sum_stride, blocks);
+    }
     if (batch_push_smem(max_S) > (size_t)kMaxSmemPerBlock) {
         delete b;
         return record_error(PIC_ERR_ARG, "deposit tile plus guard too large for shared memory");
@@ -440,11 +481,25 @@ int pic_batch_bind_workspace(pic_batch_t b, void *arena, size_t bytes, void *str
         batch_destroy_plans(b);
         return record_error(PIC_ERR_CAPACITY, "cuFFT needs %zu work bytes, %zu reserved", ws, b->fft_reserve);
     }
-    for (SizeClass &c : b->cls)
+    for (SizeClass &c : b->cls) {
+        if (c.own) {
+            FftTables tab{};
+            fft_tables(c.ax, tab);
+            std::vector<float> k((size_t)c.m * (c.n[0] / 2 + 1 + c.n[1] + c.n[2]));
+            for (int j = 0; j < c.m; ++j)
+                green_table(b->desc[c.first + j].g, b->desc[c.first + j].L_d,
+                            k.data() + (size_t)j * (c.n[0] / 2 + 1 + c.n[1] + c.n[2]));
+            B_CUDA(fft_prepare());
+            B_CUDA(cudaMemcpyAsync(b->arena + c.o_tab, &tab, sizeof(tab), cudaMemcpyHostToDevice, b->st));
+            B_CUDA(cudaMemcpyAsync(b->arena + c.o_ktab, k.data(), k.size() * 4, cudaMemcpyHostToDevice, b->st));
+            B_CUDA(cudaStreamSynchronize(b->st));
+            continue;
+        }
         for (cufftHandle p : {c.r2c, c.c2r}) {
             B_CUFFT(cufftSetWorkArea(p, b->arena + b->o_fft));
             B_CUFFT(cufftSetStream(p, b->st));
         }
+    }
     B_CUDA(batch_sort_prepare());
     Ctrl h;
     memset(&h, 0, sizeof(h));
@@ -529,14 +584,15 @@ int pic_batch_step(pic_batch_t b, int n) {
     for (int s = 0; s < n; ++s) {
         if (b->prm.sort_period > 0 && b->since_sort >= b->prm.sort_period && (r = b_sort(b))) return r;
         if (!b->rho_current && (r = b_deposit_pass(b, false, false))) return r;
-        if ((r = b_solve(b))) return r;
         const bool diag = b->prm.diag_every > 0 && ((b->step + 1) % b->prm.diag_every == 0);
+        if ((r = b_solve(b, diag))) return r;
         if (diag)
-            B_CUDA(launch_b_diag(b->at<InstDesc>(b->o_desc), b->n_inst, b->diag_blocks, b->at<float>(b->o_rho),
+            B_CUDA(launch_b_diag(b->at<InstDesc>(b->o_desc), b->n_inst, b->diag_blocks, b->sum_stride,
+                                 b->at<float>(b->o_rho),
                                  b->at<float4>(b->o_E4), b->at<double>(b->o_fpart), b->st));
         if ((r = b_deposit_pass(b, true, diag))) return r;
         if (diag)
-            B_CUDA(launch_b_diag_finalize(b->at<InstDesc>(b->o_desc), b->n_inst,
+            B_CUDA(launch_b_diag_finalize(b->at<InstDesc>(b->o_desc), b->n_inst, b->sum_stride,
                                           b->at<int32_t>(b->o_titems), b->at<double>(b->o_fpart),
                                           b->at<double>(b->o_ppart), b->at<double>(b->o_modes),
                                           b->ctrl(), b->prm.dt, b->at<pic_diag_t>(b->o_ring),
@@ -612,7 +668,8 @@ int pic_batch_set_stream(pic_batch_t b, void *stream) {
     if (r) return r;
     b->st = static_cast<cudaStream_t>(stream);
     for (SizeClass &c : b->cls)
-        for (cufftHandle p : {c.r2c, c.c2r}) B_CUFFT(cufftSetStream(p, b->st));
+        if (!c.own)
+            for (cufftHandle p : {c.r2c, c.c2r}) B_CUFFT(cufftSetStream(p, b->st));
     return PIC_OK;
 }
 

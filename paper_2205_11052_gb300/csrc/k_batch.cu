@@ -362,19 +362,13 @@ __global__ void k_b_green(const InstDesc *__restrict__ desc, int first, int m, i
 // and FP64 across threads, in a fixed order.  One block per instance with FP64
 // sums kept 24 of 152 SMs busy for 0.29 ms a step on 24 instances of up to
 // 48^3 nodes; 4096 nodes a block take 19.2 us.
-__host__ __device__ __forceinline__ int diag_blocks_of(const Geom &g) {
-    const int64_t ng = (int64_t)g.n[0] * g.n[1] * g.n[2];
-    const int64_t b = (ng + 4095) / 4096;
-    return (int)(b < kBatchDiagBlocks ? b : kBatchDiagBlocks);
-}
-
 __global__ void __launch_bounds__(256) k_b_diag_field(const InstDesc *__restrict__ desc,
                                                       const float *__restrict__ rho,
                                                       const float4 *__restrict__ E4,
-                                                      double *__restrict__ fpart) {
+                                                      double *__restrict__ fpart, int fstride) {
     const InstDesc &D = desc[blockIdx.x];
-    const int nb = diag_blocks_of(D.g);
-    if ((int)blockIdx.y >= nb) return;
+    const int nb = D.sum_blocks;
+    if (D.own_fft || (int)blockIdx.y >= nb) return;
     const int64_t ng = (int64_t)D.g.n[0] * D.g.n[1] * D.g.n[2];
     const int64_t per = (ng + nb - 1) / nb;
     const int64_t q1 = D.g0 + ((blockIdx.y + 1) * per < ng ? (blockIdx.y + 1) * per : ng);
@@ -387,7 +381,7 @@ __global__ void __launch_bounds__(256) k_b_diag_field(const InstDesc *__restrict
         ff_add(hi[3], lo[3], rho[q]);
     }
     block_field_sums<256>(hi, lo,
-                          fpart + 4 * ((int64_t)blockIdx.x * kBatchDiagBlocks + blockIdx.y));
+                          fpart + 4 * ((int64_t)blockIdx.x * fstride + blockIdx.y));
 }
 
 // One record per instance, one block each: the instance's items are
@@ -396,7 +390,7 @@ __global__ void __launch_bounds__(256) k_b_diag_field(const InstDesc *__restrict
 // instance walked up to 2000 items in a row: 0.84 ms a step on 24 instances of
 // up to 48^3 cells, now 12.7 us.
 __global__ void __launch_bounds__(256) k_b_diag_finalize(const InstDesc *__restrict__ desc,
-                                                         int n_inst,
+                                                         int n_inst, int fstride,
                                                          const int32_t *__restrict__ item_off,
                                                          const double *__restrict__ fpart,
                                                          const double *__restrict__ ppart,
@@ -407,10 +401,8 @@ __global__ void __launch_bounds__(256) k_b_diag_finalize(const InstDesc *__restr
     const InstDesc &D = desc[i];
     __shared__ double red[8][256];
     double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    const int nb = diag_blocks_of(D.g);
-    if ((int)threadIdx.x < nb)
-        for (int q = 0; q < 4; ++q)
-            s[q] = fpart[4 * ((int64_t)i * kBatchDiagBlocks + threadIdx.x) + q];
+    for (int b = threadIdx.x; b < D.sum_blocks; b += blockDim.x)
+        for (int q = 0; q < 4; ++q) s[q] += fpart[4 * ((int64_t)i * fstride + b) + q];
     const int it1 = item_off[D.tile0 + D.ntiles];
     for (int it = item_off[D.tile0] + threadIdx.x; it < it1; it += blockDim.x)
         for (int q = 0; q < 4; ++q) s[4 + q] += ppart[4 * (int64_t)it + q];
@@ -492,7 +484,9 @@ cudaError_t launch_b_sort(int64_t n, const InstDesc *desc, const long long *p0, 
                            n > 0 ? 1 : 0, st);
 }
 
-int batch_diag_blocks(const Geom &g) { return diag_blocks_of(g); }
+int batch_diag_blocks(const Geom &g) {
+    return (int)std::min<int64_t>(64, ((int64_t)g.n[0] * g.n[1] * g.n[2] + 4095) / 4096);
+}
 
 cudaError_t batch_sort_prepare() { return staged_prepare<BatchKey>(); }
 
@@ -558,19 +552,20 @@ cudaError_t launch_b_green(const InstDesc *desc, int first, int m, int64_t nhalf
     return cudaGetLastError();
 }
 
-cudaError_t launch_b_diag(const InstDesc *desc, int n_inst, int max_blocks, const float *rho,
-                          const float4 *E4, double *fpart, cudaStream_t st) {
-    const dim3 grid((unsigned)n_inst, (unsigned)std::max(1, std::min(max_blocks, kBatchDiagBlocks)));
-    k_b_diag_field<<<grid, 256, 0, st>>>(desc, rho, E4, fpart);
+cudaError_t launch_b_diag(const InstDesc *desc, int n_inst, int max_blocks, int fstride,
+                          const float *rho, const float4 *E4, double *fpart, cudaStream_t st) {
+    if (max_blocks <= 0) return cudaSuccess;
+    k_b_diag_field<<<dim3((unsigned)n_inst, (unsigned)max_blocks), 256, 0, st>>>(desc, rho, E4, fpart,
+                                                                                fstride);
     return cudaGetLastError();
 }
 
-cudaError_t launch_b_diag_finalize(const InstDesc *desc, int n_inst, const int32_t *item_off,
-                                   const double *fpart, const double *ppart, const double *modes,
-                                   Ctrl *ctrl, double dt, pic_diag_t *ring, int ring_cap,
-                                   cudaStream_t st) {
-    k_b_diag_finalize<<<n_inst, 256, 0, st>>>(desc, n_inst, item_off, fpart, ppart, modes, ctrl, dt,
-                                              ring, ring_cap);
+cudaError_t launch_b_diag_finalize(const InstDesc *desc, int n_inst, int fstride,
+                                   const int32_t *item_off, const double *fpart, const double *ppart,
+                                   const double *modes, Ctrl *ctrl, double dt, pic_diag_t *ring,
+                                   int ring_cap, cudaStream_t st) {
+    k_b_diag_finalize<<<n_inst, 256, 0, st>>>(desc, n_inst, fstride, item_off, fpart, ppart, modes, ctrl,
+                                              dt, ring, ring_cap);
     return cudaGetLastError();
 }
 

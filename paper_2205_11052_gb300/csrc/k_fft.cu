@@ -52,6 +52,10 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_forward(int ny, int nz, int
                                                              const float *__restrict__ rho,
                                                              float4 *__restrict__ lE4,
                                                              float2 *__restrict__ out, int64_t nhalf) {
+    if (COMPS == 1) {   // blockIdx.z: one of several grids in a row
+        rho += blockIdx.z * ((int64_t)ax.n * ny * nz);
+        out += blockIdx.z * nhalf;
+    }
     constexpr int ROWS = COMPS == 1 ? kRowsF : kRowsB;
     constexpr int PAIRS = ROWS / 2;
     extern __shared__ float2 sm[];
@@ -102,13 +106,18 @@ __device__ __forceinline__ void load_plane(float2 *s, const float2 *__restrict__
     }
 }
 
-// out_d = symbol_d(in) over one plane (blockIdx.x: x frequency, blockIdx.y: d)
+// out_d = symbol_d(in) over one plane (blockIdx.x: x frequency, blockIdx.y: d,
+// blockIdx.z: grid; each grid has its own wavenumbers)
 __global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, FftAxis ay, FftAxis az,
                                                 const FftTables *__restrict__ tab,
                                                 const float *__restrict__ ktab, float inv_ng,
                                                 const float2 *__restrict__ in,
                                                 float2 *__restrict__ out, int64_t nhalf, int mi, int mj,
-                                                int mk, int mode_comp, int mode_conj, Ctrl *ctrl) {
+                                                int mk, int mode_comp, int mode_conj,
+                                                double *__restrict__ mode) {
+    in += blockIdx.z * nhalf;
+    out += blockIdx.z * 3 * nhalf;
+    ktab += blockIdx.z * (nh + ny + nz);
     extern __shared__ float2 sm[];
     const int pitch = ny | 1, a = blockIdx.x, d = blockIdx.y;
     float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
@@ -135,8 +144,8 @@ __global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, 
         }
         e = v;
         if (d == mode_comp && a == mi && b == mj && c == mk) {
-            ctrl->mode[0] = (double)v.x;
-            ctrl->mode[1] = mode_conj ? -(double)v.y : (double)v.y;
+            mode[2 * blockIdx.z] = (double)v.x;
+            mode[2 * blockIdx.z + 1] = mode_conj ? -(double)v.y : (double)v.y;
         }
     }
     __syncthreads();
@@ -229,7 +238,12 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
                                                               int64_t nhalf, float4 *__restrict__ E4,
                                                               float4 *__restrict__ E8,
                                                               const float *__restrict__ rho,
-                                                              double *__restrict__ fpart) {
+                                                              double *__restrict__ fpart, int fstride) {
+    const int64_t grid0 = blockIdx.z * ((int64_t)ax.n * ny * nz);
+    in += blockIdx.z * 3 * nhalf;
+    E4 += grid0;
+    E8 += 2 * grid0;
+    rho += grid0;
     constexpr int PAIRS = kRowsB / 2;
     extern __shared__ float2 sm[];
     const int n = ax.n, pitch = n | 1;
@@ -253,7 +267,9 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
             ff_add(hi[3], lo[3], rho[g]);
         }
     }
-    if (fpart) block_field_sums<kXThreads>(hi, lo, fpart + 4 * ((int64_t)blockIdx.y * gridDim.x + blockIdx.x));
+    if (fpart)
+        block_field_sums<kXThreads>(hi, lo, fpart + 4 * ((int64_t)blockIdx.z * fstride +
+                                                         blockIdx.y * gridDim.x + blockIdx.x));
 }
 
 // lrho rows -> the x-paired copy read by the deposit-term gathers; the largest
@@ -359,20 +375,21 @@ cudaError_t fft_prepare() {
     return cudaFuncSetAttribute(k_fft_yz_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
-cudaError_t launch_fft_solve(const Geom &g, const FftAxis ax[3], const FftTables *tab, const float *ktab,
-                             const float *rho, float2 *rho_hat, float2 *E_hat, int64_t nhalf,
-                             const int *mode_idx, int mode_comp, int mode_conj, Ctrl *ctrl, float4 *E4,
-                             float4 *E8, double *fpart, cudaStream_t st) {
+cudaError_t launch_fft_solve(const Geom &g, int m, const FftAxis ax[3], const FftTables *tab,
+                             const float *ktab, const float *rho, float2 *rho_hat, float2 *E_hat,
+                             int64_t nhalf, const int *mode_idx, int mode_comp, int mode_conj,
+                             double *mode, float4 *E4, float4 *E8, double *fpart, int fstride,
+                             cudaStream_t st) {
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const float inv_ng = (float)(1.0 / ((double)nx * ny * nz));
-    k_fft_x_forward<1><<<dim3((ny + kRowsF - 1) / kRowsF, nz), kXThreads, x_smem(g, kRowsF / 2), st>>>(
+    k_fft_x_forward<1><<<dim3((ny + kRowsF - 1) / kRowsF, nz, m), kXThreads, x_smem(g, kRowsF / 2), st>>>(
         ny, nz, g.nh, ax[0], tab, rho, nullptr, rho_hat, nhalf);
-    k_fft_yz<<<dim3(g.nh, 3), yz_threads(g), yz_smem(g), st>>>(nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab,
-                                                              inv_ng, rho_hat, E_hat, nhalf, mode_idx[0],
-                                                              mode_idx[1], mode_idx[2], mode_comp, mode_conj,
-                                                              ctrl);
-    k_fft_x_backward<<<dim3((ny + kRowsB - 1) / kRowsB, nz), kXThreads, x_smem(g, 3 * kRowsB / 2), st>>>(
-        ny, nz, g.nh, ax[0], tab, E_hat, nhalf, E4, E8, rho, fpart);
+    k_fft_yz<<<dim3(g.nh, 3, m), yz_threads(g), yz_smem(g), st>>>(nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab,
+                                                                 inv_ng, rho_hat, E_hat, nhalf, mode_idx[0],
+                                                                 mode_idx[1], mode_idx[2], mode_comp,
+                                                                 mode_conj, mode);
+    k_fft_x_backward<<<dim3((ny + kRowsB - 1) / kRowsB, nz, m), kXThreads, x_smem(g, 3 * kRowsB / 2), st>>>(
+        ny, nz, g.nh, ax[0], tab, E_hat, nhalf, E4, E8, rho, fpart, fstride);
     return cudaGetLastError();
 }
 

@@ -377,12 +377,12 @@ int do_solve(pic_ctx *c, bool sums = false) {
     int r = timer_begin(c, PIC_PHASE_SOLVE);
     if (r) return r;
     if (c->own_fft) {
-        PIC_CUDA(launch_fft_solve(c->geom, c->ax, c->at<FftTables>(c->lay.fft_tab),
+        PIC_CUDA(launch_fft_solve(c->geom, 1, c->ax, c->at<FftTables>(c->lay.fft_tab),
                                   c->at<float>(c->lay.ktab), c->at<float>(c->lay.rho),
                                   c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat), c->nhalf,
-                                  c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl(),
+                                  c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl()->mode,
                                   c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8),
-                                  sums ? c->at<double>(c->lay.fpart) : nullptr, c->st));
+                                  sums ? c->at<double>(c->lay.fpart) : nullptr, 0, c->st));
         return timer_end(c, PIC_PHASE_SOLVE, 3);
     }
     PIC_CUFFT(cufftExecR2C(c->r2c, c->at<cufftReal>(c->lay.rho), c->at<cufftComplex>(c->lay.rho_hat)));

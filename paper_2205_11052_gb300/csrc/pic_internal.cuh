@@ -336,11 +336,15 @@ bool fft_axis(int n, FftAxis &a);   // false: not supported
 void fft_tables(const FftAxis ax[3], FftTables &t);
 int fft_sum_blocks(const Geom &g);   // blocks that leave partial field sums
 cudaError_t fft_prepare();           // kernel attributes; outside any stream capture
-// rho -> E4 and E8 (and fpart, 4 doubles per block, unless null)
-cudaError_t launch_fft_solve(const Geom &g, const FftAxis ax[3], const FftTables *tab, const float *ktab,
-                             const float *rho, float2 *rho_hat, float2 *E_hat, int64_t nhalf,
-                             const int *mode_idx, int mode_comp, int mode_conj, Ctrl *ctrl, float4 *E4,
-                             float4 *E8, double *fpart, cudaStream_t st);
+// rho -> E4 and E8 (and fpart, 4 doubles per block, unless null) of m <= 65535
+// grids of one size in a row, spectra in a row too; grid j has the wavenumbers
+// ktab + j (nh + ny + nz), leaves its tracked mode in mode[2 j] and [2 j + 1] and its
+// sums from fpart + 4 j fstride on
+cudaError_t launch_fft_solve(const Geom &g, int m, const FftAxis ax[3], const FftTables *tab,
+                             const float *ktab, const float *rho, float2 *rho_hat, float2 *E_hat,
+                             int64_t nhalf, const int *mode_idx, int mode_comp, int mode_conj,
+                             double *mode, float4 *E4, float4 *E8, double *fpart, int fstride,
+                             cudaStream_t st);
 // lE4 (cleared) -> lrho2, with the bound bookkeeping of launch_adj_pair_rho
 cudaError_t launch_fft_adj_solve(const Geom &g, const FftAxis ax[3], const FftTables *tab,
                                  const float *ktab, float4 *lE4, float2 *lE_hat, float2 *lrho_hat,
