@@ -19,7 +19,8 @@ struct InstDesc {
     long long g0;              // its first node in the concatenated grids
     int tile0, ntiles;         // its global tile ids: [tile0, tile0 + ntiles)
     float qscale;              // q_p / h^3
-    double qscale_d, mp, dV;   // FP64 copies for the conversions and reductions
+    double mp, dV;             // for the reductions
+    float fix_hi, fix_lo;      // qscale / 2^20 as an FP32 pair (fixed_density)
     double inv_h_d[3], h_d[3], L_d[3], two_pi_over_L[3];
     double inv_ng;             // 1 / N_g (folded into the Green kernel)
     int mode_idx[3], mode_comp, mode_conj;

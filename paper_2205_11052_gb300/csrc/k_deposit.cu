@@ -28,6 +28,7 @@
 #include <algorithm>
 
 #include "cic.cuh"
+#include "ffsum.cuh"
 
 namespace pic {
 
@@ -120,20 +121,18 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
 // two nodes per thread and iteration (16-byte loads and stores of the 8-byte
 // words, 8-byte stores of the densities), the odd last node by thread 0
 __global__ void __launch_bounds__(256) k_rho_finish(int64_t ng, unsigned long long *__restrict__ rho64,
-                                                    float *__restrict__ rho, double scale) {
+                                                    float *__restrict__ rho, float sh, float sl) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t n2 = ng >> 1;
     ulonglong2 *r2 = reinterpret_cast<ulonglong2 *>(rho64);
     float2 *f2 = reinterpret_cast<float2 *>(rho);
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n2; q += stride) {
         const ulonglong2 v = __ldcs(r2 + q);
-        __stcs(f2 + q, make_float2((float)((double)(long long)v.x * scale),
-                                   (float)((double)(long long)v.y * scale)));
+        __stcs(f2 + q, make_float2(fixed_density(v.x, sh, sl), fixed_density(v.y, sh, sl)));
         __stcs(r2 + q, make_ulonglong2(0ull, 0ull));
     }
     if ((ng & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
-        const long long v = (long long)rho64[ng - 1];
-        rho[ng - 1] = (float)((double)v * scale);
+        rho[ng - 1] = fixed_density(rho64[ng - 1], sh, sl);
         rho64[ng - 1] = 0ull;
     }
 }
@@ -144,7 +143,9 @@ cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *r
                               cudaStream_t st) {
     const int64_t ng = (int64_t)g.n[0] * g.n[1] * g.n[2];
     const int fb = (int)std::max<int64_t>(1, std::min<int64_t>((ng / 2 + 255) / 256, 152 * 8));
-    k_rho_finish<<<fb, 256, 0, st>>>(ng, rho64, rho, qscale / (double)kFixOne);
+    const double scale = qscale / (double)kFixOne;
+    const float sh = (float)scale, sl = (float)(scale - (double)sh);
+    k_rho_finish<<<fb, 256, 0, st>>>(ng, rho64, rho, sh, sl);
     return cudaGetLastError();
 }
 

@@ -462,6 +462,50 @@ __global__ void __launch_bounds__(256) k_histogram_staged(int64_t n, Key key_par
 }
 
 
+// Histogram of few keys: every key has a counter in shared memory (equal keys of
+// a warp are added up by the atomic unit), and a block adds those of its
+// contiguous share of the particles to the global counts at the end.  The hashed
+// version spends 86 instructions a particle on finding runs and slots; at 134M
+// particles and 4096 keys it took 420 us, this one 172 (reading the cells at
+// memory speed: 80).
+constexpr int kDirectBins = 8192;
+template <class Key>
+__global__ void __launch_bounds__(256) k_histogram_direct(int64_t n, int64_t per, Key key_param,
+                                                           Ctrl *ctrl, int32_t *bins, int nb,
+                                                           SortRange rg, PassEnd pe,
+                                                           const int32_t *gate) {
+    if (gate && !*gate) return;
+    Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
+    extern __shared__ __align__(16) int32_t cnt[];
+    for (int b = threadIdx.x; b < nb; b += 256) cnt[b] = 0;
+    __syncthreads();
+    const int32_t *cell = ctrl->sets[ctrl->cur ^ rg.rel].cell + rg.o;
+    const int64_t b0 = blockIdx.x * per, b1 = b0 + per < n ? b0 + per : n;
+    int bad = 0;
+    // four cells a thread and load, two loads in flight (b0 is a multiple of 1024)
+    int64_t j = b0 + 4 * threadIdx.x;
+    for (; j + 1024 + 3 < b1; j += 2048) {
+        const int4 a = __ldcs(reinterpret_cast<const int4 *>(cell + j));
+        const int4 c = __ldcs(reinterpret_cast<const int4 *>(cell + j + 1024));
+        atomicAdd(cnt + key_of(a.x, rg.o + j, bad), 1);
+        atomicAdd(cnt + key_of(a.y, rg.o + j + 1, bad), 1);
+        atomicAdd(cnt + key_of(a.z, rg.o + j + 2, bad), 1);
+        atomicAdd(cnt + key_of(a.w, rg.o + j + 3, bad), 1);
+        atomicAdd(cnt + key_of(c.x, rg.o + j + 1024, bad), 1);
+        atomicAdd(cnt + key_of(c.y, rg.o + j + 1025, bad), 1);
+        atomicAdd(cnt + key_of(c.z, rg.o + j + 1026, bad), 1);
+        atomicAdd(cnt + key_of(c.w, rg.o + j + 1027, bad), 1);
+    }
+    for (; j < b1; j += 1024)
+        for (int64_t q = j; q < j + 4 && q < b1; ++q)
+            atomicAdd(cnt + key_of(__ldcs(cell + q), rg.o + q, bad), 1);
+    __syncthreads();
+    for (int b = threadIdx.x; b < nb; b += 256)
+        if (cnt[b] > 0) atomicAdd(bins + b, cnt[b]);
+    if (bad) atomicOr(&ctrl->flags, PIC_FLAG_BAD_CELL);
+    if (pe.fused && last_block(&ctrl->done[0])) finish_bins(bins, nb, pe, ctrl);
+}
+
 // One pass by key_of over particles [rg.o, rg.o + n) of set cur ^ rg.rel
 // into the same range of the other set; nb keys (bins holds nb + 1 ints).
 template <class Key>
@@ -472,11 +516,17 @@ cudaError_t staged_pass(int64_t n, const Key &key_of, int64_t nb, Ctrl *ctrl, in
     if (e != cudaSuccess) return e;
     const int T = 256;
     if (n > 0) {
+        // a block of the direct histogram clears and adds up all counters, so it
+        // wants several particles for each
+        const int64_t dblocks = std::min<int64_t>((n + 2047) / 2048, kNumSMs * (nb <= 4096 ? 8 : 6));
+        const int64_t dper = ((n + dblocks - 1) / dblocks + 1023) / 1024 * 1024;
         // short slices while long ones would leave SMs without one
         const int per = n <= (int64_t)kNumSMs * kHistStage ? 4 : kHistPer;
         const int64_t slice = 256 * per;
         const int hblocks = (int)std::min<int64_t>((n + slice - 1) / slice, kNumSMs * 8);
-        if (per == 4) k_histogram_staged<Key, 4><<<hblocks, T, 0, st>>>(n, key_of, ctrl, bins, (int)nb, rg, pe, gate);
+        if (nb <= kDirectBins && dper >= 4 * nb)
+            k_histogram_direct<Key><<<(unsigned)((n + dper - 1) / dper), T, sizeof(int32_t) * (size_t)nb, st>>>(n, dper, key_of, ctrl, bins, (int)nb, rg, pe, gate);
+        else if (per == 4) k_histogram_staged<Key, 4><<<hblocks, T, 0, st>>>(n, key_of, ctrl, bins, (int)nb, rg, pe, gate);
         else k_histogram_staged<Key, kHistPer><<<hblocks, T, 0, st>>>(n, key_of, ctrl, bins, (int)nb, rg, pe, gate);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
