@@ -42,6 +42,7 @@ struct SizeClass {
     bool own;                 // solved by k_fft.cu: axes, tables, wavenumber tables of its instances
     FftAxis ax[3];
     size_t o_tab, o_ktab;
+    int mode_pos[3];          // the tracked mode's position in those spectra
     cufftHandle r2c, c2r;
 };
 
@@ -167,7 +168,7 @@ void batch_layout(pic_batch *b) {
     b->o_fpart = take((size_t)b->n_inst * b->sum_stride * 4 * 8);
     for (SizeClass &c : b->cls) {
         c.o_tab = take(sizeof(FftTables));
-        c.o_ktab = take((size_t)c.m * (c.n[0] / 2 + 1 + c.n[1] + c.n[2]) * 4);
+        c.o_ktab = take((size_t)c.m * fft_ktab_size(b->desc[c.first].g) * 4);
     }
     b->o_ppart = take((size_t)b->max_items * 4 * 8);
     b->o_modes = take((size_t)b->n_inst * 2 * 8);
@@ -233,13 +234,13 @@ int b_solve(pic_batch *b, bool sums) {
     for (SizeClass &c : b->cls) {
         if (c.own) {
             const InstDesc &D = b->desc[c.first];   // same grid and mode indices for the class
-            const int64_t kt = c.n[0] / 2 + 1 + c.n[1] + c.n[2];
+            const int64_t kt = fft_ktab_size(D.g);
             for (int j = 0; j < c.m; j += 65535) {   // grid.z
                 const int m = std::min(c.m - j, 65535);
                 const int64_t g0 = c.g0 + j * c.ng, h0 = c.h0 + j * c.nhalf;
                 B_CUDA(launch_fft_solve(D.g, m, c.ax, b->at<FftTables>(c.o_tab),
                                         b->at<float>(c.o_ktab) + j * kt, rho + g0, rhoh + h0, Eh + 3 * h0,
-                                        c.nhalf, D.mode_idx, D.mode_comp, D.mode_conj,
+                                        c.nhalf, c.mode_pos, D.mode_comp, D.mode_conj,
                                         b->at<double>(b->o_modes) + 2 * (c.first + j),
                                         reinterpret_cast<float4 *>(E) + g0, b->at<float4>(b->o_E8) + 2 * g0,
                                         sums ? b->at<double>(b->o_fpart) + 4 * (int64_t)b->sum_stride *
@@ -423,9 +424,8 @@ int pic_batch_create(const pic_instance_t *inst, int n_inst, double q_over_m,
     b->diag_blocks = 0;
     b->sum_stride = 1;
     for (SizeClass &c : b->cls) {
-        c.own = true;
-        for (int d = 0; d < 3; ++d) c.own = fft_axis(c.n[d], c.ax[d]) && c.own;
         const Geom &g = b->desc[c.first].g;
+        c.own = fft_supported(g, c.ax);
         const int blocks = c.own ? fft_sum_blocks(g) : batch_diag_blocks(g);
         for (int j = c.first; j < c.first + c.m; ++j) {
             b->desc[j].own_fft = c.own;
@@ -487,10 +487,13 @@ int pic_batch_bind_workspace(pic_batch_t b, void *arena, size_t bytes, void *str
         if (c.own) {
             FftTables tab{};
             fft_tables(c.ax, tab);
-            std::vector<float> k((size_t)c.m * (c.n[0] / 2 + 1 + c.n[1] + c.n[2]));
+            const InstDesc &D = b->desc[c.first];
+            const size_t kt = (size_t)fft_ktab_size(D.g);
+            std::vector<float> k(c.m * kt);
             for (int j = 0; j < c.m; ++j)
-                green_table(b->desc[c.first + j].g, b->desc[c.first + j].L_d,
-                            k.data() + (size_t)j * (c.n[0] / 2 + 1 + c.n[1] + c.n[2]));
+                fft_ktab(D.g, b->desc[c.first + j].L_d, tab, k.data() + j * kt);
+            for (int d = 0; d < 3; ++d)
+                c.mode_pos[d] = d == 0 ? D.mode_idx[0] : tab.pos[d][D.mode_idx[d]];
             B_CUDA(fft_prepare());
             B_CUDA(cudaMemcpyAsync(b->arena + c.o_tab, &tab, sizeof(tab), cudaMemcpyHostToDevice, b->st));
             B_CUDA(cudaMemcpyAsync(b->arena + c.o_ktab, k.data(), k.size() * 4, cudaMemcpyHostToDevice, b->st));

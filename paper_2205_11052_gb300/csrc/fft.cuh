@@ -14,6 +14,15 @@ namespace pic {
 
 namespace fft {
 
+// w / d and w % d for 0 <= w < 2^20 by the reciprocal (the half keeps quotients off
+// the integers, and their rounding error is far below 1 / d)
+struct FastDiv {
+    int d;
+    float inv;
+    __device__ __forceinline__ explicit FastDiv(int d_) : d(d_), inv(1.0f / (float)d_) {}
+    __device__ __forceinline__ int quot(int w) const { return (int)(((float)w + 0.5f) * inv); }
+};
+
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
@@ -174,13 +183,11 @@ template <int R, bool INV>
 __device__ __forceinline__ void stage(float2 *s, int lines, int line_stride, int elem_stride, int n,
                                       int M, const float2 *tw) {
     const int sub = M / R, per_line = n / R, work = lines * per_line;
-    const float inv_lines = 1.0f / (float)lines, inv_sub = 1.0f / (float)sub;
+    const FastDiv by_lines(lines), by_sub(sub);
     const int tstep = n / M;
     for (int w = threadIdx.x; w < work; w += blockDim.x) {
-        const int u = (int)(((float)w + 0.5f) * inv_lines);   // exact: work < 2^18
-        const int line = w - u * lines;
-        const int b = (int)(((float)u + 0.5f) * inv_sub);
-        const int j = u - b * sub;
+        const int u = by_lines.quot(w), line = w - u * lines;
+        const int b = by_sub.quot(u), j = u - b * sub;
         float2 *p = s + line * line_stride + (b * M + j) * elem_stride;
         const int step = sub * elem_stride;
         float2 x[R];
@@ -253,10 +260,11 @@ __device__ __forceinline__ void stage_prime(float2 *s, int lines, int line_strid
 }
 
 // all stages of one axis over `lines` lines in shared memory; every thread of
-// the block calls it, with the data written and a barrier passed
+// the block calls it, with the data written and a barrier passed.  Not inlined:
+// one copy of the stages per kernel and direction keeps its code small.
 template <bool INV>
-__device__ __forceinline__ void lines(float2 *s, int nlines, int line_stride, int elem_stride,
-                                      const FftAxis &ax, const float2 *tw) {
+__device__ __noinline__ void lines(float2 *s, int nlines, int line_stride, int elem_stride,
+                                   const FftAxis &ax, const float2 *tw) {
     int M = INV ? 1 : ax.n;
     for (int i = 0; i < ax.stages; ++i) {
         const int R = ax.radix[INV ? ax.stages - 1 - i : i];

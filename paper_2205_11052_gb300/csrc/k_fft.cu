@@ -18,6 +18,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "ffsum.cuh"
 #include "fft.cuh"
@@ -64,8 +65,9 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_forward(int ny, int nz, int
     const int z = blockIdx.y, y0 = blockIdx.x * ROWS, rows = min(ROWS, ny - y0);
     load_twiddles(tw, tab, 0, n);
     float *sf = reinterpret_cast<float *>(s);
+    const fft::FastDiv by_n(n), by_nh(nh);
     for (int w = threadIdx.x; w < ROWS * n; w += kXThreads) {
-        const int r = w / n, x = w - r * n;
+        const int r = by_n.quot(w), x = w - r * n;
         const int64_t g = ((int64_t)z * ny + y0 + r) * n + x;
         float v[3] = {0.f, 0.f, 0.f};
         if (r < rows) {
@@ -87,7 +89,7 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_forward(int ny, int nz, int
     // lanes over the rows: runs of ROWS values at one frequency
     for (int w = threadIdx.x; w < COMPS * nh * PAIRS; w += kXThreads) {
         const int q = w % PAIRS, u = w / PAIRS;
-        const int d = u / nh, k = u - d * nh;
+        const int d = COMPS == 1 ? 0 : by_nh.quot(u), k = u - d * nh;
         const float2 *line = s + (d * PAIRS + q) * pitch;
         float2 a, b;
         unpack_rows(line[tab->pos[0][k]], line[tab->pos[0][k == 0 ? 0 : n - k]], a, b);
@@ -100,9 +102,18 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_forward(int ny, int nz, int
 // plane of one x frequency: [z][y] in global memory, pitch ny | 1 in shared
 __device__ __forceinline__ void load_plane(float2 *s, const float2 *__restrict__ in, int ny, int nz,
                                            int pitch) {
+    const fft::FastDiv by_ny(ny);
     for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
-        const int z = w / ny;
+        const int z = by_ny.quot(w);
         s[z * pitch + (w - z * ny)] = in[w];
+    }
+}
+__device__ __forceinline__ void store_plane(float2 *__restrict__ out, const float2 *s, int ny, int nz,
+                                            int pitch) {
+    const fft::FastDiv by_ny(ny);
+    for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
+        const int z = by_ny.quot(w);
+        out[w] = s[z * pitch + (w - z * ny)];
     }
 }
 
@@ -117,7 +128,7 @@ __global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, 
                                                 double *__restrict__ mode) {
     in += blockIdx.z * nhalf;
     out += blockIdx.z * 3 * nhalf;
-    ktab += blockIdx.z * (nh + ny + nz);
+    ktab += blockIdx.z * (nh + 2 * (ny + nz));
     extern __shared__ float2 sm[];
     const int pitch = ny | 1, a = blockIdx.x, d = blockIdx.y;
     float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
@@ -127,23 +138,23 @@ __global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, 
     __syncthreads();
     lines<false>(s, nz, pitch, 1, ay, twy);
     lines<false>(s, ny, 1, pitch, az, twz);
+    const float *kyp = ktab + nh, *gyp = kyp + ny, *kzp = gyp + ny, *gzp = kzp + nz;
     const float kx = ktab[a];
     const float gx = ((nx & 1) == 0 && a == nx / 2) ? 0.0f : kx;
+    const fft::FastDiv by_ny(ny);
     for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
-        const int pz = w / ny, py = w - pz * ny;
-        const int b = tab->freq[1][py], c = tab->freq[2][pz];
-        const float ky = ktab[nh + b], kz = ktab[nh + ny + c];
-        const float gy = ((ny & 1) == 0 && b == ny / 2) ? 0.0f : ky;
-        const float gz = ((nz & 1) == 0 && c == nz / 2) ? 0.0f : kz;
+        const int pz = by_ny.quot(w), py = w - pz * ny;
+        const float ky = kyp[py], kz = kzp[pz];
         float2 &e = s[pz * pitch + py];
         const float2 rh = e;
         float2 v = make_float2(0.f, 0.f);
-        if ((a | b | c) != 0) {
-            const float sc = inv_ng / (kx * kx + ky * ky + kz * kz) * (d == 0 ? gx : (d == 1 ? gy : gz));
+        if ((a | py | pz) != 0) {   // frequency 0 stays at position 0
+            const float sc = inv_ng / (kx * kx + ky * ky + kz * kz) *
+                             (d == 0 ? gx : (d == 1 ? gyp[py] : gzp[pz]));
             v = make_float2(sc * rh.y, -sc * rh.x);   // -i g rh
         }
         e = v;
-        if (d == mode_comp && a == mi && b == mj && c == mk) {
+        if (d == mode_comp && a == mi && py == mj && pz == mk) {
             mode[2 * blockIdx.z] = (double)v.x;
             mode[2 * blockIdx.z + 1] = mode_conj ? -(double)v.y : (double)v.y;
         }
@@ -152,10 +163,7 @@ __global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, 
     lines<true>(s, ny, 1, pitch, az, twz);
     lines<true>(s, nz, pitch, 1, ay, twy);
     float2 *o = out + d * nhalf + (int64_t)a * ny * nz;
-    for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
-        const int z = w / ny;
-        o[w] = s[z * pitch + (w - z * ny)];
-    }
+    store_plane(o, s, ny, nz, pitch);
 }
 
 // lrho^ = sum_d (+i g_d / |k|^2) lE^_d / N_g of one x frequency: three planes
@@ -171,7 +179,10 @@ __global__ void __launch_bounds__(512) k_fft_yz_adj(int nx, int ny, int nz, int 
     load_twiddles(twy, tab, 1, ny);
     load_twiddles(twz, tab, 2, nz);
     float2 *o = out + (int64_t)a * ny * nz;
+    const float *kyp = ktab + nh, *gyp = kyp + ny, *kzp = gyp + ny, *gzp = kzp + nz;
     const float kx = ktab[a];
+    const float gx = ((nx & 1) == 0 && a == nx / 2) ? 0.0f : kx;
+    const fft::FastDiv by_ny(ny);
     for (int d = 0; d < 3; ++d) {
         __syncthreads();
         load_plane(s, in + d * nhalf + (int64_t)a * ny * nz, ny, nz, pitch);
@@ -179,17 +190,14 @@ __global__ void __launch_bounds__(512) k_fft_yz_adj(int nx, int ny, int nz, int 
         lines<false>(s, nz, pitch, 1, ay, twy);
         lines<false>(s, ny, 1, pitch, az, twz);
         for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
-            const int pz = w / ny, py = w - pz * ny;
-            const int b = tab->freq[1][py], c = tab->freq[2][pz];
-            const float ky = ktab[nh + b], kz = ktab[nh + ny + c];
-            float g = d == 0 ? kx : (d == 1 ? ky : kz);
-            const int m = d == 0 ? a : (d == 1 ? b : c), n = d == 0 ? nx : (d == 1 ? ny : nz);
-            if ((n & 1) == 0 && m == n / 2) g = 0.0f;
+            const int pz = by_ny.quot(w), py = w - pz * ny;
+            const float g = d == 0 ? gx : (d == 1 ? gyp[py] : gzp[pz]);
             const float2 e = s[pz * pitch + py];
             float2 v = make_float2(-g * e.y, g * e.x);   // +i g e
             if (d > 0) v = fft::cadd(v, o[w]);
             if (d == 2) {
-                const float sc = (a | b | c) != 0 ? inv_ng / (kx * kx + ky * ky + kz * kz) : 0.0f;
+                const float ky = kyp[py], kz = kzp[pz];
+                const float sc = (a | py | pz) != 0 ? inv_ng / (kx * kx + ky * ky + kz * kz) : 0.0f;
                 s[pz * pitch + py] = make_float2(sc * v.x, sc * v.y);
             } else {
                 o[w] = v;
@@ -199,10 +207,7 @@ __global__ void __launch_bounds__(512) k_fft_yz_adj(int nx, int ny, int nz, int 
     __syncthreads();
     lines<true>(s, ny, 1, pitch, az, twz);
     lines<true>(s, nz, pitch, 1, ay, twy);
-    for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
-        const int z = w / ny;
-        o[w] = s[z * pitch + (w - z * ny)];
-    }
+    store_plane(o, s, ny, nz, pitch);
 }
 
 // rows y0.. of plane z of COMPS components, from spectra by x frequency to two
@@ -215,9 +220,10 @@ __device__ __forceinline__ void rows_backward(float2 *s, float2 *tw, const float
     constexpr int PAIRS = kRowsB / 2;
     const int n = ax.n, pitch = n | 1;
     load_twiddles(tw, tab, 0, n);
+    const fft::FastDiv by_nh(nh);
     for (int w = threadIdx.x; w < COMPS * nh * PAIRS; w += kXThreads) {
         const int q = w % PAIRS, u = w / PAIRS;
-        const int d = u / nh, k = u - d * nh;
+        const int d = COMPS == 1 ? 0 : by_nh.quot(u), k = u - d * nh;
         const float2 *p = in + d * nhalf + ((int64_t)k * nz + z) * ny + y0;
         float2 a = make_float2(0.f, 0.f), b = a;
         if (2 * q < rows) a = p[2 * q];
@@ -251,8 +257,9 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
     rows_backward<3>(sm, sm + 3 * PAIRS * pitch, in, nhalf, ny, nz, nh, z, y0, rows, ax, tab);
     const float *sf = reinterpret_cast<const float *>(sm);
     float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+    const fft::FastDiv by_n(n);
     for (int w = threadIdx.x; w < rows * n; w += kXThreads) {
-        const int r = w / n, x = w - r * n, x1 = x + 1 == n ? 0 : x + 1;
+        const int r = by_n.quot(w), x = w - r * n, x1 = x + 1 == n ? 0 : x + 1;
         const float *f0 = sf + 2 * ((r >> 1) * pitch) + (r & 1);
         const float *f1 = f0 + 2 * PAIRS * pitch, *f2 = f1 + 2 * PAIRS * pitch;
         const float4 e = make_float4(f0[2 * x], f1[2 * x], f2[2 * x], 0.0f);
@@ -290,8 +297,9 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward_adj(int ny, int nz
     rows_backward<1>(sm, sm + PAIRS * pitch, in, 0, ny, nz, nh, z, y0, rows, ax, tab);
     const float *sf = reinterpret_cast<const float *>(sm);
     float m = 0.0f;
+    const fft::FastDiv by_n(n);
     for (int w = threadIdx.x; w < rows * n; w += kXThreads) {
-        const int r = w / n, x = w - r * n, x1 = x + 1 == n ? 0 : x + 1;
+        const int r = by_n.quot(w), x = w - r * n, x1 = x + 1 == n ? 0 : x + 1;
         const float *f = sf + 2 * ((r >> 1) * pitch) + (r & 1);
         lrho2[((int64_t)z * ny + y0 + r) * n + x] = make_float2(f[2 * x], f[2 * x1]);
         m = fmaxf(m, fabsf(f[2 * x]));
@@ -306,6 +314,8 @@ void split(int m, int depth, int *cur, int &best, int &best_sum, FftAxis &a) {
     if (m == 1) {
         int sum = 0;
         for (int i = 0; i < depth; ++i) sum += cur[i];
+        // a lone 16 leaves one thread a line: two stages of 4 keep more busy
+        if (depth == 1 && cur[0] == 16) depth = 2, cur[0] = cur[1] = 4, sum = 8;
         if (depth < best || (depth == best && sum < best_sum)) {
             best = depth;
             best_sum = sum;
@@ -333,7 +343,7 @@ size_t x_smem(const Geom &g, int line_count) {
 }
 int yz_threads(const Geom &g) {
     const int pts = g.n[1] * g.n[2];
-    return pts >= 2048 ? 512 : (pts >= 512 ? 256 : 128);
+    return pts >= 2048 ? 512 : (pts >= 1024 ? 256 : 128);
 }
 
 }  // namespace
@@ -365,11 +375,40 @@ void fft_tables(const FftAxis ax[3], FftTables &t) {
     }
 }
 
+// One (y, z) plane has to leave room for a second block on an SM: 128^3 grids, at
+// one block per SM (195 blocks on 152), took 157 us a solve with sums against 102.
+bool fft_supported(const Geom &g, FftAxis ax[3]) {
+    for (int d = 0; d < 3; ++d)
+        if (!fft_axis(g.n[d], ax[d])) return false;
+    return 2 * (yz_smem(g) + 1024) <= (size_t)228 * 1024;
+}
+
+// x: nh wavenumbers; y and z: those at each position, then the gradient's (zero at
+// the Nyquist frequency)
+int fft_ktab_size(const Geom &g) { return g.nh + 2 * (g.n[1] + g.n[2]); }
+void fft_ktab(const Geom &g, const double *L_d, const FftTables &t, float *out) {
+    std::vector<float> k((size_t)(g.nh + g.n[1] + g.n[2]));
+    green_table(g, L_d, k.data());
+    for (int a = 0; a < g.nh; ++a) out[a] = k[a];
+    float *o = out + g.nh;
+    int off = g.nh;
+    for (int d = 1; d < 3; ++d) {
+        const int n = g.n[d];
+        for (int p = 0; p < n; ++p) {
+            const int f = t.freq[d][p];
+            o[p] = k[off + f];
+            o[n + p] = (n & 1) == 0 && f == n / 2 ? 0.0f : k[off + f];
+        }
+        o += 2 * n;
+        off += n;
+    }
+}
+
 int fft_sum_blocks(const Geom &g) { return (g.n[1] + kRowsB - 1) / kRowsB * g.n[2]; }
 
 cudaError_t fft_prepare() {
     cudaError_t e;
-    const int most = (int)(sizeof(float2) * (kFftMaxN * (kFftMaxN | 1) + 2 * kFftMaxN));
+    const int most = 114 * 1024;   // see fft_supported
     if ((e = cudaFuncSetAttribute(k_fft_yz, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess)
         return e;
     return cudaFuncSetAttribute(k_fft_yz_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, most);

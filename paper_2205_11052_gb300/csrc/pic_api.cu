@@ -77,6 +77,7 @@ struct pic_ctx {
     int64_t cap, ng, nhalf, nbins, ntiles, max_items, staging;
     int chunk, block, sparse_below, deposit_blocks;
     int mode_idx[3], mode_conj;
+    int mode_pos[3];          // its position in spectra of k_fft.cu
     size_t fft_reserve;
     Layout lay;
     // bound state
@@ -225,7 +226,7 @@ void compute_layout(pic_ctx *c) {
     L.stage_v = take((size_t)c->staging * 24);
     L.adjE4 = take((size_t)c->ng * 16);
     L.lrho2 = take((size_t)c->ng * 8);
-    L.ktab = take((size_t)(c->geom.nh + c->grid.n[1] + c->grid.n[2]) * 4);
+    L.ktab = take((size_t)fft_ktab_size(c->geom) * 4);
     L.node_pos = take((size_t)3 * kMaxN * 8);
     L.fft_tab = take(sizeof(FftTables));
     L.fft = take(c->fft_reserve);
@@ -380,7 +381,7 @@ int do_solve(pic_ctx *c, bool sums = false) {
         PIC_CUDA(launch_fft_solve(c->geom, 1, c->ax, c->at<FftTables>(c->lay.fft_tab),
                                   c->at<float>(c->lay.ktab), c->at<float>(c->lay.rho),
                                   c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat), c->nhalf,
-                                  c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl()->mode,
+                                  c->mode_pos, c->prm.mode_comp, c->mode_conj, c->ctrl()->mode,
                                   c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8),
                                   sums ? c->at<double>(c->lay.fpart) : nullptr, 0, c->st));
         return timer_end(c, PIC_PHASE_SOLVE, 3);
@@ -929,8 +930,7 @@ int pic_create(const pic_grid_t *grid, const pic_species_t *species, const pic_p
     c->mode_idx[1] = ((m[1] % grid->n[1]) + grid->n[1]) % grid->n[1];
     c->mode_idx[2] = ((m[2] % grid->n[2]) + grid->n[2]) % grid->n[2];
 
-    c->own_fft = true;
-    for (int d = 0; d < 3; ++d) c->own_fft = fft_axis(g.n[d], c->ax[d]) && c->own_fft;
+    c->own_fft = fft_supported(g, c->ax);
     c->fft_reserve = 0;
     if (!c->own_fft) {
         // cuFFT work area: the library's own size query when it works here,
@@ -967,12 +967,15 @@ int pic_bind_workspace(pic_handle_t c, void *arena, size_t bytes, void *stream) 
     c->adj.ready = false;
     c->arena = static_cast<char *>(arena);
     c->st = static_cast<cudaStream_t>(stream);
+    std::vector<float> ktab((size_t)fft_ktab_size(c->geom));
     if (c->own_fft) {
         FftTables tab{};
         fft_tables(c->ax, tab);
         PIC_CUDA(fft_prepare());
         PIC_CUDA(cudaMemcpyAsync(c->at<FftTables>(c->lay.fft_tab), &tab, sizeof(tab),
                                  cudaMemcpyHostToDevice, c->st));
+        fft_ktab(c->geom, c->L, tab, ktab.data());
+        for (int d = 0; d < 3; ++d) c->mode_pos[d] = d == 0 ? c->mode_idx[0] : tab.pos[d][c->mode_idx[d]];
         PIC_CUDA(cudaStreamSynchronize(c->st));
     } else {
         size_t wmax = 0;
@@ -1007,8 +1010,7 @@ int pic_bind_workspace(pic_handle_t c, void *arena, size_t bytes, void *stream) 
     c->hsets[0] = h.sets[0];
     c->hsets[1] = h.sets[1];
     PIC_CUDA(cudaMemcpyAsync(c->ctrl(), &h, sizeof(h), cudaMemcpyHostToDevice, c->st));
-    std::vector<float> ktab((size_t)(c->geom.nh + c->grid.n[1] + c->grid.n[2]));
-    green_table(c->geom, c->L, ktab.data());
+    if (!c->own_fft) green_table(c->geom, c->L, ktab.data());
     PIC_CUDA(cudaMemcpyAsync(c->at<float>(c->lay.ktab), ktab.data(), ktab.size() * 4,
                              cudaMemcpyHostToDevice, c->st));
     std::vector<double> npos((size_t)3 * kMaxN);

@@ -316,9 +316,8 @@ cudaError_t launch_diag_finalize(const double *field_part, int field_blocks,
                                  Ctrl *ctrl, pic_diag_t *ring, int ring_cap, cudaStream_t st);
 
 // Field solve by the library's own line transforms (k_fft.cu), for grids whose
-// axes are at most kFftMaxN long with no prime factor above kFftMaxPrime (one
-// (y, z) plane of a spectrum then fits a block's shared memory); others go
-// through cuFFT.
+// axes are at most kFftMaxN long with no prime factor above kFftMaxPrime and whose
+// (y, z) planes fit (fft_supported); others go through cuFFT.
 constexpr int kFftMaxN = 128;
 constexpr int kFftMaxPrime = 31;
 constexpr int kFftMaxStages = 4;
@@ -333,12 +332,16 @@ struct FftTables {
     int pos[3][kFftMaxN], freq[3][kFftMaxN];
 };
 bool fft_axis(int n, FftAxis &a);   // false: not supported
+bool fft_supported(const Geom &g, FftAxis ax[3]);
+int fft_ktab_size(const Geom &g);   // wavenumber table of one grid for these kernels
+void fft_ktab(const Geom &g, const double *L_d, const FftTables &t, float *out);
 void fft_tables(const FftAxis ax[3], FftTables &t);
 int fft_sum_blocks(const Geom &g);   // blocks that leave partial field sums
 cudaError_t fft_prepare();           // kernel attributes; outside any stream capture
 // rho -> E4 and E8 (and fpart, 4 doubles per block, unless null) of m <= 65535
-// grids of one size in a row, spectra in a row too; grid j has the wavenumbers
-// ktab + j (nh + ny + nz), leaves its tracked mode in mode[2 j] and [2 j + 1] and its
+// grids of one size in a row, spectra in a row too; mode_idx are positions in y
+// and z; grid j has the wavenumbers
+// ktab + j fft_ktab_size, leaves its tracked mode in mode[2 j] and [2 j + 1] and its
 // sums from fpart + 4 j fstride on
 cudaError_t launch_fft_solve(const Geom &g, int m, const FftAxis ax[3], const FftTables *tab,
                              const float *ktab, const float *rho, float2 *rho_hat, float2 *E_hat,
