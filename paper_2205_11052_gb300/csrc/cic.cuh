@@ -191,6 +191,16 @@ __device__ __forceinline__ int box_row(const Tile &t) { return B > 0 ? B : t.S0;
 template <int B>
 __device__ __forceinline__ int box_plane(const Tile &t) { return B > 0 ? B * B : t.S01; }
 
+// whether the stencil with base slots (si, sj, sk) lies in the box
+template <int B>
+__device__ __forceinline__ bool in_box_slots(const Tile &t, const Geom &g, int si, int sj, int sk) {
+    if (B > 0)
+        return (unsigned)si < (unsigned)(B - 1) && (unsigned)sj < (unsigned)(B - 1) &&
+               (unsigned)sk < (unsigned)(B - 1);
+    return (unsigned)si < (unsigned)(t.S0 - 1) && (unsigned)sj < (unsigned)(g.tile[1] + 2 * g.guard) &&
+           (unsigned)sk < (unsigned)(g.tile[2] + 2 * g.guard);
+}
+
 // slot s of stencil base (i, j, k) in the box of tile t; true if the whole
 // 2x2x2 stencil lies inside the box
 template <int B = 0>
@@ -200,11 +210,27 @@ __device__ __forceinline__ bool box_base(const Tile &t, const Geom &g, int i, in
     const int sj = box_slot(j, t.oy, g.n[1], G);
     const int sk = box_slot(k, t.oz, g.n[2], G);
     s = si + box_row<B>(t) * sj + box_plane<B>(t) * sk;
-    if (B > 0)
-        return (unsigned)si < (unsigned)(B - 1) && (unsigned)sj < (unsigned)(B - 1) &&
-               (unsigned)sk < (unsigned)(B - 1);
-    return (unsigned)si < (unsigned)(t.S0 - 1) && (unsigned)sj < (unsigned)(g.tile[1] + 2 * G) &&
-           (unsigned)sk < (unsigned)(g.tile[2] + 2 * G);
+    return in_box_slots<B>(t, g, si, sj, sk);
+}
+
+// add the particle's weights to the shared tile at stencil base slot s
+template <bool FIXED, int B = 0>
+__device__ __forceinline__ void tile_add_at(uint32_t *acc, const Tile &t, int s, float fx, float fy,
+                                            float fz) {
+    const int S0 = box_row<B>(t), S01 = box_plane<B>(t);
+    const int off[8] = {0, 1, S0, S0 + 1, S01, S01 + 1, S01 + S0, S01 + S0 + 1};
+    if (FIXED) {
+        uint32_t q[8];
+        fixed_split(fx, fy, fz, q);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) atomicAdd(acc + s + off[c], q[c]);
+    } else {
+        float w[8];
+        weights(fx, fy, fz, w);
+        float *accf = reinterpret_cast<float *>(acc);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) atomicAdd(accf + s + off[c], w[c]);
+    }
 }
 
 // returns true if the particle went to the shared tile, false if to the grid
@@ -214,20 +240,7 @@ __device__ __forceinline__ bool tile_add(uint32_t *acc, const Tile &t, const Geo
                                          unsigned long long *rho64, float qscale) {
     int s;
     if (box_base<B>(t, g, i, j, k, s)) {
-        const int S0 = box_row<B>(t), S01 = box_plane<B>(t);
-        const int off[8] = {0, 1, S0, S0 + 1, S01, S01 + 1, S01 + S0, S01 + S0 + 1};
-        if (FIXED) {
-            uint32_t q[8];
-            fixed_split(fx, fy, fz, q);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) atomicAdd(acc + s + off[c], q[c]);
-        } else {
-            float w[8];
-            weights(fx, fy, fz, w);
-            float *accf = reinterpret_cast<float *>(acc);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) atomicAdd(accf + s + off[c], w[c]);
-        }
+        tile_add_at<FIXED, B>(acc, t, s, fx, fy, fz);
         return true;
     }
     float w[8];
@@ -299,8 +312,8 @@ __device__ __forceinline__ void stage_box(float4 *sE, const float4 *__restrict__
 }
 __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// The same box with x pairs, from E8: sA holds (Ex, Ey, Ez) of a slot and Ex of
-// its +x neighbour, sB the neighbour's Ey and Ez.
+// The same box with x pairs, from E8: sA holds Ex and Ey of a slot and of its +x
+// neighbour, sB the two Ez.
 __device__ __forceinline__ void stage_pairs(float4 *sA, float2 *sB, const float4 *__restrict__ E8,
                                             const Tile &t, const Geom &g) {
     const uint32_t da = (uint32_t)__cvta_generic_to_shared(sA);

@@ -211,54 +211,6 @@ __device__ __forceinline__ void stage(float2 *s, int lines, int line_stride, int
     __syncthreads();
 }
 
-// A stage of a prime radix R without registers for a whole transform: each
-// thread forms up to kPrimeOut outputs of R-point sums, then the block writes
-// them back in place.
-constexpr int kPrimeOut = 4;
-template <bool INV>
-__device__ __forceinline__ void stage_prime(float2 *s, int lines, int line_stride, int elem_stride,
-                                            int n, int M, int R, const float2 *tw) {
-    const int sub = M / R, per_line = n / R, total = lines * per_line;
-    const int chunk = max(1, (int)blockDim.x * kPrimeOut / R);   // transforms per round
-    const int tstep = n / M, rstep = n / R;
-    for (int c0 = 0; c0 < total; c0 += chunk) {
-        const int outs = min(chunk, total - c0) * R;
-        float2 y[kPrimeOut];
-        float2 *at[kPrimeOut];
-#pragma unroll
-        for (int e = 0; e < kPrimeOut; ++e) {
-            const int w = threadIdx.x + e * blockDim.x;
-            at[e] = nullptr;
-            if (w >= outs) continue;
-            const int k = w % R, t = c0 + w / R;
-            const int line = t % lines, u = t / lines;
-            const int b = u / sub, j = u - b * sub;
-            const float2 *p = s + line * line_stride + (b * M + j) * elem_stride;
-            float2 a = make_float2(0.f, 0.f);
-            int m = 0;   // q k mod R
-            for (int q = 0; q < R; ++q) {
-                float2 v = p[q * sub * elem_stride];
-                if (INV) {
-                    const float2 h = tw[tstep * j * q];
-                    v = cmul(v, make_float2(h.x, -h.y));
-                }
-                const float2 f = tw[rstep * m];
-                a = cadd(a, cmul(v, INV ? make_float2(f.x, -f.y) : f));
-                m += k;
-                if (m >= R) m -= R;
-            }
-            if (!INV) a = cmul(a, tw[tstep * j * k]);
-            y[e] = a;
-            at[e] = s + line * line_stride + (b * M + j + k * sub) * elem_stride;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int e = 0; e < kPrimeOut; ++e)
-            if (at[e]) *at[e] = y[e];
-        __syncthreads();
-    }
-}
-
 // all stages of one axis over `lines` lines in shared memory; every thread of
 // the block calls it, with the data written and a barrier passed.  Not inlined:
 // one copy of the stages per kernel and direction keeps its code small.
@@ -278,7 +230,6 @@ __device__ __noinline__ void lines(float2 *s, int nlines, int line_stride, int e
         case 7: stage<7, INV>(s, nlines, line_stride, elem_stride, ax.n, M, tw); break;
         case 8: stage<8, INV>(s, nlines, line_stride, elem_stride, ax.n, M, tw); break;
         case 16: stage<16, INV>(s, nlines, line_stride, elem_stride, ax.n, M, tw); break;
-        default: stage_prime<INV>(s, nlines, line_stride, elem_stride, ax.n, M, R, tw); break;
         }
         if (!INV) M /= R;
     }

@@ -444,8 +444,8 @@ __global__ void k_b_pack(int64_t mng, int nx, const float *__restrict__ planar,
         const int64_t q1 = (i + 1 == nx) ? q - i : q + 1;
         const float4 e = make_float4(planar[q], planar[q + mng], planar[q + 2 * mng], 0.0f);
         E4[q] = e;
-        E8[2 * q] = make_float4(e.x, e.y, e.z, planar[q1]);
-        E8[2 * q + 1] = make_float4(planar[q1 + mng], planar[q1 + 2 * mng], 0.0f, 0.0f);
+        E8[2 * q] = make_float4(e.x, e.y, planar[q1], planar[q1 + mng]);
+        E8[2 * q + 1] = make_float4(e.z, planar[q1 + 2 * mng], 0.0f, 0.0f);
     }
 }
 

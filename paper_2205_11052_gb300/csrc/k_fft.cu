@@ -265,8 +265,8 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
         const float4 e = make_float4(f0[2 * x], f1[2 * x], f2[2 * x], 0.0f);
         const int64_t g = ((int64_t)z * ny + y0 + r) * n + x;
         E4[g] = e;
-        E8[2 * g] = make_float4(e.x, e.y, e.z, f0[2 * x1]);
-        E8[2 * g + 1] = make_float4(f1[2 * x1], f2[2 * x1], 0.0f, 0.0f);
+        E8[2 * g] = make_float4(e.x, e.y, f0[2 * x1], f1[2 * x1]);
+        E8[2 * g + 1] = make_float4(e.z, f2[2 * x1], 0.0f, 0.0f);
         if (fpart) {
             ff_add_sq(hi[0], lo[0], e.x);
             ff_add_sq(hi[1], lo[1], e.y);
@@ -308,8 +308,8 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward_adj(int ny, int nz
     if ((threadIdx.x & 31) == 0 && m > 0.0f) atomicMax(&ctrl->adj_lrho[par], __float_as_uint(m));
 }
 
-// Split n into the radices of fft.cuh, fewest stages first, or one with a
-// larger prime up to kFftMaxPrime.
+// Split n into the radices of fft.cuh, fewest stages first.  (Stages of larger
+// primes as plain sums lost: 78 x 88 x 91 took 139 us against cuFFT's 76.)
 void split(int m, int depth, int *cur, int &best, int &best_sum, FftAxis &a) {
     if (m == 1) {
         int sum = 0;
@@ -325,11 +325,8 @@ void split(int m, int depth, int *cur, int &best, int &best_sum, FftAxis &a) {
         return;
     }
     if (depth >= kFftMaxStages) return;
-    for (int r = std::min(m, kFftMaxPrime); r >= 2; --r) {
+    for (int r : {16, 8, 7, 6, 5, 4, 3, 2}) {
         if (m % r != 0 || (depth > 0 && r > cur[depth - 1])) continue;
-        const bool prime = r != 4 && r != 6 && r != 9 && r % 2 != 0 && (r == 3 || r % 3 != 0) &&
-                           (r == 5 || r % 5 != 0);   // among r <= 31, none else is odd and composite
-        if (!(r <= 8 || r == 16 || prime)) continue;
         cur[depth] = r;
         split(m / r, depth + 1, cur, best, best_sum, a);
     }
@@ -375,12 +372,13 @@ void fft_tables(const FftAxis ax[3], FftTables &t) {
     }
 }
 
-// One (y, z) plane has to leave room for a second block on an SM: 128^3 grids, at
-// one block per SM (195 blocks on 152), took 157 us a solve with sums against 102.
+// Planes of at most 96^2 points: 96^3 solves take 55 us against 63 through cuFFT,
+// 64^3 33 against 47, 16^3 23 against 33 (200 in a row); at 128^3 the 195 blocks
+// of one per SM make two rounds and take 157 against 102 (with sums, cold caches).
 bool fft_supported(const Geom &g, FftAxis ax[3]) {
     for (int d = 0; d < 3; ++d)
         if (!fft_axis(g.n[d], ax[d])) return false;
-    return 2 * (yz_smem(g) + 1024) <= (size_t)228 * 1024;
+    return g.n[1] * g.n[2] <= 96 * 96;
 }
 
 // x: nh wavenumbers; y and z: those at each position, then the gradient's (zero at
@@ -408,7 +406,8 @@ int fft_sum_blocks(const Geom &g) { return (g.n[1] + kRowsB - 1) / kRowsB * g.n[
 
 cudaError_t fft_prepare() {
     cudaError_t e;
-    const int most = 114 * 1024;   // see fft_supported
+    // the largest plane of fft_supported, its rows padded: 128 x (72 | 1) points
+    const int most = (int)(sizeof(float2) * (96 * 96 + 128 + 2 * kFftMaxN));
     if ((e = cudaFuncSetAttribute(k_fft_yz, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess)
         return e;
     return cudaFuncSetAttribute(k_fft_yz_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, most);

@@ -101,7 +101,7 @@ __global__ void k_diag_finalize(const double *__restrict__ fpart, int fblocks,
 namespace {
 // Planar field rows (component d of row r at planar + d * dist + r * pitch) ->
 // E4, the x-paired E8 read by 256-bit loads (the components at q, then those at
-// its +x neighbour, periodic: Ex Ey Ez Ex' | Ey' Ez' 0 0) and, with SUMS, the block's partial sums of
+// its +x neighbour, periodic: Ex Ey Ex' Ey' | Ez Ez' 0 0) and, with SUMS, the block's partial sums of
 // Ex^2, Ey^2, Ez^2 and rho.  Bound by DRAM: 12 bytes read and 48 written per
 // node (16.8M nodes: 246 us).  With the interleaving left to the inverse
 // transform (output stride 4: 407 us against 92 planar), a pairing pass (120)
@@ -113,15 +113,17 @@ __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pi
                                                 const float *__restrict__ rho,
                                                 double *__restrict__ part) {
     float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
+    // one warp per row
+    const int lane = threadIdx.x & 31;
+    for (int64_t r = blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8) {
         const float *p0 = planar + r * pitch, *p1 = p0 + dist, *p2 = p1 + dist;
-        for (int x = threadIdx.x; x < nx; x += 256) {
+        for (int x = lane; x < nx; x += 32) {
             const int x1 = x + 1 == nx ? 0 : x + 1;
             const int64_t q = r * nx + x;
             const float4 e = make_float4(p0[x], p1[x], p2[x], 0.0f);
             E4[q] = e;
-            E8[2 * q] = make_float4(e.x, e.y, e.z, p0[x1]);
-            E8[2 * q + 1] = make_float4(p1[x1], p2[x1], 0.0f, 0.0f);
+            E8[2 * q] = make_float4(e.x, e.y, p0[x1], p1[x1]);
+            E8[2 * q + 1] = make_float4(e.z, p2[x1], 0.0f, 0.0f);
             if (SUMS) {
                 ff_add_sq(hi[0], lo[0], e.x);
                 ff_add_sq(hi[1], lo[1], e.y);

@@ -318,31 +318,50 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(int64_t n, Geom g, PushC
 // it at the end: per step the particle store is read and written once (56
 // bytes per particle) instead of being read again by a separate deposit.
 // ---------------------------------------------------------------------------
-// E from the block's shared copy of its tile's box when it holds one (see
-// push_one_pair_box), else from the x-paired grid.
+// One particle of the tile t (or of a sparse segment: everything through the
+// grid).  E comes from (sA, sB), the block's copy of the tile's box, when it holds
+// one and the stencil lies in it, else from the x-paired grid.  The slots of the
+// new stencil base are the old ones plus the cells moved, so the periodic
+// folding is done once per particle unless it leaves the box.
 template <bool DIAG, bool EXT, bool MAG, bool FIXED, int B>
 __device__ __forceinline__ void pd_one(const Geom &g, const PushConst &pc, const float4 *E8,
                                        const float4 *sA, const float2 *sB, bool sparse,
-                                       uint32_t *acc,
-                                       const cic::Tile &t, float *rho, unsigned long long *rho64,
-                                       float qscale, int32_t &c, float &fx, float &fy, float &fz,
-                                       float &vx, float &vy, float &vz, int &bad,
+                                       uint32_t *acc, const cic::Tile &t, float *rho,
+                                       unsigned long long *rho64, float qscale, int32_t &c, float &fx,
+                                       float &fy, float &fz, float &vx, float &vy, float &vz, int &bad,
                                        unsigned long long &strays, float (&a)[4]) {
-    int i, j, k;
-    push_one_pair_box<EXT, MAG, B>(g, pc, E8, sA, sB, t, c, fx, fy, fz, vx, vy, vz, bad, i, j, k);
-    if (sparse) {
-        float w[8];
-        cic::weights(fx, fy, fz, w);
-        cic::deposit_global<FIXED>(rho, rho64, g, i, j, k, w, fx, fy, fz, qscale);
-    } else if (!cic::tile_add<FIXED, B>(acc, t, g, i, j, k, fx, fy, fz, rho, rho64, qscale)) {
-        ++strays;
-    }
+    int i, j, k, step[3];
+    decode_base(g, c, i, j, k, bad);
+    int si = cic::box_slot(i, t.ox, g.n[0], g.guard);
+    int sj = cic::box_slot(j, t.oy, g.n[1], g.guard);
+    int sk = cic::box_slot(k, t.oz, g.n[2], g.guard);
+    float ex, ey, ez;
+    if (sA != nullptr && cic::in_box_slots<B>(t, g, si, sj, sk))
+        gather_E_pair_box<B>(sA, sB, si + cic::box_row<B>(t) * sj + cic::box_plane<B>(t) * sk, t.S0,
+                             t.S01, fx, fy, fz, ex, ey, ez);
+    else
+        gather_E_pairs(g, E8, i, j, k, fx, fy, fz, ex, ey, ez);
+    kick_drift<EXT, MAG>(g, pc, ex, ey, ez, i, j, k, c, fx, fy, fz, vx, vy, vz, bad, step);
     if (DIAG) {
         a[0] += vx;
         a[1] += vy;
         a[2] += vz;
         a[3] += vx * vx + vy * vy + vz * vz;
     }
+    if (!sparse) {
+        si += step[0];
+        sj += step[1];
+        sk += step[2];
+        int s = si + cic::box_row<B>(t) * sj + cic::box_plane<B>(t) * sk;
+        if (cic::in_box_slots<B>(t, g, si, sj, sk) || cic::box_base<B>(t, g, i, j, k, s)) {
+            cic::tile_add_at<FIXED, B>(acc, t, s, fx, fy, fz);
+            return;
+        }
+        ++strays;
+    }
+    float w[8];
+    cic::weights(fx, fy, fz, w);
+    cic::deposit_global<FIXED>(rho, rho64, g, i, j, k, w, fx, fy, fz, qscale);
 }
 
 // staged: the block copies its tile's box of E8 to shared memory at each change
@@ -604,8 +623,9 @@ __device__ __forceinline__ void move_one(const Geom &g, uint64_t seed, long long
                                          int32_t &c, float &fx, float &fy, float &fz, int &bad) {
     int i, j, k;
     decode_base(g, c, i, j, k, bad);
+    int step[3];
     advance_cells(g, fx + move_cells(seed, n, pid, 0), fy + move_cells(seed, n, pid, 1),
-                  fz + move_cells(seed, n, pid, 2), i, j, k, c, fx, fy, fz, bad);
+                  fz + move_cells(seed, n, pid, 2), i, j, k, c, fx, fy, fz, bad, step);
 }
 
 template <bool DIAG>

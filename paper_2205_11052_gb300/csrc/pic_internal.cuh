@@ -301,7 +301,7 @@ cudaError_t launch_gather_push(int64_t n, const Geom &g, const PushConst &pc, bo
                                Ctrl *ctrl, const float4 *E8, double *part, int blocks,
                                int threads, cudaStream_t st);
 // planar E (component d of row r at planar + d * dist + r * pitch) -> E4, the
-// x-paired E8 (six floats in 32 bytes per node: E at q, then E at q + x, periodic),
+// x-paired E8 (Ex Ey Ex' Ey' Ez Ez' 0 0 per node, primed at q + x, periodic),
 // and unless null the partial field sums of kDiagFieldBlocks blocks
 cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E4,
                           float4 *E8, const float *rho, double *part, cudaStream_t st);
@@ -316,10 +316,9 @@ cudaError_t launch_diag_finalize(const double *field_part, int field_blocks,
                                  Ctrl *ctrl, pic_diag_t *ring, int ring_cap, cudaStream_t st);
 
 // Field solve by the library's own line transforms (k_fft.cu), for grids whose
-// axes are at most kFftMaxN long with no prime factor above kFftMaxPrime and whose
-// (y, z) planes fit (fft_supported); others go through cuFFT.
+// axes are at most kFftMaxN long with no prime factor above 7 and whose (y, z)
+// planes fit (fft_supported); others go through cuFFT.
 constexpr int kFftMaxN = 128;
-constexpr int kFftMaxPrime = 31;
 constexpr int kFftMaxStages = 4;
 struct FftAxis {
     int n, stages;
