@@ -328,6 +328,16 @@ __device__ __forceinline__ void stage_pairs(float4 *sA, float2 *sB, const float4
     }
 }
 
+// ... and of an array of one float2 per node
+__device__ __forceinline__ void stage_float2(float2 *sR, const float2 *__restrict__ v, const Tile &t,
+                                             const Geom &g) {
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sR);
+    for (int s = threadIdx.x; s < t.S; s += blockDim.x)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst + 8u * (uint32_t)s),
+                     "l"(v + slot_node(t, g, s))
+                     : "memory");
+}
+
 // byte offset of a staged box of S slots in the push kernels' shared memory,
 // after the item tile and the tile sums
 __host__ __device__ __forceinline__ size_t stage_offset(int S) {

@@ -84,14 +84,16 @@ __device__ __forceinline__ void interp_grad(float fx, float fy, float fz, const 
          fx * fy * (sc[7] - sc[3]);
 }
 
-__device__ __forceinline__ int tile_slot(int a, int o, int n, int T, int G) {
-    int d = a - o;
-    if (d < 0) d += n;
-    if (d >= T + G) {
-        d -= n;
-        if (d < -G) return -1;
-    }
-    return d + G;
+// w q rounded to the nearest integer, |w q| < 2^22: one fused multiply-add with
+// 1.5 2^23, whose rounding leaves the integer in the mantissa (conversions run at
+// an eighth of the FP32 rate, and a particle has 24)
+__device__ __forceinline__ int round_product(float w, float q) {
+    return __float_as_int(__fmaf_rn(w, q, 12582912.0f)) - 0x4B400000;
+}
+
+// byte offset of the staged boxes after the 3 S int32 accumulators
+__host__ __device__ __forceinline__ size_t adj_stage_offset(int S) {
+    return ((size_t)S * 12 + 15) & ~(size_t)15;
 }
 
 // lE = 2 h^3 w_d E_d  (terminal seed)
@@ -112,8 +114,14 @@ __global__ void k_adj_seed(int64_t ng, const float4 *__restrict__ E4, float4 *__
 //
 // The gather term is the offset gradient (interp_grad) of the CIC
 // interpolation of s_abc = le . E at the 8 corners.
-template <bool PG>
-__global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, const Ctrl *__restrict__ ctrl,
+//
+// staged: each change of tile copies E (x pairs) and lrho (x pairs) on the tile's
+// box to shared memory, where both gathers read them while the stencil lies in
+// the box; through the L1 they cost one wavefront per particle and row, eight of
+// the eleven a particle needs.  B > 0: every tile box is B slots long on each axis.
+// 4.2M particles on 64^3 cells: 160 us, staged 142.
+template <bool PG, int B>
+__global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bool staged, const Ctrl *__restrict__ ctrl,
                                                       const int4 *__restrict__ items,
                                                       const int32_t *__restrict__ ycell,
                                                       const float *__restrict__ yo0,
@@ -154,8 +162,10 @@ __global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, co
     const int n_items = ctrl->n_items;
     const int G = g.guard;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
-    const int S0 = g.tile[0] + 2 * G + 1, S1 = g.tile[1] + 2 * G + 1, S2 = g.tile[2] + 2 * G + 1;
-    const int S01 = S0 * S1, S = S01 * S2;
+    const int S0 = B > 0 ? B : g.tile[0] + 2 * G + 1, S01 = B > 0 ? B * B : S0 * (g.tile[1] + 2 * G + 1);
+    const int S = B > 0 ? B * B * B : S01 * (g.tile[2] + 2 * G + 1);
+    float4 *sA = reinterpret_cast<float4 *>(reinterpret_cast<char *>(acc) + adj_stage_offset(S));
+    float2 *sB = reinterpret_cast<float2 *>(sA + S), *sR = sB + S;
     int bad = 0;
     // PG: sum_p lv_tot_i vm_j (row-major) and sum_p le . Q
     float pa[kPGradTerms];
@@ -194,9 +204,14 @@ __global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, co
             nlv0 = lam.v[0][p]; nlv1 = lam.v[1][p]; nlv2 = lam.v[2][p];
         }
         __syncthreads();
+        const cic::Tile tn = cic::tile_of(g, tile);
+        if (staged) {
+            cic::stage_pairs(sA, sB, E8, tn, g);
+            if (rt.cell) cic::stage_float2(sR, rt.lrho2, tn, g);
+        }
         flush();
-        tb = cic::tile_of(g, tile);
-        const int ox = tb.ox, oy = tb.oy, oz = tb.oz;
+        tb = tn;
+        cic::stage_wait();
         __syncthreads();
         for (int done = begin;;) {
             done += min(end - done, cic::fill_limit() * (int)blockDim.x);
@@ -220,7 +235,18 @@ __global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, co
                     int ri, rj, rk;
                     decode(rt.cell[p], g, ri, rj, rk);
                     float rs[8];
-                    corners_from_pairs(rt.lrho2, ri, rj, rk, nx, ny, nz, rs);
+                    int s;
+                    if (staged && cic::box_base<B>(tb, g, ri, rj, rk, s)) {
+                        const int row[4] = {0, S0, S01, S01 + S0};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float2 v = sR[s + row[q]];
+                            rs[2 * q] = v.x;
+                            rs[2 * q + 1] = v.y;
+                        }
+                    } else {
+                        corners_from_pairs(rt.lrho2, ri, rj, rk, nx, ny, nz, rs);
+                    }
                     float rx, ry, rz;
                     interp_grad(rt.o[0][p], rt.o[1][p], rt.o[2][p], rs, rx, ry, rz);
                     ly0 += rt.sx * rx;
@@ -249,14 +275,29 @@ __global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, co
                     le1 = c_kick * lv1;
                     le2 = c_kick * lv2;
                 }
-                int nd[8];
-                corners(i, j, k, nx, ny, nz, nd);
+                int s0;
+                const bool in = cic::box_base<B>(tb, g, i, j, k, s0);
+                float4 row[4][2];   // E at the x corners of the four (y, z) rows
+                if (staged && in) {
+                    const int off[4] = {0, S0, S01, S01 + S0};
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        const float4 a = sA[s0 + off[r]];
+                        const float2 b = sB[s0 + off[r]];
+                        row[r][0] = make_float4(a.x, a.y, b.x, 0.0f);
+                        row[r][1] = make_float4(a.z, a.w, b.y, 0.0f);
+                    }
+                } else {
+                    int nd[8];
+                    corners(i, j, k, nx, ny, nz, nd);
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) ld_pair(E8 + 2 * (int64_t)nd[2 * r], row[r][0], row[r][1]);
+                }
                 float sc[8];
                 float ex = 0.0f, ey = 0.0f, ez = 0.0f;   // E at y (PG)
 #pragma unroll
                 for (int r = 0; r < 4; ++r) {
-                    float4 e0, e1;
-                    ld_pair(E8 + 2 * nd[2 * r], e0, e1);
+                    const float4 e0 = row[r][0], e1 = row[r][1];
                     sc[2 * r] = le0 * e0.x + le1 * e0.y + le2 * e0.z;
                     sc[2 * r + 1] = le0 * e1.x + le1 * e1.y + le2 * e1.z;
                     if (PG) {
@@ -305,20 +346,18 @@ __global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, co
                 const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
                 const float w[8] = {gx * gy * gz, fx * gy * gz, gx * fy * gz, fx * fy * gz,
                                     gx * gy * fz, fx * gy * fz, gx * fy * fz, fx * fy * fz};
-                const int si = tile_slot(i, ox, nx, g.tile[0], G);
-                const int sj = tile_slot(j, oy, ny, g.tile[1], G);
-                const int sk = tile_slot(k, oz, nz, g.tile[2], G);
-                if (si >= 0 && sj >= 0 && sk >= 0) {
-                    const int s = si + S0 * sj + S01 * sk;
+                if (in) {
                     const int off[8] = {0, 1, S0, S0 + 1, S01, S01 + 1, S01 + S0, S01 + S0 + 1};
-                    const float q0 = qs * le0, q1 = qs * le1, q2 = qs * le2;
+                    const float q0 = qs * le0, q1 = qs * le1, q2 = qs * le2;   // below 2^18
 #pragma unroll
                     for (int cc = 0; cc < 8; ++cc) {
-                        atomicAdd(acc + s + off[cc], __float2int_rn(w[cc] * q0));
-                        atomicAdd(acc + S + s + off[cc], __float2int_rn(w[cc] * q1));
-                        atomicAdd(acc + 2 * S + s + off[cc], __float2int_rn(w[cc] * q2));
+                        atomicAdd(acc + s0 + off[cc], round_product(w[cc], q0));
+                        atomicAdd(acc + S + s0 + off[cc], round_product(w[cc], q1));
+                        atomicAdd(acc + 2 * S + s0 + off[cc], round_product(w[cc], q2));
                     }
                 } else {
+                    int nd[8];
+                    corners(i, j, k, nx, ny, nz, nd);
 #pragma unroll
                     for (int cc = 0; cc < 8; ++cc)
                         atomicAdd(lE4 + nd[cc], make_float4(w[cc] * le0, w[cc] * le1, w[cc] * le2, 0.0f));
@@ -338,7 +377,7 @@ __global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, co
     if (nonfinite) atomicOr(&ctrl_w->flags, PIC_FLAG_NONFINITE);
     if (PG) {
         // block sums in FP64, fixed order: warp shuffles, then the 8 warps
-        __shared__ double red[kPGradTerms][8];
+        __shared__ double red[kPGradTerms][kAdjThreadsPerSM / 64];
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
         for (int q = 0; q < kPGradTerms; ++q) {
@@ -355,22 +394,15 @@ __global__ void __launch_bounds__(256, PIC_ADJ_MIN_BLOCKS) k_adj_push(Geom g, co
     }
 }
 
-// acc[q] += sum over blocks of part[b][q]: strided per-thread sums, then a
-// fixed tree (one block of 256 threads)
-__global__ void k_pgrad_acc(const double *__restrict__ part, int blocks, double *acc) {
-    __shared__ double red[kPGradTerms][256];
-    double s[kPGradTerms];
-    for (int q = 0; q < kPGradTerms; ++q) s[q] = 0.0;
-    for (int b = threadIdx.x; b < blocks; b += blockDim.x)
-        for (int q = 0; q < kPGradTerms; ++q) s[q] += part[(size_t)kPGradTerms * b + q];
-    for (int q = 0; q < kPGradTerms; ++q) red[q][threadIdx.x] = s[q];
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w)
-            for (int q = 0; q < kPGradTerms; ++q) red[q][threadIdx.x] += red[q][threadIdx.x + w];
-        __syncthreads();
-    }
-    if ((int)threadIdx.x < kPGradTerms) acc[threadIdx.x] += red[threadIdx.x][0];
+// acc[q] += sum over blocks of part[b][q]: one warp per term, strided sums per
+// lane, then a fixed tree (a block tree over all terms took 8.2 us)
+__global__ void __launch_bounds__(32 * kPGradTerms) k_pgrad_acc(const double *__restrict__ part,
+                                                                int blocks, double *acc) {
+    const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
+    double s = 0.0;
+    for (int b = lane; b < blocks; b += 32) s += part[(size_t)kPGradTerms * b + q];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) acc[q] += s;
 }
 
 // lrho^ = sum_d (+i g_d / |k|^2) lE^_d / N_g   (S^T, with the C2R 1/N_g folded in)
@@ -575,31 +607,49 @@ cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, 
                             int item_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
                             float4 *lE4, float c_kick, float dt, float wz2, const AdjRhoTerm &rt,
                             const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, cudaStream_t st) {
-    const int S = (g.tile[0] + 2 * g.guard + 1) * (g.tile[1] + 2 * g.guard + 1) *
-                  (g.tile[2] + 2 * g.guard + 1);
-    const size_t smem = sizeof(int) * 3 * (size_t)S;
-    const int blocks = std::max(1, std::min(kAdjPushMaxBlocks, max_items));
-#define PIC_ADJ(PGV)                                                                            \
+    const AdjShape a = adj_shape(g);
+    const int blocks = adj_blocks(g, max_items);
+    const bool cbox = const_box(g);
+#define PIC_ADJ(PGV, BV)                                                                        \
     do {                                                                                        \
-        if (smem > 48 * 1024) {                                                                 \
-            cudaError_t e = cudaFuncSetAttribute(k_adj_push<PGV>,                               \
+        if (a.smem > 48 * 1024) {                                                               \
+            cudaError_t e = cudaFuncSetAttribute(k_adj_push<PGV, BV>,                           \
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                                 (int)smem);                                    \
+                                                 (int)a.smem);                                  \
             if (e != cudaSuccess) return e;                                                     \
         }                                                                                       \
-        k_adj_push<PGV><<<blocks, 256, smem, st>>>(g, ctrl, items, ycell, yo[0], yo[1], yo[2],  \
-                                                   E8, lE4, c_kick, dt, wz2, rt, ab, pg,        \
-                                                   item_cost, ctrl_w);                                     \
+        k_adj_push<PGV, BV><<<blocks, a.threads, a.smem, st>>>(g, a.staged, ctrl, items, ycell, \
+                                                               yo[0], yo[1], yo[2], E8, lE4,    \
+                                                               c_kick, dt, wz2, rt, ab, pg,     \
+                                                               item_cost, ctrl_w);              \
     } while (0)
-    if (pg.part) PIC_ADJ(true);
-    else PIC_ADJ(false);
+    if (pg.part) {
+        if (cbox) PIC_ADJ(true, kConstBox);
+        else PIC_ADJ(true, 0);
+    } else {
+        if (cbox) PIC_ADJ(false, kConstBox);
+        else PIC_ADJ(false, 0);
+    }
 #undef PIC_ADJ
     return cudaGetLastError();
 }
 
-cudaError_t launch_pgrad_acc(const double *part, int max_items, double *acc, cudaStream_t st) {
-    const int blocks = std::max(1, std::min(kAdjPushMaxBlocks, max_items));
-    k_pgrad_acc<<<1, 256, 0, st>>>(part, blocks, acc);
+// Blocks of the reverse push: two of 384 threads per SM with the staged boxes (32
+// bytes a slot after the accumulators' 12) while two fit, else three of 256.
+AdjShape adj_shape(const Geom &g) {
+    const int S = cic::tile_of(g, 0).S;
+    const size_t box = adj_stage_offset(S) + 32 * (size_t)S;
+    if (2 * (box + 2048) <= (size_t)228 * 1024) return AdjShape{kAdjThreadsPerSM / 2, 2, true, box};
+    return AdjShape{kAdjThreadsPerSM / 3, 3, false, adj_stage_offset(S)};
+}
+int adj_blocks(const Geom &g, int max_items) {
+    return std::max(1, std::min(kNumSMs * adj_shape(g).per_sm, max_items));
+}
+
+cudaError_t launch_pgrad_acc(const Geom &g, const double *part, int max_items, double *acc,
+                             cudaStream_t st) {
+    const int blocks = adj_blocks(g, max_items);
+    k_pgrad_acc<<<1, 32 * kPGradTerms, 0, st>>>(part, blocks, acc);
     return cudaGetLastError();
 }
 

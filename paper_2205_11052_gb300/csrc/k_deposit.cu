@@ -158,9 +158,7 @@ cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int
     const size_t smem = tile_deposit_smem(g);   // item tile + the block's tile sums
     const int blocks = grid_blocks < max_items ? grid_blocks : (max_items > 0 ? max_items : 1);
     cudaError_t e;
-    // the default geometry (8^3 tiles, two guard layers) as a constant box
-    bool cbox = true;
-    for (int d = 0; d < 3; ++d) cbox = cbox && g.tile[d] + 2 * g.guard + 1 == 13;
+    const bool cbox = const_box(g);
 #define PIC_DT(F, B)                                                                           \
     do {                                                                                       \
         if (smem > 48 * 1024 &&                                                                \
@@ -172,7 +170,7 @@ cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int
                                                          ctrl_w, sparse_below, item_cost);                \
     } while (0)
     if (fixed) {
-        if (cbox) PIC_DT(true, 13);
+        if (cbox) PIC_DT(true, kConstBox);
         else PIC_DT(true, 0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         return launch_rho_finish(g, rho64, rho, qscale_d, st);

@@ -780,9 +780,6 @@ __global__ void k_step_inc(Ctrl *ctrl) {
     ctrl->since_sort += 1;
 }
 
-// the box edge compiled as a constant into the fixed-point push and move:
-// 8^3 tiles with two guard layers (the default geometry)
-constexpr int kConstBox = 13;
 bool const_box(const Geom &g) {
     for (int d = 0; d < 3; ++d)
         if (g.tile[d] + 2 * g.guard + 1 != kConstBox) return false;

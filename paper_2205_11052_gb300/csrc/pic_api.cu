@@ -1448,7 +1448,7 @@ int pic_adjoint_backward(pic_handle_t c, double scale, double *gx, double *gv, i
             PIC_CUDA(launch_adj_push(c->geom, c->ctrl(), c->at<int4>(c->lay.items),
                                      (int)c->max_items, item_cost_of(c), ycell, yo, En, lE4, c_kick, dt, wz2, rt,
                                      step_bound(ab, n & 1), pg, c->ctrl(), c->st));
-            if (pgrad) PIC_CUDA(launch_pgrad_acc(pg_part, (int)c->max_items, pg_acc, c->st));
+            if (pgrad) PIC_CUDA(launch_pgrad_acc(c->geom, pg_part, (int)c->max_items, pg_acc, c->st));
             if ((r = adj_solve(c, n & 1))) return r;
             rt.cell = ycell;
             for (int d = 0; d < 3; ++d) rt.o[d] = yo[d];

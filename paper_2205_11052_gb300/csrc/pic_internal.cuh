@@ -114,10 +114,6 @@ constexpr int kPushThreadsPerSM = 768;
 #ifndef PIC_ZERO_COPY
 #define PIC_ZERO_COPY 1
 #endif
-// resident blocks per SM the reverse push is compiled for
-#ifndef PIC_ADJ_MIN_BLOCKS
-#define PIC_ADJ_MIN_BLOCKS 3
-#endif
 constexpr int kMaxChunk = 4095;   // fixed-point tile slots stay below 2^32
 
 // Set the thread-local message returned by pic_last_error(); returns `code`.
@@ -283,6 +279,10 @@ struct PushShape {
 };
 PushShape push_shape(const Geom &g);
 size_t tile_deposit_smem(const Geom &g);   // the deposit tiles alone (unstaged kernels)
+// the box edge compiled as a constant into the tiled kernels: 8^3 tiles with two
+// guard layers (the default geometry)
+constexpr int kConstBox = 13;
+bool const_box(const Geom &g);
 cudaError_t push_deposit_prepare(const Geom &g);
 // Optional copy of the positions a push starts from (cell, o[3]), written by
 // the fused kernel as it reads them (the adjoint keeps each step's y).
@@ -394,14 +394,25 @@ struct PGrad {
     float half_n[3], h[3];
 };
 constexpr int kPGradTerms = 10;
-constexpr int kAdjPushMaxBlocks = kNumSMs * PIC_ADJ_MIN_BLOCKS * 2;
+// threads per SM the reverse push is compiled for (80 registers), its blocks for
+// geometry g (see k_adjoint.cu) and the most of them
+constexpr int kAdjThreadsPerSM = 768;
+constexpr int kAdjPushMaxBlocks = kNumSMs * 3;
+struct AdjShape {
+    int threads, per_sm;
+    bool staged;
+    size_t smem;
+};
+AdjShape adj_shape(const Geom &g);
+int adj_blocks(const Geom &g, int max_items);
 cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, int max_items,
                             int item_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
                             float4 *lE4, float c_kick, float dt, float wz2, const AdjRhoTerm &rt,
                             const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, cudaStream_t st);
 // acc[q] += the fixed-order sum of the kPGradTerms partials of the blocks the
 // last launch_adj_push used (max_items caps them as there)
-cudaError_t launch_pgrad_acc(const double *part, int max_items, double *acc, cudaStream_t st);
+cudaError_t launch_pgrad_acc(const Geom &g, const double *part, int max_items, double *acc,
+                             cudaStream_t st);
 cudaError_t launch_green_adj(const Geom &g, const double *L_d, const float2 *lE_hat,
                              float2 *lrho_hat, int64_t nhalf, cudaStream_t st);
 // where k_adj_rho writes the updated multipliers (o[0] == nullptr: in place)

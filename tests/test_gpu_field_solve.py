@@ -23,7 +23,7 @@ from paper_2205_11052_gb300.sim import Simulation  # noqa: E402
 build()
 
 GRIDS = [(2, 1, 1), (3, 2, 1), (4, 1, 5), (16, 16, 16), (24, 36, 28), (45, 49, 20), (33, 17, 31),
-         (62, 29, 26), (64, 64, 64), (96, 7, 100), (19, 23, 121), (127, 16, 8), (112, 112, 16),
+         (62, 29, 26), (26, 33, 39), (64, 64, 64), (96, 7, 100), (19, 23, 121), (127, 16, 8), (112, 112, 16),
          (128, 128, 12), (130, 24, 9), (8, 74, 12)]
 
 
