@@ -97,12 +97,12 @@ __host__ __device__ __forceinline__ size_t adj_stage_offset(int S) {
 }
 
 // lE = 2 h^3 w_d E_d  (terminal seed)
-__global__ void k_adj_seed(int64_t ng, const float4 *__restrict__ E4, float4 *__restrict__ lE4,
+__global__ void k_adj_seed(int64_t ng, const float4 *__restrict__ E8, float4 *__restrict__ lE4,
                            float sx, float sy, float sz) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < ng; q += stride) {
-        const float4 e = E4[q];
-        lE4[q] = make_float4(sx * e.x, sy * e.y, sz * e.z, 0.0f);
+        const float4 e = E8[2 * q];
+        lE4[q] = make_float4(sx * e.x, sy * e.y, sz * E8[2 * q + 1].x, 0.0f);
     }
 }
 
@@ -595,10 +595,10 @@ __global__ void k_dot_final(const double *__restrict__ part, int nb, double *out
 
 }  // namespace
 
-cudaError_t launch_adj_seed(int64_t ng, const float4 *E4, float4 *lE4, const double *scale3,
+cudaError_t launch_adj_seed(int64_t ng, const float4 *E8, float4 *lE4, const double *scale3,
                             cudaStream_t st) {
     const int b = (int)std::min<int64_t>((ng + 255) / 256, 152 * 8);
-    k_adj_seed<<<b, 256, 0, st>>>(ng, E4, lE4, (float)scale3[0], (float)scale3[1],
+    k_adj_seed<<<b, 256, 0, st>>>(ng, E8, lE4, (float)scale3[0], (float)scale3[1],
                                   (float)scale3[2]);
     return cudaGetLastError();
 }

@@ -6,8 +6,8 @@
 //   k_fft_yz          one (y, z) plane of one x frequency and one component per
 //                     block, in shared memory: forward over y and z, the Green
 //                     kernel of k_green, back over z and y
-//   k_fft_x_backward  rows of the three components -> E4, its x-paired copy E8
-//                     and, when asked, the block's partial field sums
+//   k_fft_x_backward  rows of the three components -> the x-paired E8, E4 where the
+//                     caller keeps it and, when asked, the block's partial sums
 // The adjoint's solve runs the mirrored kernels (three components forward, the
 // conjugate symbol, one density backward).
 //
@@ -78,13 +78,16 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_forward(int ny, int nz, int
                 v[0] = e.x;
                 v[1] = e.y;
                 v[2] = e.z;
-                lE4[g] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
 #pragma unroll
         for (int d = 0; d < COMPS; ++d) sf[2 * ((d * PAIRS + (r >> 1)) * pitch + x) + (r & 1)] = v[d];
     }
     __syncthreads();
+    if (COMPS == 3) {   // in a loop of its own, so that the loads above overlap
+        float4 *row = lE4 + ((int64_t)z * ny + y0) * n;
+        for (int w = threadIdx.x; w < rows * n; w += kXThreads) row[w] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     lines<false>(s, COMPS * PAIRS, pitch, 1, ax, tw);
     // lanes over the rows: runs of ROWS values at one frequency
     for (int w = threadIdx.x; w < COMPS * nh * PAIRS; w += kXThreads) {
@@ -166,48 +169,61 @@ __global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, 
     store_plane(o, s, ny, nz, pitch);
 }
 
-// lrho^ = sum_d (+i g_d / |k|^2) lE^_d / N_g of one x frequency: three planes
-// forward, summed in global memory (each element by one thread), one plane back
+// lrho^ = sum_d (+i g_d / |k|^2) lE^_d / N_g of one x frequency, in two kernels: a
+// block per component transforms its plane forward in place and applies +i g_d
+// (blockIdx.y: d), then a block adds the three, applies 1 / (|k|^2 N_g) and
+// transforms back.  One block for all four planes took 43 us at 64^3 (33 blocks),
+// the two kernels 27.
 __global__ void __launch_bounds__(512) k_fft_yz_adj(int nx, int ny, int nz, int nh, FftAxis ay,
                                                     FftAxis az, const FftTables *__restrict__ tab,
-                                                    const float *__restrict__ ktab, float inv_ng,
-                                                    const float2 *__restrict__ in,
-                                                    float2 *__restrict__ out, int64_t nhalf) {
+                                                    const float *__restrict__ ktab,
+                                                    float2 *__restrict__ lE_hat, int64_t nhalf) {
+    extern __shared__ float2 sm[];
+    const int pitch = ny | 1, a = blockIdx.x, d = blockIdx.y;
+    float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
+    float2 *io = lE_hat + d * nhalf + (int64_t)a * ny * nz;
+    load_twiddles(twy, tab, 1, ny);
+    load_twiddles(twz, tab, 2, nz);
+    load_plane(s, io, ny, nz, pitch);
+    __syncthreads();
+    lines<false>(s, nz, pitch, 1, ay, twy);
+    lines<false>(s, ny, 1, pitch, az, twz);
+    const float *gyp = ktab + nh + ny, *gzp = gyp + ny + nz;
+    const float gx = ((nx & 1) == 0 && a == nx / 2) ? 0.0f : ktab[a];
+    const fft::FastDiv by_ny(ny);
+    for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
+        const int pz = by_ny.quot(w), py = w - pz * ny;
+        const float g = d == 0 ? gx : (d == 1 ? gyp[py] : gzp[pz]);
+        const float2 e = s[pz * pitch + py];
+        io[w] = make_float2(-g * e.y, g * e.x);   // +i g e
+    }
+}
+
+__global__ void __launch_bounds__(512) k_fft_yz_adj_back(int ny, int nz, int nh, FftAxis ay, FftAxis az,
+                                                         const FftTables *__restrict__ tab,
+                                                         const float *__restrict__ ktab, float inv_ng,
+                                                         const float2 *__restrict__ lE_hat,
+                                                         float2 *__restrict__ out, int64_t nhalf) {
     extern __shared__ float2 sm[];
     const int pitch = ny | 1, a = blockIdx.x;
     float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
     load_twiddles(twy, tab, 1, ny);
     load_twiddles(twz, tab, 2, nz);
-    float2 *o = out + (int64_t)a * ny * nz;
-    const float *kyp = ktab + nh, *gyp = kyp + ny, *kzp = gyp + ny, *gzp = kzp + nz;
+    const float2 *in = lE_hat + (int64_t)a * ny * nz;
+    const float *kyp = ktab + nh, *kzp = kyp + 2 * ny;
     const float kx = ktab[a];
-    const float gx = ((nx & 1) == 0 && a == nx / 2) ? 0.0f : kx;
     const fft::FastDiv by_ny(ny);
-    for (int d = 0; d < 3; ++d) {
-        __syncthreads();
-        load_plane(s, in + d * nhalf + (int64_t)a * ny * nz, ny, nz, pitch);
-        __syncthreads();
-        lines<false>(s, nz, pitch, 1, ay, twy);
-        lines<false>(s, ny, 1, pitch, az, twz);
-        for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
-            const int pz = by_ny.quot(w), py = w - pz * ny;
-            const float g = d == 0 ? gx : (d == 1 ? gyp[py] : gzp[pz]);
-            const float2 e = s[pz * pitch + py];
-            float2 v = make_float2(-g * e.y, g * e.x);   // +i g e
-            if (d > 0) v = fft::cadd(v, o[w]);
-            if (d == 2) {
-                const float ky = kyp[py], kz = kzp[pz];
-                const float sc = (a | py | pz) != 0 ? inv_ng / (kx * kx + ky * ky + kz * kz) : 0.0f;
-                s[pz * pitch + py] = make_float2(sc * v.x, sc * v.y);
-            } else {
-                o[w] = v;
-            }
-        }
+    for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
+        const int pz = by_ny.quot(w), py = w - pz * ny;
+        const float ky = kyp[py], kz = kzp[pz];
+        const float2 v = fft::cadd(fft::cadd(in[w], in[w + nhalf]), in[w + 2 * nhalf]);
+        const float sc = (a | py | pz) != 0 ? inv_ng / (kx * kx + ky * ky + kz * kz) : 0.0f;
+        s[pz * pitch + py] = make_float2(sc * v.x, sc * v.y);
     }
     __syncthreads();
     lines<true>(s, ny, 1, pitch, az, twz);
     lines<true>(s, nz, pitch, 1, ay, twy);
-    store_plane(o, s, ny, nz, pitch);
+    store_plane(out + (int64_t)a * ny * nz, s, ny, nz, pitch);
 }
 
 // rows y0.. of plane z of COMPS components, from spectra by x frequency to two
@@ -247,7 +263,7 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
                                                               double *__restrict__ fpart, int fstride) {
     const int64_t grid0 = blockIdx.z * ((int64_t)ax.n * ny * nz);
     in += blockIdx.z * 3 * nhalf;
-    E4 += grid0;
+    if (E4) E4 += grid0;
     E8 += 2 * grid0;
     rho += grid0;
     constexpr int PAIRS = kRowsB / 2;
@@ -264,7 +280,7 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
         const float *f1 = f0 + 2 * PAIRS * pitch, *f2 = f1 + 2 * PAIRS * pitch;
         const float4 e = make_float4(f0[2 * x], f1[2 * x], f2[2 * x], 0.0f);
         const int64_t g = ((int64_t)z * ny + y0 + r) * n + x;
-        E4[g] = e;
+        if (E4) E4[g] = e;
         E8[2 * g] = make_float4(e.x, e.y, f0[2 * x1], f1[2 * x1]);
         E8[2 * g + 1] = make_float4(e.z, f2[2 * x1], 0.0f, 0.0f);
         if (fpart) {
@@ -410,7 +426,10 @@ cudaError_t fft_prepare() {
     const int most = (int)(sizeof(float2) * (96 * 96 + 128 + 2 * kFftMaxN));
     if ((e = cudaFuncSetAttribute(k_fft_yz, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) != cudaSuccess)
         return e;
-    return cudaFuncSetAttribute(k_fft_yz_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if ((e = cudaFuncSetAttribute(k_fft_yz_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, most)) !=
+        cudaSuccess)
+        return e;
+    return cudaFuncSetAttribute(k_fft_yz_adj_back, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 cudaError_t launch_fft_solve(const Geom &g, int m, const FftAxis ax[3], const FftTables *tab,
@@ -439,8 +458,10 @@ cudaError_t launch_fft_adj_solve(const Geom &g, const FftAxis ax[3], const FftTa
     const dim3 rows((ny + kRowsB - 1) / kRowsB, nz);
     k_fft_x_forward<3><<<rows, kXThreads, x_smem(g, 3 * kRowsB / 2), st>>>(ny, nz, g.nh, ax[0], tab, nullptr,
                                                                            lE4, lE_hat, nhalf);
-    k_fft_yz_adj<<<g.nh, yz_threads(g), yz_smem(g), st>>>(nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab, inv_ng,
-                                                          lE_hat, lrho_hat, nhalf);
+    k_fft_yz_adj<<<dim3(g.nh, 3), yz_threads(g), yz_smem(g), st>>>(nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab,
+                                                                  lE_hat, nhalf);
+    k_fft_yz_adj_back<<<g.nh, yz_threads(g), yz_smem(g), st>>>(ny, nz, g.nh, ax[1], ax[2], tab, ktab, inv_ng,
+                                                              lE_hat, lrho_hat, nhalf);
     k_fft_x_backward_adj<<<rows, kXThreads, x_smem(g, kRowsB / 2), st>>>(ny, nz, g.nh, ax[0], tab, lrho_hat,
                                                                          lrho2, ctrl, par);
     return cudaGetLastError();

@@ -100,16 +100,16 @@ __global__ void k_diag_finalize(const double *__restrict__ fpart, int fblocks,
 
 namespace {
 // Planar field rows (component d of row r at planar + d * dist + r * pitch) ->
-// E4, the x-paired E8 read by 256-bit loads (the components at q, then those at
-// its +x neighbour, periodic: Ex Ey Ex' Ey' | Ez Ez' 0 0) and, with SUMS, the block's partial sums of
-// Ex^2, Ey^2, Ez^2 and rho.  Bound by DRAM: 12 bytes read and 48 written per
-// node (16.8M nodes: 246 us).  With the interleaving left to the inverse
+// the x-paired E8 read by 256-bit loads (the components at q, then those at
+// its +x neighbour, periodic: Ex Ey Ex' Ey' | Ez Ez' 0 0) and, with SUMS, the
+// block's partial sums of Ex^2, Ey^2, Ez^2 and rho.  Bound by DRAM: 12 bytes read
+// and 32 written per node (16.8M nodes: 163 us; with E4 written too 246 us).  With the interleaving left to the inverse
 // transform (output stride 4: 407 us against 92 planar), a pairing pass (120)
-// and a pass for the sums (81), a 256^3 solve with sums took 0.85 ms, now 0.54.
+// and a pass for the sums (81), a 256^3 solve with sums took 0.85 ms.
 template <bool SUMS>
 __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pitch, int64_t dist,
                                                 const float *__restrict__ planar,
-                                                float4 *__restrict__ E4, float4 *__restrict__ E8,
+                                                float4 *__restrict__ E8,
                                                 const float *__restrict__ rho,
                                                 double *__restrict__ part) {
     float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
@@ -121,7 +121,6 @@ __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pi
             const int x1 = x + 1 == nx ? 0 : x + 1;
             const int64_t q = r * nx + x;
             const float4 e = make_float4(p0[x], p1[x], p2[x], 0.0f);
-            E4[q] = e;
             E8[2 * q] = make_float4(e.x, e.y, p0[x1], p1[x1]);
             E8[2 * q + 1] = make_float4(e.z, p2[x1], 0.0f, 0.0f);
             if (SUMS) {
@@ -136,13 +135,29 @@ __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pi
 }
 }  // namespace
 
-cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E4,
-                          float4 *E8, const float *rho, double *part, cudaStream_t st) {
+namespace {
+// E8 -> one float4 (Ex, Ey, Ez, 0) per node, the layout of pic_get_field
+__global__ void __launch_bounds__(256) k_unpair_E(int64_t ng, const float4 *__restrict__ E8,
+                                                  float4 *__restrict__ E4) {
+    const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (q >= ng) return;
+    const float4 a = E8[2 * q];
+    E4[q] = make_float4(a.x, a.y, E8[2 * q + 1].x, 0.0f);
+}
+}  // namespace
+
+cudaError_t launch_unpair_E(int64_t ng, const float4 *E8, float4 *E4, cudaStream_t st) {
+    k_unpair_E<<<(unsigned)((ng + 255) / 256), 256, 0, st>>>(ng, E8, E4);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E8,
+                          const float *rho, double *part, cudaStream_t st) {
     const int64_t rows = (int64_t)g.n[1] * g.n[2];
     if (part)
-        k_pack_E<true><<<kDiagFieldBlocks, 256, 0, st>>>(g.n[0], rows, pitch, dist, planar, E4, E8, rho, part);
+        k_pack_E<true><<<kDiagFieldBlocks, 256, 0, st>>>(g.n[0], rows, pitch, dist, planar, E8, rho, part);
     else
-        k_pack_E<false><<<kDiagFieldBlocks, 256, 0, st>>>(g.n[0], rows, pitch, dist, planar, E4, E8, rho, part);
+        k_pack_E<false><<<kDiagFieldBlocks, 256, 0, st>>>(g.n[0], rows, pitch, dist, planar, E8, rho, part);
     return cudaGetLastError();
 }
 

@@ -48,7 +48,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 // Byte offsets of every device buffer inside the caller's arena.
 struct Layout {
-    size_t ctrl, sets, rho, rho64, rho_hat, E_hat, E4, E8, lrho2, bins, scan_tmp, tile_items, tile_range,
+    size_t ctrl, sets, rho, rho64, rho_hat, E_hat, E8, lrho2, bins, scan_tmp, tile_items, tile_range,
         items, fpart, ppart, ring, inv, stage_x, stage_v, adjE4, ktab, node_pos, fft_tab, fft, total;
     size_t set_stride;   // bytes of one per-particle array
 };
@@ -210,7 +210,6 @@ void compute_layout(pic_ctx *c) {
     L.rho64 = take((size_t)c->ng * 8);
     L.rho_hat = take((size_t)c->nhalf * 8);
     L.E_hat = take((size_t)c->nhalf * 8 * 3);
-    L.E4 = take((size_t)c->ng * 16);
     L.E8 = take((size_t)c->ng * 32);
     L.bins = take((size_t)(c->nbins + 1) * 4);
     const int64_t scan_n = std::max(c->nbins, c->ntiles);
@@ -382,7 +381,7 @@ int do_solve(pic_ctx *c, bool sums = false) {
                                   c->at<float>(c->lay.ktab), c->at<float>(c->lay.rho),
                                   c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat), c->nhalf,
                                   c->mode_pos, c->prm.mode_comp, c->mode_conj, c->ctrl()->mode,
-                                  c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8),
+                                  nullptr, c->at<float4>(c->lay.E8),
                                   sums ? c->at<double>(c->lay.fpart) : nullptr, 0, c->st));
         return timer_end(c, PIC_PHASE_SOLVE, 3);
     }
@@ -391,7 +390,7 @@ int do_solve(pic_ctx *c, bool sums = false) {
                           c->nhalf, c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl(), c->st));
     PIC_CUFFT(cufftExecC2R(c->c2r, c->at<cufftComplex>(c->lay.E_hat), c->at<cufftReal>(c->lay.E_hat)));
     PIC_CUDA(launch_pack_E(c->geom, c->at<float>(c->lay.E_hat), 2 * (int64_t)c->geom.nh, 2 * c->nhalf,
-                           c->at<float4>(c->lay.E4), c->at<float4>(c->lay.E8), c->at<float>(c->lay.rho),
+                           c->at<float4>(c->lay.E8), c->at<float>(c->lay.rho),
                            sums ? c->at<double>(c->lay.fpart) : nullptr, c->st));
     return timer_end(c, PIC_PHASE_SOLVE, 2);
 }
@@ -1017,7 +1016,7 @@ int pic_bind_workspace(pic_handle_t c, void *arena, size_t bytes, void *stream) 
     node_positions(c->h, npos.data());
     PIC_CUDA(cudaMemcpyAsync(c->at<double>(c->lay.node_pos), npos.data(), npos.size() * 8,
                              cudaMemcpyHostToDevice, c->st));
-    PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.E4), 0, (size_t)c->ng * 16, c->st));
+    PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.E8), 0, (size_t)c->ng * 32, c->st));
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.rho), 0, (size_t)c->ng * 4, c->st));
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.rho64), 0, (size_t)c->ng * 8, c->st));
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.ring), 0,
@@ -1175,7 +1174,15 @@ int pic_get_field(pic_handle_t c, float *rho, float *E, int dst_is_device) {
     if (r) return r;
     const cudaMemcpyKind k = dst_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (rho) PIC_CUDA(cudaMemcpyAsync(rho, c->at<float>(c->lay.rho), (size_t)c->ng * 4, k, c->st));
-    if (E) PIC_CUDA(cudaMemcpyAsync(E, c->at<float>(c->lay.E4), (size_t)c->ng * 16, k, c->st));
+    if (E) {
+        // the field is kept x-paired; one float4 per node goes straight to an
+        // aligned device destination, to others through the adjoint's field
+        // array (scratch outside a backward sweep)
+        const bool direct = dst_is_device && (uintptr_t)E % 16 == 0;
+        float4 *E4 = direct ? reinterpret_cast<float4 *>(E) : c->at<float4>(c->lay.adjE4);
+        PIC_CUDA(launch_unpair_E(c->ng, c->at<float4>(c->lay.E8), E4, c->st));
+        if (!direct) PIC_CUDA(cudaMemcpyAsync(E, E4, (size_t)c->ng * 16, k, c->st));
+    }
     if (!dst_is_device) PIC_CUDA(cudaStreamSynchronize(c->st));
     return PIC_OK;
 }
@@ -1397,7 +1404,7 @@ int pic_adjoint_backward(pic_handle_t c, double scale, double *gx, double *gv, i
         PIC_CUDA(launch_adj_zero(c->np, c->ctrl(), c->st));
         const double seed[3] = {2.0 * c->dV * c->adj.w[0], 2.0 * c->dV * c->adj.w[1],
                                 2.0 * c->dV * c->adj.w[2]};
-        PIC_CUDA(launch_adj_seed(c->ng, c->at<float4>(c->lay.E4), lE4, seed, c->st));
+        PIC_CUDA(launch_adj_seed(c->ng, c->at<float4>(c->lay.E8), lE4, seed, c->st));
         const int last = c->adj.n_steps - 1;   // the step whose field J measures
         if ((r = adj_solve(c, last & 1))) return r;
         PIC_CUDA(launch_adj_rho(c->np, c->geom, c->ctrl(), cs.cell, cyo, lrho2, qsc, LamOut{},

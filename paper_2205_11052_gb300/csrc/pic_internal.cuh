@@ -300,11 +300,13 @@ cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, b
 cudaError_t launch_gather_push(int64_t n, const Geom &g, const PushConst &pc, bool diag,
                                Ctrl *ctrl, const float4 *E8, double *part, int blocks,
                                int threads, cudaStream_t st);
-// planar E (component d of row r at planar + d * dist + r * pitch) -> E4, the
-// x-paired E8 (Ex Ey Ex' Ey' Ez Ez' 0 0 per node, primed at q + x, periodic),
+// planar E (component d of row r at planar + d * dist + r * pitch) -> the x-paired
+// E8 (Ex Ey Ex' Ey' Ez Ez' 0 0 per node, primed at q + x, periodic),
 // and unless null the partial field sums of kDiagFieldBlocks blocks
-cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E4,
-                          float4 *E8, const float *rho, double *part, cudaStream_t st);
+cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E8,
+                          const float *rho, double *part, cudaStream_t st);
+// E8 -> (Ex, Ey, Ez, 0) per node
+cudaError_t launch_unpair_E(int64_t ng, const float4 *E8, float4 *E4, cudaStream_t st);
 
 // FP32 wavenumbers of every FFT index per axis (x: nh, y: ny, z: nz entries)
 void green_table(const Geom &g, const double *L_d, float *ktab);
@@ -337,7 +339,7 @@ void fft_ktab(const Geom &g, const double *L_d, const FftTables &t, float *out);
 void fft_tables(const FftAxis ax[3], FftTables &t);
 int fft_sum_blocks(const Geom &g);   // blocks that leave partial field sums
 cudaError_t fft_prepare();           // kernel attributes; outside any stream capture
-// rho -> E4 and E8 (and fpart, 4 doubles per block, unless null) of m <= 65535
+// rho -> E8 (and E4 and fpart, 4 doubles per block, unless null) of m <= 65535
 // grids of one size in a row, spectra in a row too; mode_idx are positions in y
 // and z; grid j has the wavenumbers
 // ktab + j fft_ktab_size, leaves its tracked mode in mode[2 j] and [2 j + 1] and its
@@ -353,7 +355,7 @@ cudaError_t launch_fft_adj_solve(const Geom &g, const FftAxis ax[3], const FftTa
                                  int64_t nhalf, float2 *lrho2, Ctrl *ctrl, int par, cudaStream_t st);
 
 // adjoint (k_adjoint.cu)
-cudaError_t launch_adj_seed(int64_t ng, const float4 *E4, float4 *lE4, const double *scale3,
+cudaError_t launch_adj_seed(int64_t ng, const float4 *E8, float4 *lE4, const double *scale3,
                             cudaStream_t st);
 // up to 8 device-to-device copies in one launch (pointers 16-byte aligned)
 struct CopyList {
