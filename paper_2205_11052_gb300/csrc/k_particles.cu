@@ -21,18 +21,6 @@ namespace {
 
 __device__ __forceinline__ void raise_flag(Ctrl *ctrl, int bit) { atomicOr(&ctrl->flags, bit); }
 
-// Velocity moments (sum v, sum |v|^2) are summed per thread in FP32 over a
-// few particles (one work item's share, or one loop iteration) and then
-// added to the thread's FP64 totals, so no FP32 sum runs over more than a
-// few dozen terms.
-__device__ __forceinline__ void fold_moments(float (&a)[4], double (&d)[4]) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        d[q] += (double)a[q];
-        a[q] = 0.f;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // load: FP64 (x_0, v_0) -> x_{1/2} = x_0 + dt/2 v_0 -> (cell, offset, v)
 // ---------------------------------------------------------------------------
@@ -329,7 +317,7 @@ __device__ __forceinline__ void pd_one(const Geom &g, const PushConst &pc, const
                                        uint32_t *acc, const cic::Tile &t, float *rho,
                                        unsigned long long *rho64, float qscale, int32_t &c, float &fx,
                                        float &fy, float &fz, float &vx, float &vy, float &vz, int &bad,
-                                       unsigned long long &strays, float (&a)[4]) {
+                                       unsigned long long &strays, Moments &mo) {
     int i, j, k, step[3];
     decode_base(g, c, i, j, k, bad);
     int si = cic::box_slot(i, t.ox, g.n[0], g.guard);
@@ -342,12 +330,7 @@ __device__ __forceinline__ void pd_one(const Geom &g, const PushConst &pc, const
     else
         gather_E_pairs(g, E8, i, j, k, fx, fy, fz, ex, ey, ez);
     kick_drift<EXT, MAG>(g, pc, ex, ey, ez, i, j, k, c, fx, fy, fz, vx, vy, vz, bad, step);
-    if (DIAG) {
-        a[0] += vx;
-        a[1] += vy;
-        a[2] += vz;
-        a[3] += vx * vx + vy * vy + vz * vz;
-    }
+    if (DIAG) mo.add(vx, vy, vz);
     if (!sparse) {
         si += step[0];
         sj += step[1];
@@ -379,8 +362,7 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
-    float a[4] = {0.f, 0.f, 0.f, 0.f};
-    double dm[4] = {0.0, 0.0, 0.0, 0.0};
+    Moments mo;
     int bad = 0;
     unsigned long long strays = 0;
     // a contiguous run of work items per block, walked tile by tile
@@ -446,7 +428,7 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
                     }
                 }
                 pd_one<DIAG, EXT, MAG, FIXED, B>(g, pc, E8, sAi, sB, sparse, acc, t, rho, rho64, qscale,
-                                              c, fx, fy, fz, vx, vy, vz, bad, strays, a);
+                                              c, fx, fy, fz, vx, vy, vz, bad, strays, mo);
                 __stcs(ps.cell + p, c);
                 __stcs(ps.o[0] + p, fx);
                 __stcs(ps.o[1] + p, fy);
@@ -455,7 +437,7 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
                 __stcs(ps.v[1] + p, vy);
                 __stcs(ps.v[2] + p, vz);
             }
-            if (DIAG) fold_moments(a, dm);
+            if (DIAG) mo.fold();
             if (done == end) break;
             __syncthreads();
             cic::tile_fold<FIXED>(acc, sum, S);
@@ -471,11 +453,10 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
         atomicAdd(&ctrl->stray_step, strays);
     }
     if (DIAG) {
-        const double *d = dm;
         __shared__ double red[4][kPushThreadsPerSM / 64];
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
         for (int q = 0; q < 4; ++q) {
-            double tt = d[q];
+            double tt = mo.total(q);
             for (int o = 16; o > 0; o >>= 1) tt += __shfl_down_sync(0xffffffffu, tt, o);
             if (lane == 0) red[q][wid] = tt;
         }
@@ -629,12 +610,12 @@ __device__ __forceinline__ void move_one(const Geom &g, uint64_t seed, long long
 }
 
 template <bool DIAG>
-__device__ __forceinline__ void block_moments(const double (&d)[4], double *part) {
+__device__ __forceinline__ void block_moments(const Moments &mo, double *part) {
     if (!DIAG) return;
     __shared__ double red[4][8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int q = 0; q < 4; ++q) {
-        double tt = d[q];
+        double tt = mo.total(q);
         for (int o = 16; o > 0; o >>= 1) tt += __shfl_down_sync(0xffffffffu, tt, o);
         if (lane == 0) red[q][wid] = tt;
     }
@@ -658,8 +639,7 @@ __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
     const long long n = ctrl->step;   // advanced after this kernel (k_step_inc)
-    float a[4] = {0.f, 0.f, 0.f, 0.f};
-    double dm[4] = {0.0, 0.0, 0.0, 0.0};
+    Moments mo;
     int bad = 0;
     unsigned long long strays = 0;
     Segments run = run_segments(items, n_items, item_cost);
@@ -714,19 +694,13 @@ __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
                 } else if (!cic::tile_add<FIXED, B>(acc, t, g, i, j, k, fx, fy, fz, rho, rho64, qscale)) {
                     ++strays;
                 }
-                if (DIAG) {
-                    const float vx = ps.v[0][p], vy = ps.v[1][p], vz = ps.v[2][p];
-                    a[0] += vx;
-                    a[1] += vy;
-                    a[2] += vz;
-                    a[3] += vx * vx + vy * vy + vz * vz;
-                }
+                if (DIAG) mo.add(ps.v[0][p], ps.v[1][p], ps.v[2][p]);
                 __stcs(ps.cell + p, c);
                 __stcs(ps.o[0] + p, fx);
                 __stcs(ps.o[1] + p, fy);
                 __stcs(ps.o[2] + p, fz);
             }
-            if (DIAG) fold_moments(a, dm);
+            if (DIAG) mo.fold();
             if (done == end) break;
             __syncthreads();
             cic::tile_fold<FIXED>(acc, sum, S);
@@ -741,7 +715,7 @@ __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
         atomicAdd(&ctrl->stray, strays);
         atomicAdd(&ctrl->stray_step, strays);
     }
-    block_moments<DIAG>(dm, part);
+    block_moments<DIAG>(mo, part);
 }
 
 // the random move alone (split calls: pic_gather_push)
@@ -750,8 +724,7 @@ __global__ void __launch_bounds__(256) k_move(int64_t np, Geom g, uint64_t seed,
                                                double *__restrict__ part) {
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const long long n = ctrl->step;
-    float a[4] = {0.f, 0.f, 0.f, 0.f};
-    double dm[4] = {0.0, 0.0, 0.0, 0.0};
+    Moments mo;
     int bad = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += stride) {
@@ -763,16 +736,12 @@ __global__ void __launch_bounds__(256) k_move(int64_t np, Geom g, uint64_t seed,
         ps.o[1][p] = fy;
         ps.o[2][p] = fz;
         if (DIAG) {
-            const float vx = ps.v[0][p], vy = ps.v[1][p], vz = ps.v[2][p];
-            a[0] += vx;
-            a[1] += vy;
-            a[2] += vz;
-            a[3] += vx * vx + vy * vy + vz * vz;
-            fold_moments(a, dm);
+            mo.add(ps.v[0][p], ps.v[1][p], ps.v[2][p]);
+            mo.fold();
         }
     }
     if (bad) raise_flag(ctrl, bad);
-    block_moments<DIAG>(dm, part);
+    block_moments<DIAG>(mo, part);
 }
 
 __global__ void k_step_inc(Ctrl *ctrl) {
