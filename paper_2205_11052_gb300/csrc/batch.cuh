@@ -30,15 +30,15 @@ struct InstDesc {
 
 cudaError_t launch_b_load(const double *x, const double *v, int64_t m, int64_t base,
                           const InstDesc *desc, const long long *p0, int n_inst, double dt,
-                          Ctrl *ctrl, cudaStream_t st);
+                          Ctrl *ctrl, LStream st);
 // after launch_unload_records over all particles; c0 (one entry per instance,
 // its first particle in the caller's order) or null: see k_b_unload
 cudaError_t launch_b_unload(int64_t o0, int64_t m, const InstDesc *desc, const long long *p0,
                             int n_inst, const long long *c0, double dt, const Ctrl *ctrl, double *x,
-                            double *v, cudaStream_t st);
+                            double *v, LStream st);
 cudaError_t launch_b_sort(int64_t n, const InstDesc *desc, const long long *p0, int n_inst,
                           int ntiles, int chunk, Ctrl *ctrl, int32_t *bins, int32_t *scan_tmp,
-                          int32_t *tile_items, int2 *tile_range, int4 *items, cudaStream_t st);
+                          int32_t *tile_items, int2 *tile_range, int4 *items, LStream st);
 cudaError_t batch_sort_prepare();   // kernel attributes; once per device outside capture
 // shared memory of the batched push + deposit: u32 tile slots + 64-bit per-tile sums
 // dynamic shared memory of the batched push + deposit for tiles of up to
@@ -53,24 +53,24 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
                                   const int4 *items, int blocks, int threads, int max_S,
                                   const float4 *E4, const float4 *E8,
                                   float *rho, unsigned long long *rho64, int sparse_below,
-                                  int item_cost, double *part, cudaStream_t st);
+                                  int item_cost, double *part, LStream st);
 cudaError_t launch_b_rho_finish(int64_t ng, const InstDesc *desc, const long long *g0, int n_inst,
-                                unsigned long long *rho64, float *rho, cudaStream_t st);
+                                unsigned long long *rho64, float *rho, LStream st);
 cudaError_t launch_b_green(const InstDesc *desc, int first, int m, int64_t nhalf,
-                           const float2 *rho_hat, float2 *E_hat, double *modes, cudaStream_t st);
+                           const float2 *rho_hat, float2 *E_hat, double *modes, LStream st);
 // partial field sums of the instances whose solve leaves none (fpart: fstride x 4
 // doubles per instance); max_blocks: the largest sum_blocks of any of them
 int batch_diag_blocks(const Geom &g);
 cudaError_t launch_b_diag(const InstDesc *desc, int n_inst, int max_blocks, int fstride,
-                          const float *rho, const float4 *E4, double *fpart, cudaStream_t st);
+                          const float *rho, const float4 *E4, double *fpart, LStream st);
 cudaError_t launch_b_diag_finalize(const InstDesc *desc, int n_inst, int fstride,
                                    const int32_t *item_off,
                                    const double *fpart, const double *ppart, const double *modes,
                                    Ctrl *ctrl, double dt, pic_diag_t *ring, int ring_cap,
-                                   cudaStream_t st);
+                                   LStream st);
 // planar E of a size class (grids of nx points per row) -> E4 and x-paired E8
 cudaError_t launch_b_pack(int64_t mng, int nx, const float *planar, float4 *E4, float4 *E8,
-                          cudaStream_t st);
-cudaError_t launch_b_step_done(Ctrl *ctrl, bool diag, cudaStream_t st);
+                          LStream st);
+cudaError_t launch_b_step_done(Ctrl *ctrl, bool diag, LStream st);
 
 }  // namespace pic

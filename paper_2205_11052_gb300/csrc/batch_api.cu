@@ -72,7 +72,7 @@ struct pic_batch {
         o_Eh, o_Epl, o_bins, o_scan, o_titems, o_trange, o_items, o_fpart, o_ppart, o_modes, o_ring, o_c0,
         o_sx, o_sv, o_fft, total;
     char *arena;
-    cudaStream_t st;
+    LStream st;
     bool bound, loaded, plans, rho_current;
     int64_t step;
     int since_sort;
@@ -239,7 +239,8 @@ int b_solve(pic_batch *b, bool sums) {
                 const int m = std::min(c.m - j, 65535);
                 const int64_t g0 = c.g0 + j * c.ng, h0 = c.h0 + j * c.nhalf;
                 B_CUDA(launch_fft_solve(D.g, m, c.ax, b->at<FftTables>(c.o_tab),
-                                        b->at<float>(c.o_ktab) + j * kt, rho + g0, rhoh + h0, Eh + 3 * h0,
+                                        b->at<float>(c.o_ktab) + j * kt, rho + g0, false, rhoh + h0,
+                                        Eh + 3 * h0,
                                         c.nhalf, c.mode_pos, D.mode_comp, D.mode_conj,
                                         b->at<double>(b->o_modes) + 2 * (c.first + j),
                                         reinterpret_cast<float4 *>(E) + g0, b->at<float4>(b->o_E8) + 2 * g0,
@@ -537,6 +538,7 @@ int pic_batch_bind_workspace(pic_batch_t b, void *arena, size_t bytes, void *str
     B_CUDA(cudaMemsetAsync(b->at<char>(b->o_E8), 0, (size_t)b->ng * 32, b->st));
     B_CUDA(cudaMemsetAsync(b->at<char>(b->o_rho), 0, (size_t)b->ng * 4, b->st));
     B_CUDA(cudaMemsetAsync(b->at<char>(b->o_rho64), 0, (size_t)b->ng * 8, b->st));
+    B_CUDA(cudaMemsetAsync(b->at<char>(b->o_bins), 0, (size_t)(b->ntiles + 1) * 4, b->st));
     B_CUDA(cudaMemsetAsync(b->at<char>(b->o_modes), 0, (size_t)b->n_inst * 16, b->st));
     B_CUDA(cudaStreamSynchronize(b->st));
     b->bound = true;
@@ -586,6 +588,7 @@ int pic_batch_step(pic_batch_t b, int n) {
     int r = b_loaded(b);
     if (r) return r;
     if (n < 0) return record_error(PIC_ERR_ARG, "negative step count");
+    const DepScope dep(b->st, b->np <= kDepMaxParticles);
     for (int s = 0; s < n; ++s) {
         if (b->prm.sort_period > 0 && b->since_sort >= b->prm.sort_period && (r = b_sort(b))) return r;
         if (!b->rho_current && (r = b_deposit_pass(b, false, false))) return r;

@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bo
                                                       float dt, float wz2, AdjRhoTerm rt,
                                                       AdjBound ab, PGrad pg, int item_cost,
                                                       Ctrl *ctrl_w) {
+    dep_begin();
     // 3 * S integer accumulators (x, y, z components) in units of 1 / qs
     extern __shared__ int acc[];
     const int cur = ctrl->cur;
@@ -398,6 +399,7 @@ __global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bo
 // lane, then a fixed tree (a block tree over all terms took 8.2 us)
 __global__ void __launch_bounds__(32 * kPGradTerms) k_pgrad_acc(const double *__restrict__ part,
                                                                 int blocks, double *acc) {
+    dep_begin();
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
     double s = 0.0;
     for (int b = lane; b < blocks; b += 32) s += part[(size_t)kPGradTerms * b + q];
@@ -441,6 +443,7 @@ __global__ void k_adj_rho(int64_t n, Geom g, Ctrl *ctrl, const int32_t *__restri
                           const float *__restrict__ yo0, const float *__restrict__ yo1,
                           const float *__restrict__ yo2, const float2 *__restrict__ lrho2,
                           float qscale, LamOut out, int par) {
+    dep_begin();
     const ParticleSet lam = ctrl->sets[1 - ctrl->cur];
     float mly = 0.0f;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
@@ -537,6 +540,7 @@ __global__ void __launch_bounds__(256) k_adj_unload(int64_t o0, int64_t m,
 // pid_prev[i]) takes the multipliers from slot pos[pid_prev[i]].
 __global__ void k_adj_reorder(int64_t n, const int32_t *__restrict__ pos,
                               const int32_t *__restrict__ pid_prev, ReorderArgs a) {
+    dep_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int32_t j = pos[pid_prev[i]];
@@ -596,7 +600,7 @@ __global__ void k_dot_final(const double *__restrict__ part, int nb, double *out
 }  // namespace
 
 cudaError_t launch_adj_seed(int64_t ng, const float4 *E8, float4 *lE4, const double *scale3,
-                            cudaStream_t st) {
+                            LStream st) {
     const int b = (int)std::min<int64_t>((ng + 255) / 256, 152 * 8);
     k_adj_seed<<<b, 256, 0, st>>>(ng, E8, lE4, (float)scale3[0], (float)scale3[1],
                                   (float)scale3[2]);
@@ -606,7 +610,7 @@ cudaError_t launch_adj_seed(int64_t ng, const float4 *E8, float4 *lE4, const dou
 cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, int max_items,
                             int item_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
                             float4 *lE4, float c_kick, float dt, float wz2, const AdjRhoTerm &rt,
-                            const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, cudaStream_t st) {
+                            const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, LStream st) {
     const AdjShape a = adj_shape(g);
     const int blocks = adj_blocks(g, max_items);
     const bool cbox = const_box(g);
@@ -618,7 +622,7 @@ cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, 
                                                  (int)a.smem);                                  \
             if (e != cudaSuccess) return e;                                                     \
         }                                                                                       \
-        k_adj_push<PGV, BV><<<blocks, a.threads, a.smem, st>>>(g, a.staged, ctrl, items, ycell, \
+        launch_dep(k_adj_push<PGV, BV>, blocks, a.threads, a.smem, st, g, a.staged, ctrl, items, ycell, \
                                                                yo[0], yo[1], yo[2], E8, lE4,    \
                                                                c_kick, dt, wz2, rt, ab, pg,     \
                                                                item_cost, ctrl_w);              \
@@ -647,14 +651,14 @@ int adj_blocks(const Geom &g, int max_items) {
 }
 
 cudaError_t launch_pgrad_acc(const Geom &g, const double *part, int max_items, double *acc,
-                             cudaStream_t st) {
+                             LStream st) {
     const int blocks = adj_blocks(g, max_items);
-    k_pgrad_acc<<<1, 32 * kPGradTerms, 0, st>>>(part, blocks, acc);
+    launch_dep(k_pgrad_acc, 1, 32 * kPGradTerms, 0, st, part, blocks, acc);
     return cudaGetLastError();
 }
 
 cudaError_t launch_green_adj(const Geom &g, const double *L_d, const float2 *lE_hat,
-                             float2 *lrho_hat, int64_t nhalf, cudaStream_t st) {
+                             float2 *lrho_hat, int64_t nhalf, LStream st) {
     const double two_pi = 6.283185307179586476925286766559;
     const double ng = (double)g.n[0] * g.n[1] * g.n[2];
     k_green_adj<<<(unsigned)((nhalf + 255) / 256), 256, 0, st>>>(
@@ -691,7 +695,7 @@ __global__ void k_adj_pair_rho(int nx, int64_t ng, const float *__restrict__ lrh
 }
 
 cudaError_t launch_adj_pair_rho(const Geom &g, const float *lrho, float2 *lrho2, float4 *lE4,
-                                Ctrl *ctrl, int par, cudaStream_t st) {
+                                Ctrl *ctrl, int par, LStream st) {
     const int64_t ng = (int64_t)g.n[0] * g.n[1] * g.n[2];
     k_adj_pair_rho<<<(unsigned)((ng + 255) / 256), 256, 0, st>>>(g.n[0], ng, lrho, lrho2, lE4,
                                                                  ctrl, par);
@@ -700,14 +704,14 @@ cudaError_t launch_adj_pair_rho(const Geom &g, const float *lrho, float2 *lrho2,
 
 cudaError_t launch_adj_rho(int64_t n, const Geom &g, Ctrl *ctrl, const int32_t *ycell,
                            const float *const yo[3], const float2 *lrho2, float qscale,
-                           const LamOut &out, int par, cudaStream_t st) {
+                           const LamOut &out, int par, LStream st) {
     if (n <= 0) return cudaSuccess;
     const int b = (int)std::min<int64_t>((n + 255) / 256, 152 * 8);
-    k_adj_rho<<<b, 256, 0, st>>>(n, g, ctrl, ycell, yo[0], yo[1], yo[2], lrho2, qscale, out, par);
+    launch_dep(k_adj_rho, b, 256, 0, st, n, g, ctrl, ycell, yo[0], yo[1], yo[2], lrho2, qscale, out, par);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_zero(int64_t n, const Ctrl *ctrl, cudaStream_t st) {
+cudaError_t launch_adj_zero(int64_t n, const Ctrl *ctrl, LStream st) {
     if (n <= 0) return cudaSuccess;
     const int b = (int)std::min<int64_t>((n + 255) / 256, 152 * 8);
     k_adj_zero<<<b, 256, 0, st>>>(n, ctrl);
@@ -716,7 +720,7 @@ cudaError_t launch_adj_zero(int64_t n, const Ctrl *ctrl, cudaStream_t st) {
 
 cudaError_t launch_adj_reorder(int64_t n, const int32_t *pos, const int32_t *pid_prev,
                                const float *const in_o[3], const float *const in_v[3],
-                               float *const out_o[3], float *const out_v[3], cudaStream_t st) {
+                               float *const out_o[3], float *const out_v[3], LStream st) {
     if (n <= 0) return cudaSuccess;
     ReorderArgs a;
     for (int d = 0; d < 3; ++d) {
@@ -725,31 +729,31 @@ cudaError_t launch_adj_reorder(int64_t n, const int32_t *pos, const int32_t *pid
         a.out_o[d] = out_o[d];
         a.out_v[d] = out_v[d];
     }
-    k_adj_reorder<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, pos, pid_prev, a);
+    launch_dep(k_adj_reorder, (unsigned)((n + 255) / 256), 256, 0, st, n, pos, pid_prev, a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_adj_unload_records(int64_t n, const Ctrl *ctrl, float4 *rec, cudaStream_t st) {
+cudaError_t launch_adj_unload_records(int64_t n, const Ctrl *ctrl, float4 *rec, LStream st) {
     if (n <= 0) return cudaSuccess;
     k_adj_unload_records<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ctrl, rec);
     return cudaGetLastError();
 }
 
 cudaError_t launch_adj_unload(int64_t o0, int64_t m, const float4 *rec, double half_dt,
-                              double scale, double *gx, double *gv, cudaStream_t st) {
+                              double scale, double *gx, double *gv, LStream st) {
     if (m <= 0) return cudaSuccess;
     k_adj_unload<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(o0, m, rec, half_dt, scale, gx, gv);
     return cudaGetLastError();
 }
 
 cudaError_t launch_objective(const double *fpart, int nb, double dV, const double *w,
-                             double *out, cudaStream_t st) {
+                             double *out, LStream st) {
     k_objective<<<1, 256, 0, st>>>(fpart, nb, dV, w[0], w[1], w[2], out);
     return cudaGetLastError();
 }
 
 cudaError_t launch_dot(int64_t n, const double *a, const double *b, double *part, int max_part,
-                       double *out, cudaStream_t st) {
+                       double *out, LStream st) {
     const int nb = (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, max_part));
     k_dot_partials<<<nb, 256, 0, st>>>(n, a, b, part);
     k_dot_final<<<1, 256, 0, st>>>(part, nb, out);

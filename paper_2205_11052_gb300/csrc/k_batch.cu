@@ -86,6 +86,7 @@ __global__ void __launch_bounds__(256) k_b_unload(int64_t o0, int64_t m,
                                                   const long long *__restrict__ c0, double half_dt,
                                                   const Ctrl *ctrl, double *__restrict__ x,
                                                   double *__restrict__ v) {
+    dep_begin();
     const float4 *rec = reinterpret_cast<const float4 *>(ctrl->sets[1 - ctrl->cur].cell);
     __shared__ double sx[3 * 256], sv[3 * 256];
     __shared__ long long dst[256];
@@ -172,6 +173,7 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
     const int4 *__restrict__ items, const float4 *__restrict__ E4, const float4 *__restrict__ E8,
     float *rho, unsigned long long *rho64, int sparse_below, int item_cost, int max_S,
     double *__restrict__ part) {
+    dep_begin();
     extern __shared__ __align__(16) uint32_t acc[];
     __shared__ double red[4][8];
     void *sum = reinterpret_cast<char *>(acc) + cic::sum_offset(max_S);
@@ -316,6 +318,7 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
 __global__ void k_b_rho_finish(int64_t ng, const InstDesc *__restrict__ desc,
                                const long long *__restrict__ g0, int n_inst,
                                unsigned long long *__restrict__ rho64, float *__restrict__ rho) {
+    dep_begin();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int inst = 0;
     for (int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gidx < ng; gidx += stride) {
@@ -406,6 +409,7 @@ __global__ void __launch_bounds__(256) k_b_diag_finalize(const InstDesc *__restr
                                                          const double *__restrict__ modes,
                                                          Ctrl *ctrl, double dt, pic_diag_t *ring,
                                                          int ring_cap) {
+    dep_begin();
     const int i = blockIdx.x;
     const InstDesc &D = desc[i];
     __shared__ double red[8][256];
@@ -460,6 +464,7 @@ __global__ void k_b_pack(int64_t mng, int nx, const float *__restrict__ planar,
 }
 
 __global__ void k_b_step_done(Ctrl *ctrl, int diag) {
+    dep_begin();
     ctrl->step += 1;
     if (diag) ctrl->diag_written += 1;
 }
@@ -468,7 +473,7 @@ __global__ void k_b_step_done(Ctrl *ctrl, int diag) {
 
 cudaError_t launch_b_load(const double *x, const double *v, int64_t m, int64_t base,
                           const InstDesc *desc, const long long *p0, int n_inst, double dt,
-                          Ctrl *ctrl, cudaStream_t st) {
+                          Ctrl *ctrl, LStream st) {
     if (m <= 0) return cudaSuccess;
     k_b_load<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(x, v, m, base, desc, p0, n_inst, dt, ctrl);
     return cudaGetLastError();
@@ -476,16 +481,16 @@ cudaError_t launch_b_load(const double *x, const double *v, int64_t m, int64_t b
 
 cudaError_t launch_b_unload(int64_t o0, int64_t m, const InstDesc *desc, const long long *p0,
                             int n_inst, const long long *c0, double dt, const Ctrl *ctrl, double *x,
-                            double *v, cudaStream_t st) {
+                            double *v, LStream st) {
     if (m <= 0) return cudaSuccess;
-    k_b_unload<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(o0, m, desc, p0, n_inst, c0,
+    launch_dep(k_b_unload, (unsigned)((m + 255) / 256), 256, 0, st, o0, m, desc, p0, n_inst, c0,
                                                             0.5 * dt, ctrl, x, v);
     return cudaGetLastError();
 }
 
 cudaError_t launch_b_sort(int64_t n, const InstDesc *desc, const long long *p0, int n_inst,
                           int ntiles, int chunk, Ctrl *ctrl, int32_t *bins, int32_t *scan_tmp,
-                          int32_t *tile_items, int2 *tile_range, int4 *items, cudaStream_t st) {
+                          int32_t *tile_items, int2 *tile_range, int4 *items, LStream st) {
     const PassEnd pe{n > 0 && ntiles <= kFusedBins, true, chunk, tile_items, tile_range, items};
     cudaError_t e = staged_pass(n, BatchKey{desc, p0, n_inst}, ntiles, ctrl, bins, scan_tmp, pe, st);
     if (e != cudaSuccess || pe.fused) return e;
@@ -515,7 +520,7 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
                                   const int4 *items, int blocks, int threads, int max_S,
                                   const float4 *E4, const float4 *E8,
                                   float *rho, unsigned long long *rho64, int sparse_below,
-                                  int item_cost, double *part, cudaStream_t st) {
+                                  int item_cost, double *part, LStream st) {
     const size_t smem = batch_push_smem(max_S, E4 != nullptr && push);
     cudaError_t e = cudaSuccess;
 #define PIC_BPD(P, D, X, M, F)                                                                  \
@@ -525,7 +530,7 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
             (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
                                       (int)smem)) != cudaSuccess)                               \
             return e;                                                                           \
-        kern<<<blocks, threads, smem, st>>>(desc, tile_inst, ctrl, items, push ? E4 : nullptr, \
+        launch_dep(kern, blocks, threads, smem, st, desc, tile_inst, ctrl, items, push ? E4 : nullptr, \
                                             E8, rho, rho64, sparse_below, item_cost, max_S,     \
                                             part);                                              \
     } while (0)
@@ -546,14 +551,14 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
 }
 
 cudaError_t launch_b_rho_finish(int64_t ng, const InstDesc *desc, const long long *g0, int n_inst,
-                                unsigned long long *rho64, float *rho, cudaStream_t st) {
+                                unsigned long long *rho64, float *rho, LStream st) {
     const int b = (int)std::max<int64_t>(1, std::min<int64_t>((ng + 255) / 256, 152 * 8));
-    k_b_rho_finish<<<b, 256, 0, st>>>(ng, desc, g0, n_inst, rho64, rho);
+    launch_dep(k_b_rho_finish, b, 256, 0, st, ng, desc, g0, n_inst, rho64, rho);
     return cudaGetLastError();
 }
 
 cudaError_t launch_b_green(const InstDesc *desc, int first, int m, int64_t nhalf,
-                           const float2 *rho_hat, float2 *E_hat, double *modes, cudaStream_t st) {
+                           const float2 *rho_hat, float2 *E_hat, double *modes, LStream st) {
     const int64_t tot = (int64_t)m * nhalf;
     if (tot <= 0) return cudaSuccess;
     k_b_green<<<(unsigned)((tot + 255) / 256), 256, 0, st>>>(desc, first, m, nhalf, rho_hat, E_hat,
@@ -562,7 +567,7 @@ cudaError_t launch_b_green(const InstDesc *desc, int first, int m, int64_t nhalf
 }
 
 cudaError_t launch_b_diag(const InstDesc *desc, int n_inst, int max_blocks, int fstride,
-                          const float *rho, const float4 *E4, double *fpart, cudaStream_t st) {
+                          const float *rho, const float4 *E4, double *fpart, LStream st) {
     if (max_blocks <= 0) return cudaSuccess;
     k_b_diag_field<<<dim3((unsigned)n_inst, (unsigned)max_blocks), 256, 0, st>>>(desc, rho, E4, fpart,
                                                                                 fstride);
@@ -572,21 +577,21 @@ cudaError_t launch_b_diag(const InstDesc *desc, int n_inst, int max_blocks, int 
 cudaError_t launch_b_diag_finalize(const InstDesc *desc, int n_inst, int fstride,
                                    const int32_t *item_off, const double *fpart, const double *ppart,
                                    const double *modes, Ctrl *ctrl, double dt, pic_diag_t *ring,
-                                   int ring_cap, cudaStream_t st) {
-    k_b_diag_finalize<<<n_inst, 256, 0, st>>>(desc, n_inst, fstride, item_off, fpart, ppart, modes, ctrl,
+                                   int ring_cap, LStream st) {
+    launch_dep(k_b_diag_finalize, n_inst, 256, 0, st, desc, n_inst, fstride, item_off, fpart, ppart, modes, ctrl,
                                               dt, ring, ring_cap);
     return cudaGetLastError();
 }
 
 cudaError_t launch_b_pack(int64_t mng, int nx, const float *planar, float4 *E4, float4 *E8,
-                          cudaStream_t st) {
+                          LStream st) {
     const int b = (int)std::max<int64_t>(1, std::min<int64_t>((mng + 255) / 256, 152 * 8));
     k_b_pack<<<b, 256, 0, st>>>(mng, nx, planar, E4, E8);
     return cudaGetLastError();
 }
 
-cudaError_t launch_b_step_done(Ctrl *ctrl, bool diag, cudaStream_t st) {
-    k_b_step_done<<<1, 1, 0, st>>>(ctrl, diag ? 1 : 0);
+cudaError_t launch_b_step_done(Ctrl *ctrl, bool diag, LStream st) {
+    launch_dep(k_b_step_done, 1, 1, 0, st, ctrl, diag ? 1 : 0);
     return cudaGetLastError();
 }
 

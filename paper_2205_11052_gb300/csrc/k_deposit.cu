@@ -43,6 +43,7 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
                                                            float qscale, float *rho,
                                                            unsigned long long *rho64, Ctrl *ctrl_w,
                                                            int sparse_below, int item_cost) {
+    dep_begin();
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
@@ -122,6 +123,7 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
 // words, 8-byte stores of the densities), the odd last node by thread 0
 __global__ void __launch_bounds__(256) k_rho_finish(int64_t ng, unsigned long long *__restrict__ rho64,
                                                     float *__restrict__ rho, float sh, float sl) {
+    dep_begin();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t n2 = ng >> 1;
     ulonglong2 *r2 = reinterpret_cast<ulonglong2 *>(rho64);
@@ -140,19 +142,19 @@ __global__ void __launch_bounds__(256) k_rho_finish(int64_t ng, unsigned long lo
 }  // namespace
 
 cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *rho, double qscale,
-                              cudaStream_t st) {
+                              LStream st) {
     const int64_t ng = (int64_t)g.n[0] * g.n[1] * g.n[2];
     const int fb = (int)std::max<int64_t>(1, std::min<int64_t>((ng / 2 + 255) / 256, 152 * 8));
     const double scale = qscale / (double)kFixOne;
     const float sh = (float)scale, sl = (float)(scale - (double)sh);
-    k_rho_finish<<<fb, 256, 0, st>>>(ng, rho64, rho, sh, sl);
+    launch_dep(k_rho_finish, fb, 256, 0, st, ng, rho64, rho, sh, sl);
     return cudaGetLastError();
 }
 
 cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int4 *items,
                            int max_items, double qscale_d, float *rho, unsigned long long *rho64,
                            bool fixed, Ctrl *ctrl_w, int grid_blocks, int sparse_below,
-                           int item_cost, cudaStream_t st) {
+                           int item_cost, LStream st) {
     (void)n;
     const float qscale = (float)qscale_d;
     const size_t smem = tile_deposit_smem(g);   // item tile + the block's tile sums
@@ -166,7 +168,7 @@ cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int
                                       cudaFuncAttributeMaxDynamicSharedMemorySize,             \
                                       (int)smem)) != cudaSuccess)                              \
             return e;                                                                          \
-        k_deposit_tiles<F, B><<<blocks, 256, smem, st>>>(g, ctrl, items, qscale, rho, rho64,   \
+        launch_dep(k_deposit_tiles<F, B>, blocks, 256, smem, st, g, ctrl, items, qscale, rho, rho64,   \
                                                          ctrl_w, sparse_below, item_cost);                \
     } while (0)
     if (fixed) {

@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_forward(int ny, int nz, int
                                                              const float *__restrict__ rho,
                                                              float4 *__restrict__ lE4,
                                                              float2 *__restrict__ out, int64_t nhalf) {
+    dep_begin();
     if (COMPS == 1) {   // blockIdx.z: one of several grids in a row
         rho += blockIdx.z * ((int64_t)ax.n * ny * nz);
         out += blockIdx.z * nhalf;
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, 
                                                 float2 *__restrict__ out, int64_t nhalf, int mi, int mj,
                                                 int mk, int mode_comp, int mode_conj,
                                                 double *__restrict__ mode) {
+    dep_begin();
     in += blockIdx.z * nhalf;
     out += blockIdx.z * 3 * nhalf;
     ktab += blockIdx.z * (nh + 2 * (ny + nz));
@@ -178,6 +180,7 @@ __global__ void __launch_bounds__(512) k_fft_yz_adj(int nx, int ny, int nz, int 
                                                     FftAxis az, const FftTables *__restrict__ tab,
                                                     const float *__restrict__ ktab,
                                                     float2 *__restrict__ lE_hat, int64_t nhalf) {
+    dep_begin();
     extern __shared__ float2 sm[];
     const int pitch = ny | 1, a = blockIdx.x, d = blockIdx.y;
     float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
@@ -204,6 +207,7 @@ __global__ void __launch_bounds__(512) k_fft_yz_adj_back(int ny, int nz, int nh,
                                                          const float *__restrict__ ktab, float inv_ng,
                                                          const float2 *__restrict__ lE_hat,
                                                          float2 *__restrict__ out, int64_t nhalf) {
+    dep_begin();
     extern __shared__ float2 sm[];
     const int pitch = ny | 1, a = blockIdx.x;
     float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
@@ -259,8 +263,9 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
                                                               const float2 *__restrict__ in,
                                                               int64_t nhalf, float4 *__restrict__ E4,
                                                               float4 *__restrict__ E8,
-                                                              const float *__restrict__ rho,
+                                                              float *__restrict__ rho, bool clear_rho,
                                                               double *__restrict__ fpart, int fstride) {
+    dep_begin();
     const int64_t grid0 = blockIdx.z * ((int64_t)ax.n * ny * nz);
     in += blockIdx.z * 3 * nhalf;
     if (E4) E4 += grid0;
@@ -289,6 +294,7 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
             ff_add_sq(hi[2], lo[2], e.z);
             ff_add(hi[3], lo[3], rho[g]);
         }
+        if (clear_rho) rho[g] = 0.0f;
     }
     if (fpart)
         block_field_sums<kXThreads>(hi, lo, fpart + 4 * ((int64_t)blockIdx.z * fstride +
@@ -302,6 +308,7 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward_adj(int ny, int nz
                                                                   const float2 *__restrict__ in,
                                                                   float2 *__restrict__ lrho2, Ctrl *ctrl,
                                                                   int par) {
+    dep_begin();
     constexpr int PAIRS = kRowsB / 2;
     extern __shared__ float2 sm[];
     const int n = ax.n, pitch = n | 1;
@@ -433,36 +440,36 @@ cudaError_t fft_prepare() {
 }
 
 cudaError_t launch_fft_solve(const Geom &g, int m, const FftAxis ax[3], const FftTables *tab,
-                             const float *ktab, const float *rho, float2 *rho_hat, float2 *E_hat,
+                             const float *ktab, float *rho, bool clear_rho, float2 *rho_hat, float2 *E_hat,
                              int64_t nhalf, const int *mode_idx, int mode_comp, int mode_conj,
                              double *mode, float4 *E4, float4 *E8, double *fpart, int fstride,
-                             cudaStream_t st) {
+                             LStream st) {
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const float inv_ng = (float)(1.0 / ((double)nx * ny * nz));
-    k_fft_x_forward<1><<<dim3((ny + kRowsF - 1) / kRowsF, nz, m), kXThreads, x_smem(g, kRowsF / 2), st>>>(
+    launch_dep(k_fft_x_forward<1>, dim3((ny + kRowsF - 1) / kRowsF, nz, m), kXThreads, x_smem(g, kRowsF / 2), st, 
         ny, nz, g.nh, ax[0], tab, rho, nullptr, rho_hat, nhalf);
-    k_fft_yz<<<dim3(g.nh, 3, m), yz_threads(g), yz_smem(g), st>>>(nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab,
+    launch_dep(k_fft_yz, dim3(g.nh, 3, m), yz_threads(g), yz_smem(g), st, nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab,
                                                                  inv_ng, rho_hat, E_hat, nhalf, mode_idx[0],
                                                                  mode_idx[1], mode_idx[2], mode_comp,
                                                                  mode_conj, mode);
-    k_fft_x_backward<<<dim3((ny + kRowsB - 1) / kRowsB, nz, m), kXThreads, x_smem(g, 3 * kRowsB / 2), st>>>(
-        ny, nz, g.nh, ax[0], tab, E_hat, nhalf, E4, E8, rho, fpart, fstride);
+    launch_dep(k_fft_x_backward, dim3((ny + kRowsB - 1) / kRowsB, nz, m), kXThreads, x_smem(g, 3 * kRowsB / 2), st, 
+        ny, nz, g.nh, ax[0], tab, E_hat, nhalf, E4, E8, rho, clear_rho, fpart, fstride);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fft_adj_solve(const Geom &g, const FftAxis ax[3], const FftTables *tab,
                                  const float *ktab, float4 *lE4, float2 *lE_hat, float2 *lrho_hat,
-                                 int64_t nhalf, float2 *lrho2, Ctrl *ctrl, int par, cudaStream_t st) {
+                                 int64_t nhalf, float2 *lrho2, Ctrl *ctrl, int par, LStream st) {
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
     const float inv_ng = (float)(1.0 / ((double)nx * ny * nz));
     const dim3 rows((ny + kRowsB - 1) / kRowsB, nz);
-    k_fft_x_forward<3><<<rows, kXThreads, x_smem(g, 3 * kRowsB / 2), st>>>(ny, nz, g.nh, ax[0], tab, nullptr,
+    launch_dep(k_fft_x_forward<3>, rows, kXThreads, x_smem(g, 3 * kRowsB / 2), st, ny, nz, g.nh, ax[0], tab, nullptr,
                                                                            lE4, lE_hat, nhalf);
-    k_fft_yz_adj<<<dim3(g.nh, 3), yz_threads(g), yz_smem(g), st>>>(nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab,
+    launch_dep(k_fft_yz_adj, dim3(g.nh, 3), yz_threads(g), yz_smem(g), st, nx, ny, nz, g.nh, ax[1], ax[2], tab, ktab,
                                                                   lE_hat, nhalf);
-    k_fft_yz_adj_back<<<g.nh, yz_threads(g), yz_smem(g), st>>>(ny, nz, g.nh, ax[1], ax[2], tab, ktab, inv_ng,
+    launch_dep(k_fft_yz_adj_back, g.nh, yz_threads(g), yz_smem(g), st, ny, nz, g.nh, ax[1], ax[2], tab, ktab, inv_ng,
                                                               lE_hat, lrho_hat, nhalf);
-    k_fft_x_backward_adj<<<rows, kXThreads, x_smem(g, kRowsB / 2), st>>>(ny, nz, g.nh, ax[0], tab, lrho_hat,
+    launch_dep(k_fft_x_backward_adj, rows, kXThreads, x_smem(g, kRowsB / 2), st, ny, nz, g.nh, ax[0], tab, lrho_hat,
                                                                          lrho2, ctrl, par);
     return cudaGetLastError();
 }

@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(128) k_green(int nx, int ny, int nz, int nh,
                                                float2 *__restrict__ E_hat, int64_t nhalf, int mi,
                                                int mj, int mk, int mode_comp, int mode_conj,
                                                Ctrl *ctrl) {
+    dep_begin();
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= nh) return;
     const int b = blockIdx.y, c = blockIdx.z;
@@ -63,6 +64,7 @@ __global__ void k_diag_finalize(const double *__restrict__ fpart, int fblocks,
                                 const double *__restrict__ ppart, int pblocks, double dV,
                                 double mp, double dt, Ctrl *ctrl, pic_diag_t *ring,
                                 int ring_cap) {
+    dep_begin();
     // one warp per quantity: strided sums per lane, then a fixed tree (a block
     // tree over 256 x 8 FP64 values took 9.6 us, mostly its 64 barriers' adds)
     __shared__ double red[8];
@@ -110,8 +112,9 @@ template <bool SUMS>
 __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pitch, int64_t dist,
                                                 const float *__restrict__ planar,
                                                 float4 *__restrict__ E8,
-                                                const float *__restrict__ rho,
+                                                float *__restrict__ rho, bool clear_rho,
                                                 double *__restrict__ part) {
+    dep_begin();
     float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
     // one warp per row
     const int lane = threadIdx.x & 31;
@@ -129,6 +132,7 @@ __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pi
                 ff_add_sq(hi[2], lo[2], e.z);
                 ff_add(hi[3], lo[3], rho[q]);
             }
+            if (clear_rho) rho[q] = 0.0f;
         }
     }
     if (SUMS) block_field_sums<256>(hi, lo, part + 4 * (int64_t)blockIdx.x);
@@ -139,6 +143,7 @@ namespace {
 // E8 -> one float4 (Ex, Ey, Ez, 0) per node, the layout of pic_get_field
 __global__ void __launch_bounds__(256) k_unpair_E(int64_t ng, const float4 *__restrict__ E8,
                                                   float4 *__restrict__ E4) {
+    dep_begin();
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= ng) return;
     const float4 a = E8[2 * q];
@@ -146,18 +151,18 @@ __global__ void __launch_bounds__(256) k_unpair_E(int64_t ng, const float4 *__re
 }
 }  // namespace
 
-cudaError_t launch_unpair_E(int64_t ng, const float4 *E8, float4 *E4, cudaStream_t st) {
-    k_unpair_E<<<(unsigned)((ng + 255) / 256), 256, 0, st>>>(ng, E8, E4);
+cudaError_t launch_unpair_E(int64_t ng, const float4 *E8, float4 *E4, LStream st) {
+    launch_dep(k_unpair_E, (unsigned)((ng + 255) / 256), 256, 0, st, ng, E8, E4);
     return cudaGetLastError();
 }
 
 cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E8,
-                          const float *rho, double *part, cudaStream_t st) {
+                          float *rho, bool clear_rho, double *part, LStream st) {
     const int64_t rows = (int64_t)g.n[1] * g.n[2];
     if (part)
-        k_pack_E<true><<<kDiagFieldBlocks, 256, 0, st>>>(g.n[0], rows, pitch, dist, planar, E8, rho, part);
+        launch_dep(k_pack_E<true>, kDiagFieldBlocks, 256, 0, st, g.n[0], rows, pitch, dist, planar, E8, rho, clear_rho, part);
     else
-        k_pack_E<false><<<kDiagFieldBlocks, 256, 0, st>>>(g.n[0], rows, pitch, dist, planar, E8, rho, part);
+        launch_dep(k_pack_E<false>, kDiagFieldBlocks, 256, 0, st, g.n[0], rows, pitch, dist, planar, E8, rho, clear_rho, part);
     return cudaGetLastError();
 }
 
@@ -177,11 +182,11 @@ void green_table(const Geom &g, const double *L_d, float *ktab) {
 
 cudaError_t launch_green(const Geom &g, const float *ktab, const float2 *rho_hat, float2 *E_hat,
                          int64_t nhalf, const int *mode_idx, int mode_comp, int mode_conj,
-                         Ctrl *ctrl, cudaStream_t st) {
+                         Ctrl *ctrl, LStream st) {
     const double ng = (double)g.n[0] * g.n[1] * g.n[2];
     const int T = 128;
     const dim3 grid((unsigned)((g.nh + T - 1) / T), (unsigned)g.n[1], (unsigned)g.n[2]);
-    k_green<<<grid, T, 0, st>>>(g.n[0], g.n[1], g.n[2], g.nh, ktab, (float)(1.0 / ng), rho_hat,
+    launch_dep(k_green, grid, T, 0, st, g.n[0], g.n[1], g.n[2], g.nh, ktab, (float)(1.0 / ng), rho_hat,
                                 E_hat, nhalf, mode_idx[0], mode_idx[1], mode_idx[2], mode_comp,
                                 mode_conj, ctrl);
     return cudaGetLastError();
@@ -189,8 +194,8 @@ cudaError_t launch_green(const Geom &g, const float *ktab, const float2 *rho_hat
 
 cudaError_t launch_diag_finalize(const double *field_part, int field_blocks,
                                  const double *push_part, int push_blocks, double dV, double mp, double dt, Ctrl *ctrl,
-                                 pic_diag_t *ring, int ring_cap, cudaStream_t st) {
-    k_diag_finalize<<<1, 256, 0, st>>>(field_part, field_blocks, push_part, push_blocks, dV,
+                                 pic_diag_t *ring, int ring_cap, LStream st) {
+    launch_dep(k_diag_finalize, 1, 256, 0, st, field_part, field_blocks, push_part, push_blocks, dV,
                                        mp, dt, ctrl, ring, ring_cap);
     return cudaGetLastError();
 }

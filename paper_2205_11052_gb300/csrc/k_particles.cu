@@ -132,6 +132,7 @@ __global__ void k_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv) {
 }
 
 __global__ void __launch_bounds__(256) k_unload_records(int64_t n, const Ctrl *__restrict__ ctrl) {
+    dep_begin();
     const int cur = ctrl->cur;
     const ParticleSet ps = ctrl->sets[cur];
     float4 *rec = reinterpret_cast<float4 *>(ctrl->sets[1 - cur].cell);
@@ -159,6 +160,7 @@ __global__ void __launch_bounds__(kLoadThreads) k_unload(int64_t o0, int64_t m,
                                                         double half_dt, const Ctrl *ctrl,
                                                         double *__restrict__ x,
                                                         double *__restrict__ v) {
+    dep_begin();
     // results are staged in shared memory and written as contiguous runs (the
     // destination may be host memory written over the chip-to-chip link)
     __shared__ double sx[3 * kLoadThreads], sv[3 * kLoadThreads];
@@ -211,6 +213,7 @@ template <bool DIAG, bool EXT, bool MAG>
 __global__ void __launch_bounds__(256, 3) k_gather_push(int64_t n, Geom g, PushConst pc, Ctrl *ctrl,
                                                       const float4 *__restrict__ E8,
                                                       double *__restrict__ part) {
+    dep_begin();
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     float a_vx = 0.f, a_vy = 0.f, a_vz = 0.f, a_v2 = 0.f;
     double d_v[4] = {0.0, 0.0, 0.0, 0.0};
@@ -359,6 +362,7 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
                                                           float qscale, int sparse_below, int item_cost,
                                                           double *__restrict__ part,
                                                           SaveY save) {
+    dep_begin();
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
@@ -477,7 +481,7 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
 }  // namespace
 
 cudaError_t launch_load(const double *x, const double *v, int64_t m, int64_t base, const Geom &g,
-                        const double *inv_h_d, double dt, Ctrl *ctrl, cudaStream_t st,
+                        const double *inv_h_d, double dt, Ctrl *ctrl, LStream st,
                         int max_blocks) {
     if (m <= 0) return cudaSuccess;
     const int T = kLoadThreads;
@@ -492,6 +496,7 @@ cudaError_t launch_load(const double *x, const double *v, int64_t m, int64_t bas
 // byte tail of each array by the first threads).  Copies inside the arena run
 // on the SMs at HBM speed rather than through a copy engine.
 __global__ void __launch_bounds__(256) k_copy(CopyList cl) {
+    dep_begin();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int a = 0; a < cl.count; ++a) {
@@ -504,7 +509,7 @@ __global__ void __launch_bounds__(256) k_copy(CopyList cl) {
     }
 }
 
-cudaError_t launch_copy(const CopyList &cl, cudaStream_t st) {
+cudaError_t launch_copy(const CopyList &cl, LStream st) {
     int64_t total = 0;
     for (int a = 0; a < cl.count; ++a) {
         if ((reinterpret_cast<uintptr_t>(cl.dst[a]) | reinterpret_cast<uintptr_t>(cl.src[a])) & 15)
@@ -513,28 +518,29 @@ cudaError_t launch_copy(const CopyList &cl, cudaStream_t st) {
     }
     if (total == 0 && cl.count == 0) return cudaSuccess;
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 8));
-    k_copy<<<blocks, 256, 0, st>>>(cl);
+    launch_dep(k_copy, blocks, 256, 0, st, cl);
     return cudaGetLastError();
 }
 
 __global__ void k_pid_positions(int64_t n, const int32_t *__restrict__ pid, int32_t *pos) {
+    dep_begin();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p < n) pos[pid[p]] = (int32_t)p;
 }
 
-cudaError_t launch_pid_positions(int64_t n, const int32_t *pid, int32_t *pos, cudaStream_t st) {
+cudaError_t launch_pid_positions(int64_t n, const int32_t *pid, int32_t *pos, LStream st) {
     if (n <= 0) return cudaSuccess;
-    k_pid_positions<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, pid, pos);
+    launch_dep(k_pid_positions, (unsigned)((n + 255) / 256), 256, 0, st, n, pid, pos);
     return cudaGetLastError();
 }
 
-cudaError_t launch_unload_records(int64_t n, const Ctrl *ctrl, cudaStream_t st) {
+cudaError_t launch_unload_records(int64_t n, const Ctrl *ctrl, LStream st) {
     if (n <= 0) return cudaSuccess;
-    k_unload_records<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ctrl);
+    launch_dep(k_unload_records, (unsigned)((n + 255) / 256), 256, 0, st, n, ctrl);
     return cudaGetLastError();
 }
 
-cudaError_t launch_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv, cudaStream_t st) {
+cudaError_t launch_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv, LStream st) {
     if (n <= 0) return cudaSuccess;
     k_invperm<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, ctrl, inv);
     return cudaGetLastError();
@@ -547,11 +553,11 @@ void node_positions(const double *h_d, double *node_pos) {
 
 cudaError_t launch_unload(int64_t o0, int64_t m, const int32_t *inv, const double *node_pos,
                           const double *h_d, const double *L_d, double dt, const Ctrl *ctrl,
-                          double *x, double *v, cudaStream_t st) {
+                          double *x, double *v, LStream st) {
     if (m <= 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((m + kLoadThreads - 1) / kLoadThreads);
 #define PIC_UL(G)                                                                            \
-    k_unload<G><<<blocks, kLoadThreads, 0, st>>>(o0, m, inv, node_pos, h_d[0], h_d[1], h_d[2], \
+    launch_dep(k_unload<G>, blocks, kLoadThreads, 0, st, o0, m, inv, node_pos, h_d[0], h_d[1], h_d[2], \
                                                  L_d[0], L_d[1], L_d[2], 0.5 * dt, ctrl, x, v)
     if (inv) PIC_UL(true);
     else PIC_UL(false);
@@ -561,10 +567,10 @@ cudaError_t launch_unload(int64_t o0, int64_t m, const int32_t *inv, const doubl
 
 cudaError_t launch_gather_push(int64_t n, const Geom &g, const PushConst &pc, bool diag,
                                Ctrl *ctrl, const float4 *E8, double *part, int blocks,
-                               int threads, cudaStream_t st) {
+                               int threads, LStream st) {
     const bool ext = pc.wz2 != 0.0f;
     const bool mag = pc.t[0] != 0.0f || pc.t[1] != 0.0f || pc.t[2] != 0.0f;
-#define PIC_GP(D, X, M) k_gather_push<D, X, M><<<blocks, threads, 0, st>>>(n, g, pc, ctrl, E8, part)
+#define PIC_GP(D, X, M) launch_dep(k_gather_push<D, X, M>, blocks, threads, 0, st, n, g, pc, ctrl, E8, part)
     if (diag) {
         if (ext) { if (mag) PIC_GP(true, true, true); else PIC_GP(true, true, false); }
         else     { if (mag) PIC_GP(true, false, true); else PIC_GP(true, false, false); }
@@ -635,6 +641,7 @@ __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
     Geom g, uint64_t seed, Ctrl *ctrl, const int4 *__restrict__ items, float *rho,
     unsigned long long *rho64, float qscale, int sparse_below, int item_cost,
     double *__restrict__ part) {
+    dep_begin();
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
@@ -745,6 +752,7 @@ __global__ void __launch_bounds__(256) k_move(int64_t np, Geom g, uint64_t seed,
 }
 
 __global__ void k_step_inc(Ctrl *ctrl) {
+    dep_begin();
     ctrl->step += 1;
     ctrl->since_sort += 1;
 }
@@ -758,14 +766,14 @@ bool const_box(const Geom &g) {
 cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, bool fixed, bool deposit,
                         Ctrl *ctrl, const int4 *items, int max_items, float *rho,
                         unsigned long long *rho64, double qscale, int sparse_below, int item_cost,
-                        double *part, int blocks, cudaStream_t st) {
+                        double *part, int blocks, LStream st) {
     const int nb = std::max(1, std::min(blocks, deposit ? max_items : blocks));
     if (deposit) {
         const size_t smem = tile_deposit_smem(g);
         const float qs = (float)qscale;
         const bool cbox = const_box(g);
 #define PIC_MV(D, F, B) \
-    k_move_deposit<D, F, B><<<nb, 256, smem, st>>>(g, seed, ctrl, items, rho, rho64, qs, sparse_below, \
+    launch_dep(k_move_deposit<D, F, B>, nb, 256, smem, st, g, seed, ctrl, items, rho, rho64, qs, sparse_below, \
                                                    item_cost, part)
         if (diag) {
             if (!fixed) PIC_MV(true, false, 0);
@@ -783,7 +791,7 @@ cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, boo
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_step_inc<<<1, 1, 0, st>>>(ctrl);
+    launch_dep(k_step_inc, 1, 1, 0, st, ctrl);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return (deposit && fixed) ? launch_rho_finish(g, rho64, rho, qscale, st) : cudaSuccess;
 }
@@ -844,7 +852,7 @@ cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, b
                                 Ctrl *ctrl, const int4 *items, int max_items,
                                 const float4 *E8, float *rho, unsigned long long *rho64,
                                 double qscale, int sparse_below, int item_cost, double *part,
-                                int blocks, const SaveY &save, cudaStream_t st) {
+                                int blocks, const SaveY &save, LStream st) {
     const bool ext = pc.wz2 != 0.0f;
     const bool mag = pc.t[0] != 0.0f || pc.t[1] != 0.0f || pc.t[2] != 0.0f;
     const PushShape ps = push_shape(g);
@@ -853,7 +861,7 @@ cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, b
     cudaError_t e = cudaSuccess;
     const bool cbox = const_box(g);
 #define PIC_PD(D, X, M, F, B)                                                                   \
-    k_push_deposit<D, X, M, F, B><<<nb, ps.threads, ps.smem, st>>>(g, pc, ctrl, items, ps.staged, E8, \
+    launch_dep(k_push_deposit<D, X, M, F, B>, nb, ps.threads, ps.smem, st, g, pc, ctrl, items, ps.staged, E8, \
                                                                     rho, rho64, qs,             \
                                                                     sparse_below, item_cost, part, save)
 #define PIC_PD_F(D, X, M)                                  \

@@ -109,7 +109,7 @@ __global__ void k_scan_apply(int32_t *data, int64_t n, const int32_t *sums, int 
     if (blockIdx.x == 0 && threadIdx.x == 0) data[n] = sums[nb];
 }
 
-cudaError_t exclusive_scan_impl(int32_t *data, int64_t n, int32_t *tmp, cudaStream_t st,
+cudaError_t exclusive_scan_impl(int32_t *data, int64_t n, int32_t *tmp, LStream st,
                                 const int32_t *gate = nullptr) {
     const int nb = (int)((n + kScanSeg - 1) / kScanSeg);
     if (nb == 0) {
@@ -151,13 +151,14 @@ __global__ void k_flip(Ctrl *ctrl) { ctrl->cur = 1 - ctrl->cur; }
 
 }  // namespace
 
-cudaError_t exclusive_scan(int32_t *data, int64_t n, int32_t *tmp, cudaStream_t st,
+cudaError_t exclusive_scan(int32_t *data, int64_t n, int32_t *tmp, LStream st,
                            const int32_t *gate) {
     return exclusive_scan_impl(data, n, tmp, st, gate);
 }
 
 namespace {
 __global__ void k_rebin_decide(Ctrl *ctrl, long long max_strays, int period) {
+    dep_begin();
     const bool due = (period > 0 && ctrl->since_sort >= period) ||
                      ctrl->stray_step > (unsigned long long)max_strays;
     ctrl->rebin = due ? 1 : 0;
@@ -165,8 +166,8 @@ __global__ void k_rebin_decide(Ctrl *ctrl, long long max_strays, int period) {
 }
 }  // namespace
 
-cudaError_t launch_rebin_decide(Ctrl *ctrl, long long max_strays, int period, cudaStream_t st) {
-    k_rebin_decide<<<1, 1, 0, st>>>(ctrl, max_strays < 0 ? 0 : max_strays, period);
+cudaError_t launch_rebin_decide(Ctrl *ctrl, long long max_strays, int period, LStream st) {
+    launch_dep(k_rebin_decide, 1, 1, 0, st, ctrl, max_strays < 0 ? 0 : max_strays, period);
     return cudaGetLastError();
 }
 
@@ -174,7 +175,7 @@ namespace {
 // per-tile ranges from the bin ends left by a scatter, then the work items
 cudaError_t worklist(const int32_t *bin_end, int ntiles, int chunk, int32_t *tile_items,
                      int2 *tile_range, int4 *items, int32_t *scan_tmp, Ctrl *ctrl, int flip,
-                     cudaStream_t st, const int32_t *gate) {
+                     LStream st, const int32_t *gate) {
     const int T = 256;
     const int tb = (ntiles + T - 1) / T;
     k_tile_ranges<<<tb, T, 0, st>>>(bin_end, ntiles, chunk, tile_items, tile_range, gate);
@@ -188,7 +189,7 @@ cudaError_t worklist(const int32_t *bin_end, int ntiles, int chunk, int32_t *til
 
 cudaError_t launch_worklist(const int32_t *bin_end, int ntiles, int chunk, int32_t *tile_items,
                             int2 *tile_range, int4 *items, int32_t *scan_tmp, Ctrl *ctrl, int flip,
-                            cudaStream_t st) {
+                            LStream st) {
     return worklist(bin_end, ntiles, chunk, tile_items, tile_range, items, scan_tmp, ctrl, flip, st,
                     nullptr);
 }
@@ -234,7 +235,7 @@ int sort_launches(int64_t n, int64_t ntiles, bool presort) {
 
 cudaError_t launch_sort(int64_t n, const Geom &g, int chunk, Ctrl *ctrl, int32_t *bins,
                         int64_t nbins, int32_t *scan_tmp, int32_t *tile_items,
-                        int2 *tile_range, int4 *items, bool presort, cudaStream_t st,
+                        int2 *tile_range, int4 *items, bool presort, LStream st,
                         const int32_t *gate) {
     cudaError_t e;
     const int nt = g.ntile[0] * g.ntile[1] * g.ntile[2];
@@ -267,7 +268,7 @@ cudaError_t launch_sort(int64_t n, const Geom &g, int chunk, Ctrl *ctrl, int32_t
 // being loaded; o must be a multiple of 4 (bulk copies start on 16 bytes).
 cudaError_t launch_sort_range(int64_t n, int64_t o, const Geom &g, Ctrl *ctrl, int32_t *bins,
                               int64_t nbins, int32_t *scan_tmp, int *passes, int *kernels,
-                              cudaStream_t st) {
+                              LStream st) {
     *passes = 0;
     *kernels = 0;
     if (n <= 0) return cudaSuccess;
@@ -304,12 +305,12 @@ __global__ void k_timeout_selftest(Ctrl *ctrl) {
 }
 }  // namespace
 
-cudaError_t launch_timeout_selftest(Ctrl *ctrl, cudaStream_t st) {
+cudaError_t launch_timeout_selftest(Ctrl *ctrl, LStream st) {
     k_timeout_selftest<<<1, 32, 0, st>>>(ctrl);
     return cudaGetLastError();
 }
 
-cudaError_t launch_flip(Ctrl *ctrl, cudaStream_t st) {
+cudaError_t launch_flip(Ctrl *ctrl, LStream st) {
     k_flip<<<1, 1, 0, st>>>(ctrl);
     return cudaGetLastError();
 }

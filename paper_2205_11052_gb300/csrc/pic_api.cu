@@ -83,7 +83,7 @@ struct pic_ctx {
     // bound state
     bool bound;
     char *arena;
-    cudaStream_t st;
+    LStream st;
     cufftHandle r2c, c2r;     // rho -> rho^ ; 3 x E^ -> planar E, in place
     cufftHandle r2c3, c2r1;   // adjoint: lE4 (stride 4) -> 3 x lE^ ; lrho^ -> lrho
     bool plans;
@@ -372,13 +372,18 @@ int field_blocks_of(const pic_ctx *c) {
     return c->own_fft ? fft_sum_blocks(c->geom) : kDiagFieldBlocks;
 }
 
-// sums: also leave the partial field sums of the diagnostics
-int do_solve(pic_ctx *c, bool sums = false) {
+// whether the push of a step adds into a cleared FP32 rho (the fixed-point path
+// overwrites every node)
+bool fp32_rho(const pic_ctx *c) { return !(c->prm.options & PIC_OPT_FIXED_DEPOSIT) || c->np <= 0; }
+
+// sums: also leave the partial field sums of the diagnostics; clear_rho: leave rho
+// cleared for the push of the step
+int do_solve(pic_ctx *c, bool sums = false, bool clear_rho = false) {
     int r = timer_begin(c, PIC_PHASE_SOLVE);
     if (r) return r;
     if (c->own_fft) {
         PIC_CUDA(launch_fft_solve(c->geom, 1, c->ax, c->at<FftTables>(c->lay.fft_tab),
-                                  c->at<float>(c->lay.ktab), c->at<float>(c->lay.rho),
+                                  c->at<float>(c->lay.ktab), c->at<float>(c->lay.rho), clear_rho,
                                   c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat), c->nhalf,
                                   c->mode_pos, c->prm.mode_comp, c->mode_conj, c->ctrl()->mode,
                                   nullptr, c->at<float4>(c->lay.E8),
@@ -390,7 +395,7 @@ int do_solve(pic_ctx *c, bool sums = false) {
                           c->nhalf, c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl(), c->st));
     PIC_CUFFT(cufftExecC2R(c->c2r, c->at<cufftComplex>(c->lay.E_hat), c->at<cufftReal>(c->lay.E_hat)));
     PIC_CUDA(launch_pack_E(c->geom, c->at<float>(c->lay.E_hat), 2 * (int64_t)c->geom.nh, 2 * c->nhalf,
-                           c->at<float4>(c->lay.E8), c->at<float>(c->lay.rho),
+                           c->at<float4>(c->lay.E8), c->at<float>(c->lay.rho), clear_rho,
                            sums ? c->at<double>(c->lay.fpart) : nullptr, c->st));
     return timer_end(c, PIC_PHASE_SOLVE, 2);
 }
@@ -439,11 +444,10 @@ int fused_blocks_of(const pic_ctx *c) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(c->max_items, std::min(kMaxPushBlocks, 152 * per)));
 }
 
-// gather + push + deposit of the new positions in one kernel (pic_step)
+// gather + push + deposit of the new positions in one kernel (pic_step), after a
+// solve that cleared rho if fp32_rho
 int do_push_deposit(pic_ctx *c, bool diag, const SaveY &save = SaveY{}) {
     const bool fixed = (c->prm.options & PIC_OPT_FIXED_DEPOSIT) != 0;
-    if (!fixed || c->np <= 0)
-        PIC_CUDA(cudaMemsetAsync(c->at<float>(c->lay.rho), 0, (size_t)c->ng * 4, c->st));
     int r = timer_begin(c, PIC_PHASE_PUSH);
     if (r) return r;
     if (c->np > 0 && uniform_move(c)) {
@@ -739,7 +743,7 @@ int adj_keep_step(pic_ctx *c, const AdjLayout &L, int seg, int a0, int n, int *c
             return r;
     }
     if (!c->rho_current && (r = do_deposit(c))) return r;
-    if ((r = do_solve(c)) || (r = adj_keep_E(c, L, n - a0))) return r;
+    if ((r = do_solve(c, false, fp32_rho(c))) || (r = adj_keep_E(c, L, n - a0))) return r;
     if (c->np == 0) return do_push_deposit(c, false);
     // y_n is written by the push that reads it
     char *y[7];
@@ -1019,6 +1023,7 @@ int pic_bind_workspace(pic_handle_t c, void *arena, size_t bytes, void *stream) 
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.E8), 0, (size_t)c->ng * 32, c->st));
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.rho), 0, (size_t)c->ng * 4, c->st));
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.rho64), 0, (size_t)c->ng * 8, c->st));
+    PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.bins), 0, (size_t)(c->nbins + 1) * 4, c->st));
     PIC_CUDA(cudaMemsetAsync(c->at<char>(c->lay.ring), 0,
                              (size_t)c->prm.diag_capacity * sizeof(pic_diag_t), c->st));
     PIC_CUDA(cudaStreamSynchronize(c->st));
@@ -1233,6 +1238,7 @@ int pic_step(pic_handle_t c, int n) {
     int r = check_loaded(c);
     if (r) return r;
     if (n < 0) return fail(PIC_ERR_ARG, "negative step count");
+    const DepScope dep(c->st, c->np <= kDepMaxParticles);
     // each step: [re-bin] -> (deposit, only if rho is stale) -> solve ->
     // [field diagnostics, before rho is replaced] -> fused gather + push +
     // deposit of the new positions -> [particle diagnostics]
@@ -1244,7 +1250,7 @@ int pic_step(pic_handle_t c, int n) {
         }
         if (!c->rho_current && (r = do_deposit(c))) return r;
         const bool diag = c->prm.diag_every > 0 && ((c->step + 1) % c->prm.diag_every == 0);
-        if ((r = do_solve(c, diag))) return r;
+        if ((r = do_solve(c, diag, fp32_rho(c)))) return r;
         if ((r = do_push_deposit(c, diag))) return r;
         if (diag && (r = do_diag_finalize(c, c->np > 0 ? fused_blocks_of(c) : 1))) return r;
     }
@@ -1327,6 +1333,7 @@ int pic_adjoint_forward(pic_handle_t c, int n_steps, int K, const double *w, voi
     const AdjLayout L = adj_layout(c, n_steps, K);
     if (bytes < L.total)
         return fail(PIC_ERR_CAPACITY, "adjoint buffer of %zu bytes < required %zu", bytes, L.total);
+    const DepScope dep(c->st, c->np <= kDepMaxParticles);
     PIC_CUDA(cudaStreamSynchronize(c->st));
     int32_t cur = 0;
     PIC_CUDA(cudaMemcpy(&cur, &c->ctrl()->cur, sizeof(cur), cudaMemcpyDeviceToHost));
@@ -1356,7 +1363,7 @@ int pic_adjoint_forward(pic_handle_t c, int n_steps, int K, const double *w, voi
             }
             if (n > a0 && (n - a0) % L.R == 0 && (r = adj_rebin(c, &cur))) return r;
             if (!c->rho_current && (r = do_deposit(c))) return r;
-            if ((r = do_solve(c)) || (r = do_push_deposit(c, false))) return r;
+            if ((r = do_solve(c, false, fp32_rho(c))) || (r = do_push_deposit(c, false))) return r;
         }
     }
     c->adj.cur_end = cur;
@@ -1375,6 +1382,7 @@ int pic_adjoint_backward(pic_handle_t c, double scale, double *gx, double *gv, i
     if (r) return r;
     if (!c->adj.ready) return fail(PIC_ERR_STATE, "no pic_adjoint_forward to reverse");
     if (c->np > 0 && (!gx || !gv)) return fail(PIC_ERR_ARG, "null output array");
+    const DepScope dep(c->st, c->np <= kDepMaxParticles);
     const AdjLayout L = adj_layout(c, c->adj.n_steps, c->adj.K);
     const int K = c->adj.K;
     int cur = c->adj.cur_end;

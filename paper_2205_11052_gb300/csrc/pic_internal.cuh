@@ -11,6 +11,52 @@
 namespace pic {
 
 // ----------------------------------------------------------------------------
+// Dependent launches.  A kernel launched by launch_dep on a stream with dep set may
+// be put on the SMs while the kernel before it in the stream still runs
+// (programmatic dependent launch); its first statement, dep_begin, lets the kernel
+// after it do the same and waits until the one before has finished, its writes
+// visible.  A kernel that begins so may also be launched plainly.
+//
+// Small runs spend a quarter of their time between kernels: 20 steps of 16^3 x 8
+// took 1.41 ms, now 1.08; a gradient in a 24^3 trap 2.74, now 2.26.  Large ones lose:
+// the waiting blocks' shared memory is taken from the L1 that gathers rely on (the
+// split cycle at 16.8M particles went from 4.06 to 6.25 ms, the 130M Penning bunch
+// from 49.8 to 51.4), so only whole steps of at most kDepMaxParticles set it.
+// ----------------------------------------------------------------------------
+struct LStream {
+    cudaStream_t s;
+    bool dep;
+    LStream(cudaStream_t s_ = nullptr, bool dep_ = false) : s(s_), dep(dep_) {}
+    operator cudaStream_t() const { return s; }
+};
+constexpr int64_t kDepMaxParticles = (int64_t)1 << 23;
+// dependent launches on `st` within a scope
+struct DepScope {
+    LStream &st;
+    DepScope(LStream &st_, bool on) : st(st_) { st.dep = on; }
+    ~DepScope() { st.dep = false; }
+};
+__device__ __forceinline__ void dep_begin() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, const LStream &st,
+                              A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st.s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = st.dep ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// ----------------------------------------------------------------------------
 // Particle store: structure of arrays, 32 bytes per particle.
 //   cell  packed stencil-base cell (i | j << 10 | k << 20), i.e. the node
 //         index of the lower corner of the particle's CIC stencil
@@ -214,35 +260,35 @@ __device__ __forceinline__ bool next_segment(Segments &r, int &tile, int &begin,
 // max_blocks > 0 caps the grid (blocks then stride over the particles)
 cudaError_t launch_load(const double *x, const double *v, int64_t m, int64_t base,
                         const Geom &g, const double *inv_h_d, double dt, Ctrl *ctrl,
-                        cudaStream_t st, int max_blocks = 0);
+                        LStream st, int max_blocks = 0);
 // readback in load order: the current set's particles as 32-byte records (by
 // pid) in the other set, or the inverse of the store's order (inv[pid]); then
 // particles [o0, o0 + m) as FP64 triples from the records (inv null) or through
 // inv; node_pos: kMaxN node positions (i + 1/2) h per axis
-cudaError_t launch_unload_records(int64_t n, const Ctrl *ctrl, cudaStream_t st);
-cudaError_t launch_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv, cudaStream_t st);
+cudaError_t launch_unload_records(int64_t n, const Ctrl *ctrl, LStream st);
+cudaError_t launch_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv, LStream st);
 void node_positions(const double *h_d, double *node_pos);
 cudaError_t launch_unload(int64_t o0, int64_t m, const int32_t *inv, const double *node_pos,
                           const double *h_d, const double *L_d, double dt, const Ctrl *ctrl,
-                          double *x, double *v, cudaStream_t st);
+                          double *x, double *v, LStream st);
 
-cudaError_t exclusive_scan(int32_t *data, int64_t n, int32_t *tmp, cudaStream_t st,
+cudaError_t exclusive_scan(int32_t *data, int64_t n, int32_t *tmp, LStream st,
                            const int32_t *gate = nullptr);
 cudaError_t sort_prepare();   // kernel attributes; call once per device outside capture
 cudaError_t launch_worklist(const int32_t *bin_end, int ntiles, int chunk, int32_t *tile_items,
                             int2 *tile_range, int4 *items, int32_t *scan_tmp, Ctrl *ctrl, int flip,
-                            cudaStream_t st);
+                            LStream st);
 // presort: the particles are in arbitrary order (just loaded); coarse passes
 // by tile key >> shift run first so that no slice overflows the staged table
 // gate != nullptr: every kernel of the sort returns at once unless *gate is
 // nonzero on the device (the stray-triggered re-binning of pic_step)
 cudaError_t launch_sort(int64_t n, const Geom &g, int chunk, Ctrl *ctrl, int32_t *bins,
                         int64_t nbins, int32_t *scan_tmp, int32_t *tile_items,
-                        int2 *tile_range, int4 *items, bool presort, cudaStream_t st,
+                        int2 *tile_range, int4 *items, bool presort, LStream st,
                         const int32_t *gate = nullptr);
 // ctrl->rebin = (period > 0 and ctrl->since_sort >= period) or
 // ctrl->stray_step > max_strays; clears ctrl->stray_step
-cudaError_t launch_rebin_decide(Ctrl *ctrl, long long max_strays, int period, cudaStream_t st);
+cudaError_t launch_rebin_decide(Ctrl *ctrl, long long max_strays, int period, LStream st);
 // kernels launch_sort issues
 int sort_launches(int64_t n, int64_t ntiles, bool presort);
 int presort_passes(int64_t ntiles);   // coarse passes of a presort
@@ -250,25 +296,25 @@ int presort_passes(int64_t ntiles);   // coarse passes of a presort
 // (which stays unchanged); the range ends in set cur ^ (*passes & 1)
 cudaError_t launch_sort_range(int64_t n, int64_t o, const Geom &g, Ctrl *ctrl, int32_t *bins,
                               int64_t nbins, int32_t *scan_tmp, int *passes, int *kernels,
-                              cudaStream_t st);
-cudaError_t launch_flip(Ctrl *ctrl, cudaStream_t st);   // ctrl->cur = 1 - ctrl->cur
+                              LStream st);
+cudaError_t launch_flip(Ctrl *ctrl, LStream st);   // ctrl->cur = 1 - ctrl->cur
 // one bounded wait that nothing completes: raises PIC_FLAG_TIMEOUT (pic_selftest_timeout)
-cudaError_t launch_timeout_selftest(Ctrl *ctrl, cudaStream_t st);
+cudaError_t launch_timeout_selftest(Ctrl *ctrl, LStream st);
 
 cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int4 *items,
                            int max_items, double qscale, float *rho, unsigned long long *rho64,
                            bool fixed, Ctrl *ctrl_w, int grid_blocks, int sparse_below,
-                           int item_cost, cudaStream_t st);
+                           int item_cost, LStream st);
 
 cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *rho, double qscale,
-                              cudaStream_t st);
+                              LStream st);
 // the uniform-plasma random move (PIC_OPT_UNIFORM_MOVE) of every particle,
 // with the deposit of the new positions when `deposit` (then over the work
 // items, like launch_push_deposit); advances the device step counter
 cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, bool fixed, bool deposit,
                         Ctrl *ctrl, const int4 *items, int max_items, float *rho,
                         unsigned long long *rho64, double qscale, int sparse_below, int item_cost,
-                        double *part, int blocks, cudaStream_t st);
+                        double *part, int blocks, LStream st);
 // block size, blocks per SM, whether the blocks stage E, and the dynamic shared
 // memory of the fused push + deposit kernel for geometry g; the one-time
 // attribute setting it needs above 48 KiB
@@ -296,26 +342,26 @@ cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, b
                                 Ctrl *ctrl, const int4 *items, int max_items, const float4 *E8,
                                 float *rho, unsigned long long *rho64, double qscale,
                                 int sparse_below, int item_cost, double *part, int blocks,
-                                const SaveY &save, cudaStream_t st);
+                                const SaveY &save, LStream st);
 cudaError_t launch_gather_push(int64_t n, const Geom &g, const PushConst &pc, bool diag,
                                Ctrl *ctrl, const float4 *E8, double *part, int blocks,
-                               int threads, cudaStream_t st);
+                               int threads, LStream st);
 // planar E (component d of row r at planar + d * dist + r * pitch) -> the x-paired
 // E8 (Ex Ey Ex' Ey' Ez Ez' 0 0 per node, primed at q + x, periodic),
 // and unless null the partial field sums of kDiagFieldBlocks blocks
 cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E8,
-                          const float *rho, double *part, cudaStream_t st);
+                          float *rho, bool clear_rho, double *part, LStream st);
 // E8 -> (Ex, Ey, Ez, 0) per node
-cudaError_t launch_unpair_E(int64_t ng, const float4 *E8, float4 *E4, cudaStream_t st);
+cudaError_t launch_unpair_E(int64_t ng, const float4 *E8, float4 *E4, LStream st);
 
 // FP32 wavenumbers of every FFT index per axis (x: nh, y: ny, z: nz entries)
 void green_table(const Geom &g, const double *L_d, float *ktab);
 cudaError_t launch_green(const Geom &g, const float *ktab, const float2 *rho_hat,
                          float2 *E_hat, int64_t nhalf, const int *mode_idx, int mode_comp,
-                         int mode_conj, Ctrl *ctrl, cudaStream_t st);
+                         int mode_conj, Ctrl *ctrl, LStream st);
 cudaError_t launch_diag_finalize(const double *field_part, int field_blocks,
                                  const double *push_part, int push_blocks, double dV, double mp, double dt,
-                                 Ctrl *ctrl, pic_diag_t *ring, int ring_cap, cudaStream_t st);
+                                 Ctrl *ctrl, pic_diag_t *ring, int ring_cap, LStream st);
 
 // Field solve by the library's own line transforms (k_fft.cu), for grids whose
 // axes are at most kFftMaxN long with no prime factor above 7 and whose (y, z)
@@ -339,24 +385,25 @@ void fft_ktab(const Geom &g, const double *L_d, const FftTables &t, float *out);
 void fft_tables(const FftAxis ax[3], FftTables &t);
 int fft_sum_blocks(const Geom &g);   // blocks that leave partial field sums
 cudaError_t fft_prepare();           // kernel attributes; outside any stream capture
-// rho -> E8 (and E4 and fpart, 4 doubles per block, unless null) of m <= 65535
+// rho (cleared on the way for an FP32 deposit with clear_rho) -> E8 (and E4 and
+// fpart, 4 doubles per block, unless null) of m <= 65535
 // grids of one size in a row, spectra in a row too; mode_idx are positions in y
 // and z; grid j has the wavenumbers
 // ktab + j fft_ktab_size, leaves its tracked mode in mode[2 j] and [2 j + 1] and its
 // sums from fpart + 4 j fstride on
 cudaError_t launch_fft_solve(const Geom &g, int m, const FftAxis ax[3], const FftTables *tab,
-                             const float *ktab, const float *rho, float2 *rho_hat, float2 *E_hat,
+                             const float *ktab, float *rho, bool clear_rho, float2 *rho_hat, float2 *E_hat,
                              int64_t nhalf, const int *mode_idx, int mode_comp, int mode_conj,
                              double *mode, float4 *E4, float4 *E8, double *fpart, int fstride,
-                             cudaStream_t st);
+                             LStream st);
 // lE4 (cleared) -> lrho2, with the bound bookkeeping of launch_adj_pair_rho
 cudaError_t launch_fft_adj_solve(const Geom &g, const FftAxis ax[3], const FftTables *tab,
                                  const float *ktab, float4 *lE4, float2 *lE_hat, float2 *lrho_hat,
-                                 int64_t nhalf, float2 *lrho2, Ctrl *ctrl, int par, cudaStream_t st);
+                                 int64_t nhalf, float2 *lrho2, Ctrl *ctrl, int par, LStream st);
 
 // adjoint (k_adjoint.cu)
 cudaError_t launch_adj_seed(int64_t ng, const float4 *E8, float4 *lE4, const double *scale3,
-                            cudaStream_t st);
+                            LStream st);
 // up to 8 device-to-device copies in one launch (pointers 16-byte aligned)
 struct CopyList {
     int count;
@@ -364,7 +411,7 @@ struct CopyList {
     const char *src[8];
     int64_t bytes[8];
 };
-cudaError_t launch_copy(const CopyList &cl, cudaStream_t st);
+cudaError_t launch_copy(const CopyList &cl, LStream st);
 
 // The deposit term of the adjoint of one step, (dD/dy)^T lrho evaluated at
 // that step's positions (cell, o) and scaled by q/h_d, folded into the
@@ -410,13 +457,13 @@ int adj_blocks(const Geom &g, int max_items);
 cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, int max_items,
                             int item_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
                             float4 *lE4, float c_kick, float dt, float wz2, const AdjRhoTerm &rt,
-                            const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, cudaStream_t st);
+                            const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, LStream st);
 // acc[q] += the fixed-order sum of the kPGradTerms partials of the blocks the
 // last launch_adj_push used (max_items caps them as there)
 cudaError_t launch_pgrad_acc(const Geom &g, const double *part, int max_items, double *acc,
-                             cudaStream_t st);
+                             LStream st);
 cudaError_t launch_green_adj(const Geom &g, const double *L_d, const float2 *lE_hat,
-                             float2 *lrho_hat, int64_t nhalf, cudaStream_t st);
+                             float2 *lrho_hat, int64_t nhalf, LStream st);
 // where k_adj_rho writes the updated multipliers (o[0] == nullptr: in place)
 struct LamOut {
     float *o[3];
@@ -424,11 +471,11 @@ struct LamOut {
 };
 cudaError_t launch_adj_rho(int64_t n, const Geom &g, Ctrl *ctrl, const int32_t *ycell,
                            const float *const yo[3], const float2 *lrho2, float qscale,
-                           const LamOut &out, int par, cudaStream_t st);
+                           const LamOut &out, int par, LStream st);
 // lrho2[q] = (lrho[q], lrho[q + x (periodic)]); lE4 cleared
 cudaError_t launch_adj_pair_rho(const Geom &g, const float *lrho, float2 *lrho2, float4 *lE4,
-                                Ctrl *ctrl, int par, cudaStream_t st);
-cudaError_t launch_adj_zero(int64_t n, const Ctrl *ctrl, cudaStream_t st);
+                                Ctrl *ctrl, int par, LStream st);
+cudaError_t launch_adj_zero(int64_t n, const Ctrl *ctrl, LStream st);
 struct ReorderArgs {
     const float *in_o[3];
     const float *in_v[3];
@@ -437,17 +484,17 @@ struct ReorderArgs {
 };
 cudaError_t launch_adj_reorder(int64_t n, const int32_t *pos, const int32_t *pid_prev,
                                const float *const in_o[3], const float *const in_v[3],
-                               float *const out_o[3], float *const out_v[3], cudaStream_t st);
+                               float *const out_o[3], float *const out_v[3], LStream st);
 // pos[pid[j]] = j for j < n (the inverse of a particle order)
-cudaError_t launch_pid_positions(int64_t n, const int32_t *pid, int32_t *pos, cudaStream_t st);
+cudaError_t launch_pid_positions(int64_t n, const int32_t *pid, int32_t *pos, LStream st);
 // the multipliers in load order: records (by pid) in `rec` (32 bytes per
 // particle, caller's scratch), then records [o0, o0 + m) as the gradients
-cudaError_t launch_adj_unload_records(int64_t n, const Ctrl *ctrl, float4 *rec, cudaStream_t st);
+cudaError_t launch_adj_unload_records(int64_t n, const Ctrl *ctrl, float4 *rec, LStream st);
 cudaError_t launch_adj_unload(int64_t o0, int64_t m, const float4 *rec, double half_dt,
-                              double scale, double *gx, double *gv, cudaStream_t st);
+                              double scale, double *gx, double *gv, LStream st);
 cudaError_t launch_objective(const double *fpart, int nb, double dV, const double *w,
-                             double *out, cudaStream_t st);
+                             double *out, LStream st);
 cudaError_t launch_dot(int64_t n, const double *a, const double *b, double *part, int max_part,
-                       double *out, cudaStream_t st);
+                       double *out, LStream st);
 
 }  // namespace pic

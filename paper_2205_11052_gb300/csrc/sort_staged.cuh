@@ -46,7 +46,7 @@ __device__ __forceinline__ int block_exclusive_scan(int val, int *total) {
 
 // What the last block of a pass does besides: the histogram's scans its counts
 // into bin starts (and, for the full-key pass, lays out the work items), the
-// scatter's flips the current set.  One launch each instead of eleven per
+// scatter's clears the bins and flips the current set.  One launch each instead of eleven per
 // re-binning (three of a scan twice, ranges, items): those took 30 of 38 us a
 // re-binning of 33k particles.  One block walks the bins, so passes of more than
 // kFusedBins keys keep the separate kernels (fused = false).  A step of 33k
@@ -221,6 +221,7 @@ template <class Key>
 __global__ void __launch_bounds__(256) k_scatter_staged(int64_t n, Key key_param, Ctrl *ctrl,
                                                          int32_t *bins, int nb, SortRange rg,
                                                          PassEnd pe, const int32_t *gate) {
+    dep_begin();
     if (gate && !*gate) return;
     Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
     extern __shared__ __align__(128) unsigned char smem[];
@@ -243,9 +244,11 @@ __global__ void __launch_bounds__(256) k_scatter_staged(int64_t n, Key key_param
     if (pe.fused && pe.chunk > 0)
         for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nb; t += gridDim.x * blockDim.x)
             fill_tile(t, pe.tile_range[t], pe.tile_items[t], pe.chunk, pe.items);
-    // every block has read ctrl->cur by the time it gets here
+    // every block has read ctrl->cur and claimed its ranges by the time it gets here
     auto finish = [&]() {
-        if (pe.fused && pe.flip && last_block(&ctrl->done[1]) && threadIdx.x == 0) {
+        if (!pe.fused || !last_block(&ctrl->done[1])) return;
+        for (int t = threadIdx.x; t < nb; t += blockDim.x) bins[t] = 0;   // for the next pass
+        if (pe.flip && threadIdx.x == 0) {
             if (pe.chunk > 0) rebinned(ctrl, true);
             else ctrl->cur = 1 - ctrl->cur;
         }
@@ -416,6 +419,7 @@ template <class Key, int PER>
 __global__ void __launch_bounds__(256) k_histogram_staged(int64_t n, Key key_param, Ctrl *ctrl,
                                                            int32_t *bins, int nb, SortRange rg,
                                                            PassEnd pe, const int32_t *gate) {
+    dep_begin();
     if (gate && !*gate) return;
     Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
     __shared__ int32_t hkey[kHash];
@@ -474,6 +478,7 @@ __global__ void __launch_bounds__(256) k_histogram_direct(int64_t n, int64_t per
                                                            Ctrl *ctrl, int32_t *bins, int nb,
                                                            SortRange rg, PassEnd pe,
                                                            const int32_t *gate) {
+    dep_begin();
     if (gate && !*gate) return;
     Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
     extern __shared__ __align__(16) int32_t cnt[];
@@ -510,10 +515,12 @@ __global__ void __launch_bounds__(256) k_histogram_direct(int64_t n, int64_t per
 // into the same range of the other set; nb keys (bins holds nb + 1 ints).
 template <class Key>
 cudaError_t staged_pass(int64_t n, const Key &key_of, int64_t nb, Ctrl *ctrl, int32_t *bins,
-                        int32_t *scan_tmp, const PassEnd &pe, cudaStream_t st,
+                        int32_t *scan_tmp, const PassEnd &pe, LStream st,
                         SortRange rg = SortRange{0, 0}, const int32_t *gate = nullptr) {
-    cudaError_t e = cudaMemsetAsync(bins, 0, sizeof(int32_t) * (size_t)(nb + 1), st);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;   // fused passes find the bins clear and leave them so
+    if (!(pe.fused && n > 0) &&
+        (e = cudaMemsetAsync(bins, 0, sizeof(int32_t) * (size_t)(nb + 1), st)) != cudaSuccess)
+        return e;
     const int T = 256;
     if (n > 0) {
         // a block of the direct histogram clears and adds up all counters, so it
@@ -525,10 +532,16 @@ cudaError_t staged_pass(int64_t n, const Key &key_of, int64_t nb, Ctrl *ctrl, in
         const int64_t slice = 256 * per;
         const int hblocks = (int)std::min<int64_t>((n + slice - 1) / slice, kNumSMs * 8);
         if (nb <= kDirectBins && dper >= 4 * nb)
-            k_histogram_direct<Key><<<(unsigned)((n + dper - 1) / dper), T, sizeof(int32_t) * (size_t)nb, st>>>(n, dper, key_of, ctrl, bins, (int)nb, rg, pe, gate);
-        else if (per == 4) k_histogram_staged<Key, 4><<<hblocks, T, 0, st>>>(n, key_of, ctrl, bins, (int)nb, rg, pe, gate);
-        else k_histogram_staged<Key, kHistPer><<<hblocks, T, 0, st>>>(n, key_of, ctrl, bins, (int)nb, rg, pe, gate);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            e = launch_dep(k_histogram_direct<Key>, (unsigned)((n + dper - 1) / dper), T,
+                           sizeof(int32_t) * (size_t)nb, st, n, dper, key_of, ctrl, bins, (int)nb, rg, pe,
+                           gate);
+        else if (per == 4)
+            e = launch_dep(k_histogram_staged<Key, 4>, hblocks, T, 0, st, n, key_of, ctrl, bins, (int)nb,
+                           rg, pe, gate);
+        else
+            e = launch_dep(k_histogram_staged<Key, kHistPer>, hblocks, T, 0, st, n, key_of, ctrl, bins,
+                           (int)nb, rg, pe, gate);
+        if (e != cudaSuccess) return e;
     }
     if (!(pe.fused && n > 0) && (e = exclusive_scan(bins, nb, scan_tmp, st, gate)) != cudaSuccess)
         return e;
@@ -537,8 +550,9 @@ cudaError_t staged_pass(int64_t n, const Key &key_of, int64_t nb, Ctrl *ctrl, in
         const int per_sm =
             (int)std::max<size_t>(1, std::min<size_t>(8, (228 * 1024) / (kStageSmem + 1024)));
         const int sblocks = (int)std::min<int64_t>((n + kStage - 1) / kStage, 152 * per_sm);
-        k_scatter_staged<Key><<<sblocks, T, kStageSmem, st>>>(n, key_of, ctrl, bins, (int)nb, rg, pe, gate);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_dep(k_scatter_staged<Key>, sblocks, T, kStageSmem, st, n, key_of, ctrl, bins,
+                            (int)nb, rg, pe, gate)) != cudaSuccess)
+            return e;
     }
     return cudaSuccess;
 }
