@@ -378,7 +378,9 @@ bool fp32_rho(const pic_ctx *c) { return !(c->prm.options & PIC_OPT_FIXED_DEPOSI
 
 // sums: also leave the partial field sums of the diagnostics; clear_rho: leave rho
 // cleared for the push of the step
-int do_solve(pic_ctx *c, bool sums = false, bool clear_rho = false) {
+// (E8: where the field goes, by default the run's own array)
+int do_solve(pic_ctx *c, bool sums = false, bool clear_rho = false, float4 *E8 = nullptr) {
+    if (!E8) E8 = c->at<float4>(c->lay.E8);
     int r = timer_begin(c, PIC_PHASE_SOLVE);
     if (r) return r;
     if (c->own_fft) {
@@ -386,8 +388,7 @@ int do_solve(pic_ctx *c, bool sums = false, bool clear_rho = false) {
                                   c->at<float>(c->lay.ktab), c->at<float>(c->lay.rho), clear_rho,
                                   c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat), c->nhalf,
                                   c->mode_pos, c->prm.mode_comp, c->mode_conj, c->ctrl()->mode,
-                                  nullptr, c->at<float4>(c->lay.E8),
-                                  sums ? c->at<double>(c->lay.fpart) : nullptr, 0, c->st));
+                                  nullptr, E8, sums ? c->at<double>(c->lay.fpart) : nullptr, 0, c->st));
         return timer_end(c, PIC_PHASE_SOLVE, 3);
     }
     PIC_CUFFT(cufftExecR2C(c->r2c, c->at<cufftReal>(c->lay.rho), c->at<cufftComplex>(c->lay.rho_hat)));
@@ -395,7 +396,7 @@ int do_solve(pic_ctx *c, bool sums = false, bool clear_rho = false) {
                           c->nhalf, c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl(), c->st));
     PIC_CUFFT(cufftExecC2R(c->c2r, c->at<cufftComplex>(c->lay.E_hat), c->at<cufftReal>(c->lay.E_hat)));
     PIC_CUDA(launch_pack_E(c->geom, c->at<float>(c->lay.E_hat), 2 * (int64_t)c->geom.nh, 2 * c->nhalf,
-                           c->at<float4>(c->lay.E8), c->at<float>(c->lay.rho), clear_rho,
+                           E8, c->at<float>(c->lay.rho), clear_rho,
                            sums ? c->at<double>(c->lay.fpart) : nullptr, c->st));
     return timer_end(c, PIC_PHASE_SOLVE, 2);
 }
@@ -446,7 +447,8 @@ int fused_blocks_of(const pic_ctx *c) {
 
 // gather + push + deposit of the new positions in one kernel (pic_step), after a
 // solve that cleared rho if fp32_rho
-int do_push_deposit(pic_ctx *c, bool diag, const SaveY &save = SaveY{}) {
+int do_push_deposit(pic_ctx *c, bool diag, const SaveY &save = SaveY{}, float4 *E8 = nullptr) {
+    if (!E8) E8 = c->at<float4>(c->lay.E8);
     const bool fixed = (c->prm.options & PIC_OPT_FIXED_DEPOSIT) != 0;
     int r = timer_begin(c, PIC_PHASE_PUSH);
     if (r) return r;
@@ -459,7 +461,7 @@ int do_push_deposit(pic_ctx *c, bool diag, const SaveY &save = SaveY{}) {
     } else if (c->np > 0) {
         PIC_CUDA(launch_push_deposit(c->geom, push_const(c), diag, fixed, c->ctrl(),
                                      c->at<int4>(c->lay.items), (int)c->max_items,
-                                     c->at<float4>(c->lay.E8), c->at<float>(c->lay.rho),
+                                     E8, c->at<float>(c->lay.rho),
                                      c->at<unsigned long long>(c->lay.rho64), qscale_of(c),
                                      c->sparse_below, item_cost_of(c), c->at<double>(c->lay.ppart),
                                      fused_blocks_of(c), save, c->st));
@@ -671,15 +673,11 @@ AdjBound step_bound(const AdjBound &ab, int par) {
     return b;
 }
 
-// field (x-paired) of step `slot` of the segment being reversed
-int adj_keep_E(pic_ctx *c, const AdjLayout &L, int slot) {
-    CopyList cl{};
-    cl.count = 1;
-    cl.dst[0] = c->adj.buf + L.off_segE + (size_t)slot * L.segE;
-    cl.src[0] = c->at<char>(c->lay.E8);
-    cl.bytes[0] = c->ng * 32;
-    PIC_CUDA(launch_copy(cl, c->st));
-    return PIC_OK;
+// where the field (x-paired) of step `slot` of the segment being reversed is kept:
+// the solve writes it there and the push reads it from there (a copy of the run's
+// own array took 17 us of 250 a kept step at 64^3)
+float4 *adj_field(const pic_ctx *c, const AdjLayout &L, int slot) {
+    return reinterpret_cast<float4 *>(c->adj.buf + L.off_segE + (size_t)slot * L.segE);
 }
 
 // Re-bin; *cur follows the particles (the sort moves a non-empty store to the
@@ -743,8 +741,9 @@ int adj_keep_step(pic_ctx *c, const AdjLayout &L, int seg, int a0, int n, int *c
             return r;
     }
     if (!c->rho_current && (r = do_deposit(c))) return r;
-    if ((r = do_solve(c, false, fp32_rho(c))) || (r = adj_keep_E(c, L, n - a0))) return r;
-    if (c->np == 0) return do_push_deposit(c, false);
+    float4 *E8 = adj_field(c, L, n - a0);
+    if ((r = do_solve(c, false, fp32_rho(c), E8))) return r;
+    if (c->np == 0) return do_push_deposit(c, false, SaveY{}, E8);
     // y_n is written by the push that reads it
     char *y[7];
     buf_arrays(c->adj.buf + L.off_segy + (size_t)(n - a0) * L.segy, L.arr, L.ny, y);
@@ -753,7 +752,7 @@ int adj_keep_step(pic_ctx *c, const AdjLayout &L, int seg, int a0, int n, int *c
     for (int d = 0; d < 3; ++d) save.o[d] = reinterpret_cast<float *>(y[1 + d]);
     if (L.ny == 7)
         for (int d = 0; d < 3; ++d) save.v[d] = reinterpret_cast<float *>(y[4 + d]);
-    return do_push_deposit(c, false, save);
+    return do_push_deposit(c, false, save, E8);
 }
 
 // the adjoint field solve of step m (par = m & 1: its bound bookkeeping slot)
@@ -1449,8 +1448,7 @@ int pic_adjoint_backward(pic_handle_t c, double scale, double *gx, double *gv, i
             const float *yo[3] = {reinterpret_cast<const float *>(y[1]),
                                   reinterpret_cast<const float *>(y[2]),
                                   reinterpret_cast<const float *>(y[3])};
-            const float4 *En = reinterpret_cast<const float4 *>(c->adj.buf + L.off_segE +
-                                                                (size_t)(n - a0) * L.segE);
+            const float4 *En = adj_field(c, L, n - a0);
             PGrad pg{};
             if (pgrad) {
                 for (int d = 0; d < 3; ++d) {
