@@ -115,6 +115,7 @@ __device__ __forceinline__ void deposit_global(float *rho, unsigned long long *r
 // origin o; add one particle (or send it to the grid if it left the guard).
 struct Tile {
     int ox, oy, oz, S0, S01, S;
+    int G;              // guard layers of the box
     unsigned m0, m01;   // ceil(2^32 / S0), ceil(2^32 / S01): slot -> (a, b, c) by multiply-high
     bool inside;        // the box crosses no periodic boundary
     int node0;          // its first node if so
@@ -143,7 +144,8 @@ __host__ __device__ __forceinline__ int wrap_index(int v, int n) {
     return v;
 }
 
-__host__ __device__ __forceinline__ Tile tile_of(const Geom &g, int tile) {
+// the box of a tile with the deposit's guard layers, or with `guard` (>= 0)
+__host__ __device__ __forceinline__ Tile tile_of(const Geom &g, int tile, int guard = -1) {
     Tile t;
     const int tx = tile % g.ntile[0];
     const int ty = (tile / g.ntile[0]) % g.ntile[1];
@@ -151,7 +153,8 @@ __host__ __device__ __forceinline__ Tile tile_of(const Geom &g, int tile) {
     t.ox = tx * g.tile[0];
     t.oy = ty * g.tile[1];
     t.oz = tz * g.tile[2];
-    const int G = g.guard;
+    const int G = guard >= 0 ? guard : g.guard;
+    t.G = G;
     t.S0 = g.tile[0] + 2 * G + 1;
     t.S01 = t.S0 * (g.tile[1] + 2 * G + 1);
     t.S = t.S01 * (g.tile[2] + 2 * G + 1);
@@ -168,7 +171,7 @@ __device__ __forceinline__ int slot_node(const Tile &t, const Geom &g, int s) {
     int a, b, c;
     tile_pos(t, s, a, b, c);
     if (t.inside) return t.node0 + a + g.n[0] * (b + g.n[1] * c);
-    const int G = g.guard;
+    const int G = t.G;
     return wrap_index(t.ox - G + a, g.n[0]) +
            g.n[0] * (wrap_index(t.oy - G + b, g.n[1]) + g.n[1] * wrap_index(t.oz - G + c, g.n[2]));
 }

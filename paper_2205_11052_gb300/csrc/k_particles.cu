@@ -309,14 +309,40 @@ __global__ void __launch_bounds__(256, 3) k_gather_push(int64_t n, Geom g, PushC
 // it at the end: per step the particle store is read and written once (56
 // bytes per particle) instead of being read again by a separate deposit.
 // ---------------------------------------------------------------------------
+// The staged field box of a tile: its guard layers (at most the deposit's) and
+// extents.  BE > 0: BE slots on each axis.
+struct EBox {
+    int guard, row, plane, S;
+};
+template <int BE>
+__device__ __forceinline__ EBox e_box(const Geom &g, int guard) {
+    EBox e;
+    e.guard = guard;
+    e.row = BE > 0 ? BE : g.tile[0] + 2 * guard + 1;
+    e.plane = BE > 0 ? BE * BE : e.row * (g.tile[1] + 2 * guard + 1);
+    e.S = BE > 0 ? BE * BE * BE : e.plane * (g.tile[2] + 2 * guard + 1);
+    return e;
+}
+// slot of the stencil base with deposit slots (si, sj, sk) in the staged box; false
+// if its stencil leaves it
+template <int BE>
+__device__ __forceinline__ bool e_slot(const Geom &g, const EBox &e, int si, int sj, int sk, int &s) {
+    const int dg = g.guard - e.guard;
+    const unsigned a = (unsigned)(si - dg), b = (unsigned)(sj - dg), c = (unsigned)(sk - dg);
+    s = (int)a + e.row * (int)b + e.plane * (int)c;
+    if (BE > 0) return a < (unsigned)(BE - 1) && b < (unsigned)(BE - 1) && c < (unsigned)(BE - 1);
+    return a < (unsigned)(g.tile[0] + 2 * e.guard) && b < (unsigned)(g.tile[1] + 2 * e.guard) &&
+           c < (unsigned)(g.tile[2] + 2 * e.guard);
+}
+
 // One particle of the tile t (or of a sparse segment: everything through the
 // grid).  E comes from (sA, sB), the block's copy of the tile's box, when it holds
 // one and the stencil lies in it, else from the x-paired grid.  The slots of the
 // new stencil base are the old ones plus the cells moved, so the periodic
 // folding is done once per particle unless it leaves the box.
-template <bool DIAG, bool EXT, bool MAG, bool FIXED, int B>
+template <bool DIAG, bool EXT, bool MAG, bool FIXED, int B, int BE>
 __device__ __forceinline__ void pd_one(const Geom &g, const PushConst &pc, const float4 *E8,
-                                       const float4 *sA, const float2 *sB, bool sparse,
+                                       const float4 *sA, const float2 *sB, const EBox &eb, bool sparse,
                                        uint32_t *acc, const cic::Tile &t, float *rho,
                                        unsigned long long *rho64, float qscale, int32_t &c, float &fx,
                                        float &fy, float &fz, float &vx, float &vy, float &vz, int &bad,
@@ -327,9 +353,9 @@ __device__ __forceinline__ void pd_one(const Geom &g, const PushConst &pc, const
     int sj = cic::box_slot(j, t.oy, g.n[1], g.guard);
     int sk = cic::box_slot(k, t.oz, g.n[2], g.guard);
     float ex, ey, ez;
-    if (sA != nullptr && cic::in_box_slots<B>(t, g, si, sj, sk))
-        gather_E_pair_box<B>(sA, sB, si + cic::box_row<B>(t) * sj + cic::box_plane<B>(t) * sk, t.S0,
-                             t.S01, fx, fy, fz, ex, ey, ez);
+    int es;
+    if (sA != nullptr && e_slot<BE>(g, eb, si, sj, sk, es))
+        gather_E_pair_box<BE>(sA, sB, es, eb.row, eb.plane, fx, fy, fz, ex, ey, ez);
     else
         gather_E_pairs(g, E8, i, j, k, fx, fy, fz, ex, ey, ez);
     kick_drift<EXT, MAG>(g, pc, ex, ey, ez, i, j, k, c, fx, fy, fz, vx, vy, vz, bad, step);
@@ -351,12 +377,13 @@ __device__ __forceinline__ void pd_one(const Geom &g, const PushConst &pc, const
 }
 
 // staged: the block copies its tile's box of E8 to shared memory at each change
-// of tile and gathers there (see pd_one).  B > 0: every tile box
-// is B slots long on each axis (see cic::box_row).
-template <bool DIAG, bool EXT, bool MAG, bool FIXED, int B>
+// of tile, with e_guard guard layers, and gathers there (see pd_one).  BE > 0:
+// that box is BE slots long on each axis; B > 0: the deposit's is B slots long
+// (see cic::box_row).
+template <bool DIAG, bool EXT, bool MAG, bool FIXED, int B, int BE>
 __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom g, PushConst pc, Ctrl *ctrl,
                                                           const int4 *__restrict__ items,
-                                                          bool staged,
+                                                          bool staged, int e_guard,
                                                           const float4 *__restrict__ E8,
                                                           float *rho, unsigned long long *rho64,
                                                           float qscale, int sparse_below, int item_cost,
@@ -374,7 +401,8 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
     const int S = cic::tile_of(g, 0).S;
     void *sum = reinterpret_cast<char *>(acc) + cic::sum_offset(S);
     float4 *sA = reinterpret_cast<float4 *>(reinterpret_cast<char *>(acc) + cic::stage_offset(S));
-    float2 *sB = reinterpret_cast<float2 *>(sA + S);
+    const EBox eb = e_box<BE>(g, e_guard);
+    float2 *sB = reinterpret_cast<float2 *>(sA + eb.S);
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
         acc[s] = 0u;
         if (FIXED) reinterpret_cast<unsigned long long *>(sum)[s] = 0ull;
@@ -399,7 +427,7 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
         if (!sparse) {
             __syncthreads();   // every add to the tile and read of its box is done
             const cic::Tile tn = cic::tile_of(g, tile);
-            if (staged) cic::stage_pairs(sA, sB, E8, tn, g);
+            if (staged) cic::stage_pairs(sA, sB, E8, cic::tile_of(g, tile, e_guard), g);
             if (any) cic::tile_flush<FIXED>(acc, sum, folded, t, g, rho, rho64, qscale);
             any = true;
             folded = false;
@@ -431,7 +459,7 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
                         __stcs(save.v[2] + p, vz);
                     }
                 }
-                pd_one<DIAG, EXT, MAG, FIXED, B>(g, pc, E8, sAi, sB, sparse, acc, t, rho, rho64, qscale,
+                pd_one<DIAG, EXT, MAG, FIXED, B, BE>(g, pc, E8, sAi, sB, eb, sparse, acc, t, rho, rho64, qscale,
                                               c, fx, fy, fz, vx, vy, vz, bad, strays, mo);
                 __stcs(ps.cell + p, c);
                 __stcs(ps.o[0] + p, fx);
@@ -804,16 +832,26 @@ size_t tile_deposit_smem(const Geom &g) {
 // Blocks of the fused push + deposit: two of 384 threads per SM with the x-paired
 // box (24 bytes a slot after the deposit tiles' 12) while two fit in its 228 KiB
 // (plus the kernel's static shared memory and the runtime's 1 KiB per block), else
-// three of 256 that read the grid.  13^3 slots (8^3 tiles, two guard layers) take
-// the first: 20 steps of 128^3 x 64 64.1 ms, with whole nodes in the box (16 bytes
-// a slot, three blocks of 256) 66.9.  15^3 slots (three guard layers) take the
-// second: one block of 768 threads with the box made the Penning bunch's 10 steps
-// 53.7 ms instead of 50.7.
+// three of 256 that read the grid.  13^3 slots (8^3 tiles, two guard layers): 20
+// steps of 128^3 x 64 64.1 ms, with whole nodes in the box (16 bytes a slot, three
+// blocks of 256) 66.9.  With more guard layers the box takes as many as fit, two at
+// least: the Penning bunch's (three, of which the box takes two) 10 steps took 49.8
+// ms reading the grid, now 46.9; one block of 768 threads with all three 53.7.
 PushShape push_shape(const Geom &g) {
-    const int S = cic::tile_of(g, 0).S;
-    const size_t box = cic::stage_offset(S) + 24 * (size_t)S;
-    if (2 * (box + 2048) <= (size_t)228 * 1024) return PushShape{kPushThreadsPerSM / 2, 2, true, box};
-    return PushShape{kPushThreadsPerSM / 3, 3, false, tile_deposit_smem(g)};
+    const size_t tiles = cic::stage_offset(cic::tile_of(g, 0).S);
+    for (int eg = g.guard; eg >= std::min(g.guard, 2); --eg) {
+        const size_t box = tiles + 24 * (size_t)cic::tile_of(g, 0, eg).S;
+        if (2 * (box + 2048) <= (size_t)228 * 1024)
+            return PushShape{kPushThreadsPerSM / 2, 2, true, eg, box};
+    }
+    return PushShape{kPushThreadsPerSM / 3, 3, false, 0, tile_deposit_smem(g)};
+}
+// boxes compiled as constants: the default's, and a three-layer guard's with the
+// field box of two
+bool const_box15(const Geom &g, const PushShape &ps) {
+    for (int d = 0; d < 3; ++d)
+        if (g.tile[d] != 8) return false;
+    return g.guard == 3 && ps.staged && ps.e_guard == 2;
 }
 
 // Allow the fused kernels' shared memory (call outside any stream capture)
@@ -832,13 +870,14 @@ cudaError_t push_deposit_prepare(const Geom &g) {
     }
     const size_t smem = push_shape(g).smem;
     if (smem <= 48 * 1024) return cudaSuccess;
-#define PIC_PDA(D, X, M, F, B)                                                                \
-    if ((e = cudaFuncSetAttribute(k_push_deposit<D, X, M, F, B>,                              \
+#define PIC_PDA(D, X, M, F, B, BE)                                                            \
+    if ((e = cudaFuncSetAttribute(k_push_deposit<D, X, M, F, B, BE>,                          \
                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != \
         cudaSuccess)                                                                          \
         return e
 #define PIC_PDA2(D, X, M) \
-    PIC_PDA(D, X, M, false, 0); PIC_PDA(D, X, M, true, 0); PIC_PDA(D, X, M, true, kConstBox)
+    PIC_PDA(D, X, M, false, 0, 0); PIC_PDA(D, X, M, true, 0, 0);          \
+    PIC_PDA(D, X, M, true, kConstBox, kConstBox); PIC_PDA(D, X, M, true, 15, kConstBox)
     PIC_PDA2(false, false, false); PIC_PDA2(false, false, true);
     PIC_PDA2(false, true, false);  PIC_PDA2(false, true, true);
     PIC_PDA2(true, false, false);  PIC_PDA2(true, false, true);
@@ -859,16 +898,16 @@ cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, b
     const int nb = std::max(1, std::min(blocks, max_items));
     const float qs = (float)qscale;
     cudaError_t e = cudaSuccess;
-    const bool cbox = const_box(g);
-#define PIC_PD(D, X, M, F, B)                                                                   \
-    launch_dep(k_push_deposit<D, X, M, F, B>, nb, ps.threads, ps.smem, st, g, pc, ctrl, items, ps.staged, E8, \
-                                                                    rho, rho64, qs,             \
-                                                                    sparse_below, item_cost, part, save)
-#define PIC_PD_F(D, X, M)                                  \
-    do {                                                   \
-        if (!fixed) PIC_PD(D, X, M, false, 0);             \
-        else if (cbox) PIC_PD(D, X, M, true, kConstBox);   \
-        else PIC_PD(D, X, M, true, 0);                     \
+    const bool cbox = const_box(g) && ps.staged, cbox15 = const_box15(g, ps);
+#define PIC_PD(D, X, M, F, B, BE)                                                             \
+    launch_dep(k_push_deposit<D, X, M, F, B, BE>, nb, ps.threads, ps.smem, st, g, pc, ctrl, items, \
+               ps.staged, ps.e_guard, E8, rho, rho64, qs, sparse_below, item_cost, part, save)
+#define PIC_PD_F(D, X, M)                                            \
+    do {                                                             \
+        if (!fixed) PIC_PD(D, X, M, false, 0, 0);                    \
+        else if (cbox) PIC_PD(D, X, M, true, kConstBox, kConstBox);  \
+        else if (cbox15) PIC_PD(D, X, M, true, 15, kConstBox);       \
+        else PIC_PD(D, X, M, true, 0, 0);                            \
     } while (0)
     if (diag) {
         if (ext) { if (mag) PIC_PD_F(true, true, true); else PIC_PD_F(true, true, false); }

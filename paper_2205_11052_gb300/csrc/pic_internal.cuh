@@ -321,6 +321,7 @@ cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, boo
 struct PushShape {
     int threads, per_sm;
     bool staged;
+    int e_guard;   // guard layers of the staged box
     size_t smem;
 };
 PushShape push_shape(const Geom &g);

@@ -84,6 +84,31 @@ def test_more_tiles_than_the_fused_passes_take():
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
+# (tile, guard): field boxes of the deposit's guard layers (2, 1), of fewer (3, 4 and
+# an uneven tile) and none at all (5)
+BOXES = [((8, 8, 8), 3), ((8, 8, 8), 4), ((8, 8, 8), 5), ((8, 6, 8), 3), ((4, 8, 8), 5), ((4, 4, 4), 1)]
+
+
+@pytest.mark.parametrize("tile,guard", BOXES)
+def test_field_boxes_of_fewer_layers_give_the_same_bits(tile, guard):
+    w = pi.landau(n=24, ppc=8, alpha=0.2, seed=22, dt=0.3)   # 0.6 cells a step
+    out = []
+    for kw in (dict(tile=(8, 8, 8), guard=2), dict(tile=tile, guard=guard)):
+        sim = Simulation.from_workload(w, sort_period=-1, options=FIXED, **kw)
+        sim.step(6)
+        out.append((*sim.particles(), sim.field()[0]))
+        assert sim.flags() == 0
+        sim.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("tile,guard", BOXES[:4])
+def test_field_boxes_of_fewer_layers_with_fp32_deposit(tile, guard):
+    _check_steps((24, 24, 24), (2.0, 2.0, 2.0), 20_011, 0, guard, steps=4, tile=tile, guard=guard,
+                 sort_period=-1)
+
+
 @pytest.mark.parametrize("kw", [dict(), dict(guard=3), dict(tile=(4, 4, 4), guard=1), dict(guard=8)],
                          ids=["staged", "grid", "small-box", "large-box"])
 def test_reverse_push_shapes(kw):
