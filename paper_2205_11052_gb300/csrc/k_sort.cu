@@ -25,6 +25,7 @@ namespace pic {
 
 namespace {
 
+constexpr int kScanThreads = 256;
 constexpr int kScanItems = 16;
 constexpr int kScanSeg = kScanThreads * kScanItems;   // 4096 elements per block
 

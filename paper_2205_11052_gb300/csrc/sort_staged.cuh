@@ -16,10 +16,10 @@ namespace pic {
 
 namespace {
 
-constexpr int kScanThreads = 256;
-
+// exclusive scan over the block (at most 1024 threads), its total to *total
 __device__ __forceinline__ int block_exclusive_scan(int val, int *total) {
-    __shared__ int warp_tot[kScanThreads / 32];
+    __shared__ int warp_tot[32];
+    const int warps = blockDim.x >> 5;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int inc = val;
     for (int o = 1; o < 32; o <<= 1) {
@@ -29,14 +29,14 @@ __device__ __forceinline__ int block_exclusive_scan(int val, int *total) {
     if (lane == 31) warp_tot[wid] = inc;
     __syncthreads();
     if (wid == 0) {
-        int w = (lane < kScanThreads / 32) ? warp_tot[lane] : 0;
+        int w = (lane < warps) ? warp_tot[lane] : 0;
         int wi = w;
         for (int o = 1; o < 32; o <<= 1) {
             const int t = __shfl_up_sync(0xffffffffu, wi, o);
             if (lane >= o) wi += t;
         }
-        if (lane < kScanThreads / 32) warp_tot[lane] = wi - w;   // exclusive warp offsets
-        if (lane == kScanThreads / 32 - 1) *total = wi;
+        if (lane < warps) warp_tot[lane] = wi - w;   // exclusive warp offsets
+        if (lane == warps - 1) *total = wi;
     }
     __syncthreads();
     const int r = warp_tot[wid] + inc - val;
@@ -76,10 +76,10 @@ __device__ __forceinline__ bool last_block(unsigned int *done) {
 __device__ __forceinline__ int items_of(int cnt, int chunk) { return (cnt + chunk - 1) / chunk; }
 
 // counts -> exclusive starts in place, ranges and first items per tile; one
-// block of kScanThreads, each thread a contiguous run of bins
+// block, each thread a contiguous run of bins
 __device__ __forceinline__ void finish_bins(int32_t *bins, int nb, const PassEnd &pe, Ctrl *ctrl) {
     __shared__ int tot;
-    const int per = ((nb + kScanThreads - 1) / kScanThreads + 3) & ~3;
+    const int per = (nb + (int)blockDim.x - 1) / (int)blockDim.x;
     const int t0 = threadIdx.x * per, t1 = min(nb, t0 + per);
     int cnt = 0, it = 0;
     for (int t = t0; t < t1; ++t) {
@@ -471,10 +471,11 @@ __global__ void __launch_bounds__(256) k_histogram_staged(int64_t n, Key key_par
 // contiguous share of the particles to the global counts at the end.  The hashed
 // version spends 86 instructions a particle on finding runs and slots; at 134M
 // particles and 4096 keys it took 420 us, this one 172 (reading the cells at
-// memory speed: 80).
+// memory speed: 80).  Above kDirectBins the counters take one block of 1024 threads
+// per SM: 32768 keys 545 us, now 265 (134M particles).
 constexpr int kDirectBins = 8192;
-template <class Key>
-__global__ void __launch_bounds__(256) k_histogram_direct(int64_t n, int64_t per, Key key_param,
+template <class Key, int T>
+__global__ void __launch_bounds__(T) k_histogram_direct(int64_t n, int64_t per, Key key_param,
                                                            Ctrl *ctrl, int32_t *bins, int nb,
                                                            SortRange rg, PassEnd pe,
                                                            const int32_t *gate) {
@@ -482,30 +483,30 @@ __global__ void __launch_bounds__(256) k_histogram_direct(int64_t n, int64_t per
     if (gate && !*gate) return;
     Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
     extern __shared__ __align__(16) int32_t cnt[];
-    for (int b = threadIdx.x; b < nb; b += 256) cnt[b] = 0;
+    for (int b = threadIdx.x; b < nb; b += T) cnt[b] = 0;
     __syncthreads();
     const int32_t *cell = ctrl->sets[ctrl->cur ^ rg.rel].cell + rg.o;
     const int64_t b0 = blockIdx.x * per, b1 = b0 + per < n ? b0 + per : n;
     int bad = 0;
-    // four cells a thread and load, two loads in flight (b0 is a multiple of 1024)
+    // four cells a thread and load, two loads in flight (b0 is a multiple of 4 T)
     int64_t j = b0 + 4 * threadIdx.x;
-    for (; j + 1024 + 3 < b1; j += 2048) {
+    for (; j + 4 * T + 3 < b1; j += 8 * T) {
         const int4 a = __ldcs(reinterpret_cast<const int4 *>(cell + j));
-        const int4 c = __ldcs(reinterpret_cast<const int4 *>(cell + j + 1024));
+        const int4 c = __ldcs(reinterpret_cast<const int4 *>(cell + j + 4 * T));
         atomicAdd(cnt + key_of(a.x, rg.o + j, bad), 1);
         atomicAdd(cnt + key_of(a.y, rg.o + j + 1, bad), 1);
         atomicAdd(cnt + key_of(a.z, rg.o + j + 2, bad), 1);
         atomicAdd(cnt + key_of(a.w, rg.o + j + 3, bad), 1);
-        atomicAdd(cnt + key_of(c.x, rg.o + j + 1024, bad), 1);
-        atomicAdd(cnt + key_of(c.y, rg.o + j + 1025, bad), 1);
-        atomicAdd(cnt + key_of(c.z, rg.o + j + 1026, bad), 1);
-        atomicAdd(cnt + key_of(c.w, rg.o + j + 1027, bad), 1);
+        atomicAdd(cnt + key_of(c.x, rg.o + j + 4 * T, bad), 1);
+        atomicAdd(cnt + key_of(c.y, rg.o + j + 4 * T + 1, bad), 1);
+        atomicAdd(cnt + key_of(c.z, rg.o + j + 4 * T + 2, bad), 1);
+        atomicAdd(cnt + key_of(c.w, rg.o + j + 4 * T + 3, bad), 1);
     }
-    for (; j < b1; j += 1024)
+    for (; j < b1; j += 4 * T)
         for (int64_t q = j; q < j + 4 && q < b1; ++q)
             atomicAdd(cnt + key_of(__ldcs(cell + q), rg.o + q, bad), 1);
     __syncthreads();
-    for (int b = threadIdx.x; b < nb; b += 256)
+    for (int b = threadIdx.x; b < nb; b += T)
         if (cnt[b] > 0) atomicAdd(bins + b, cnt[b]);
     if (bad) atomicOr(&ctrl->flags, PIC_FLAG_BAD_CELL);
     if (pe.fused && last_block(&ctrl->done[0])) finish_bins(bins, nb, pe, ctrl);
@@ -525,16 +526,23 @@ cudaError_t staged_pass(int64_t n, const Key &key_of, int64_t nb, Ctrl *ctrl, in
     if (n > 0) {
         // a block of the direct histogram clears and adds up all counters, so it
         // wants several particles for each
-        const int64_t dblocks = std::min<int64_t>((n + 2047) / 2048, kNumSMs * (nb <= 4096 ? 8 : 6));
-        const int64_t dper = ((n + dblocks - 1) / dblocks + 1023) / 1024 * 1024;
+        const int64_t dt = nb <= kDirectBins ? 256 : 1024;
+        const int64_t dblocks = std::min<int64_t>((n + 8 * dt - 1) / (8 * dt),
+                                                  kNumSMs * (dt == 256 ? (nb <= 4096 ? 8 : 6) : 1));
+        const int64_t dper = ((n + dblocks - 1) / dblocks + 4 * dt - 1) / (4 * dt) * (4 * dt);
+        const unsigned dgrid = (unsigned)((n + dper - 1) / dper);
+        const size_t dsmem = sizeof(int32_t) * (size_t)nb;
+        const bool direct = nb <= kFusedBins && dper >= 4 * nb;
         // short slices while long ones would leave SMs without one
         const int per = n <= (int64_t)kNumSMs * kHistStage ? 4 : kHistPer;
         const int64_t slice = 256 * per;
         const int hblocks = (int)std::min<int64_t>((n + slice - 1) / slice, kNumSMs * 8);
-        if (nb <= kDirectBins && dper >= 4 * nb)
-            e = launch_dep(k_histogram_direct<Key>, (unsigned)((n + dper - 1) / dper), T,
-                           sizeof(int32_t) * (size_t)nb, st, n, dper, key_of, ctrl, bins, (int)nb, rg, pe,
-                           gate);
+        if (direct && dt == 256)
+            e = launch_dep(k_histogram_direct<Key, 256>, dgrid, 256, dsmem, st, n, dper, key_of, ctrl, bins,
+                           (int)nb, rg, pe, gate);
+        else if (direct)
+            e = launch_dep(k_histogram_direct<Key, 1024>, dgrid, 1024, dsmem, st, n, dper, key_of, ctrl,
+                           bins, (int)nb, rg, pe, gate);
         else if (per == 4)
             e = launch_dep(k_histogram_staged<Key, 4>, hblocks, T, 0, st, n, key_of, ctrl, bins, (int)nb,
                            rg, pe, gate);
@@ -557,10 +565,14 @@ cudaError_t staged_pass(int64_t n, const Key &key_of, int64_t nb, Ctrl *ctrl, in
     return cudaSuccess;
 }
 
-// the scatter's shared memory (above the default 48 KB); once per device,
-// outside any stream capture
+// the shared memory of the scatter and the large histogram (above the default
+// 48 KB); once per device, outside any stream capture
 template <class Key>
 cudaError_t staged_prepare() {
+    const cudaError_t e = cudaFuncSetAttribute(k_histogram_direct<Key, 1024>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)(sizeof(int32_t) * kFusedBins));
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_scatter_staged<Key>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)kStageSmem);
 }

@@ -84,6 +84,23 @@ def test_more_tiles_than_the_fused_passes_take():
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
+def test_histogram_of_more_keys_than_small_blocks_take():
+    """21^3 = 9261 tiles and enough particles for counters in shared memory."""
+    n, L, N = (84, 84, 84), (4.0, 4.0, 4.0), 6_000_001
+    r = np.random.default_rng(4)
+    x, v = r.random((N, 3)) * 4.0, r.standard_normal((N, 3))
+    out = []
+    for period in (1, -1):
+        sim = Simulation(n=n, L=L, n_particles=N, dt=0.01, Q=-64.0, options=FIXED, tile=(4, 4, 4),
+                         sort_period=period)
+        sim.load(x, v)
+        sim.step(2)
+        out.append(sim.particles())
+        assert sim.flags() == 0
+        sim.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
 # (tile, guard): field boxes of the deposit's guard layers (2, 1), of fewer (3, 4 and
 # an uneven tile) and none at all (5)
 BOXES = [((8, 8, 8), 3), ((8, 8, 8), 4), ((8, 8, 8), 5), ((8, 6, 8), 3), ((4, 8, 8), 5), ((4, 4, 4), 1)]
