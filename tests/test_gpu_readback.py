@@ -83,3 +83,24 @@ def test_ensemble_orders():
     assert np.array_equal(xd.cpu().numpy(), np.concatenate(xs))
     assert np.array_equal(vd.cpu().numpy(), np.concatenate(vs))
     ens.close()
+
+
+@pytest.mark.parametrize("copies", [1, 40])
+def test_ensemble_offsets_come_back_exactly(copies):
+    """Unit spacing: node + offset is exact in FP64 for offsets down to 2^-42, around
+    2^-19 (where the sum changes from integer to FP64 instructions) and up to 1."""
+    off = np.array([0.0, 2.0**-42, 2.0**-20 * (2 - 2.0**-23), 2.0**-19, 2.0**-19 * (1 + 2.0**-23), 0.5,
+                    1 - 2.0**-24])
+    sizes = [(24, 16, 9), (1000, 8, 8), (24, 16, 9)]
+    r = np.random.default_rng(9)
+    insts = []
+    for n in sizes:
+        i = np.tile(np.arange(n[0]), copies)
+        idx = np.stack([i, r.integers(0, n[1], i.size), r.integers(0, n[2], i.size)], 1)
+        x = idx + 0.5 + off[r.integers(0, off.size, idx.shape)]
+        insts.append((n, np.array(n, dtype=float), x, np.zeros_like(x), 0.0))
+    ens = Ensemble(insts, dt=DT)
+    xs, vs = ens.particles()
+    for (n, L, x0, v0, _), x, v in zip(insts, xs, vs):
+        assert np.array_equal(x, np.mod(x0, L)) and np.array_equal(v, v0)
+    ens.close()
