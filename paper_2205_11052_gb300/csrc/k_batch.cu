@@ -210,11 +210,8 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
     auto emit = [&](int it) {
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
         __syncthreads();
-        for (int q = 0; q < 4; ++q) {
-            double t = mo.total(q);
-            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-            if (lane == 0) red[q][wid] = t;
-        }
+        const double w4 = warp_total(mo);
+        if ((lane & 7) == 0) red[lane >> 3][wid] = w4;
         __syncthreads();
         if (threadIdx.x < 4) {
             double t = 0.0;

@@ -487,11 +487,8 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
     if (DIAG) {
         __shared__ double red[4][kPushThreadsPerSM / 64];
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-        for (int q = 0; q < 4; ++q) {
-            double tt = mo.total(q);
-            for (int o = 16; o > 0; o >>= 1) tt += __shfl_down_sync(0xffffffffu, tt, o);
-            if (lane == 0) red[q][wid] = tt;
-        }
+        const double w4 = warp_total(mo);
+        if ((lane & 7) == 0) red[lane >> 3][wid] = w4;
         __syncthreads();
         if (threadIdx.x < 4) {
             double tt = 0.0;
@@ -648,11 +645,8 @@ __device__ __forceinline__ void block_moments(const Moments &mo, double *part) {
     if (!DIAG) return;
     __shared__ double red[4][8];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int q = 0; q < 4; ++q) {
-        double tt = mo.total(q);
-        for (int o = 16; o > 0; o >>= 1) tt += __shfl_down_sync(0xffffffffu, tt, o);
-        if (lane == 0) red[q][wid] = tt;
-    }
+    const double w4 = warp_total(mo);
+    if ((lane & 7) == 0) red[lane >> 3][wid] = w4;
     __syncthreads();
     if (threadIdx.x < 4) {
         double tt = 0.0;
