@@ -53,7 +53,7 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
                                   const int4 *items, int blocks, int threads, int max_S,
                                   const float4 *E4, const float4 *E8,
                                   float *rho, unsigned long long *rho64, int sparse_below,
-                                  int item_cost, double *part, LStream st);
+                                  int tile_cost, double *part, LStream st);
 cudaError_t launch_b_rho_finish(int64_t ng, const InstDesc *desc, const long long *g0, int n_inst,
                                 unsigned long long *rho64, float *rho, LStream st);
 cudaError_t launch_b_green(const InstDesc *desc, int first, int m, int64_t nhalf,

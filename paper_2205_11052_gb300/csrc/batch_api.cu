@@ -163,8 +163,8 @@ void batch_layout(pic_batch *b) {
     b->o_bins = take((size_t)(b->ntiles + 1) * 4);
     b->o_scan = take((size_t)((b->ntiles + 4095) / 4096 + 2) * 4);
     b->o_titems = take((size_t)(b->ntiles + 1) * 4);
-    b->o_trange = take((size_t)b->ntiles * 8);
-    b->o_items = take((size_t)b->max_items * 16);
+    b->o_trange = take((size_t)(b->ntiles + 1) * 8);
+    b->o_items = take(rank_bytes(b->max_items) + (size_t)b->max_items * 16) + rank_bytes(b->max_items);
     b->o_fpart = take((size_t)b->n_inst * b->sum_stride * 4 * 8);
     for (SizeClass &c : b->cls) {
         c.o_tab = take(sizeof(FftTables));
@@ -207,7 +207,7 @@ int b_deposit_pass(pic_batch *b, bool push, bool diag) {
                                  b->stage_E ? b->at<float4>(b->o_E4) : nullptr,
                                  b->at<float4>(b->o_E8),
                                  b->at<float>(b->o_rho), b->at<unsigned long long>(b->o_rho64),
-                                 b->sparse_below, std::max(1, b->chunk / 4), b->at<double>(b->o_ppart),
+                                 b->sparse_below, tile_cost_of(b->np, b->fused_blocks), b->at<double>(b->o_ppart),
                                  b->st));
     if (b_fixed(b))
         B_CUDA(launch_b_rho_finish(b->ng, b->at<InstDesc>(b->o_desc), b->at<long long>(b->o_g0),

@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bo
                                                       const float4 *__restrict__ E8,
                                                       float4 *__restrict__ lE4, float c_kick,
                                                       float dt, float wz2, AdjRhoTerm rt,
-                                                      AdjBound ab, PGrad pg, int item_cost,
+                                                      AdjBound ab, PGrad pg, int tile_cost,
                                                       Ctrl *ctrl_w) {
     dep_begin();
     // 3 * S integer accumulators (x, y, z components) in units of 1 / qs
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bo
     float pa[kPGradTerms];
 #pragma unroll
     for (int q = 0; q < kPGradTerms; ++q) pa[q] = 0.0f;
-    Segments run = run_segments(items, n_items, item_cost);
+    Segments run = run_segments(items, n_items, tile_cost);
     for (int q = threadIdx.x; q < 3 * S; q += blockDim.x) acc[q] = 0;
     cic::Tile tb = cic::tile_of(g, 0);
     // adds the block's tile to lE4 and clears it
@@ -608,7 +608,7 @@ cudaError_t launch_adj_seed(int64_t ng, const float4 *E8, float4 *lE4, const dou
 }
 
 cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, int max_items,
-                            int item_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
+                            int tile_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
                             float4 *lE4, float c_kick, float dt, float wz2, const AdjRhoTerm &rt,
                             const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, LStream st) {
     const AdjShape a = adj_shape(g);
@@ -625,7 +625,7 @@ cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, 
         launch_dep(k_adj_push<PGV, BV>, blocks, a.threads, a.smem, st, g, a.staged, ctrl, items, ycell, \
                                                                yo[0], yo[1], yo[2], E8, lE4,    \
                                                                c_kick, dt, wz2, rt, ab, pg,     \
-                                                               item_cost, ctrl_w);              \
+                                                               tile_cost, ctrl_w);              \
     } while (0)
     if (pg.part) {
         if (cbox) PIC_ADJ(true, kConstBox);

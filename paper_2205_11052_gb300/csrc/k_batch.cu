@@ -181,7 +181,7 @@ template <bool PUSH, bool DIAG, bool EXT, bool MAG, bool FIXED>
 __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit(
     const InstDesc *__restrict__ desc, const int32_t *__restrict__ tile_inst, Ctrl *ctrl,
     const int4 *__restrict__ items, const float4 *__restrict__ E4, const float4 *__restrict__ E8,
-    float *rho, unsigned long long *rho64, int sparse_below, int item_cost, int max_S,
+    float *rho, unsigned long long *rho64, int sparse_below, int tile_cost, int max_S,
     double *__restrict__ part) {
     dep_begin();
     extern __shared__ __align__(16) uint32_t acc[];
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
     int it0, it1;
-    item_run(items, n_items, item_cost, it0, it1);
+    item_run(items, n_items, tile_cost, it0, it1);
     for (int s = threadIdx.x; s < max_S; s += blockDim.x) {
         acc[s] = 0u;
         if (FIXED) reinterpret_cast<unsigned long long *>(sum)[s] = 0ull;
@@ -527,7 +527,7 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
                                   const int4 *items, int blocks, int threads, int max_S,
                                   const float4 *E4, const float4 *E8,
                                   float *rho, unsigned long long *rho64, int sparse_below,
-                                  int item_cost, double *part, LStream st) {
+                                  int tile_cost, double *part, LStream st) {
     const size_t smem = batch_push_smem(max_S, E4 != nullptr && push);
     cudaError_t e = cudaSuccess;
 #define PIC_BPD(P, D, X, M, F)                                                                  \
@@ -538,7 +538,7 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
                                       (int)smem)) != cudaSuccess)                               \
             return e;                                                                           \
         launch_dep(kern, blocks, threads, smem, st, desc, tile_inst, ctrl, items, push ? E4 : nullptr, \
-                                            E8, rho, rho64, sparse_below, item_cost, max_S,     \
+                                            E8, rho, rho64, sparse_below, tile_cost, max_S,     \
                                             part);                                              \
     } while (0)
 #define PIC_BPD_F(P, D, X, M) \

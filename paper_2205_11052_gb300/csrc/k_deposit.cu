@@ -42,14 +42,14 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
                                                            const int4 *__restrict__ items,
                                                            float qscale, float *rho,
                                                            unsigned long long *rho64, Ctrl *ctrl_w,
-                                                           int sparse_below, int item_cost) {
+                                                           int sparse_below, int tile_cost) {
     dep_begin();
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
     unsigned long long strays = 0;
     int bad = 0;
-    Segments run = run_segments(items, n_items, item_cost);
+    Segments run = run_segments(items, n_items, tile_cost);
     const int S = tile_of(g, 0).S;
     void *sum = reinterpret_cast<char *>(acc) + sum_offset(S);
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
@@ -154,7 +154,7 @@ cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *r
 cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int4 *items,
                            int max_items, double qscale_d, float *rho, unsigned long long *rho64,
                            bool fixed, Ctrl *ctrl_w, int grid_blocks, int sparse_below,
-                           int item_cost, LStream st) {
+                           int tile_cost, LStream st) {
     (void)n;
     const float qscale = (float)qscale_d;
     const size_t smem = tile_deposit_smem(g);   // item tile + the block's tile sums
@@ -169,7 +169,7 @@ cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int
                                       (int)smem)) != cudaSuccess)                              \
             return e;                                                                          \
         launch_dep(k_deposit_tiles<F, B>, blocks, 256, smem, st, g, ctrl, items, qscale, rho, rho64,   \
-                                                         ctrl_w, sparse_below, item_cost);                \
+                                                         ctrl_w, sparse_below, tile_cost);                \
     } while (0)
     if (fixed) {
         if (cbox) PIC_DT(true, kConstBox);

@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
                                                           bool staged, int e_guard,
                                                           const float4 *__restrict__ E8,
                                                           float *rho, unsigned long long *rho64,
-                                                          float qscale, int sparse_below, int item_cost,
+                                                          float qscale, int sparse_below, int tile_cost,
                                                           double *__restrict__ part,
                                                           SaveY save) {
     dep_begin();
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
     int bad = 0;
     unsigned long long strays = 0;
     // a contiguous run of work items per block, walked tile by tile
-    Segments run = run_segments(items, n_items, item_cost);
+    Segments run = run_segments(items, n_items, tile_cost);
     const int S = cic::tile_of(g, 0).S;
     void *sum = reinterpret_cast<char *>(acc) + cic::sum_offset(S);
     float4 *sA = reinterpret_cast<float4 *>(reinterpret_cast<char *>(acc) + cic::stage_offset(S));
@@ -661,7 +661,7 @@ __device__ __forceinline__ void block_moments(const Moments &mo, double *part) {
 template <bool DIAG, bool FIXED, int B>
 __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
     Geom g, uint64_t seed, Ctrl *ctrl, const int4 *__restrict__ items, float *rho,
-    unsigned long long *rho64, float qscale, int sparse_below, int item_cost,
+    unsigned long long *rho64, float qscale, int sparse_below, int tile_cost,
     double *__restrict__ part) {
     dep_begin();
     extern __shared__ __align__(16) uint32_t acc[];
@@ -671,7 +671,7 @@ __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
     Moments mo;
     int bad = 0;
     unsigned long long strays = 0;
-    Segments run = run_segments(items, n_items, item_cost);
+    Segments run = run_segments(items, n_items, tile_cost);
     const int S = cic::tile_of(g, 0).S;
     void *sum = reinterpret_cast<char *>(acc) + cic::sum_offset(S);
     for (int s = threadIdx.x; s < S; s += blockDim.x) {
@@ -787,7 +787,7 @@ bool const_box(const Geom &g) {
 
 cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, bool fixed, bool deposit,
                         Ctrl *ctrl, const int4 *items, int max_items, float *rho,
-                        unsigned long long *rho64, double qscale, int sparse_below, int item_cost,
+                        unsigned long long *rho64, double qscale, int sparse_below, int tile_cost,
                         double *part, int blocks, LStream st) {
     const int nb = std::max(1, std::min(blocks, deposit ? max_items : blocks));
     if (deposit) {
@@ -796,7 +796,7 @@ cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, boo
         const bool cbox = const_box(g);
 #define PIC_MV(D, F, B) \
     launch_dep(k_move_deposit<D, F, B>, nb, 256, smem, st, g, seed, ctrl, items, rho, rho64, qs, sparse_below, \
-                                                   item_cost, part)
+                                                   tile_cost, part)
         if (diag) {
             if (!fixed) PIC_MV(true, false, 0);
             else if (cbox) PIC_MV(true, true, kConstBox);
@@ -884,7 +884,7 @@ cudaError_t push_deposit_prepare(const Geom &g) {
 cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, bool fixed,
                                 Ctrl *ctrl, const int4 *items, int max_items,
                                 const float4 *E8, float *rho, unsigned long long *rho64,
-                                double qscale, int sparse_below, int item_cost, double *part,
+                                double qscale, int sparse_below, int tile_cost, double *part,
                                 int blocks, const SaveY &save, LStream st) {
     const bool ext = pc.wz2 != 0.0f;
     const bool mag = pc.t[0] != 0.0f || pc.t[1] != 0.0f || pc.t[2] != 0.0f;
@@ -895,7 +895,7 @@ cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, b
     const bool cbox = const_box(g) && ps.staged, cbox15 = const_box15(g, ps);
 #define PIC_PD(D, X, M, F, B, BE)                                                             \
     launch_dep(k_push_deposit<D, X, M, F, B, BE>, nb, ps.threads, ps.smem, st, g, pc, ctrl, items, \
-               ps.staged, ps.e_guard, E8, rho, rho64, qs, sparse_below, item_cost, part, save)
+               ps.staged, ps.e_guard, E8, rho, rho64, qs, sparse_below, tile_cost, part, save)
 #define PIC_PD_F(D, X, M)                                            \
     do {                                                             \
         if (!fixed) PIC_PD(D, X, M, false, 0, 0);                    \

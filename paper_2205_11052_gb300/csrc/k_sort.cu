@@ -131,7 +131,8 @@ __global__ void k_tile_ranges(const int32_t *__restrict__ bin_end, int ntiles, i
     if (t >= ntiles) return;
     const int s = (t == 0) ? 0 : bin_end[t - 1];
     const int e = bin_end[t];
-    tile_range[t] = make_int2(s, e);
+    tile_range[t] = make_int2(s, -1);
+    if (t == ntiles - 1) tile_range[ntiles] = make_int2(e, -1);
     tile_items[t] = items_of(e - s, chunk);
 }
 
@@ -144,8 +145,7 @@ __global__ void k_fill_items(int ntiles, int chunk, const int32_t *__restrict__ 
         ctrl->n_items = item_off[ntiles];
         rebinned(ctrl, flip != 0);
     }
-    if (t >= ntiles) return;
-    fill_tile(t, tile_range[t], item_off[t], chunk, items);
+    fill_tiles(t & ~31, ntiles, tile_range, item_off, chunk, items);
 }
 
 __global__ void k_flip(Ctrl *ctrl) { ctrl->cur = 1 - ctrl->cur; }

@@ -171,23 +171,46 @@ int record_error(int code, const char *fmt, ...);
 // its run tile by tile (next_segment), so small items cost it nothing.
 //
 // The run of work items [it0, it1) of this block.  Items cover the particles
-// [0, P) in order; item i costs its particles plus item_cost for its share of
-// the tile's staging and flush, so the cost before item i is y_i + item_cost i,
-// and the block takes the items that start within its equal share of the total
-// (with fewer items than blocks, block b takes item b).
+// [0, P) in order; a tile costs its particles plus tile_cost for its staging and
+// flush, so the cost before item i is y_i + tile_cost r_i with r_i the tiles with
+// particles before the item's (kept below the items, see item_rank), and the block
+// takes the items that start within its equal share of the total (with fewer items
+// than blocks, block b takes item b).
 //
 // With at most 4095 particles an item, 4.2M particles on 512 tiles of 8192 gave
 // a block two or three items (9200 particles), and 33k particles on 8 tiles kept
 // 9 of 456 blocks busy; sixteen items a block (256..4095 particles) keep the
 // shares within a few percent (push 110 -> 101 us and 40.6 -> 17.4 us).
+//
+// A tile's cost in particles (kTileCost) shows where tiles differ: with an item's
+// cost instead, a quarter of its size, blocks among the thin tiles at the end of a
+// 41^3 grid or around a bunch switched tiles up to eighteen times while the others
+// did not (14 steps of 2.5M particles 2.25 ms, now 1.73; the Penning bunch in 256^3,
+// 10 steps, 45.2 -> 44.7; with a cost of 512 1.92
+// and 46.1, of 4096 1.79 and 45.7).  It is at most half a block's particles, as every
+// block stages one tile whatever its share.
 constexpr int kItemsPerBlock = 16;
+constexpr int kTileCost = 2048;
+inline int tile_cost_of(int64_t n, int64_t blocks) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(kTileCost, n / (2 * blocks)));
+}
 constexpr int kMinChunk = 256;
 // Called by every thread of the block (it synchronises): the two item
 // indices are found by a two-level search in which each thread tests one
 // sample per round, so a block start costs a few dependent loads (two while
 // n_items <= blockDim^2), not log2(n_items).
+// The rank of item i, kept before the items in falling order
+__device__ __forceinline__ int32_t *item_rank(int4 *items, int i) {
+    return reinterpret_cast<int32_t *>(items) - 1 - i;
+}
+__device__ __forceinline__ int item_rank(const int4 *items, int i) {
+    return reinterpret_cast<const int32_t *>(items)[-1 - i];
+}
+// bytes of the ranks before the items
+inline size_t rank_bytes(int64_t max_items) { return ((size_t)max_items * 4 + 255) / 256 * 256; }
+
 __device__ __forceinline__ void item_run(const int4 *__restrict__ items, int n_items,
-                                         long long item_cost, int &it0, int &it1) {
+                                         long long tile_cost, int &it0, int &it1) {
     if (n_items <= (int)gridDim.x) {
         // at most one item per block: consecutive blocks (spread over the SMs)
         // take consecutive items, however large
@@ -196,10 +219,10 @@ __device__ __forceinline__ void item_run(const int4 *__restrict__ items, int n_i
         return;
     }
     const long long total =
-        n_items > 0 ? (long long)items[n_items - 1].z + item_cost * n_items : 0;
+        n_items > 0 ? (long long)items[n_items - 1].z + tile_cost * (item_rank(items, n_items - 1) + 1) : 0;
     const long long c0 = total * blockIdx.x / gridDim.x;
     const long long c1 = total * (blockIdx.x + 1) / gridDim.x;
-    auto cost = [&](int i) { return (long long)items[i].y + item_cost * i; };
+    auto cost = [&](int i) { return (long long)items[i].y + tile_cost * item_rank(items, i); };
     // level 1: sample i_t = (t + 1) * step - 1; the first index with cost >= c lies
     // in the step-wide bucket after the last sample below c
     const int nt = (int)blockDim.x;
@@ -232,10 +255,10 @@ struct Segments {
     int4 next;
 };
 __device__ __forceinline__ Segments run_segments(const int4 *__restrict__ items, int n_items,
-                                                 long long item_cost) {
+                                                 long long tile_cost) {
     Segments r;
     r.items = items;
-    item_run(items, n_items, item_cost, r.it, r.it1);
+    item_run(items, n_items, tile_cost, r.it, r.it1);
     r.next = make_int4(0, 0, 0, 0);
     r.pb = 0;
     if (r.it < r.it1) {
@@ -304,7 +327,7 @@ cudaError_t launch_timeout_selftest(Ctrl *ctrl, LStream st);
 cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int4 *items,
                            int max_items, double qscale, float *rho, unsigned long long *rho64,
                            bool fixed, Ctrl *ctrl_w, int grid_blocks, int sparse_below,
-                           int item_cost, LStream st);
+                           int tile_cost, LStream st);
 
 cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *rho, double qscale,
                               LStream st);
@@ -313,7 +336,7 @@ cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *r
 // items, like launch_push_deposit); advances the device step counter
 cudaError_t launch_move(int64_t np, const Geom &g, uint64_t seed, bool diag, bool fixed, bool deposit,
                         Ctrl *ctrl, const int4 *items, int max_items, float *rho,
-                        unsigned long long *rho64, double qscale, int sparse_below, int item_cost,
+                        unsigned long long *rho64, double qscale, int sparse_below, int tile_cost,
                         double *part, int blocks, LStream st);
 // block size, blocks per SM, whether the blocks stage E, and the dynamic shared
 // memory of the fused push + deposit kernel for geometry g; the one-time
@@ -342,7 +365,7 @@ struct SaveY {
 cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, bool fixed,
                                 Ctrl *ctrl, const int4 *items, int max_items, const float4 *E8,
                                 float *rho, unsigned long long *rho64, double qscale,
-                                int sparse_below, int item_cost, double *part, int blocks,
+                                int sparse_below, int tile_cost, double *part, int blocks,
                                 const SaveY &save, LStream st);
 cudaError_t launch_gather_push(int64_t n, const Geom &g, const PushConst &pc, bool diag,
                                Ctrl *ctrl, const float4 *E8, double *part, int blocks,
@@ -456,7 +479,7 @@ struct AdjShape {
 AdjShape adj_shape(const Geom &g);
 int adj_blocks(const Geom &g, int max_items);
 cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, int max_items,
-                            int item_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
+                            int tile_cost, const int32_t *ycell, const float *const yo[3], const float4 *E8,
                             float4 *lE4, float c_kick, float dt, float wz2, const AdjRhoTerm &rt,
                             const AdjBound &ab, const PGrad &pg, Ctrl *ctrl_w, LStream st);
 // acc[q] += the fixed-order sum of the kPGradTerms partials of the blocks the

@@ -57,7 +57,8 @@ struct PassEnd {
     bool flip;             // the scatter's last block flips ctrl->cur
     int chunk;             // > 0: build the work list (particles per item)
     int32_t *tile_items;   // first item of each tile, total last
-    int2 *tile_range;      // particles of each tile
+    int2 *tile_range;      // first particle of each tile and its rank (tiles with
+                           // particles before it; -1: not known), the total last
     int4 *items;
 };
 
@@ -81,21 +82,25 @@ __device__ __forceinline__ void finish_bins(int32_t *bins, int nb, const PassEnd
     __shared__ int tot;
     const int per = (nb + (int)blockDim.x - 1) / (int)blockDim.x;
     const int t0 = threadIdx.x * per, t1 = min(nb, t0 + per);
-    int cnt = 0, it = 0;
+    int cnt = 0, it = 0, full = 0;
     for (int t = t0; t < t1; ++t) {
         const int k = __ldcg(bins + t);
         cnt += k;
+        full += k > 0;
         if (pe.chunk > 0) it += items_of(k, pe.chunk);
     }
     int run = block_exclusive_scan(cnt, &tot);
+    int rank = pe.chunk > 0 ? block_exclusive_scan(full, &tot) : 0;
     int item = pe.chunk > 0 ? block_exclusive_scan(it, &tot) : 0;
     for (int t = t0; t < t1; ++t) {
         const int k = __ldcg(bins + t);
         bins[t] = run;
         if (pe.chunk > 0) {
-            pe.tile_range[t] = make_int2(run, run + k);
+            pe.tile_range[t] = make_int2(run, rank);
             pe.tile_items[t] = item;
             item += items_of(k, pe.chunk);
+            rank += k > 0;
+            if (t == nb - 1) pe.tile_range[nb] = make_int2(run + k, rank);
         }
         run += k;
     }
@@ -105,12 +110,41 @@ __device__ __forceinline__ void finish_bins(int32_t *bins, int nb, const PassEnd
     }
 }
 
-// tile t's items: begins of equal shares of its particles, the tile's end and
-// the next tile's first item
-__device__ __forceinline__ void fill_tile(int t, int2 r, int o, int chunk, int4 *items) {
-    const int cnt = r.y - r.x, k = items_of(cnt, chunk);
-    for (int i = 0; i < k; ++i)
-        items[o + i] = make_int4(t, r.x + (int)((long long)cnt * i / k), r.y, o + k);
+// The items of tiles t0..t0 + 31 by one warp (all its lanes), lane l's tile t0 + l:
+// begins of equal shares of its particles, the tile's end and the next tile's first
+// item, and the items' ranks (the item's own index where the tile's is not known).
+// A lane writes a few items by itself, the warp the many of a dense tile together
+// (with a thread per tile a bunch of 900 thousand particles in a few tiles waited 40
+// us for them at every re-binning).
+__device__ __forceinline__ void fill_tiles(int t0, int ntiles, const int2 *__restrict__ range,
+                                           const int32_t *__restrict__ first, int chunk, int4 *items) {
+    const int lane = threadIdx.x & 31, t = t0 + lane;
+    int2 r = make_int2(0, 0);
+    int o = 0, end = 0;
+    if (t < ntiles) {
+        r = range[t];
+        o = first[t];
+        end = range[t + 1].x;
+    }
+    const int k = items_of(end - r.x, chunk);
+    const int q = k > 0 ? (end - r.x) / k : 0, rest = end - r.x - q * k;
+    constexpr int kAlone = 4;
+    if (k <= kAlone)
+        for (int i = 0; i < k; ++i) {
+            items[o + i] = make_int4(t, r.x + q * i + min(i, rest), end, o + k);
+            *item_rank(items, o + i) = r.y >= 0 ? r.y : o + i;
+        }
+    for (unsigned m = __ballot_sync(0xffffffffu, k > kAlone); m; m &= m - 1) {
+        const int l = __ffs(m) - 1;
+        const int kl = __shfl_sync(0xffffffffu, k, l), ol = __shfl_sync(0xffffffffu, o, l);
+        const int ql = __shfl_sync(0xffffffffu, q, l), dl = __shfl_sync(0xffffffffu, rest, l);
+        const int xl = __shfl_sync(0xffffffffu, r.x, l), rl = __shfl_sync(0xffffffffu, r.y, l);
+        const int el = __shfl_sync(0xffffffffu, end, l);
+        for (int i = lane; i < kl; i += 32) {
+            items[ol + i] = make_int4(t0 + l, xl + ql * i + min(i, dl), el, ol + kl);
+            *item_rank(items, ol + i) = rl >= 0 ? rl : ol + i;
+        }
+    }
 }
 
 // a re-binning is complete: the particles are in the other set, each inside its tile
@@ -242,8 +276,9 @@ __global__ void __launch_bounds__(256) k_scatter_staged(int64_t n, Key key_param
     const int64_t nslices = (n + kStage - 1) / kStage;
     int bad = 0;
     if (pe.fused && pe.chunk > 0)
-        for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < nb; t += gridDim.x * blockDim.x)
-            fill_tile(t, pe.tile_range[t], pe.tile_items[t], pe.chunk, pe.items);
+        for (int t0 = 32 * (int)(blockIdx.x + (threadIdx.x >> 5) * gridDim.x); t0 < nb;
+             t0 += (int)(gridDim.x * blockDim.x))
+            fill_tiles(t0, nb, pe.tile_range, pe.tile_items, pe.chunk, pe.items);
     // every block has read ctrl->cur and claimed its ranges by the time it gets here
     auto finish = [&]() {
         if (!pe.fused || !last_block(&ctrl->done[1])) return;

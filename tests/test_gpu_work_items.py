@@ -126,6 +126,28 @@ def test_field_boxes_of_fewer_layers_with_fp32_deposit(tile, guard):
                  sort_period=-1)
 
 
+@pytest.mark.parametrize("n", [(17, 9, 25), (41, 41, 41), (64, 64, 8)])
+@pytest.mark.parametrize("N", [5000, 174_646, 1_500_001])
+def test_shares_of_a_bunch_among_thin_tiles(n, N):
+    """Half the particles in a few cells, half anywhere: whatever the items and the
+    blocks' shares, the fixed-point deposit gives the same bits."""
+    L = np.asarray(n) * 0.1
+    r = np.random.default_rng(N)
+    x, v = r.random((N, 3)) * L, r.standard_normal((N, 3))
+    x[::2] = (0.6 + 0.05 * r.standard_normal((x[::2].shape))) % L
+    out = []
+    for chunk in (0, 32, 4095):
+        sim = Simulation(n=n, L=L, n_particles=N, dt=0.01, Q=-float(np.prod(L)), options=FIXED,
+                         sort_period=2, chunk=chunk)
+        sim.load(x, v)
+        sim.step(3)
+        out.append((*sim.particles(), sim.field()[0]))
+        assert sim.flags() == 0
+        sim.close()
+    for o in out[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(out[0], o))
+
+
 @pytest.mark.parametrize("kw", [dict(), dict(guard=3), dict(tile=(4, 4, 4), guard=1), dict(guard=8)],
                          ids=["staged", "grid", "small-box", "large-box"])
 def test_reverse_push_shapes(kw):
