@@ -468,9 +468,11 @@ struct PGrad {
 };
 constexpr int kPGradTerms = 10;
 // threads per SM the reverse push is compiled for (80 registers), its blocks for
-// geometry g (see k_adjoint.cu) and the most of them
+// geometry g (see k_adjoint.cu)
 constexpr int kAdjThreadsPerSM = 768;
-constexpr int kAdjPushMaxBlocks = kNumSMs * 3;
+// room in the caller's buffer, whose size is part of the interface; at most half of
+// it is launched (adj_blocks)
+constexpr int kAdjPushMaxBlocks = kNumSMs * 3 * 2;
 struct AdjShape {
     int threads, per_sm;
     bool staged;
