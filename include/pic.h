@@ -89,8 +89,8 @@ typedef struct {
     int32_t block;         /* threads per block of the particle kernels (256);
                               ensembles: of the batched push + deposit, a
                               multiple of 32 in 64..256 (autotuned)          */
-    int32_t chunk;         /* max particles per deposit work item, 32..4095
-                              (default 4095)                                     */
+    int32_t chunk;         /* max particles per work item, 32..4095 (0: chosen
+                              from the particle count)                           */
     int32_t options;       /* PIC_OPT_* bits (default 0)                         */
     uint64_t seed;         /* random stream of PIC_OPT_UNIFORM_MOVE              */
     double  stray_rebin;   /* stray-triggered re-binning in pic_step (default 0 =
@@ -288,11 +288,11 @@ int pic_selftest_timeout(pic_handle_t h);
  * bound stream around its kernels; the library also counts its own kernel
  * launches (cuFFT's kernels excluded).  Do not enable timers while the
  * stream is being captured into a CUDA graph. */
-#define PIC_PHASE_SORT     0   /* binning: histogram, scan, scatter, work list   */
+#define PIC_PHASE_SORT     0   /* binning: histogram, scatter, work list          */
 #define PIC_PHASE_DEPOSIT  1   /* the deposit kernel                              */
-#define PIC_PHASE_SOLVE    2   /* R2C FFT, Green kernel, C2R FFT                  */
-#define PIC_PHASE_PUSH     3   /* the fused gather + push kernel                  */
-#define PIC_PHASE_DIAG     4   /* FP64 diagnostic reductions                      */
+#define PIC_PHASE_SOLVE    2   /* FFT, Green kernel, inverse FFT; field sums      */
+#define PIC_PHASE_PUSH     3   /* the fused gather + push (+ deposit) kernel      */
+#define PIC_PHASE_DIAG     4   /* the record from the partial sums                */
 #define PIC_PHASE_COUNT    5
 
 /* Enable (1) or disable (0) the timers; either way the accumulators and the

@@ -27,18 +27,6 @@ __device__ __forceinline__ bool decode_cell(int32_t c, const Geom &g, int &i, in
     return true;
 }
 
-// place axis index a (0 <= a < n) relative to tile origin o with guard G:
-// the slot in [0, T + 2G), or -1 if farther than G cells from the tile
-__device__ __forceinline__ int tile_slot(int a, int o, int n, int T, int G) {
-    int d = a - o;
-    if (d < 0) d += n;
-    if (d >= T + G) {
-        d -= n;
-        if (d < -G) return -1;
-    }
-    return d + G;
-}
-
 __device__ __forceinline__ void weights(float fx, float fy, float fz, float w[8]) {
     const float x0 = 1.0f - fx, y0 = 1.0f - fy, z0 = 1.0f - fz;
     const float a = y0 * z0, b = fy * z0, c = y0 * fz, d = fy * fz;

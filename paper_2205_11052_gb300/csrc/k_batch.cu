@@ -144,12 +144,6 @@ __device__ __forceinline__ int b_key(int32_t c, const InstDesc &D, int &bad) {
     return D.tile0 + ti + D.g.ntile[0] * (tj + D.g.ntile[1] * tk);
 }
 
-__device__ __forceinline__ void b_slice(int64_t n, int64_t &b0, int64_t &b1) {
-    const int64_t per = ((n + gridDim.x - 1) / gridDim.x + blockDim.x - 1) / blockDim.x * blockDim.x;
-    b0 = (int64_t)blockIdx.x * per;
-    b1 = b0 + per < n ? b0 + per : n;
-}
-
 // binning key of particle p: the global tile id of its instance's tile.  A
 // thread's copy remembers the particle range of the last instance it looked
 // up (a thread meets consecutive particles of one instance), so the binary
