@@ -827,10 +827,10 @@ size_t tile_deposit_smem(const Geom &g) {
 // box (24 bytes a slot after the deposit tiles' 12) while two fit in its 228 KiB
 // (plus the kernel's static shared memory and the runtime's 1 KiB per block), else
 // three of 256 that read the grid.  13^3 slots (8^3 tiles, two guard layers): 20
-// steps of 128^3 x 64 64.1 ms, with whole nodes in the box (16 bytes a slot, three
-// blocks of 256) 66.9.  With more guard layers the box takes as many as fit, two at
+// steps of 128^3 x 64 64.1 ms (62.4 since), with whole nodes in the box (16 bytes a
+// slot, three blocks of 256) 66.9.  With more guard layers the box takes as many as fit, two at
 // least: the Penning bunch's (three, of which the box takes two) 10 steps took 49.8
-// ms reading the grid, now 46.9; one block of 768 threads with all three 53.7.
+// ms reading the grid, 46.9 with the box (44.7 since kTileCost); one block of 768 threads with all three 53.7.
 PushShape push_shape(const Geom &g) {
     const size_t tiles = cic::stage_offset(cic::tile_of(g, 0).S);
     for (int eg = g.guard; eg >= std::min(g.guard, 2); --eg) {
