@@ -40,7 +40,7 @@ __device__ __forceinline__ int inst_of_particle(const long long *__restrict__ p0
 
 __global__ void k_b_load(const double *__restrict__ x, const double *__restrict__ v, int64_t m,
                          int64_t base, const InstDesc *__restrict__ desc,
-                         const long long *__restrict__ p0, int n_inst, double dt, Ctrl *ctrl) {
+                         const long long *__restrict__ p0, int n_inst, double half_dt, Ctrl *ctrl) {
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= m) return;
     const int64_t p = base + q;
@@ -51,22 +51,28 @@ __global__ void k_b_load(const double *__restrict__ x, const double *__restrict_
     bool ok = true;
     for (int d = 0; d < 3; ++d) {
         const double vd = v[3 * q + d];
-        double s = (x[3 * q + d] + 0.5 * dt * vd) * D.inv_h_d[d] - 0.5;
+        double s = (x[3 * q + d] + half_dt * vd) * D.inv_h_d[d] - 0.5;
         if (!isfinite(s) || !isfinite(vd) || fabs(s) > 4.0e15) {
             ok = false;
             s = 0.0;
         }
-        const double fl = floor(s);
-        long long il = (long long)fl % D.g.n[d];
-        if (il < 0) il += D.g.n[d];
-        float ff = (float)(s - fl);
+        const FloorRest fr = floor_rest(s);
+        long long il = fr.whole;
+        if ((unsigned long long)il >= (unsigned long long)D.g.n[d]) {   // outside: wrap
+            il += il < 0 ? D.g.n[d] : -D.g.n[d];
+            if ((unsigned long long)il >= (unsigned long long)D.g.n[d]) {   // a box away
+                il %= D.g.n[d];
+                if (il < 0) il += D.g.n[d];
+            }
+        }
+        float ff = fr.rest;
         if (ff >= 1.0f) {
             ff = 0.0f;
             if (++il == D.g.n[d]) il = 0;
         }
         idx[d] = (int)il;
         off[d] = ff;
-        ps.v[d][p] = ok ? (float)vd : 0.0f;
+        ps.v[d][p] = ok ? narrow(vd) : 0.0f;
     }
     if (!ok) atomicOr(&ctrl->flags, PIC_FLAG_NONFINITE);
     ps.cell[p] = pack_cell(idx[0], idx[1], idx[2]);
@@ -476,7 +482,7 @@ cudaError_t launch_b_load(const double *x, const double *v, int64_t m, int64_t b
                           const InstDesc *desc, const long long *p0, int n_inst, double dt,
                           Ctrl *ctrl, LStream st) {
     if (m <= 0) return cudaSuccess;
-    k_b_load<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(x, v, m, base, desc, p0, n_inst, dt, ctrl);
+    k_b_load<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(x, v, m, base, desc, p0, n_inst, 0.5 * dt, ctrl);
     return cudaGetLastError();
 }
 

@@ -35,6 +35,47 @@ __device__ __forceinline__ double widen(float f) {
     return __hiloint2double((int)(((b >> 3) + bias) | sign), (int)(b << 29));
 }
 
+// (float)x, round to nearest with ties to even, by integer instructions; values
+// outside the range of normal floats take the conversion.  (The rare paths here and
+// below are calls: predicated instructions would hold the FP64 units all the same.)
+static __device__ __noinline__ float narrow_any(double x) { return (float)x; }
+__device__ __forceinline__ float narrow(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+    if (b < 0x3810000000000000ull || b >= 0x47E0000000000000ull) return narrow_any(x);
+    const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
+    return __uint_as_float((unsigned)((r >> 29) - 0x1C0000000ull) |
+                           ((unsigned)__double2hiint(x) & 0x80000000u));
+}
+
+// Floor of s and the rest rounded to FP32, for |s| < 2^52.  For 2^-26 <= |s| < 2^10
+// and a rest of at least 2^-17 by integer instructions: s in units of 2^-53, what lies
+// below them kept as the last bit; of the rest's 53 bits the first 23 and the next 23,
+// the last seven as one bit, become floats by their bits and are added exactly, so
+// that it is rounded once.
+struct FloorRest {
+    long long whole;
+    float rest;
+};
+static __device__ __noinline__ FloorRest floor_rest_any(double s) {
+    const double fl = floor(s);
+    return FloorRest{(long long)fl, (float)(s - fl)};
+}
+__device__ __forceinline__ FloorRest floor_rest(double s) {
+    const unsigned es = (unsigned)(__double2hiint(s) >> 20) & 0x7ffu;
+    const unsigned long long m =
+        ((unsigned long long)__double_as_longlong(s) & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int up = min(max((int)es - 1022, -25), 10);   // |s| = m 2^(up - 53)
+    unsigned long long u = m << max(up, 0);
+    if (up < 0) u = (m >> -up) | ((m & ((1ull << -up) - 1ull)) != 0ull);
+    const long long q = __double2hiint(s) < 0 ? -(long long)u : (long long)u;
+    const unsigned hi = (unsigned)((unsigned long long)q >> 30) & 0x7fffffu;
+    const unsigned lo = (unsigned)q & 0x3fffffffu;
+    if (es - (1023u - 26u) >= 36u || hi < 64u) return floor_rest_any(s);
+    const float h = __uint_as_float(0x4b000000u | hi) - 8388608.0f;
+    const float l = __uint_as_float(0x4b000000u | (lo >> 7) | ((lo & 127u) != 0u)) - 8388608.0f;
+    return FloorRest{q >> 53, fmaf(h, 1.1920928955078125e-7f, l * 1.4210854715202004e-14f)};
+}
+
 // i + 1/2 in FP64 for 0 <= i < 2^31: 2^51 + (2 i + 1) / 2 built from its bits
 __device__ __forceinline__ double half_node(int i) {
     return __hiloint2double(0x43200000, 2 * i + 1) - 2251799813685248.0;

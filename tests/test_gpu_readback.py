@@ -104,3 +104,28 @@ def test_ensemble_offsets_come_back_exactly(copies):
     for (n, L, x0, v0, _), x, v in zip(insts, xs, vs):
         assert np.array_equal(x, np.mod(x0, L)) and np.array_equal(v, v0)
     ens.close()
+
+
+@pytest.mark.parametrize("shift", [0, -1, 1, 37, -2**20, 2**30])
+def test_positions_load_exactly(shift):
+    """Unit spacing: nodes plus offsets that FP32 and FP64 both hold, whole boxes away,
+    the first half cell (below node 0) and offsets around 2^-26 included, where the
+    load goes from integer to FP64 instructions."""
+    n = (24, 16, 9)
+    L = np.array(n, dtype=float)
+    tiny = 2.0**-40 if abs(shift) < 2 else 2.0**-12
+    off = np.array([0.0, tiny, 2.0**-26, 2.0**-27, 2.0**-26 * (1 + 2.0**-10), 0.25, 0.5, 1 - 2.0**-12])
+    off = off[off >= tiny] if abs(shift) >= 2 else off
+    r = np.random.default_rng(3)
+    N = 5000
+    idx = np.stack([r.integers(0, m, N) for m in n], 1)
+    x = idx + 0.5 + off[r.integers(0, off.size, idx.shape)] + shift * L
+    x[:10] = [[0.25, 0.5 - 2.0**-20, 2.0**-10]] * 10 + shift * L     # below node 0
+    v = r.standard_normal((N, 3)) * 10.0 ** r.integers(-42, 30, (N, 3))
+    sim = Simulation(n=n, L=L, n_particles=N, dt=0.0 + 1e-300, Q=0.0)
+    sim.load(x, v)
+    xg, vg = sim.particles()
+    v32 = v.astype(np.float32).astype(np.float64)
+    assert np.array_equal(vg, v32)
+    assert np.array_equal(xg, np.mod(x, L))
+    sim.close()
