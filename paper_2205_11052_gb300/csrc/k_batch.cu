@@ -88,9 +88,9 @@ __global__ void k_b_load(const double *__restrict__ x, const double *__restrict_
 // without, one instance's records go out contiguously.
 //
 // Bound by FP64 instructions (about two lanes per clock and SM: the product, the
-// half step back and some wraps; 55 % of their rate) and by DRAM.  With a search
-// per thread and (i + 1/2) + o by FP64 instructions 43M particles took 1.17 ms, now
-// 0.77 (the bytes 0.51).  Blocks of several runs, the next one's records loaded
+// half step back) and by DRAM.  With a search per thread and (i + 1/2) + o by FP64
+// instructions 43M particles took 1.17 ms, without 0.77, and without a wrap for every
+// particle of the last half cell 0.71 (the bytes 0.51).  Blocks of several runs, the next one's records loaded
 // ahead, measured the same.
 __global__ void __launch_bounds__(256) k_b_unload(int64_t o0, int64_t m,
                                                   const InstDesc *__restrict__ desc,
@@ -121,7 +121,9 @@ __global__ void __launch_bounds__(256) k_b_unload(int64_t o0, int64_t m,
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const double vd = widen(w[d]);
-            const double pos = half_node_plus(idx[d], o[d]) * D.h_d[d];
+            // beyond the last half cell at its place below the first node: no wrap
+            const int i = idx[d] == D.g.n[d] - 1 && o[d] >= 0.5f ? -1 : idx[d];
+            const double pos = half_node_plus(i, o[d]) * D.h_d[d];
             sx[3 * threadIdx.x + d] = wrap_position(fma(-half_dt, vd, pos), D.L_d[d]);
             sv[3 * threadIdx.x + d] = vd;
         }

@@ -81,13 +81,14 @@ __device__ __forceinline__ double half_node(int i) {
     return __hiloint2double(0x43200000, 2 * i + 1) - 2251799813685248.0;
 }
 
-// (i + 1/2) + o in FP64 for 0 <= i < 2^10, rounded once.  For 2^-19 <= o < 1 the sum
+// (i + 1/2) + o in FP64 for 0 <= i < 2^10, or i = -1 and o >= 1/2, rounded once.  For 2^-19 <= o < 1 the sum
 // is exact, and an integer in units of 2^-42 below 2^53 gives its bits
 __device__ __forceinline__ double half_node_plus(int i, float o) {
     const unsigned b = __float_as_uint(o), e = b >> 23;
     if (e - 108u >= 19u) return half_node(i) + widen(o);
     const unsigned long long f = ((unsigned long long)(2 * i + 1) << 41) +
                                  ((unsigned long long)((b & 0x7fffffu) | 0x800000u) << (e - 108u));
+    if (f == 0ull) return 0.0;   // i = -1, o = 1/2
     const int z = __clzll((long long)f) - 11;   // to the mantissa's leading bit
     return __longlong_as_double((long long)((f << z) + ((unsigned long long)(1032 - z) << 52)));
 }
