@@ -1067,6 +1067,12 @@ void pic_destroy(pic_handle_t c) {
 
 namespace {
 
+// blocks that read page-locked host particles: enough to fill the link, and SMs left
+// for the binning of the range before.  8M particles loaded, 4 steps and read back
+// with 152 blocks 5.75 ms, 114 5.49, 104 5.47, 76 5.48, 48 5.60; 134M loaded and one
+// step with 152 3.65e9 particles/s, 104 3.71, 76 3.66, 48 3.2
+constexpr int kLinkBlocks = 104;
+
 int load_overlapped(pic_ctx *c, const double *mx, const double *mv, int64_t n) {
     if (!c->side_made) {
         PIC_CUDA(cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking));
@@ -1081,7 +1087,7 @@ int load_overlapped(pic_ctx *c, const double *mx, const double *mv, int64_t n) {
         if (o >= n) break;
         const int64_t m = std::min(per, n - o);
         PIC_CUDA(launch_load(mx + 3 * o, mv + 3 * o, m, o, c->geom, c->inv_h, c->prm.dt, c->ctrl(),
-                             c->st, kNumSMs));
+                             c->st, kLinkBlocks));
         c->launches += 1;
         PIC_CUDA(cudaEventRecord(c->side_ev[k], c->st));
         PIC_CUDA(cudaStreamWaitEvent(c->side, c->side_ev[k], 0));
@@ -1117,7 +1123,7 @@ int pic_load_particles(pic_handle_t c, const double *x, const double *v, int64_t
         PIC_CUDA(launch_load(x, v, n, 0, c->geom, c->inv_h, c->prm.dt, c->ctrl(), c->st));
     } else if (mx && mv && n >= kOverlapMin && presort_passes(c->ntiles) > 0) {
         // page-locked host arrays, read in place by the load kernel one range
-        // at a time on one block per SM (the host link, not the SMs, bounds
+        // at a time on kLinkBlocks blocks (the host link, not the SMs, bounds
         // it); each loaded range is binned on the side stream meanwhile, so
         // the final full-key pass sees tile-ordered runs
         if ((r = load_overlapped(c, mx, mv, n))) return r;
