@@ -101,14 +101,14 @@ __global__ void k_diag_finalize(const double *__restrict__ fpart, int fblocks,
 }  // namespace
 
 namespace {
-// Planar field rows (component d of row r at planar + d * dist + r * pitch) ->
-// the x-paired E8 read by 256-bit loads (the components at q, then those at
+// Field rows (component d of row r from planar + d * dist + r * pitch on, every
+// ES-th float) -> the x-paired E8 read by 256-bit loads (the components at q, then those at
 // its +x neighbour, periodic: Ex Ey Ex' Ey' | Ez Ez' 0 0) and, with SUMS, the
 // block's partial sums of Ex^2, Ey^2, Ez^2 and rho.  Bound by DRAM: 12 bytes read
 // and 32 written per node (16.8M nodes: 163 us; with E4 written too 246 us).  With the interleaving left to the inverse
 // transform (output stride 4: 407 us against 92 planar), a pairing pass (120)
 // and a pass for the sums (81), a 256^3 solve with sums took 0.85 ms.
-template <bool SUMS>
+template <int ES, bool SUMS>
 __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pitch, int64_t dist,
                                                 const float *__restrict__ planar,
                                                 float4 *__restrict__ E8,
@@ -123,9 +123,9 @@ __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pi
         for (int x = lane; x < nx; x += 32) {
             const int x1 = x + 1 == nx ? 0 : x + 1;
             const int64_t q = r * nx + x;
-            const float4 e = make_float4(p0[x], p1[x], p2[x], 0.0f);
-            E8[2 * q] = make_float4(e.x, e.y, p0[x1], p1[x1]);
-            E8[2 * q + 1] = make_float4(e.z, p2[x1], 0.0f, 0.0f);
+            const float4 e = make_float4(p0[ES * x], p1[ES * x], p2[ES * x], 0.0f);
+            E8[2 * q] = make_float4(e.x, e.y, p0[ES * x1], p1[ES * x1]);
+            E8[2 * q + 1] = make_float4(e.z, p2[ES * x1], 0.0f, 0.0f);
             if (SUMS) {
                 ff_add_sq(hi[0], lo[0], e.x);
                 ff_add_sq(hi[1], lo[1], e.y);
@@ -156,13 +156,17 @@ cudaError_t launch_unpair_E(int64_t ng, const float4 *E8, float4 *E4, LStream st
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E8,
-                          float *rho, bool clear_rho, double *part, LStream st) {
+cudaError_t launch_pack_E(const Geom &g, const float *E, bool interleaved, float4 *E8, float *rho,
+                          bool clear_rho, double *part, LStream st) {
     const int64_t rows = (int64_t)g.n[1] * g.n[2];
-    if (part)
-        launch_dep(k_pack_E<true>, kDiagFieldBlocks, 256, 0, st, g.n[0], rows, pitch, dist, planar, E8, rho, clear_rho, part);
-    else
-        launch_dep(k_pack_E<false>, kDiagFieldBlocks, 256, 0, st, g.n[0], rows, pitch, dist, planar, E8, rho, clear_rho, part);
+    const int64_t pitch = interleaved ? 4 * (int64_t)g.n[0] : 2 * (int64_t)g.nh;
+    const int64_t dist = interleaved ? 1 : pitch * rows;
+#define PIC_PACK(ES, SUMS)                                                                          \
+    launch_dep(k_pack_E<ES, SUMS>, kDiagFieldBlocks, 256, 0, st, g.n[0], rows, pitch, dist, E, E8, rho, \
+               clear_rho, part)
+    if (interleaved) { if (part) PIC_PACK(4, true); else PIC_PACK(4, false); }
+    else             { if (part) PIC_PACK(1, true); else PIC_PACK(1, false); }
+#undef PIC_PACK
     return cudaGetLastError();
 }
 

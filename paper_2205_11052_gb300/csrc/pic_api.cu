@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <initializer_list>
 #include <new>
 #include <vector>
 
@@ -49,7 +50,7 @@ size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 // Byte offsets of every device buffer inside the caller's arena.
 struct Layout {
     size_t ctrl, sets, rho, rho64, rho_hat, E_hat, E8, lrho2, bins, scan_tmp, tile_items, tile_range,
-        items, fpart, ppart, ring, inv, stage_x, stage_v, adjE4, ktab, node_pos, fft_tab, fft, total;
+        items, fpart, ppart, ring, inv, stage_x, stage_v, adjE4, ktab, ktab_fft, node_pos, fft_tab, fft, total;
     size_t set_stride;   // bytes of one per-particle array
 };
 
@@ -84,9 +85,8 @@ struct pic_ctx {
     bool bound;
     char *arena;
     LStream st;
-    cufftHandle r2c, c2r;     // rho -> rho^ ; 3 x E^ -> planar E, in place
-    cufftHandle r2c3, c2r1;   // adjoint: lE4 (stride 4) -> 3 x lE^ ; lrho^ -> lrho
-    bool plans;
+    cufftHandle plan[5];      // see make_plan
+    bool planned[5];          // which of them are made
     bool own_fft;             // the field solve runs on k_fft.cu instead of cuFFT
     FftAxis ax[3];
     ParticleSet hsets[2];     // host copies of the device set descriptors
@@ -142,56 +142,58 @@ int fft_dims(const pic_ctx *c, long long *n, long long *nin, long long *npad) {
     return r;
 }
 
-// The four transforms: rho -> rho^ (R2C), 3 x E^ -> planar E in its place (C2R,
-// batch 3, rows padded to their half spectra), lE4 -> 3 x lE^ (R2C, batch 3, input stride 4), lrho^ -> lrho (C2R).
-int make_plans(pic_ctx *c, bool estimate_only, size_t *ws_max) {
+// The transforms: rho -> rho^ (R2C), 3 x E^ -> planar E in its place (C2R, batch 3,
+// rows padded to their half spectra), lE4 -> 3 x lE^ (R2C, batch 3, input stride 4),
+// lrho^ -> lrho (C2R), 3 x E^ -> E4 (C2R, batch 3, output stride 4).
+enum { kR2C, kC2R, kR2C3, kC2R1, kC2R4, kPlans };
+cufftResult make_plan(const pic_ctx *c, int which, bool estimate_only, cufftHandle *p, size_t *ws) {
     long long n[3], nh[3], npad[3];
     const int rank = fft_dims(c, n, nh, npad);
-    cufftHandle p[4] = {0, 0, 0, 0};
-    size_t ws[4] = {0, 0, 0, 0};
-    cufftResult r = CUFFT_SUCCESS;
-    int made = 0;
-    for (; made < 4 && r == CUFFT_SUCCESS; ++made) {
-        r = cufftCreate(&p[made]);
-        if (r != CUFFT_SUCCESS) break;
-        cufftSetAutoAllocation(p[made], 0);
-    }
-    auto plan = [&](int q, long long *inembed, long long istride, long long idist,
-                    long long *onembed, long long ostride, long long odist, cufftType t,
-                    long long batch) {
+    cufftResult r = cufftCreate(p);
+    if (r != CUFFT_SUCCESS) return r;
+    cufftSetAutoAllocation(*p, 0);
+    auto plan = [&](long long *inembed, long long istride, long long idist, long long *onembed,
+                    long long ostride, long long odist, cufftType t, long long batch) {
         if (estimate_only)
-            return cufftGetSizeMany64(p[q], rank, n, inembed, istride, idist, onembed, ostride,
-                                      odist, t, batch, &ws[q]);
-        return cufftMakePlanMany64(p[q], rank, n, inembed, istride, idist, onembed, ostride, odist,
-                                   t, batch, &ws[q]);
+            return cufftGetSizeMany64(*p, rank, n, inembed, istride, idist, onembed, ostride, odist, t,
+                                      batch, ws);
+        return cufftMakePlanMany64(*p, rank, n, inembed, istride, idist, onembed, ostride, odist, t,
+                                   batch, ws);
     };
-    if (r == CUFFT_SUCCESS) r = plan(0, nullptr, 1, 0, nullptr, 1, 0, CUFFT_R2C, 1);
-    if (r == CUFFT_SUCCESS) r = plan(1, nh, 1, c->nhalf, npad, 1, 2 * c->nhalf, CUFFT_C2R, 3);
-    if (r == CUFFT_SUCCESS) r = plan(2, n, 4, 1, nh, 1, c->nhalf, CUFFT_R2C, 3);
-    if (r == CUFFT_SUCCESS) r = plan(3, nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 1);
-    if (r != CUFFT_SUCCESS || estimate_only) {
-        for (int q = 0; q < made && q < 4; ++q)
-            if (p[q]) cufftDestroy(p[q]);
-        if (r != CUFFT_SUCCESS) return fail(PIC_ERR_CUFFT, "cuFFT plan setup failed: %d", (int)r);
-        *ws_max = std::max(std::max(ws[0], ws[1]), std::max(ws[2], ws[3]));
-        return PIC_OK;
+    switch (which) {
+    case kR2C: r = plan(nullptr, 1, 0, nullptr, 1, 0, CUFFT_R2C, 1); break;
+    case kC2R: r = plan(nh, 1, c->nhalf, npad, 1, 2 * c->nhalf, CUFFT_C2R, 3); break;
+    case kR2C3: r = plan(n, 4, 1, nh, 1, c->nhalf, CUFFT_R2C, 3); break;
+    case kC2R1: r = plan(nullptr, 1, 0, nullptr, 1, 0, CUFFT_C2R, 1); break;
+    case kC2R4: r = plan(nh, 1, c->nhalf, n, 4, 1, CUFFT_C2R, 3); break;
     }
-    c->r2c = p[0];
-    c->c2r = p[1];
-    c->r2c3 = p[2];
-    c->c2r1 = p[3];
-    c->plans = true;
-    *ws_max = std::max(std::max(ws[0], ws[1]), std::max(ws[2], ws[3]));
+    if (r != CUFFT_SUCCESS || estimate_only) cufftDestroy(*p);
+    return r;
+}
+
+// Makes the plans of `which` that are not there yet, on the handle's work area and stream
+int make_plans(pic_ctx *c, std::initializer_list<int> which) {
+    for (int q : which) {
+        if (c->planned[q]) continue;
+        size_t ws = 0;
+        cufftResult r = make_plan(c, q, false, &c->plan[q], &ws);
+        if (r != CUFFT_SUCCESS) return fail(PIC_ERR_CUFFT, "cuFFT plan setup failed: %d", (int)r);
+        if (ws > c->fft_reserve) {
+            cufftDestroy(c->plan[q]);
+            return fail(PIC_ERR_CAPACITY, "cuFFT needs %zu work bytes, %zu reserved", ws, c->fft_reserve);
+        }
+        c->planned[q] = true;
+        PIC_CUFFT(cufftSetWorkArea(c->plan[q], c->arena + c->lay.fft));
+        PIC_CUFFT(cufftSetStream(c->plan[q], c->st));
+    }
     return PIC_OK;
 }
 
 void destroy_plans(pic_ctx *c) {
-    if (!c->plans) return;
-    cufftDestroy(c->r2c);
-    cufftDestroy(c->c2r);
-    cufftDestroy(c->r2c3);
-    cufftDestroy(c->c2r1);
-    c->plans = false;
+    for (int q = 0; q < kPlans; ++q) {
+        if (c->planned[q]) cufftDestroy(c->plan[q]);
+        c->planned[q] = false;
+    }
 }
 
 // the work items and their ranks before them
@@ -228,7 +230,8 @@ void compute_layout(pic_ctx *c) {
     L.stage_v = take((size_t)c->staging * 24);
     L.adjE4 = take((size_t)c->ng * 16);
     L.lrho2 = take((size_t)c->ng * 8);
-    L.ktab = take((size_t)fft_ktab_size(c->geom) * 4);
+    L.ktab = take((size_t)(c->geom.nh + c->grid.n[1] + c->grid.n[2]) * 4);
+    L.ktab_fft = take(c->own_fft ? (size_t)fft_ktab_size(c->geom) * 4 : 0);
     L.node_pos = take((size_t)3 * kMaxN * 8);
     L.fft_tab = take(sizeof(FftTables));
     L.fft = take(c->fft_reserve);
@@ -388,24 +391,35 @@ bool fp32_rho(const pic_ctx *c) { return !(c->prm.options & PIC_OPT_FIXED_DEPOSI
 // sums: also leave the partial field sums of the diagnostics; clear_rho: leave rho
 // cleared for the push of the step
 // (E8: where the field goes, by default the run's own array)
-int do_solve(pic_ctx *c, bool sums = false, bool clear_rho = false, float4 *E8 = nullptr) {
+//
+// sweep: a solve of pic_adjoint_forward or of a segment recomputed from a checkpoint.
+// These go through cuFFT on every grid, the field interleaved by the transform (in
+// adjE4, which is scratch then): the derivative of the cloud-in-cell weights jumps
+// where a particle crosses a cell face, and the last step's deposit enters the
+// gradient without a factor dt, so the components of a particle that sits on a face
+// there hang on the last bit of E.  4.2M particles on 64^3 nodes have a few such; with
+// the solve by k_fft.cu, as exact but rounded otherwise, one of them moved a gradient
+// by 0.13 of the largest (2e-4 in the mean square).  That gradient of 20 steps takes
+// 11.5 ms, with k_fft.cu 11.2 (12 steps in a 24^3 trap 2.3 and 2.1).
+int do_solve(pic_ctx *c, bool sums = false, bool clear_rho = false, float4 *E8 = nullptr,
+             bool sweep = false) {
     if (!E8) E8 = c->at<float4>(c->lay.E8);
     int r = timer_begin(c, PIC_PHASE_SOLVE);
     if (r) return r;
-    if (c->own_fft) {
+    if (c->own_fft && !sweep) {
         PIC_CUDA(launch_fft_solve(c->geom, 1, c->ax, c->at<FftTables>(c->lay.fft_tab),
-                                  c->at<float>(c->lay.ktab), c->at<float>(c->lay.rho), clear_rho,
+                                  c->at<float>(c->lay.ktab_fft), c->at<float>(c->lay.rho), clear_rho,
                                   c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat), c->nhalf,
                                   c->mode_pos, c->prm.mode_comp, c->mode_conj, c->ctrl()->mode,
                                   nullptr, E8, sums ? c->at<double>(c->lay.fpart) : nullptr, 0, c->st));
         return timer_end(c, PIC_PHASE_SOLVE, 3);
     }
-    PIC_CUFFT(cufftExecR2C(c->r2c, c->at<cufftReal>(c->lay.rho), c->at<cufftComplex>(c->lay.rho_hat)));
+    PIC_CUFFT(cufftExecR2C(c->plan[kR2C], c->at<cufftReal>(c->lay.rho), c->at<cufftComplex>(c->lay.rho_hat)));
     PIC_CUDA(launch_green(c->geom, c->at<float>(c->lay.ktab), c->at<float2>(c->lay.rho_hat), c->at<float2>(c->lay.E_hat),
                           c->nhalf, c->mode_idx, c->prm.mode_comp, c->mode_conj, c->ctrl(), c->st));
-    PIC_CUFFT(cufftExecC2R(c->c2r, c->at<cufftComplex>(c->lay.E_hat), c->at<cufftReal>(c->lay.E_hat)));
-    PIC_CUDA(launch_pack_E(c->geom, c->at<float>(c->lay.E_hat), 2 * (int64_t)c->geom.nh, 2 * c->nhalf,
-                           E8, c->at<float>(c->lay.rho), clear_rho,
+    float *out = c->at<float>(sweep ? c->lay.adjE4 : c->lay.E_hat);
+    PIC_CUFFT(cufftExecC2R(c->plan[sweep ? kC2R4 : kC2R], c->at<cufftComplex>(c->lay.E_hat), out));
+    PIC_CUDA(launch_pack_E(c->geom, out, sweep, E8, c->at<float>(c->lay.rho), clear_rho,
                            sums ? c->at<double>(c->lay.fpart) : nullptr, c->st));
     return timer_end(c, PIC_PHASE_SOLVE, 2);
 }
@@ -751,7 +765,7 @@ int adj_keep_step(pic_ctx *c, const AdjLayout &L, int seg, int a0, int n, int *c
     }
     if (!c->rho_current && (r = do_deposit(c))) return r;
     float4 *E8 = adj_field(c, L, n - a0);
-    if ((r = do_solve(c, false, fp32_rho(c), E8))) return r;
+    if ((r = do_solve(c, false, fp32_rho(c), E8, true))) return r;
     if (c->np == 0) return do_push_deposit(c, false, SaveY{}, E8);
     // y_n is written by the push that reads it
     char *y[7];
@@ -768,15 +782,15 @@ int adj_keep_step(pic_ctx *c, const AdjLayout &L, int seg, int a0, int n, int *c
 int adj_solve(pic_ctx *c, int par) {
     if (c->own_fft) {
         PIC_CUDA(launch_fft_adj_solve(c->geom, c->ax, c->at<FftTables>(c->lay.fft_tab),
-                                      c->at<float>(c->lay.ktab), c->at<float4>(c->lay.adjE4),
+                                      c->at<float>(c->lay.ktab_fft), c->at<float4>(c->lay.adjE4),
                                       c->at<float2>(c->lay.E_hat), c->at<float2>(c->lay.rho_hat), c->nhalf,
                                       c->at<float2>(c->lay.lrho2), c->ctrl(), par, c->st));
         return PIC_OK;
     }
-    PIC_CUFFT(cufftExecR2C(c->r2c3, c->at<cufftReal>(c->lay.adjE4), c->at<cufftComplex>(c->lay.E_hat)));
+    PIC_CUFFT(cufftExecR2C(c->plan[kR2C3], c->at<cufftReal>(c->lay.adjE4), c->at<cufftComplex>(c->lay.E_hat)));
     PIC_CUDA(launch_green_adj(c->geom, c->L, c->at<float2>(c->lay.E_hat),
                               c->at<float2>(c->lay.rho_hat), c->nhalf, c->st));
-    PIC_CUFFT(cufftExecC2R(c->c2r1, c->at<cufftComplex>(c->lay.rho_hat), c->at<cufftReal>(c->lay.rho)));
+    PIC_CUFFT(cufftExecC2R(c->plan[kC2R1], c->at<cufftComplex>(c->lay.rho_hat), c->at<cufftReal>(c->lay.rho)));
     PIC_CUDA(launch_adj_pair_rho(c->geom, c->at<float>(c->lay.rho), c->at<float2>(c->lay.lrho2),
                                  c->at<float4>(c->lay.adjE4), c->ctrl(), par, c->st));
     return PIC_OK;
@@ -942,15 +956,19 @@ int pic_create(const pic_grid_t *grid, const pic_species_t *species, const pic_p
     c->mode_idx[2] = ((m[2] % grid->n[2]) + grid->n[2]) % grid->n[2];
 
     c->own_fft = fft_supported(g, c->ax);
-    c->fft_reserve = 0;
-    if (!c->own_fft) {
-        // cuFFT work area: the library's own size query when it works here,
-        // never less than a conservative bound
-        size_t wmax = 0;
-        size_t bound = (size_t)c->nhalf * 8 * 3 + ((size_t)4 << 20);
-        if (make_plans(c, true, &wmax) == PIC_OK) bound = std::max(bound, wmax);
-        c->fft_reserve = bound;
-    }
+    // cuFFT work area.  The two transforms of a gradient sweep on a grid of k_fft.cu
+    // take at most 32 bytes a node and a kilobyte (x lengths of 75; 18 thousand grids
+    // asked); on others never less than a conservative bound, and the library's own
+    // size query when it works here
+    c->fft_reserve = c->own_fft ? (size_t)c->ng * 32 + ((size_t)64 << 10)
+                                : (size_t)c->nhalf * 8 * 3 + ((size_t)4 << 20);
+    if (!c->own_fft)
+        for (int q = 0; q < kPlans; ++q) {
+            cufftHandle p;
+            size_t ws = 0;
+            if (make_plan(c, q, true, &p, &ws) != CUFFT_SUCCESS) break;
+            c->fft_reserve = std::max(c->fft_reserve, ws);
+        }
     compute_layout(c);
     *out = c;
     snprintf(g_err, sizeof(g_err), "no error");
@@ -978,30 +996,22 @@ int pic_bind_workspace(pic_handle_t c, void *arena, size_t bytes, void *stream) 
     c->adj.ready = false;
     c->arena = static_cast<char *>(arena);
     c->st = static_cast<cudaStream_t>(stream);
-    std::vector<float> ktab((size_t)fft_ktab_size(c->geom));
+    if (!c->own_fft) {   // kC2R4: by the first gradient sweep
+        const int r = make_plans(c, {kR2C, kC2R, kR2C3, kC2R1});
+        if (r) return r;
+    }
     if (c->own_fft) {
         FftTables tab{};
         fft_tables(c->ax, tab);
         PIC_CUDA(fft_prepare());
         PIC_CUDA(cudaMemcpyAsync(c->at<FftTables>(c->lay.fft_tab), &tab, sizeof(tab),
                                  cudaMemcpyHostToDevice, c->st));
-        fft_ktab(c->geom, c->L, tab, ktab.data());
+        std::vector<float> k((size_t)fft_ktab_size(c->geom));
+        fft_ktab(c->geom, c->L, tab, k.data());
+        PIC_CUDA(cudaMemcpyAsync(c->at<float>(c->lay.ktab_fft), k.data(), k.size() * 4,
+                                 cudaMemcpyHostToDevice, c->st));
         for (int d = 0; d < 3; ++d) c->mode_pos[d] = d == 0 ? c->mode_idx[0] : tab.pos[d][c->mode_idx[d]];
         PIC_CUDA(cudaStreamSynchronize(c->st));
-    } else {
-        size_t wmax = 0;
-        int r = make_plans(c, false, &wmax);
-        if (r) return r;
-        if (wmax > c->fft_reserve) {
-            destroy_plans(c);
-            return fail(PIC_ERR_CAPACITY, "cuFFT needs %zu work bytes, %zu reserved", wmax,
-                        c->fft_reserve);
-        }
-        void *work = c->arena + c->lay.fft;
-        for (cufftHandle p : {c->r2c, c->c2r, c->r2c3, c->c2r1}) {
-            PIC_CUFFT(cufftSetWorkArea(p, work));
-            PIC_CUFFT(cufftSetStream(p, c->st));
-        }
     }
 
     PIC_CUDA(sort_prepare());
@@ -1021,7 +1031,8 @@ int pic_bind_workspace(pic_handle_t c, void *arena, size_t bytes, void *stream) 
     c->hsets[0] = h.sets[0];
     c->hsets[1] = h.sets[1];
     PIC_CUDA(cudaMemcpyAsync(c->ctrl(), &h, sizeof(h), cudaMemcpyHostToDevice, c->st));
-    if (!c->own_fft) green_table(c->geom, c->L, ktab.data());
+    std::vector<float> ktab((size_t)(c->geom.nh + c->grid.n[1] + c->grid.n[2]));
+    green_table(c->geom, c->L, ktab.data());
     PIC_CUDA(cudaMemcpyAsync(c->at<float>(c->lay.ktab), ktab.data(), ktab.size() * 4,
                              cudaMemcpyHostToDevice, c->st));
     std::vector<double> npos((size_t)3 * kMaxN);
@@ -1046,8 +1057,8 @@ int pic_set_stream(pic_handle_t c, void *stream) {
     int r = check_ready(c);
     if (r) return r;
     c->st = static_cast<cudaStream_t>(stream);
-    if (c->plans)
-        for (cufftHandle p : {c->r2c, c->c2r, c->r2c3, c->c2r1}) PIC_CUFFT(cufftSetStream(p, c->st));
+    for (int q = 0; q < kPlans; ++q)
+        if (c->planned[q]) PIC_CUFFT(cufftSetStream(c->plan[q], c->st));
     return PIC_OK;
 }
 
@@ -1347,6 +1358,7 @@ int pic_adjoint_forward(pic_handle_t c, int n_steps, int K, const double *w, voi
     const AdjLayout L = adj_layout(c, n_steps, K);
     if (bytes < L.total)
         return fail(PIC_ERR_CAPACITY, "adjoint buffer of %zu bytes < required %zu", bytes, L.total);
+    if ((r = make_plans(c, {kR2C, kC2R4}))) return r;
     const DepScope dep(c->st, c->np <= kDepMaxParticles);
     PIC_CUDA(cudaStreamSynchronize(c->st));
     int32_t cur = 0;
@@ -1377,13 +1389,14 @@ int pic_adjoint_forward(pic_handle_t c, int n_steps, int K, const double *w, voi
             }
             if (n > a0 && (n - a0) % L.R == 0 && (r = adj_rebin(c, &cur))) return r;
             if (!c->rho_current && (r = do_deposit(c))) return r;
-            if ((r = do_solve(c, false, fp32_rho(c))) || (r = do_push_deposit(c, false))) return r;
+            if ((r = do_solve(c, false, fp32_rho(c), nullptr, true)) || (r = do_push_deposit(c, false)))
+                return r;
         }
     }
     c->adj.cur_end = cur;
     if (!c->rho_current && (r = do_deposit(c))) return r;
-    if ((r = do_solve(c, true))) return r;
-    PIC_CUDA(launch_objective(c->at<double>(c->lay.fpart), field_blocks_of(c), c->dV, c->adj.w,
+    if ((r = do_solve(c, true, false, nullptr, true))) return r;
+    PIC_CUDA(launch_objective(c->at<double>(c->lay.fpart), kDiagFieldBlocks, c->dV, c->adj.w,
                               &c->ctrl()->scalar[0], c->st));
     PIC_CUDA(cudaMemcpyAsync(J, &c->ctrl()->scalar[0], sizeof(double), cudaMemcpyDeviceToHost, c->st));
     PIC_CUDA(cudaStreamSynchronize(c->st));
@@ -1447,6 +1460,8 @@ int pic_adjoint_backward(pic_handle_t c, double scale, double *gx, double *gv, i
             c->rho_current = false;
             for (int n = a0; n < b0; ++n)
                 if ((r = adj_keep_step(c, L, s, a0, n, &cur))) return r;
+            // the solves went through lE4, which a reverse push adds to
+            PIC_CUDA(cudaMemsetAsync(lE4, 0, (size_t)c->ng * 16, c->st));
             const int32_t *pid_next =
                 reinterpret_cast<const int32_t *>(order_rec(c, L, s + 1, 0).pid);
             if ((r = adj_permute_from_backup(c, L, cur, pid_next, c->hsets[cur].pid))) return r;

@@ -370,11 +370,11 @@ cudaError_t launch_push_deposit(const Geom &g, const PushConst &pc, bool diag, b
 cudaError_t launch_gather_push(int64_t n, const Geom &g, const PushConst &pc, bool diag,
                                Ctrl *ctrl, const float4 *E8, double *part, int blocks,
                                int threads, LStream st);
-// planar E (component d of row r at planar + d * dist + r * pitch) -> the x-paired
-// E8 (Ex Ey Ex' Ey' Ez Ez' 0 0 per node, primed at q + x, periodic),
+// E as cuFFT left it, one float4 per node (interleaved) or planar in the place of its
+// spectra, -> the x-paired E8 (Ex Ey Ex' Ey' Ez Ez' 0 0 per node, primed at q + x, periodic),
 // and unless null the partial field sums of kDiagFieldBlocks blocks
-cudaError_t launch_pack_E(const Geom &g, const float *planar, int64_t pitch, int64_t dist, float4 *E8,
-                          float *rho, bool clear_rho, double *part, LStream st);
+cudaError_t launch_pack_E(const Geom &g, const float *E, bool interleaved, float4 *E8, float *rho,
+                          bool clear_rho, double *part, LStream st);
 // E8 -> (Ex, Ey, Ez, 0) per node
 cudaError_t launch_unpair_E(int64_t ng, const float4 *E8, float4 *E4, LStream st);
 
