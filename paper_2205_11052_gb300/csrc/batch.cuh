@@ -2,6 +2,7 @@
 // k_batch.cu (internal; the C ABI is in pic.h).
 #pragma once
 
+#include "ffsum.cuh"
 #include "pic_internal.cuh"
 
 namespace pic {
@@ -20,7 +21,7 @@ struct InstDesc {
     int tile0, ntiles;         // its global tile ids: [tile0, tile0 + ntiles)
     float qscale;              // q_p / h^3
     double mp, dV;             // for the reductions
-    float fix_hi, fix_lo;      // qscale / 2^20 as an FP32 pair (fixed_density)
+    FixedScale fix;            // qscale / 2^20 (fixed_density)
     double inv_h_d[3], h_d[3], L_d[3], two_pi_over_L[3];
     double inv_ng;             // 1 / N_g (folded into the Green kernel)
     int mode_idx[3], mode_comp, mode_conj;

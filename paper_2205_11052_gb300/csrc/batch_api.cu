@@ -393,9 +393,7 @@ int pic_batch_create(const pic_instance_t *inst, int n_inst, double q_over_m,
             D.dV = D.h_d[0] * D.h_d[1] * D.h_d[2];
             const double qp = I.n_particles > 0 ? I.total_charge / (double)I.n_particles : 0.0;
             D.qscale = (float)(qp / D.dV);
-            const double fix = qp / D.dV * (1.0 / (double)cic::kFixOne);
-            D.fix_hi = (float)fix;
-            D.fix_lo = (float)(fix - (double)D.fix_hi);
+            D.fix = fixed_scale(qp / D.dV * (1.0 / (double)cic::kFixOne));
             D.mp = qp / q_over_m;
             D.inv_ng = 1.0 / (double)c.ng;
             int m[3] = {b->prm.mode[0], b->prm.mode[1], b->prm.mode[2]};

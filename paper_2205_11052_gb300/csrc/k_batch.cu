@@ -332,7 +332,7 @@ __global__ void k_b_rho_finish(int64_t ng, const InstDesc *__restrict__ desc,
     int inst = 0;
     for (int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gidx < ng; gidx += stride) {
         inst = inst_of_particle(g0, n_inst, gidx);
-        rho[gidx] = fixed_density(rho64[gidx], desc[inst].fix_hi, desc[inst].fix_lo);
+        rho[gidx] = fixed_density(rho64[gidx], desc[inst].fix);
         rho64[gidx] = 0ull;
     }
 }

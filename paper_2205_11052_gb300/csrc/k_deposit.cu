@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
 // two nodes per thread and iteration (16-byte loads and stores of the 8-byte
 // words, 8-byte stores of the densities), the odd last node by thread 0
 __global__ void __launch_bounds__(256) k_rho_finish(int64_t ng, unsigned long long *__restrict__ rho64,
-                                                    float *__restrict__ rho, float sh, float sl) {
+                                                    float *__restrict__ rho, FixedScale f) {
     dep_begin();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t n2 = ng >> 1;
@@ -130,11 +130,11 @@ __global__ void __launch_bounds__(256) k_rho_finish(int64_t ng, unsigned long lo
     float2 *f2 = reinterpret_cast<float2 *>(rho);
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n2; q += stride) {
         const ulonglong2 v = __ldcs(r2 + q);
-        __stcs(f2 + q, make_float2(fixed_density(v.x, sh, sl), fixed_density(v.y, sh, sl)));
+        __stcs(f2 + q, make_float2(fixed_density(v.x, f), fixed_density(v.y, f)));
         __stcs(r2 + q, make_ulonglong2(0ull, 0ull));
     }
     if ((ng & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
-        rho[ng - 1] = fixed_density(rho64[ng - 1], sh, sl);
+        rho[ng - 1] = fixed_density(rho64[ng - 1], f);
         rho64[ng - 1] = 0ull;
     }
 }
@@ -145,9 +145,7 @@ cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *r
                               LStream st) {
     const int64_t ng = (int64_t)g.n[0] * g.n[1] * g.n[2];
     const int fb = (int)std::max<int64_t>(1, std::min<int64_t>((ng / 2 + 255) / 256, 152 * 8));
-    const double scale = qscale / (double)kFixOne;
-    const float sh = (float)scale, sl = (float)(scale - (double)sh);
-    launch_dep(k_rho_finish, fb, 256, 0, st, ng, rho64, rho, sh, sl);
+    launch_dep(k_rho_finish, fb, 256, 0, st, ng, rho64, rho, fixed_scale(qscale / (double)kFixOne));
     return cudaGetLastError();
 }
 
