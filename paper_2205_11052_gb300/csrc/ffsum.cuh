@@ -3,6 +3,8 @@
 // this part), shared by the single-run and the batched reductions.
 #pragma once
 
+#include "records.cuh"
+
 namespace pic {
 
 // (hi, lo) += a, with the rounding error of the FP32 sum (Knuth's TwoSum,
@@ -50,49 +52,27 @@ __device__ __forceinline__ void block_field_sums(float (&hi)[4], float (&lo)[4],
     }
 }
 
-// A factor in FP64 and as an FP32 pair
+// A factor and what a product with it and 2^52 + q is off by
 struct FixedScale {
-    double s;
-    float hi, lo;
+    double s, off;
 };
 inline FixedScale fixed_scale(double s) {
-    const float hi = (float)s;
-    return FixedScale{s, hi, (float)(s - (double)hi)};
-}
-// (not inlined: see records.cuh)
-static __device__ __noinline__ float fixed_density_any(unsigned long long q, double s) {
-    return (float)((double)(long long)q * s);
+    const double most = 8.4527e270;   // beyond FP32's range with any q but 0, 2^52 s within FP64's
+    if (s > most) s = most;
+    if (s < -most) s = -most;
+    return FixedScale{s, -4503599627370496.0 * s};
 }
 
-// Fixed-point sum q (below 2^63) times a scale, the FP64 product rounded to FP32.  By
-// FP32: q is split into three exactly converted parts whose sum and product carry
-// their rounding errors, which gives the product within 2^-20 units in the last place
-// beside the rounded result and what that leaves over.  Results closer than 5e-6 units to
-// halfway between two floats, powers of two and the smallest and largest exponents
-// take the FP64 product (three FP64 instructions for every node bound the conversion
-// of a grid: 16.8M nodes took 92.7 us, without any 48.5, as here).
+// Fixed-point sum q (below 2^52: 2^31 particles of 2^20 units fit) times a scale, the
+// FP64 product rounded to FP32.  q's bits below an exponent of 2^52 are 2^52 + q, so one
+// fused multiply-add gives the product, and the rounding is integer instructions: FP64
+// ones run at about two lanes per clock and SM, and with three of them a node (a
+// conversion, the product, a conversion) they bound the conversion of a grid: 16.8M
+// nodes 92.7 us, now 55.8 (their bytes 50).
 __device__ __forceinline__ float fixed_density(unsigned long long q, const FixedScale &f) {
-    constexpr float kMagic = 8388608.0f;   // 2^23: its mantissa bits hold an integer
-    auto part = [](unsigned int v) { return __fsub_rn(__uint_as_float(0x4B000000u | v), kMagic); };
-    const float a = part((unsigned int)(q >> 40)) * 1099511627776.0f;
-    const float b = part((unsigned int)(q >> 20) & 0xFFFFFu) * 1048576.0f;
-    const float c = part((unsigned int)q & 0xFFFFFu);
-    const float ab = __fadd_rn(a, b);
-    float lo = __fsub_rn(b, __fsub_rn(ab, a));
-    const float t = __fadd_rn(ab, c);
-    lo = __fadd_rn(lo, __fsub_rn(c, __fsub_rn(t, ab)));
-    const float p = __fmul_rn(t, f.hi);
-    float e = __fmaf_rn(t, f.hi, -p);
-    e = __fmaf_rn(t, f.lo, e);
-    e = __fmaf_rn(lo, f.hi, e);
-    const float r = __fadd_rn(p, e);
-    const float rest = __fsub_rn(e, __fsub_rn(r, p));
-    const unsigned int bits = __float_as_uint(r) & 0x7fffffffu;
-    const float half = __uint_as_float((bits & 0x7f800000u) - (24u << 23));   // of r's last place
-    const bool sure = fabsf(rest) < 0.99999f * half && (bits & 0x7fffffu) != 0u &&
-                      bits - (64u << 23) < (184u << 23);
-    if (q == 0ull) return p;
-    return sure ? r : fixed_density_any(q, f.s);
+    const double d = fma(__longlong_as_double((long long)(q | 0x4330000000000000ull)), f.s, f.off);
+    if (q == 0ull) return __uint_as_float((unsigned)__double2hiint(f.s) & 0x80000000u);   // 0 s
+    return narrow(d);
 }
 
 }  // namespace pic

@@ -128,10 +128,17 @@ __global__ void __launch_bounds__(256) k_rho_finish(int64_t ng, unsigned long lo
     const int64_t n2 = ng >> 1;
     ulonglong2 *r2 = reinterpret_cast<ulonglong2 *>(rho64);
     float2 *f2 = reinterpret_cast<float2 *>(rho);
-    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n2; q += stride) {
+    // two loads in flight
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n2; q += 2 * stride) {
+        const bool two = q + stride < n2;
         const ulonglong2 v = __ldcs(r2 + q);
+        const ulonglong2 w = two ? __ldcs(r2 + q + stride) : make_ulonglong2(0ull, 0ull);
         __stcs(f2 + q, make_float2(fixed_density(v.x, f), fixed_density(v.y, f)));
         __stcs(r2 + q, make_ulonglong2(0ull, 0ull));
+        if (two) {
+            __stcs(f2 + q + stride, make_float2(fixed_density(w.x, f), fixed_density(w.y, f)));
+            __stcs(r2 + q + stride, make_ulonglong2(0ull, 0ull));
+        }
     }
     if ((ng & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
         rho[ng - 1] = fixed_density(rho64[ng - 1], f);
