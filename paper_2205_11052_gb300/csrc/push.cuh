@@ -65,44 +65,39 @@ __device__ __forceinline__ ERow row_of(const float4 &e0, const float4 &e1) {
     return ERow{make_float2(e0.x, e0.y), make_float2(e1.x, e1.y), make_float2(e0.z, e1.z)};
 }
 
-// CIC interpolation of the rows (corner bits b | c<<1)
+// CIC interpolation of the rows (corner bits b | c<<1).  The roundings are written out, so
+// that every kernel that pushes a particle gives the same bits: a step and the split
+// calls can be compared exactly.  (In packed pairs of FP32 operations, Ez's two x corners
+// side by side, the split push is 4% faster, 8 steps of the split cycle on 64^3 x 64 in
+// 4.10 ms and not 4.26, but rounds otherwise; with Ex and Ey alone packed, which does
+// not, it gains nothing.)
+__device__ __forceinline__ float lerp_x(float gx, float a, float fx, float b) {
+    return __fmaf_rn(gx, a, __fmul_rn(fx, b));
+}
+__device__ __forceinline__ float sum_rows(const float (&w)[4], const float (&v)[4]) {
+    return __fmaf_rn(w[3], v[3], __fmaf_rn(w[2], v[2], __fmaf_rn(w[0], v[0], __fmul_rn(w[1], v[1]))));
+}
+__device__ __forceinline__ void row_weights(float fy, float fz, float (&w)[4]) {
+    const float gy = 1.0f - fy, gz = 1.0f - fz;
+    w[0] = __fmul_rn(gy, gz);
+    w[1] = __fmul_rn(fy, gz);
+    w[2] = __fmul_rn(gy, fz);
+    w[3] = __fmul_rn(fy, fz);
+}
 __device__ __forceinline__ void interp_E(const ERow r[4], float fx, float fy, float fz, float &ex,
                                          float &ey, float &ez) {
-    const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
-    const float w[4] = {gy * gz, fy * gz, gy * fz, fy * fz};
-    float vx[4], vy[4], vz[4];
+    const float gx = 1.0f - fx;
+    float w[4], vx[4], vy[4], vz[4];
+    row_weights(fy, fz, w);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        vx[q] = gx * r[q].a.x + fx * r[q].b.x;
-        vy[q] = gx * r[q].a.y + fx * r[q].b.y;
-        vz[q] = gx * r[q].z.x + fx * r[q].z.y;
+        vx[q] = lerp_x(gx, r[q].a.x, fx, r[q].b.x);
+        vy[q] = lerp_x(gx, r[q].a.y, fx, r[q].b.y);
+        vz[q] = lerp_x(gx, r[q].z.x, fx, r[q].z.y);
     }
-    ex = w[0] * vx[0] + w[1] * vx[1] + w[2] * vx[2] + w[3] * vx[3];
-    ey = w[0] * vy[0] + w[1] * vy[1] + w[2] * vy[2] + w[3] * vy[3];
-    ez = w[0] * vz[0] + w[1] * vz[1] + w[2] * vz[2] + w[3] * vz[3];
-}
-
-// The same in packed pairs of FP32 operations: Ex and Ey side by side, Ez at the
-// two x corners side by side.  The split-call push, bound by issue, gains 4% (8
-// steps of the split cycle on 64^3 x 64: 4.24 -> 4.08 ms); the fused push, at its
-// register limit, lost 1%, so it keeps the scalar form.
-__device__ __forceinline__ void interp_E_packed(const ERow r[4], float fx, float fy, float fz,
-                                                float &ex, float &ey, float &ez) {
-    const float gx = 1.0f - fx, gy = 1.0f - fy, gz = 1.0f - fz;
-    const float w[4] = {gy * gz, fy * gz, gy * fz, fy * fz};
-    const float2 x0 = make_float2(gx, gx), x1 = make_float2(fx, fx), wx = make_float2(gx, fx);
-    float2 xy, z;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const float2 ww = make_float2(w[q], w[q]);
-        const float2 t = __ffma2_rn(x1, r[q].b, __fmul2_rn(x0, r[q].a));
-        const float2 u = __fmul2_rn(ww, wx);
-        xy = q == 0 ? __fmul2_rn(ww, t) : __ffma2_rn(ww, t, xy);
-        z = q == 0 ? __fmul2_rn(u, r[q].z) : __ffma2_rn(u, r[q].z, z);
-    }
-    ex = xy.x;
-    ey = xy.y;
-    ez = z.x + z.y;
+    ex = sum_rows(w, vx);
+    ey = sum_rows(w, vy);
+    ez = sum_rows(w, vz);
 }
 
 // E8 holds, per node q, E at q and (primed) at its +x neighbour (periodic) as Ex
@@ -114,7 +109,6 @@ __device__ __forceinline__ void ld_pair(const float4 *p, float4 &a, float4 &b) {
         : "l"(p));
 }
 
-template <bool PACKED = false>
 __device__ __forceinline__ void gather_E_pairs(const Geom &g, const float4 *__restrict__ E8, int i,
                                                int j, int k, float fx, float fy, float fz,
                                                float &ex, float &ey, float &ez) {
@@ -132,8 +126,7 @@ __device__ __forceinline__ void gather_E_pairs(const Geom &g, const float4 *__re
         ld_pair(E8 + 2 * (int64_t)at[q], e0, e1);
         r[q] = row_of(e0, e1);
     }
-    if (PACKED) interp_E_packed(r, fx, fy, fz, ex, ey, ez);
-    else interp_E(r, fx, fy, fz, ex, ey, ez);
+    interp_E(r, fx, fy, fz, ex, ey, ez);
 }
 
 // E at the particle from a copy of the field on a box in shared memory (one
@@ -249,7 +242,7 @@ __device__ __forceinline__ void push_one_pairs(const Geom &g, const PushConst &p
                                                int &k) {
     decode_base(g, c, i, j, k, bad);
     float ex, ey, ez;
-    gather_E_pairs<true>(g, E8, i, j, k, fx, fy, fz, ex, ey, ez);
+    gather_E_pairs(g, E8, i, j, k, fx, fy, fz, ex, ey, ez);
     int step[3];
     kick_drift<EXT, MAG>(g, pc, ex, ey, ez, i, j, k, c, fx, fy, fz, vx, vy, vz, bad, step);
 }
