@@ -614,19 +614,9 @@ cudaError_t launch_adj_push(const Geom &g, const Ctrl *ctrl, const int4 *items, 
     const AdjShape a = adj_shape(g);
     const int blocks = adj_blocks(g, max_items);
     const bool cbox = const_box(g);
-#define PIC_ADJ(PGV, BV)                                                                        \
-    do {                                                                                        \
-        if (a.smem > 48 * 1024) {                                                               \
-            cudaError_t e = cudaFuncSetAttribute(k_adj_push<PGV, BV>,                           \
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                                                 (int)a.smem);                                  \
-            if (e != cudaSuccess) return e;                                                     \
-        }                                                                                       \
-        launch_dep(k_adj_push<PGV, BV>, blocks, a.threads, a.smem, st, g, a.staged, ctrl, items, ycell, \
-                                                               yo[0], yo[1], yo[2], E8, lE4,    \
-                                                               c_kick, dt, wz2, rt, ab, pg,     \
-                                                               tile_cost, ctrl_w);              \
-    } while (0)
+#define PIC_ADJ(PGV, BV)                                                                          \
+    launch_dep(k_adj_push<PGV, BV>, blocks, a.threads, a.smem, st, g, a.staged, ctrl, items, ycell, yo[0], \
+               yo[1], yo[2], E8, lE4, c_kick, dt, wz2, rt, ab, pg, tile_cost, ctrl_w)
     if (pg.part) {
         if (cbox) PIC_ADJ(true, kConstBox);
         else PIC_ADJ(true, 0);
@@ -648,6 +638,16 @@ AdjShape adj_shape(const Geom &g) {
 }
 int adj_blocks(const Geom &g, int max_items) {
     return std::max(1, std::min(kNumSMs * adj_shape(g).per_sm, max_items));
+}
+
+cudaError_t adj_prepare(const Geom &g) {
+    const size_t smem = adj_shape(g).smem;
+    cudaError_t e;
+    if ((e = allow_smem(k_adj_push<true, 0>, smem)) != cudaSuccess ||
+        (e = allow_smem(k_adj_push<false, 0>, smem)) != cudaSuccess ||
+        (e = allow_smem(k_adj_push<true, kConstBox>, smem)) != cudaSuccess)
+        return e;
+    return allow_smem(k_adj_push<false, kConstBox>, smem);
 }
 
 cudaError_t launch_pgrad_acc(const Geom &g, const double *part, int max_items, double *acc,

@@ -535,10 +535,7 @@ cudaError_t launch_b_push_deposit(bool push, bool diag, bool ext, bool mag, bool
 #define PIC_BPD(P, D, X, M, F)                                                                  \
     do {                                                                                        \
         auto kern = k_b_push_deposit<P, D, X, M, F>;                                            \
-        if (smem > 48 * 1024 &&                                                                 \
-            (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
-                                      (int)smem)) != cudaSuccess)                               \
-            return e;                                                                           \
+        if ((e = allow_smem(kern, smem)) != cudaSuccess) return e;                              \
         launch_dep(kern, blocks, threads, smem, st, desc, tile_inst, ctrl, items, push ? E4 : nullptr, \
                                             E8, rho, rho64, sparse_below, tile_cost, max_S,     \
                                             part);                                              \

@@ -156,6 +156,15 @@ cudaError_t launch_rho_finish(const Geom &g, unsigned long long *rho64, float *r
     return cudaGetLastError();
 }
 
+cudaError_t deposit_prepare(const Geom &g) {
+    const size_t smem = tile_deposit_smem(g);
+    cudaError_t e;
+    if ((e = allow_smem(k_deposit_tiles<false, 0>, smem)) != cudaSuccess ||
+        (e = allow_smem(k_deposit_tiles<true, 0>, smem)) != cudaSuccess)
+        return e;
+    return allow_smem(k_deposit_tiles<true, kConstBox>, smem);
+}
+
 cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int4 *items,
                            int max_items, double qscale_d, float *rho, unsigned long long *rho64,
                            bool fixed, Ctrl *ctrl_w, int grid_blocks, int sparse_below,
@@ -166,16 +175,9 @@ cudaError_t launch_deposit(int64_t n, const Geom &g, const Ctrl *ctrl, const int
     const int blocks = grid_blocks < max_items ? grid_blocks : (max_items > 0 ? max_items : 1);
     cudaError_t e;
     const bool cbox = const_box(g);
-#define PIC_DT(F, B)                                                                           \
-    do {                                                                                       \
-        if (smem > 48 * 1024 &&                                                                \
-            (e = cudaFuncSetAttribute(k_deposit_tiles<F, B>,                                   \
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize,             \
-                                      (int)smem)) != cudaSuccess)                              \
-            return e;                                                                          \
-        launch_dep(k_deposit_tiles<F, B>, blocks, 256, smem, st, g, ctrl, items, qscale, rho, rho64,   \
-                                                         ctrl_w, sparse_below, tile_cost);                \
-    } while (0)
+#define PIC_DT(F, B)                                                                              \
+    launch_dep(k_deposit_tiles<F, B>, blocks, 256, smem, st, g, ctrl, items, qscale, rho, rho64, ctrl_w, \
+               sparse_below, tile_cost)
     if (fixed) {
         if (cbox) PIC_DT(true, kConstBox);
         else PIC_DT(true, 0);

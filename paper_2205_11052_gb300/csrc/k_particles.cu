@@ -857,24 +857,14 @@ bool const_box15(const Geom &g, const PushShape &ps) {
 // Allow the fused kernels' shared memory (call outside any stream capture)
 cudaError_t push_deposit_prepare(const Geom &g) {
     cudaError_t e = cudaSuccess;
-    const size_t tsm = tile_deposit_smem(g);
-    if (tsm > 48 * 1024) {
-#define PIC_MVA(D, F, B)                                                                       \
-        if ((e = cudaFuncSetAttribute(k_move_deposit<D, F, B>,                                  \
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm)) != \
-            cudaSuccess)                                                                        \
-            return e
-        PIC_MVA(false, false, 0); PIC_MVA(false, true, 0); PIC_MVA(true, false, 0);
-        PIC_MVA(true, true, 0); PIC_MVA(false, true, kConstBox); PIC_MVA(true, true, kConstBox);
+    const size_t tsm = tile_deposit_smem(g), smem = push_shape(g).smem;
+#define PIC_MVA(D, F, B) \
+    if ((e = allow_smem(k_move_deposit<D, F, B>, tsm)) != cudaSuccess) return e
+    PIC_MVA(false, false, 0); PIC_MVA(false, true, 0); PIC_MVA(true, false, 0);
+    PIC_MVA(true, true, 0); PIC_MVA(false, true, kConstBox); PIC_MVA(true, true, kConstBox);
 #undef PIC_MVA
-    }
-    const size_t smem = push_shape(g).smem;
-    if (smem <= 48 * 1024) return cudaSuccess;
-#define PIC_PDA(D, X, M, F, B, BE)                                                            \
-    if ((e = cudaFuncSetAttribute(k_push_deposit<D, X, M, F, B, BE>,                          \
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != \
-        cudaSuccess)                                                                          \
-        return e
+#define PIC_PDA(D, X, M, F, B, BE) \
+    if ((e = allow_smem(k_push_deposit<D, X, M, F, B, BE>, smem)) != cudaSuccess) return e
 #define PIC_PDA2(D, X, M) \
     PIC_PDA(D, X, M, false, 0, 0); PIC_PDA(D, X, M, true, 0, 0);          \
     PIC_PDA(D, X, M, true, kConstBox, kConstBox); PIC_PDA(D, X, M, true, 15, kConstBox)

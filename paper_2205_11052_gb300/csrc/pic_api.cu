@@ -1016,6 +1016,7 @@ int pic_bind_workspace(pic_handle_t c, void *arena, size_t bytes, void *stream) 
 
     PIC_CUDA(sort_prepare());
     PIC_CUDA(push_deposit_prepare(c->geom));
+    PIC_CUDA(deposit_prepare(c->geom));
     Ctrl h;
     memset(&h, 0, sizeof(h));
     for (int s = 0; s < 2; ++s) {
@@ -1359,6 +1360,7 @@ int pic_adjoint_forward(pic_handle_t c, int n_steps, int K, const double *w, voi
     if (bytes < L.total)
         return fail(PIC_ERR_CAPACITY, "adjoint buffer of %zu bytes < required %zu", bytes, L.total);
     if ((r = make_plans(c, {kR2C, kC2R4}))) return r;
+    PIC_CUDA(adj_prepare(c->geom));
     const DepScope dep(c->st, c->np <= kDepMaxParticles);
     PIC_CUDA(cudaStreamSynchronize(c->st));
     int32_t cur = 0;

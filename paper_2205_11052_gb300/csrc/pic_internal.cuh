@@ -146,6 +146,20 @@ constexpr int kDiagFieldBlocks = 152 * 8;
 constexpr int kNumSMs = 152;   // streaming multiprocessors of the GPU (two dies of 76)
 constexpr int kMaxPushBlocks = kNumSMs * 8;
 constexpr int kMaxSmemPerBlock = 227 * 1024;   // opt-in shared memory per block
+// Lets a kernel be launched with `need` bytes of dynamic shared memory.  The limit belongs
+// to the function, which every handle of the process shares, so it is always set to all
+// that its static memory leaves: set to a handle's own need, it would be lowered under
+// another handle (or a captured graph) that needs more.
+template <class K>
+inline cudaError_t allow_smem(K *kernel, size_t need) {
+    if (need <= 48 * 1024) return cudaSuccess;
+    cudaFuncAttributes a;
+    const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    const size_t most = kMaxSmemPerBlock - a.sharedSizeBytes;
+    if (need > most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
 // threads per SM the fused push + deposit kernel is compiled for (80 registers)
 constexpr int kPushThreadsPerSM = 768;
 // resident blocks per SM of the uniform-plasma move + deposit
@@ -354,6 +368,8 @@ size_t tile_deposit_smem(const Geom &g);   // the deposit tiles alone (unstaged 
 constexpr int kConstBox = 13;
 bool const_box(const Geom &g);
 cudaError_t push_deposit_prepare(const Geom &g);
+cudaError_t deposit_prepare(const Geom &g);
+cudaError_t adj_prepare(const Geom &g);
 // Optional copy of the positions a push starts from (cell, o[3]), written by
 // the fused kernel as it reads them (the adjoint keeps each step's y).
 struct SaveY {
