@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(256) k_adj_unload_records(int64_t n,
     if (p >= n) return;
     const int cur = ctrl->cur;
     const int32_t q = ctrl->sets[cur].pid[p];
-    if ((uint64_t)(int64_t)q >= (uint64_t)n) return;   // only after a sort that gave up
+    if (!is_particle(q, n)) return;
     const ParticleSet lam = ctrl->sets[1 - cur];
     st_record(rec, q, make_float4(lam.o[0][p], lam.o[1][p], lam.o[2][p], 0.0f),
               make_float4(lam.v[0][p], lam.v[1][p], lam.v[2][p], 0.0f));
@@ -543,11 +543,13 @@ __global__ void k_adj_reorder(int64_t n, const int32_t *__restrict__ pos,
     dep_begin();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    const int32_t j = pos[pid_prev[i]];
+    const int32_t q = pid_prev[i];
+    const int32_t j = is_particle(q, n) ? pos[q] : -1;
+    const bool known = is_particle(j, n);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        a.out_o[d][i] = a.in_o[d][j];
-        a.out_v[d][i] = a.in_v[d][j];
+        a.out_o[d][i] = known ? a.in_o[d][j] : 0.0f;
+        a.out_v[d][i] = known ? a.in_v[d][j] : 0.0f;
     }
 }
 

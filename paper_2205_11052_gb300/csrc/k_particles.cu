@@ -134,7 +134,7 @@ __global__ void k_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv) {
     if (p >= n) return;
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int32_t q = ps.pid[p];
-    if ((uint64_t)(int64_t)q < (uint64_t)n) inv[q] = (int32_t)p;   // else: a sort gave up
+    if (is_particle(q, n)) inv[q] = (int32_t)p;
 }
 
 __global__ void __launch_bounds__(256) k_unload_records(int64_t n, const Ctrl *__restrict__ ctrl) {
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(256) k_unload_records(int64_t n, const Ctrl *_
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const int32_t q = __ldcs(ps.pid + p);
-    if ((uint64_t)(int64_t)q >= (uint64_t)n) return;   // only after a sort that gave up
+    if (!is_particle(q, n)) return;
     st_record(rec, q,
               make_float4(__int_as_float(__ldcs(ps.cell + p)), __ldcs(ps.o[0] + p),
                           __ldcs(ps.o[1] + p), __ldcs(ps.o[2] + p)),
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(256) k_unload_records(int64_t n, const Ctrl *_
 // come from a table, floats are widened and the wrap is tested on the bits (with
 // conversions and divisions the FP64 pipe was 85% busy: 5.0 ms at 134M).
 template <bool GATHER>
-__global__ void __launch_bounds__(kLoadThreads) k_unload(int64_t o0, int64_t m,
+__global__ void __launch_bounds__(kLoadThreads) k_unload(int64_t o0, int64_t m, int64_t n,
                                                         const int32_t *__restrict__ inv,
                                                         const double *__restrict__ node_pos,
                                                         double h0, double h1, double h2,
@@ -173,12 +173,14 @@ __global__ void __launch_bounds__(kLoadThreads) k_unload(int64_t o0, int64_t m,
     const int64_t q0 = (int64_t)blockIdx.x * kLoadThreads;
     const int cnt = (int)(m - q0 < kLoadThreads ? m - q0 : kLoadThreads);
     if ((int)threadIdx.x < cnt) {
-        float4 a, b;
+        float4 a = make_float4(0.0f, 0.0f, 0.0f, 0.0f), b = a;
         if (GATHER) {
             const ParticleSet ps = ctrl->sets[ctrl->cur];
-            const int64_t p = inv[o0 + q0 + threadIdx.x];
-            a = make_float4(__int_as_float(ps.cell[p]), ps.o[0][p], ps.o[1][p], ps.o[2][p]);
-            b = make_float4(ps.v[0][p], ps.v[1][p], ps.v[2][p], 0.0f);
+            const int32_t p = inv[o0 + q0 + threadIdx.x];
+            if (is_particle(p, n)) {
+                a = make_float4(__int_as_float(ps.cell[p]), ps.o[0][p], ps.o[1][p], ps.o[2][p]);
+                b = make_float4(ps.v[0][p], ps.v[1][p], ps.v[2][p], 0.0f);
+            }
         } else {
             ld_record(reinterpret_cast<const float4 *>(ctrl->sets[1 - ctrl->cur].cell),
                       o0 + q0 + threadIdx.x, a, b);
@@ -556,7 +558,7 @@ cudaError_t launch_copy(const CopyList &cl, LStream st) {
 __global__ void k_pid_positions(int64_t n, const int32_t *__restrict__ pid, int32_t *pos) {
     dep_begin();
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) pos[pid[p]] = (int32_t)p;
+    if (p < n && is_particle(pid[p], n)) pos[pid[p]] = (int32_t)p;
 }
 
 cudaError_t launch_pid_positions(int64_t n, const int32_t *pid, int32_t *pos, LStream st) {
@@ -582,13 +584,13 @@ void node_positions(const double *h_d, double *node_pos) {
         for (int i = 0; i < kMaxN; ++i) node_pos[d * kMaxN + i] = ((double)i + 0.5) * h_d[d];
 }
 
-cudaError_t launch_unload(int64_t o0, int64_t m, const int32_t *inv, const double *node_pos,
+cudaError_t launch_unload(int64_t o0, int64_t m, int64_t n, const int32_t *inv, const double *node_pos,
                           const double *h_d, const double *L_d, double dt, const Ctrl *ctrl,
                           double *x, double *v, LStream st) {
     if (m <= 0) return cudaSuccess;
     const unsigned blocks = (unsigned)((m + kLoadThreads - 1) / kLoadThreads);
 #define PIC_UL(G)                                                                            \
-    launch_dep(k_unload<G>, blocks, kLoadThreads, 0, st, o0, m, inv, node_pos, h_d[0], h_d[1], h_d[2], \
+    launch_dep(k_unload<G>, blocks, kLoadThreads, 0, st, o0, m, n, inv, node_pos, h_d[0], h_d[1], h_d[2], \
                                                  L_d[0], L_d[1], L_d[2], 0.5 * dt, ctrl, x, v)
     if (inv) PIC_UL(true);
     else PIC_UL(false);

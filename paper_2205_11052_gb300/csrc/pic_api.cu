@@ -1174,7 +1174,7 @@ int pic_get_particles(pic_handle_t c, double *x, double *v, int dst_is_device) {
     const double *npos = c->at<double>(c->lay.node_pos);
     if (dst_is_device) {
         PIC_CUDA(launch_unload_records(c->np, c->ctrl(), c->st));
-        PIC_CUDA(launch_unload(0, c->np, nullptr, npos, c->h, c->L, c->prm.dt, c->ctrl(), x, v, c->st));
+        PIC_CUDA(launch_unload(0, c->np, c->np, nullptr, npos, c->h, c->L, c->prm.dt, c->ctrl(), x, v, c->st));
         return PIC_OK;
     }
     // host destinations: the host link is slower than the scattered reads
@@ -1185,14 +1185,14 @@ int pic_get_particles(pic_handle_t c, double *x, double *v, int dst_is_device) {
                     : nullptr;
     if (mx && mv) {
         // page-locked host arrays: written in place by the unload kernel
-        PIC_CUDA(launch_unload(0, c->np, inv, npos, c->h, c->L, c->prm.dt, c->ctrl(), mx, mv, c->st));
+        PIC_CUDA(launch_unload(0, c->np, c->np, inv, npos, c->h, c->L, c->prm.dt, c->ctrl(), mx, mv, c->st));
         PIC_CUDA(cudaStreamSynchronize(c->st));
         return PIC_OK;
     }
     double *sx = c->at<double>(c->lay.stage_x), *sv = c->at<double>(c->lay.stage_v);
     for (int64_t o = 0; o < c->np; o += c->staging) {
         const int64_t m = std::min<int64_t>(c->staging, c->np - o);
-        PIC_CUDA(launch_unload(o, m, inv, npos, c->h, c->L, c->prm.dt, c->ctrl(), sx, sv, c->st));
+        PIC_CUDA(launch_unload(o, m, c->np, inv, npos, c->h, c->L, c->prm.dt, c->ctrl(), sx, sv, c->st));
         PIC_CUDA(cudaMemcpyAsync(x + 3 * o, sx, (size_t)m * 24, cudaMemcpyDeviceToHost, c->st));
         PIC_CUDA(cudaMemcpyAsync(v + 3 * o, sv, (size_t)m * 24, cudaMemcpyDeviceToHost, c->st));
     }

@@ -112,6 +112,14 @@ __host__ __device__ __forceinline__ int cell_i(int32_t c) { return c & kCellMask
 __host__ __device__ __forceinline__ int cell_j(int32_t c) { return (c >> kCellBits) & kCellMask; }
 __host__ __device__ __forceinline__ int cell_k(int32_t c) { return (c >> (2 * kCellBits)) & kCellMask; }
 
+// Whether q names one of n particles.  A re-binning that gave up (PIC_FLAG_TIMEOUT)
+// leaves slots that it did not write, in which the other set's former contents, a
+// readback's records among them, stand for load indices, and an index that no slot holds
+// keeps whatever an inverse of the order had there: what follows such an index asks first.
+__device__ __forceinline__ bool is_particle(int32_t q, int64_t n) {
+    return (uint64_t)(int64_t)q < (uint64_t)n;
+}
+
 // Grid geometry passed by value to kernels.
 struct Geom {
     int n[3];          // nodes per axis
@@ -300,12 +308,12 @@ cudaError_t launch_load(const double *x, const double *v, int64_t m, int64_t bas
                         LStream st, int max_blocks = 0);
 // readback in load order: the current set's particles as 32-byte records (by
 // pid) in the other set, or the inverse of the store's order (inv[pid]); then
-// particles [o0, o0 + m) as FP64 triples from the records (inv null) or through
+// particles [o0, o0 + m) of n as FP64 triples from the records (inv null) or through
 // inv; node_pos: kMaxN node positions (i + 1/2) h per axis
 cudaError_t launch_unload_records(int64_t n, const Ctrl *ctrl, LStream st);
 cudaError_t launch_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv, LStream st);
 void node_positions(const double *h_d, double *node_pos);
-cudaError_t launch_unload(int64_t o0, int64_t m, const int32_t *inv, const double *node_pos,
+cudaError_t launch_unload(int64_t o0, int64_t m, int64_t n, const int32_t *inv, const double *node_pos,
                           const double *h_d, const double *L_d, double dt, const Ctrl *ctrl,
                           double *x, double *v, LStream st);
 
