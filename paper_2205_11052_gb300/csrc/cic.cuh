@@ -293,7 +293,7 @@ __host__ __device__ __forceinline__ size_t sum_offset(int S) { return ((size_t)S
 // (256^3 cells, 4096 particles a tile: the push takes 3.22 ms; with one load after
 // the other through registers 3.58).  stage_wait, then a
 // barrier, before the box is read.
-__device__ __forceinline__ void stage_box(float4 *sE, const float4 *__restrict__ E4, const Tile &t,
+__device__ __forceinline__ void stage_box(float4 *sE, const float4 *E4, const Tile &t,
                                           const Geom &g) {
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sE);
     for (int s = threadIdx.x; s < t.S; s += blockDim.x)
@@ -305,7 +305,7 @@ __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;"
 
 // The same box with x pairs, from E8: sA holds Ex and Ey of a slot and of its +x
 // neighbour, sB the two Ez.
-__device__ __forceinline__ void stage_pairs(float4 *sA, float2 *sB, const float4 *__restrict__ E8,
+__device__ __forceinline__ void stage_pairs(float4 *sA, float2 *sB, const float4 *E8,
                                             const Tile &t, const Geom &g) {
     const uint32_t da = (uint32_t)__cvta_generic_to_shared(sA);
     const uint32_t db = (uint32_t)__cvta_generic_to_shared(sB);
@@ -320,7 +320,7 @@ __device__ __forceinline__ void stage_pairs(float4 *sA, float2 *sB, const float4
 }
 
 // ... and of an array of one float2 per node
-__device__ __forceinline__ void stage_float2(float2 *sR, const float2 *__restrict__ v, const Tile &t,
+__device__ __forceinline__ void stage_float2(float2 *sR, const float2 *v, const Tile &t,
                                              const Geom &g) {
     const uint32_t dst = (uint32_t)__cvta_generic_to_shared(sR);
     for (int s = threadIdx.x; s < t.S; s += blockDim.x)

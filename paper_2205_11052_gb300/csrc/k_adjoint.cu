@@ -59,12 +59,12 @@ __device__ __forceinline__ void corners(int i, int j, int k, int nx, int ny, int
 
 // the 8 corner values of an x-paired scalar grid (v2[q] = (v[q], v[q + x])):
 // four aligned 8-byte loads, corner bits a | b<<1 | c<<2
-__device__ __forceinline__ void corners_from_pairs(const float2 *__restrict__ v2, int i, int j,
-                                                   int k, int nx, int ny, int nz, float sc[8]) {
+__device__ __forceinline__ void corners_from_pairs(const float2 *v2, int i, int j, int k, int nx, int ny,
+                                                   int nz, float sc[8]) {
     const int j1 = (j + 1 == ny) ? 0 : j + 1;
     const int k1 = (k + 1 == nz) ? 0 : k + 1;
-    const float2 a = __ldg(v2 + (j + ny * k) * nx + i), b = __ldg(v2 + (j1 + ny * k) * nx + i);
-    const float2 c = __ldg(v2 + (j + ny * k1) * nx + i), d = __ldg(v2 + (j1 + ny * k1) * nx + i);
+    const float2 a = v2[(j + ny * k) * nx + i], b = v2[(j1 + ny * k) * nx + i];
+    const float2 c = v2[(j + ny * k1) * nx + i], d = v2[(j1 + ny * k1) * nx + i];
     sc[0] = a.x; sc[1] = a.y; sc[2] = b.x; sc[3] = b.y;
     sc[4] = c.x; sc[5] = c.y; sc[6] = d.x; sc[7] = d.y;
 }
@@ -121,18 +121,18 @@ __global__ void k_adj_seed(int64_t ng, const float4 *__restrict__ E8, float4 *__
 // the eleven a particle needs.  B > 0: every tile box is B slots long on each axis.
 // 4.2M particles on 64^3 cells: 160 us, staged 142.
 template <bool PG, int B>
-__global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bool staged, const Ctrl *__restrict__ ctrl,
-                                                      const int4 *__restrict__ items,
-                                                      const int32_t *__restrict__ ycell,
-                                                      const float *__restrict__ yo0,
-                                                      const float *__restrict__ yo1,
-                                                      const float *__restrict__ yo2,
-                                                      const float4 *__restrict__ E8,
-                                                      float4 *__restrict__ lE4, float c_kick,
+__global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bool staged, const Ctrl *ctrl,
+                                                      const int4 *items,
+                                                      const int32_t *ycell,
+                                                      const float *yo0,
+                                                      const float *yo1,
+                                                      const float *yo2,
+                                                      const float4 *E8,
+                                                      float4 *lE4, float c_kick,
                                                       float dt, float wz2, AdjRhoTerm rt,
                                                       AdjBound ab, PGrad pg, int tile_cost,
                                                       Ctrl *ctrl_w) {
-    dep_begin();
+    dep_begin(ctrl, items, ycell, yo0, yo1, yo2, E8, lE4, ctrl_w);
     // 3 * S integer accumulators (x, y, z components) in units of 1 / qs
     extern __shared__ int acc[];
     const int cur = ctrl->cur;
@@ -397,9 +397,9 @@ __global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bo
 
 // acc[q] += sum over blocks of part[b][q]: one warp per term, strided sums per
 // lane, then a fixed tree (a block tree over all terms took 8.2 us)
-__global__ void __launch_bounds__(32 * kPGradTerms) k_pgrad_acc(const double *__restrict__ part,
+__global__ void __launch_bounds__(32 * kPGradTerms) k_pgrad_acc(const double *part,
                                                                 int blocks, double *acc) {
-    dep_begin();
+    dep_begin(part, acc);
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
     double s = 0.0;
     for (int b = lane; b < blocks; b += 32) s += part[(size_t)kPGradTerms * b + q];
@@ -439,11 +439,11 @@ __global__ void k_green_adj(int nx, int ny, int nz, int nh, double tpx, double t
 // ly += (q_p / h^3) sum_corner grad W lrho  ((dD/dy)^T lrho)
 // (with `out` given, the updated multipliers go there instead of in place:
 // ly + term to out.o, lv copied to out.v)
-__global__ void k_adj_rho(int64_t n, Geom g, Ctrl *ctrl, const int32_t *__restrict__ ycell,
-                          const float *__restrict__ yo0, const float *__restrict__ yo1,
-                          const float *__restrict__ yo2, const float2 *__restrict__ lrho2,
+__global__ void k_adj_rho(int64_t n, Geom g, Ctrl *ctrl, const int32_t *ycell,
+                          const float *yo0, const float *yo1,
+                          const float *yo2, const float2 *lrho2,
                           float qscale, LamOut out, int par) {
-    dep_begin();
+    dep_begin(ctrl, ycell, yo0, yo1, yo2, lrho2);
     const ParticleSet lam = ctrl->sets[1 - ctrl->cur];
     float mly = 0.0f;
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
@@ -538,9 +538,9 @@ __global__ void __launch_bounds__(256) k_adj_unload(int64_t o0, int64_t m,
 // across a re-binning is a permutation: with pos[pid] the slot of particle
 // pid in the later order, slot i of the earlier order (particle
 // pid_prev[i]) takes the multipliers from slot pos[pid_prev[i]].
-__global__ void k_adj_reorder(int64_t n, const int32_t *__restrict__ pos,
-                              const int32_t *__restrict__ pid_prev, ReorderArgs a) {
-    dep_begin();
+__global__ void k_adj_reorder(int64_t n, const int32_t *pos,
+                              const int32_t *pid_prev, ReorderArgs a) {
+    dep_begin(pos, pid_prev);
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int32_t q = pid_prev[i];

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(256) k_b_unload(int64_t o0, int64_t m,
                                                   const long long *__restrict__ c0, double half_dt,
                                                   const Ctrl *ctrl, double *__restrict__ x,
                                                   double *__restrict__ v) {
-    dep_begin();
+    dep_begin(ctrl, x, v);
     const float4 *rec = reinterpret_cast<const float4 *>(ctrl->sets[1 - ctrl->cur].cell);
     __shared__ double sx[3 * 256], sv[3 * 256];
     __shared__ long long dst[256];
@@ -182,10 +182,10 @@ struct BatchKey {
 template <bool PUSH, bool DIAG, bool EXT, bool MAG, bool FIXED>
 __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit(
     const InstDesc *__restrict__ desc, const int32_t *__restrict__ tile_inst, Ctrl *ctrl,
-    const int4 *__restrict__ items, const float4 *__restrict__ E4, const float4 *__restrict__ E8,
+    const int4 *items, const float4 *E4, const float4 *E8,
     float *rho, unsigned long long *rho64, int sparse_below, int tile_cost, int max_S,
     double *__restrict__ part) {
-    dep_begin();
+    dep_begin(ctrl, items, E4, E8, rho, rho64, part);
     extern __shared__ __align__(16) uint32_t acc[];
     __shared__ double red[4][8];
     void *sum = reinterpret_cast<char *>(acc) + cic::sum_offset(max_S);
@@ -326,8 +326,8 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
 // integer grid -> charge density of each node's instance; clears rho64
 __global__ void k_b_rho_finish(int64_t ng, const InstDesc *__restrict__ desc,
                                const long long *__restrict__ g0, int n_inst,
-                               unsigned long long *__restrict__ rho64, float *__restrict__ rho) {
-    dep_begin();
+                               unsigned long long *rho64, float *__restrict__ rho) {
+    dep_begin(rho64, rho);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int inst = 0;
     for (int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; gidx < ng; gidx += stride) {
@@ -412,13 +412,13 @@ __global__ void __launch_bounds__(256) k_b_diag_field(const InstDesc *__restrict
 // up to 48^3 cells, now 12.7 us.
 __global__ void __launch_bounds__(256) k_b_diag_finalize(const InstDesc *__restrict__ desc,
                                                          int n_inst, int fstride,
-                                                         const int32_t *__restrict__ item_off,
-                                                         const double *__restrict__ fpart,
-                                                         const double *__restrict__ ppart,
-                                                         const double *__restrict__ modes,
+                                                         const int32_t *item_off,
+                                                         const double *fpart,
+                                                         const double *ppart,
+                                                         const double *modes,
                                                          Ctrl *ctrl, double dt, pic_diag_t *ring,
                                                          int ring_cap) {
-    dep_begin();
+    dep_begin(item_off, fpart, ppart, modes, ctrl, ring);
     const int i = blockIdx.x;
     const InstDesc &D = desc[i];
     __shared__ double red[8][256];
@@ -473,7 +473,7 @@ __global__ void k_b_pack(int64_t mng, int nx, const float *__restrict__ planar,
 }
 
 __global__ void k_b_step_done(Ctrl *ctrl, int diag) {
-    dep_begin();
+    dep_begin(ctrl);
     ctrl->step += 1;
     if (diag) ctrl->diag_written += 1;
 }

@@ -38,12 +38,12 @@ using namespace cic;
 
 // B > 0: every tile box is B slots long on each axis (cic::box_row)
 template <bool FIXED, int B>
-__global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom g, const Ctrl *__restrict__ ctrl,
-                                                           const int4 *__restrict__ items,
+__global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom g, const Ctrl *ctrl,
+                                                           const int4 *items,
                                                            float qscale, float *rho,
                                                            unsigned long long *rho64, Ctrl *ctrl_w,
                                                            int sparse_below, int tile_cost) {
-    dep_begin();
+    dep_begin(ctrl, items, rho, rho64, ctrl_w);
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
@@ -121,9 +121,9 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
 // integer grid -> charge density, and clear the integer grid for next time;
 // two nodes per thread and iteration (16-byte loads and stores of the 8-byte
 // words, 8-byte stores of the densities), the odd last node by thread 0
-__global__ void __launch_bounds__(256) k_rho_finish(int64_t ng, unsigned long long *__restrict__ rho64,
+__global__ void __launch_bounds__(256) k_rho_finish(int64_t ng, unsigned long long *rho64,
                                                     float *__restrict__ rho, FixedScale f) {
-    dep_begin();
+    dep_begin(rho64, rho);
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t n2 = ng >> 1;
     ulonglong2 *r2 = reinterpret_cast<ulonglong2 *>(rho64);

@@ -50,10 +50,10 @@ __device__ __forceinline__ void unpack_rows(float2 z, float2 m, float2 &a, float
 template <int COMPS>
 __global__ void __launch_bounds__(kXThreads) k_fft_x_forward(int ny, int nz, int nh, FftAxis ax,
                                                              const FftTables *__restrict__ tab,
-                                                             const float *__restrict__ rho,
-                                                             float4 *__restrict__ lE4,
+                                                             const float *rho,
+                                                             float4 *lE4,
                                                              float2 *__restrict__ out, int64_t nhalf) {
-    dep_begin();
+    dep_begin(rho, lE4, out);
     if (COMPS == 1) {   // blockIdx.z: one of several grids in a row
         rho += blockIdx.z * ((int64_t)ax.n * ny * nz);
         out += blockIdx.z * nhalf;
@@ -104,7 +104,7 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_forward(int ny, int nz, int
 }
 
 // plane of one x frequency: [z][y] in global memory, pitch ny | 1 in shared
-__device__ __forceinline__ void load_plane(float2 *s, const float2 *__restrict__ in, int ny, int nz,
+__device__ __forceinline__ void load_plane(float2 *s, const float2 *in, int ny, int nz,
                                            int pitch) {
     const fft::FastDiv by_ny(ny);
     for (int w = threadIdx.x; w < ny * nz; w += blockDim.x) {
@@ -126,11 +126,11 @@ __device__ __forceinline__ void store_plane(float2 *__restrict__ out, const floa
 __global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, FftAxis ay, FftAxis az,
                                                 const FftTables *__restrict__ tab,
                                                 const float *__restrict__ ktab, float inv_ng,
-                                                const float2 *__restrict__ in,
+                                                const float2 *in,
                                                 float2 *__restrict__ out, int64_t nhalf, int mi, int mj,
                                                 int mk, int mode_comp, int mode_conj,
                                                 double *__restrict__ mode) {
-    dep_begin();
+    dep_begin(in, out, mode);
     in += blockIdx.z * nhalf;
     out += blockIdx.z * 3 * nhalf;
     ktab += blockIdx.z * (nh + 2 * (ny + nz));
@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(512) k_fft_yz(int nx, int ny, int nz, int nh, 
 __global__ void __launch_bounds__(512) k_fft_yz_adj(int nx, int ny, int nz, int nh, FftAxis ay,
                                                     FftAxis az, const FftTables *__restrict__ tab,
                                                     const float *__restrict__ ktab,
-                                                    float2 *__restrict__ lE_hat, int64_t nhalf) {
-    dep_begin();
+                                                    float2 *lE_hat, int64_t nhalf) {
+    dep_begin(lE_hat);
     extern __shared__ float2 sm[];
     const int pitch = ny | 1, a = blockIdx.x, d = blockIdx.y;
     float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
@@ -205,9 +205,9 @@ __global__ void __launch_bounds__(512) k_fft_yz_adj(int nx, int ny, int nz, int 
 __global__ void __launch_bounds__(512) k_fft_yz_adj_back(int ny, int nz, int nh, FftAxis ay, FftAxis az,
                                                          const FftTables *__restrict__ tab,
                                                          const float *__restrict__ ktab, float inv_ng,
-                                                         const float2 *__restrict__ lE_hat,
+                                                         const float2 *lE_hat,
                                                          float2 *__restrict__ out, int64_t nhalf) {
-    dep_begin();
+    dep_begin(lE_hat, out);
     extern __shared__ float2 sm[];
     const int pitch = ny | 1, a = blockIdx.x;
     float2 *s = sm, *twy = sm + nz * pitch, *twz = twy + ny;
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(512) k_fft_yz_adj_back(int ny, int nz, int nh,
 // rows y0.. of plane z of COMPS components, from spectra by x frequency to two
 // real rows per complex line in shared memory
 template <int COMPS>
-__device__ __forceinline__ void rows_backward(float2 *s, float2 *tw, const float2 *__restrict__ in,
+__device__ __forceinline__ void rows_backward(float2 *s, float2 *tw, const float2 *in,
                                               int64_t nhalf, int ny, int nz, int nh, int z, int y0,
                                               int rows, const FftAxis &ax,
                                               const FftTables *__restrict__ tab) {
@@ -260,12 +260,12 @@ __device__ __forceinline__ void rows_backward(float2 *s, float2 *tw, const float
 
 __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, int nh, FftAxis ax,
                                                               const FftTables *__restrict__ tab,
-                                                              const float2 *__restrict__ in,
+                                                              const float2 *in,
                                                               int64_t nhalf, float4 *__restrict__ E4,
                                                               float4 *__restrict__ E8,
                                                               float *__restrict__ rho, bool clear_rho,
                                                               double *__restrict__ fpart, int fstride) {
-    dep_begin();
+    dep_begin(in, E4, E8, rho, fpart);
     const int64_t grid0 = blockIdx.z * ((int64_t)ax.n * ny * nz);
     in += blockIdx.z * 3 * nhalf;
     if (E4) E4 += grid0;
@@ -305,10 +305,10 @@ __global__ void __launch_bounds__(kXThreads) k_fft_x_backward(int ny, int nz, in
 // |lrho| goes to adj_lrho[par], and the slots of the next reverse push are cleared
 __global__ void __launch_bounds__(kXThreads) k_fft_x_backward_adj(int ny, int nz, int nh, FftAxis ax,
                                                                   const FftTables *__restrict__ tab,
-                                                                  const float2 *__restrict__ in,
+                                                                  const float2 *in,
                                                                   float2 *__restrict__ lrho2, Ctrl *ctrl,
                                                                   int par) {
-    dep_begin();
+    dep_begin(in, lrho2, ctrl);
     constexpr int PAIRS = kRowsB / 2;
     extern __shared__ float2 sm[];
     const int n = ax.n, pitch = n | 1;

@@ -27,11 +27,11 @@ namespace {
 // entries, then y: ny, then z: nz), rounded once from FP64 on the host.
 __global__ void __launch_bounds__(128) k_green(int nx, int ny, int nz, int nh,
                                                const float *__restrict__ ktab, float inv_ng,
-                                               const float2 *__restrict__ rho_hat,
+                                               const float2 *rho_hat,
                                                float2 *__restrict__ E_hat, int64_t nhalf, int mi,
                                                int mj, int mk, int mode_comp, int mode_conj,
                                                Ctrl *ctrl) {
-    dep_begin();
+    dep_begin(rho_hat, E_hat, ctrl);
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= nh) return;
     const int b = blockIdx.y, c = blockIdx.z;
@@ -60,11 +60,11 @@ __global__ void __launch_bounds__(128) k_green(int nx, int ny, int nz, int nh,
     }
 }
 
-__global__ void k_diag_finalize(const double *__restrict__ fpart, int fblocks,
-                                const double *__restrict__ ppart, int pblocks, double dV,
+__global__ void k_diag_finalize(const double *fpart, int fblocks,
+                                const double *ppart, int pblocks, double dV,
                                 double mp, double dt, Ctrl *ctrl, pic_diag_t *ring,
                                 int ring_cap) {
-    dep_begin();
+    dep_begin(fpart, ppart, ctrl, ring);
     // one warp per quantity: strided sums per lane, then a fixed tree (a block
     // tree over 256 x 8 FP64 values took 9.6 us, mostly its 64 barriers' adds)
     __shared__ double red[8];
@@ -110,11 +110,11 @@ namespace {
 // and a pass for the sums (81), a 256^3 solve with sums took 0.85 ms.
 template <int ES, bool SUMS>
 __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pitch, int64_t dist,
-                                                const float *__restrict__ planar,
+                                                const float *planar,
                                                 float4 *__restrict__ E8,
                                                 float *__restrict__ rho, bool clear_rho,
                                                 double *__restrict__ part) {
-    dep_begin();
+    dep_begin(planar, E8, rho, part);
     float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
     // one warp per row
     const int lane = threadIdx.x & 31;
@@ -141,9 +141,9 @@ __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pi
 
 namespace {
 // E8 -> one float4 (Ex, Ey, Ez, 0) per node, the layout of pic_get_field
-__global__ void __launch_bounds__(256) k_unpair_E(int64_t ng, const float4 *__restrict__ E8,
+__global__ void __launch_bounds__(256) k_unpair_E(int64_t ng, const float4 *E8,
                                                   float4 *__restrict__ E4) {
-    dep_begin();
+    dep_begin(E8, E4);
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= ng) return;
     const float4 a = E8[2 * q];

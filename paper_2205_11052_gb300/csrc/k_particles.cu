@@ -137,8 +137,8 @@ __global__ void k_invperm(int64_t n, const Ctrl *ctrl, int32_t *inv) {
     if (is_particle(q, n)) inv[q] = (int32_t)p;
 }
 
-__global__ void __launch_bounds__(256) k_unload_records(int64_t n, const Ctrl *__restrict__ ctrl) {
-    dep_begin();
+__global__ void __launch_bounds__(256) k_unload_records(int64_t n, const Ctrl *ctrl) {
+    dep_begin(ctrl);
     const int cur = ctrl->cur;
     const ParticleSet ps = ctrl->sets[cur];
     float4 *rec = reinterpret_cast<float4 *>(ctrl->sets[1 - cur].cell);
@@ -159,14 +159,14 @@ __global__ void __launch_bounds__(256) k_unload_records(int64_t n, const Ctrl *_
 // conversions and divisions the FP64 pipe was 85% busy: 5.0 ms at 134M).
 template <bool GATHER>
 __global__ void __launch_bounds__(kLoadThreads) k_unload(int64_t o0, int64_t m, int64_t n,
-                                                        const int32_t *__restrict__ inv,
+                                                        const int32_t *inv,
                                                         const double *__restrict__ node_pos,
                                                         double h0, double h1, double h2,
                                                         double L0, double L1, double L2,
                                                         double half_dt, const Ctrl *ctrl,
                                                         double *__restrict__ x,
                                                         double *__restrict__ v) {
-    dep_begin();
+    dep_begin(inv, ctrl, x, v);
     // results are staged in shared memory and written as contiguous runs (the
     // destination may be host memory written over the chip-to-chip link)
     __shared__ double sx[3 * kLoadThreads], sv[3 * kLoadThreads];
@@ -219,9 +219,9 @@ __global__ void __launch_bounds__(kLoadThreads) k_unload(int64_t o0, int64_t m, 
 // ---------------------------------------------------------------------------
 template <bool DIAG, bool EXT, bool MAG>
 __global__ void __launch_bounds__(256, 3) k_gather_push(int64_t n, Geom g, PushConst pc, Ctrl *ctrl,
-                                                      const float4 *__restrict__ E8,
+                                                      const float4 *E8,
                                                       double *__restrict__ part) {
-    dep_begin();
+    dep_begin(ctrl, E8, part);
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     float a_vx = 0.f, a_vy = 0.f, a_vz = 0.f, a_v2 = 0.f;
     double d_v[4] = {0.0, 0.0, 0.0, 0.0};
@@ -390,14 +390,14 @@ __device__ __forceinline__ void pd_one(const Geom &g, const PushConst &pc, const
 // (see cic::box_row).
 template <bool DIAG, bool EXT, bool MAG, bool FIXED, int B, int BE>
 __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom g, PushConst pc, Ctrl *ctrl,
-                                                          const int4 *__restrict__ items,
+                                                          const int4 *items,
                                                           bool staged, int e_guard,
-                                                          const float4 *__restrict__ E8,
+                                                          const float4 *E8,
                                                           float *rho, unsigned long long *rho64,
                                                           float qscale, int sparse_below, int tile_cost,
                                                           double *__restrict__ part,
                                                           SaveY save) {
-    dep_begin();
+    dep_begin(ctrl, items, E8, rho, rho64, part);
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
@@ -555,8 +555,8 @@ cudaError_t launch_copy(const CopyList &cl, LStream st) {
     return cudaGetLastError();
 }
 
-__global__ void k_pid_positions(int64_t n, const int32_t *__restrict__ pid, int32_t *pos) {
-    dep_begin();
+__global__ void k_pid_positions(int64_t n, const int32_t *pid, int32_t *pos) {
+    dep_begin(pid, pos);
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (p < n && is_particle(pid[p], n)) pos[pid[p]] = (int32_t)p;
 }
@@ -668,10 +668,10 @@ __device__ __forceinline__ void block_moments(const Moments &mo, double *part) {
 // B > 0: every tile box is B slots long on each axis (see cic::box_row).
 template <bool DIAG, bool FIXED, int B>
 __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
-    Geom g, uint64_t seed, Ctrl *ctrl, const int4 *__restrict__ items, float *rho,
+    Geom g, uint64_t seed, Ctrl *ctrl, const int4 *items, float *rho,
     unsigned long long *rho64, float qscale, int sparse_below, int tile_cost,
     double *__restrict__ part) {
-    dep_begin();
+    dep_begin(ctrl, items, rho, rho64, part);
     extern __shared__ __align__(16) uint32_t acc[];
     const ParticleSet ps = ctrl->sets[ctrl->cur];
     const int n_items = ctrl->n_items;
@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(256) k_move(int64_t np, Geom g, uint64_t seed,
 }
 
 __global__ void k_step_inc(Ctrl *ctrl) {
-    dep_begin();
+    dep_begin(ctrl);
     ctrl->step += 1;
     ctrl->since_sort += 1;
 }

@@ -159,7 +159,7 @@ cudaError_t exclusive_scan(int32_t *data, int64_t n, int32_t *tmp, LStream st,
 
 namespace {
 __global__ void k_rebin_decide(Ctrl *ctrl, long long max_strays, int period) {
-    dep_begin();
+    dep_begin(ctrl);
     const bool due = (period > 0 && ctrl->since_sort >= period) ||
                      ctrl->stray_step > (unsigned long long)max_strays;
     ctrl->rebin = due ? 1 : 0;

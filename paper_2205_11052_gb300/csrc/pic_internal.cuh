@@ -17,6 +17,12 @@ namespace pic {
 // after it do the same and waits until the one before has finished, its writes
 // visible.  A kernel that begins so may also be launched plainly.
 //
+// Such a kernel runs while the one before writes what it is going to read, so none of
+// that may be declared constant for the kernel: dep_begin takes its pointers (all but
+// those of tables written at bind) and hands them back through an addition that the
+// compiler cannot look through, so that no access moves above the wait, and those that
+// are only read carry no __restrict__, which allows loads past the coherent cache.
+//
 // Small runs spend a quarter of their time between kernels: 20 steps of 16^3 x 8
 // took 1.41 ms, now 1.08; a gradient in a 24^3 trap 2.74, now 2.26.  Large ones lose:
 // the waiting blocks' shared memory is taken from the L1 that gathers rely on (the
@@ -36,9 +42,15 @@ struct DepScope {
     DepScope(LStream &st_, bool on) : st(st_) { st.dep = on; }
     ~DepScope() { st.dep = false; }
 };
-__device__ __forceinline__ void dep_begin() {
+template <class... P>
+__device__ __forceinline__ void dep_begin(P &...p) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if constexpr (sizeof...(P) > 0) {
+        long long zero;
+        asm volatile("mov.b64 %0, 0;" : "=l"(zero)::"memory");
+        ((p += zero), ...);
+    }
 }
 template <class... P, class... A>
 inline cudaError_t launch_dep(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, const LStream &st,
@@ -231,7 +243,7 @@ __device__ __forceinline__ int item_rank(const int4 *items, int i) {
 // bytes of the ranks before the items
 inline size_t rank_bytes(int64_t max_items) { return ((size_t)max_items * 4 + 255) / 256 * 256; }
 
-__device__ __forceinline__ void item_run(const int4 *__restrict__ items, int n_items,
+__device__ __forceinline__ void item_run(const int4 *items, int n_items,
                                          long long tile_cost, int &it0, int &it1) {
     if (n_items <= (int)gridDim.x) {
         // at most one item per block: consecutive blocks (spread over the SMs)
@@ -269,33 +281,29 @@ __device__ __forceinline__ void item_run(const int4 *__restrict__ items, int n_i
 }
 
 // The particles [begin, end) of one tile, of a block's run [it, it1) of items;
-// next_segment moves on to the next tile.  `next` holds the item it will start
-// from, loaded while the segment before is worked on.
+// next_segment moves on to the next tile.  Its item is loaded there: neighbours share a
+// line, and held over a tile's particles it costs the push, at its register limit, more
+// than the wait (256^3 x 8, four steps: 13.3 ms of pushes, so 12.85).
 struct Segments {
     const int4 *items;
     int it, it1, pb;   // pb: the run's last particle + 1
-    int4 next;
 };
-__device__ __forceinline__ Segments run_segments(const int4 *__restrict__ items, int n_items,
+__device__ __forceinline__ Segments run_segments(const int4 *items, int n_items,
                                                  long long tile_cost) {
     Segments r;
     r.items = items;
     item_run(items, n_items, tile_cost, r.it, r.it1);
-    r.next = make_int4(0, 0, 0, 0);
     r.pb = 0;
-    if (r.it < r.it1) {
-        r.next = items[r.it];
-        r.pb = r.it1 < n_items ? items[r.it1].y : items[n_items - 1].z;
-    }
+    if (r.it < r.it1) r.pb = r.it1 < n_items ? items[r.it1].y : items[n_items - 1].z;
     return r;
 }
 __device__ __forceinline__ bool next_segment(Segments &r, int &tile, int &begin, int &end) {
     if (r.it >= r.it1) return false;
-    tile = r.next.x;
-    begin = r.next.y;
-    end = min(r.next.z, r.pb);
-    r.it = r.next.w;
-    if (r.it < r.it1) r.next = r.items[r.it];
+    const int4 i = r.items[r.it];
+    tile = i.x;
+    begin = i.y;
+    end = min(i.z, r.pb);
+    r.it = i.w;
     return true;
 }
 

@@ -102,14 +102,14 @@ __device__ __forceinline__ void interp_E(const ERow r[4], float fx, float fy, fl
 
 // E8 holds, per node q, E at q and (primed) at its +x neighbour (periodic) as Ex
 // Ey Ex' Ey' Ez Ez' and two unused floats, so each of the four (y, z) corner rows of the
-// stencil is one aligned 256-bit read-only load
+// stencil is one aligned 256-bit load
 __device__ __forceinline__ void ld_pair(const float4 *p, float4 &a, float4 &b) {
-    asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+    asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
         : "=f"(a.x), "=f"(a.y), "=f"(b.x), "=f"(b.y), "=f"(a.z), "=f"(b.z), "=f"(a.w), "=f"(b.w)
         : "l"(p));
 }
 
-__device__ __forceinline__ void gather_E_pairs(const Geom &g, const float4 *__restrict__ E8, int i,
+__device__ __forceinline__ void gather_E_pairs(const Geom &g, const float4 *E8, int i,
                                                int j, int k, float fx, float fy, float fz,
                                                float &ex, float &ey, float &ez) {
     const int nx = g.n[0], ny = g.n[1], nz = g.n[2];
@@ -236,7 +236,7 @@ __device__ __forceinline__ void decode_base(const Geom &g, int32_t c, int &i, in
 // stencil base (the fields of the new packed cell c)
 template <bool EXT, bool MAG>
 __device__ __forceinline__ void push_one_pairs(const Geom &g, const PushConst &pc,
-                                               const float4 *__restrict__ E8, int32_t &c,
+                                               const float4 *E8, int32_t &c,
                                                float &fx, float &fy, float &fz, float &vx,
                                                float &vy, float &vz, int &bad, int &i, int &j,
                                                int &k) {
@@ -249,7 +249,7 @@ __device__ __forceinline__ void push_one_pairs(const Geom &g, const PushConst &p
 
 template <bool EXT, bool MAG>
 __device__ __forceinline__ void push_one_pairs(const Geom &g, const PushConst &pc,
-                                               const float4 *__restrict__ E8, int32_t &c,
+                                               const float4 *E8, int32_t &c,
                                                float &fx, float &fy, float &fz, float &vx,
                                                float &vy, float &vz, int &bad) {
     int i, j, k;
@@ -284,7 +284,7 @@ __device__ __forceinline__ void gather_E_pair_box(const float4 *sA, const float2
 // (i, j, k) receives the new stencil base.
 template <bool EXT, bool MAG, int B = 0>
 __device__ __forceinline__ void push_one_staged(const Geom &g, const PushConst &pc,
-                                                const float4 *__restrict__ E8, const float4 *sE,
+                                                const float4 *E8, const float4 *sE,
                                                 const cic::Tile &t, int32_t &c, float &fx,
                                                 float &fy, float &fz, float &vx, float &vy,
                                                 float &vz, int &bad, int &i, int &j, int &k) {

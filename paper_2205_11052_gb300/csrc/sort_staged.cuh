@@ -116,8 +116,8 @@ __device__ __forceinline__ void finish_bins(int32_t *bins, int nb, const PassEnd
 // A lane writes a few items by itself, the warp the many of a dense tile together
 // (with a thread per tile a bunch of 900 thousand particles in a few tiles waited 40
 // us for them at every re-binning).
-__device__ __forceinline__ void fill_tiles(int t0, int ntiles, const int2 *__restrict__ range,
-                                           const int32_t *__restrict__ first, int chunk, int4 *items) {
+__device__ __forceinline__ void fill_tiles(int t0, int ntiles, const int2 *range,
+                                           const int32_t *first, int chunk, int4 *items) {
     const int lane = threadIdx.x & 31, t = t0 + lane;
     int2 r = make_int2(0, 0);
     int o = 0, end = 0;
@@ -255,7 +255,7 @@ template <class Key>
 __global__ void __launch_bounds__(256) k_scatter_staged(int64_t n, Key key_param, Ctrl *ctrl,
                                                          int32_t *bins, int nb, SortRange rg,
                                                          PassEnd pe, const int32_t *gate) {
-    dep_begin();
+    dep_begin(ctrl, bins, gate);
     if (gate && !*gate) return;
     Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
     extern __shared__ __align__(128) unsigned char smem[];
@@ -454,7 +454,7 @@ template <class Key, int PER>
 __global__ void __launch_bounds__(256) k_histogram_staged(int64_t n, Key key_param, Ctrl *ctrl,
                                                            int32_t *bins, int nb, SortRange rg,
                                                            PassEnd pe, const int32_t *gate) {
-    dep_begin();
+    dep_begin(ctrl, bins, gate);
     if (gate && !*gate) return;
     Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
     __shared__ int32_t hkey[kHash];
@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(T) k_histogram_direct(int64_t n, int64_t per, 
                                                            Ctrl *ctrl, int32_t *bins, int nb,
                                                            SortRange rg, PassEnd pe,
                                                            const int32_t *gate) {
-    dep_begin();
+    dep_begin(ctrl, bins, gate);
     if (gate && !*gate) return;
     Key key_of = key_param;   // a per-thread copy (functors may cache lookups)
     extern __shared__ __align__(16) int32_t cnt[];
