@@ -246,7 +246,7 @@ __device__ __forceinline__ bool tile_add(uint32_t *acc, const Tile &t, const Geo
 // particles at most.  A tile visit that ends before needs no fold; the flush
 // adds what both hold to the grid, one global atomic per touched slot.  Each
 // slot is touched by one thread in both loops.
-__device__ __forceinline__ int fill_limit() { return kMaxChunk / (int)blockDim.x; }
+__device__ __forceinline__ unsigned fill_limit() { return kMaxChunk / blockDim.x; }
 
 template <bool FIXED>
 __device__ __forceinline__ void tile_fold(uint32_t *acc, void *sum, int S) {

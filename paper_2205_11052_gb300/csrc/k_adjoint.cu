@@ -190,11 +190,12 @@ __global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bo
     };
     // the run's particles tile by tile; the tile goes to the grid when the run
     // leaves it and after 4095 particles at most (the int32 bound above)
-    int tile, begin, end;
+    int tile;
+    PIndex begin, end;
     while (next_segment(run, tile, begin, end)) {
         // the next particle's position and multipliers are loaded before the
         // current one is reversed
-        int p = begin + threadIdx.x;
+        PIndex p = begin + threadIdx.x;
         int32_t nyc = 0;
         float nly0 = 0.f, nly1 = 0.f, nly2 = 0.f, nfx = 0.f, nfy = 0.f, nfz = 0.f;
         float nlv0 = 0.f, nlv1 = 0.f, nlv2 = 0.f;
@@ -214,8 +215,8 @@ __global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bo
         tb = tn;
         cic::stage_wait();
         __syncthreads();
-        for (int done = begin;;) {
-            done += min(end - done, cic::fill_limit() * (int)blockDim.x);
+        for (PIndex done = begin;;) {
+            done += min(end - done, cic::fill_limit() * blockDim.x);
             for (; p < done; p += blockDim.x) {
                 int i, j, k;
                 if (!decode(nyc, g, i, j, k)) bad = 1;
@@ -223,7 +224,7 @@ __global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bo
                 const float fx = nfx, fy = nfy, fz = nfz;
                 const float plv0 = nlv0, plv1 = nlv1, plv2 = nlv2;
                 {
-                    const int pn = p + (int)blockDim.x;
+                    const PIndex pn = p + blockDim.x;
                     if (pn < end) {
                         nyc = ycell[pn];
                         nly0 = lam.o[0][pn]; nly1 = lam.o[1][pn]; nly2 = lam.o[2][pn];

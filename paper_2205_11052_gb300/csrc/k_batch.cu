@@ -266,23 +266,24 @@ __global__ void __launch_bounds__(256, PIC_BATCH_PD_MIN_BLOCKS) k_b_push_deposit
         }
         const float4 *sEi = (PUSH && E4 != nullptr && !sparse) ? sE : nullptr;
         // the next particle's streams are loaded before the current one is pushed
-        int p = item.y + threadIdx.x;
+        const PIndex end = item.z;
+        PIndex p = item.y + threadIdx.x;
         int32_t nc = 0;
         float nfx = 0.f, nfy = 0.f, nfz = 0.f, nvx = 0.f, nvy = 0.f, nvz = 0.f;
-        if (p < item.z) {
+        if (p < end) {
             nc = __ldcs(ps.cell + p);
             nfx = __ldcs(ps.o[0] + p); nfy = __ldcs(ps.o[1] + p); nfz = __ldcs(ps.o[2] + p);
             if (PUSH) {
                 nvx = __ldcs(ps.v[0] + p); nvy = __ldcs(ps.v[1] + p); nvz = __ldcs(ps.v[2] + p);
             }
         }
-        for (; p < item.z; p += blockDim.x) {
+        for (; p < end; p += blockDim.x) {
             int32_t c = nc;
             float fx = nfx, fy = nfy, fz = nfz;
             const float cvx = nvx, cvy = nvy, cvz = nvz;
             {
-                const int pn = p + (int)blockDim.x;
-                if (pn < item.z) {
+                const PIndex pn = p + blockDim.x;
+                if (pn < end) {
                     nc = __ldcs(ps.cell + pn);
                     nfx = __ldcs(ps.o[0] + pn); nfy = __ldcs(ps.o[1] + pn); nfz = __ldcs(ps.o[2] + pn);
                     if (PUSH) {

@@ -60,11 +60,12 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
     // t: the tile of the dense segments (sparse ones go straight to the grid)
     bool any = false, folded = false;
     Tile t = tile_of(g, 0);
-    int tile, begin, end;
+    int tile;
+    PIndex begin, end;
     while (next_segment(run, tile, begin, end)) {
-        if (end - begin < sparse_below) {
+        if ((int)(end - begin) < sparse_below) {
             // few particles: skip the shared tile, add straight to the grid
-            for (int p = begin + threadIdx.x; p < end; p += blockDim.x) {
+            for (PIndex p = begin + threadIdx.x; p < end; p += blockDim.x) {
                 int i, j, k;
                 if (!decode_cell(ps.cell[p], g, i, j, k)) bad = 1;
                 const float fx = ps.o[0][p], fy = ps.o[1][p], fz = ps.o[2][p];
@@ -74,7 +75,7 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
             }
             continue;
         }
-        int p = begin + threadIdx.x;
+        PIndex p = begin + threadIdx.x;
         int32_t nc = 0;
         float nfx = 0.f, nfy = 0.f, nfz = 0.f;
         if (p < end) {
@@ -89,12 +90,12 @@ __global__ void __launch_bounds__(256, PIC_DEP_MIN_BLOCKS) k_deposit_tiles(Geom 
         folded = false;
         t = tile_of(g, tile);
         __syncthreads();
-        for (int done = begin;;) {
-            done += min(end - done, fill_limit() * (int)blockDim.x);
+        for (PIndex done = begin;;) {
+            done += min(end - done, fill_limit() * blockDim.x);
             for (; p < done; p += blockDim.x) {
                 const int32_t c = nc;
                 const float fx = nfx, fy = nfy, fz = nfz;
-                const int pn = p + (int)blockDim.x;
+                const PIndex pn = p + blockDim.x;
                 if (pn < end) {
                     nc = __ldcs(ps.cell + pn);
                     nfx = __ldcs(ps.o[0] + pn);

@@ -419,12 +419,13 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
     // t: the tile of the dense segments (sparse ones deposit and gather globally)
     bool any = false, folded = false;
     cic::Tile t = cic::tile_of(g, 0);
-    int tile, begin, end;
+    int tile;
+    PIndex begin, end;
     while (next_segment(run, tile, begin, end)) {
-        const bool sparse = end - begin < sparse_below;
+        const bool sparse = (int)(end - begin) < sparse_below;
         // one particle per thread and iteration (coalesced 4-byte streams);
         // the next iteration's particle is loaded before this one is pushed
-        int p = begin + threadIdx.x;
+        PIndex p = begin + threadIdx.x;
         int32_t nc = 0;
         float nfx = 0.f, nfy = 0.f, nfz = 0.f, nvx = 0.f, nvy = 0.f, nvz = 0.f;
         if (p < end) {
@@ -444,13 +445,13 @@ __global__ void __launch_bounds__(kPushThreadsPerSM / 2, 2) k_push_deposit(Geom 
             __syncthreads();
         }
         const float4 *sAi = (staged && !sparse) ? sA : nullptr;
-        for (int done = begin;;) {
+        for (PIndex done = begin;;) {
             // as many particles as the tile takes without a fold
-            done += min(end - done, cic::fill_limit() * (int)blockDim.x);
+            done += min(end - done, cic::fill_limit() * blockDim.x);
             for (; p < done; p += blockDim.x) {
                 int32_t c = nc;
                 float fx = nfx, fy = nfy, fz = nfz, vx = nvx, vy = nvy, vz = nvz;
-                const int pn = p + (int)blockDim.x;
+                const PIndex pn = p + blockDim.x;
                 if (pn < end) {
                     nc = __ldcs(ps.cell + pn);
                     nfx = __ldcs(ps.o[0] + pn); nfy = __ldcs(ps.o[1] + pn); nfz = __ldcs(ps.o[2] + pn);
@@ -690,11 +691,12 @@ __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
     // t: the tile of the dense segments (sparse ones deposit globally)
     bool any = false, folded = false;
     cic::Tile t = cic::tile_of(g, 0);
-    int tile, begin, end;
+    int tile;
+    PIndex begin, end;
     while (next_segment(run, tile, begin, end)) {
-        const bool sparse = end - begin < sparse_below;
+        const bool sparse = (int)(end - begin) < sparse_below;
         // the next particle's streams are loaded before the current one moves
-        int p = begin + threadIdx.x;
+        PIndex p = begin + threadIdx.x;
         int32_t nc = 0, npid = 0;
         float nfx = 0.f, nfy = 0.f, nfz = 0.f;
         if (p < end) {
@@ -710,13 +712,13 @@ __global__ void __launch_bounds__(256, PIC_MV_MIN_BLOCKS) k_move_deposit(
             t = cic::tile_of(g, tile);
             __syncthreads();
         }
-        for (int done = begin;;) {
-            done += min(end - done, cic::fill_limit() * (int)blockDim.x);
+        for (PIndex done = begin;;) {
+            done += min(end - done, cic::fill_limit() * blockDim.x);
             for (; p < done; p += blockDim.x) {
                 int32_t c = nc;
                 float fx = nfx, fy = nfy, fz = nfz;
                 const int32_t pid = npid;
-                const int pn = p + (int)blockDim.x;
+                const PIndex pn = p + blockDim.x;
                 if (pn < end) {
                     nc = __ldcs(ps.cell + pn);
                     nfx = __ldcs(ps.o[0] + pn); nfy = __ldcs(ps.o[1] + pn); nfz = __ldcs(ps.o[2] + pn);

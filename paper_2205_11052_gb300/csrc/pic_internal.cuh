@@ -280,6 +280,10 @@ __device__ __forceinline__ void item_run(const int4 *items, int n_items,
     it1 = blockIdx.x + 1 == gridDim.x ? n_items : min(n_items, lo1 + r1);
 }
 
+// Index of a particle in the walk over a tile.  Unsigned: a stride past the last of
+// 2^31 - 1 particles stays above it (as an int it would be negative, and so below).
+using PIndex = uint32_t;
+
 // The particles [begin, end) of one tile, of a block's run [it, it1) of items;
 // next_segment moves on to the next tile.  Its item is loaded there: neighbours share a
 // line, and held over a tile's particles it costs the push, at its register limit, more
@@ -297,7 +301,7 @@ __device__ __forceinline__ Segments run_segments(const int4 *items, int n_items,
     if (r.it < r.it1) r.pb = r.it1 < n_items ? items[r.it1].y : items[n_items - 1].z;
     return r;
 }
-__device__ __forceinline__ bool next_segment(Segments &r, int &tile, int &begin, int &end) {
+__device__ __forceinline__ bool next_segment(Segments &r, int &tile, PIndex &begin, PIndex &end) {
     if (r.it >= r.it1) return false;
     const int4 i = r.items[r.it];
     tile = i.x;
