@@ -1525,6 +1525,17 @@ int pic_adjoint_backward(pic_handle_t c, double scale, double *gx, double *gv, i
         }
     }
 
+    // pic_get_field gives the field of the last solve, a recomputed step's, which went
+    // into the buffer
+    if (c->adj.nseg > 1) {
+        CopyList cl{};
+        cl.count = 1;
+        cl.dst[0] = c->at<char>(c->lay.E8);
+        cl.src[0] = reinterpret_cast<const char *>(adj_field(c, L, K - 1));
+        cl.bytes[0] = c->ng * 32;
+        PIC_CUDA(launch_copy(cl, c->st));
+    }
+
     // The multipliers are now in the order of checkpoint 0: restore it (the
     // state the forward sweep started from, re-binned, with its work items).
     if ((r = adj_restore(c, L, 0, cur))) return r;

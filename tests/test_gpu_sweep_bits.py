@@ -99,6 +99,24 @@ def test_recomputed_segments_repeat_the_forward_sweep():
         assert np.max(np.abs(a - b)) <= 1e-5 * np.max(np.abs(a))
 
 
+@pytest.mark.parametrize("name", ["24_trap", "primes"])
+@pytest.mark.parametrize("steps,keep,last", [(8, 3, 3), (8, 8, 8), (5, 2, 2), (1, 4, 1)])
+def test_field_after_a_gradient_is_that_of_the_last_solve(name, steps, keep, last):
+    """Segments are recomputed back to front, so the last solve is that of the first
+    segment's last step (or of the objective where nothing is recomputed)."""
+    grid, n, B, wz2, kw = CASES[name]
+    out = []
+    for s, k, back in ((steps, keep, True), (last, last, False)):
+        sim = Simulation(n=grid, L=(L,) * 3, n_particles=n, dt=0.05, Q=-L ** 3, B=B, wz2=wz2, options=FIXED, **kw)
+        sim.load(*_inputs(n))
+        sim.adjoint_forward(s, checkpoint_every=k)
+        if back:
+            sim.adjoint_backward()
+        out.append(sim.field()[1])
+        sim.close()
+    assert np.array_equal(*out)
+
+
 def test_gradient_away_from_cell_faces():
     """Particles farther than 1e-4 cells (a hundred times the FP32 trajectory's error)
     from a face at the last step: 2-norm of the difference to the oracle within 1e-5
