@@ -790,9 +790,10 @@ int adj_solve(pic_ctx *c, int par) {
     PIC_CUFFT(cufftExecR2C(c->plan[kR2C3], c->at<cufftReal>(c->lay.adjE4), c->at<cufftComplex>(c->lay.E_hat)));
     PIC_CUDA(launch_green_adj(c->geom, c->L, c->at<float2>(c->lay.E_hat),
                               c->at<float2>(c->lay.rho_hat), c->nhalf, c->st));
-    PIC_CUFFT(cufftExecC2R(c->plan[kC2R1], c->at<cufftComplex>(c->lay.rho_hat), c->at<cufftReal>(c->lay.rho)));
-    PIC_CUDA(launch_adj_pair_rho(c->geom, c->at<float>(c->lay.rho), c->at<float2>(c->lay.lrho2),
-                                 c->at<float4>(c->lay.adjE4), c->ctrl(), par, c->st));
+    float *lrho = c->at<float>(c->lay.E_hat);   // lE^ is done with; rho stays the last deposit's
+    PIC_CUFFT(cufftExecC2R(c->plan[kC2R1], c->at<cufftComplex>(c->lay.rho_hat), lrho));
+    PIC_CUDA(launch_adj_pair_rho(c->geom, lrho, c->at<float2>(c->lay.lrho2), c->at<float4>(c->lay.adjE4),
+                                 c->ctrl(), par, c->st));
     return PIC_OK;
 }
 

@@ -101,20 +101,24 @@ def test_recomputed_segments_repeat_the_forward_sweep():
 
 @pytest.mark.parametrize("name", ["24_trap", "primes"])
 @pytest.mark.parametrize("steps,keep,last", [(8, 3, 3), (8, 8, 8), (5, 2, 2), (1, 4, 1)])
-def test_field_after_a_gradient_is_that_of_the_last_solve(name, steps, keep, last):
+def test_fields_after_a_gradient_are_the_last_ones(name, steps, keep, last):
     """Segments are recomputed back to front, so the last solve is that of the first
-    segment's last step (or of the objective where nothing is recomputed)."""
+    segment's last step and the last deposit that of its push (or both are the
+    objective's where nothing is recomputed)."""
     grid, n, B, wz2, kw = CASES[name]
-    out = []
-    for s, k, back in ((steps, keep, True), (last, last, False)):
+    rho, E = [], []
+    for s, k, back in ((steps, keep, True), (last, last, False), (last + (last < steps), last + 1, False)):
         sim = Simulation(n=grid, L=(L,) * 3, n_particles=n, dt=0.05, Q=-L ** 3, B=B, wz2=wz2, options=FIXED, **kw)
         sim.load(*_inputs(n))
         sim.adjoint_forward(s, checkpoint_every=k)
         if back:
             sim.adjoint_backward()
-        out.append(sim.field()[1])
+        f = sim.field()
+        rho.append(f[0])
+        E.append(f[1])
         sim.close()
-    assert np.array_equal(*out)
+    assert np.array_equal(E[0], E[1])
+    assert np.array_equal(rho[0], rho[2])
 
 
 def test_gradient_away_from_cell_faces():
