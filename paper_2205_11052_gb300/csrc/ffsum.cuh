@@ -1,6 +1,7 @@
-// FP32 (hi, lo) pair sums of the field diagnostics: about 48-bit arithmetic at
-// FP32 speed (FP64 instructions run at a small fraction of the FP32 rate on
-// this part), shared by the single-run and the batched reductions.
+// Sums of the field diagnostics: in FP64, and on the grids solved by cuFFT in FP32
+// (hi, lo) pairs, about 48-bit arithmetic at FP32 speed (FP64 instructions run at
+// a small fraction of the FP32 rate on this part); and the conversion of the
+// fixed-point density.
 #pragma once
 
 #include "records.cuh"
@@ -27,29 +28,48 @@ __device__ __forceinline__ void ff_add_sq(float &hi, float &lo, float x) {
     lo = __fadd_rn(lo, e);
 }
 
-// The block's sums of four such pairs, in out[0..3] as FP64: pairs are added
-// across the lanes in FP32 (error terms included), warps in FP64, both in a
-// fixed order.  Every thread of the THREADS-thread block calls it.
+// The warp's sums of four totals t of each lane: lane 8 q returns the q-th.  The lanes
+// trade halves of the four first: 2 + 1 + 3 FP64 additions instead of 20, at about two
+// lanes per clock and SM.
+__device__ __forceinline__ double warp_sums(const double (&t)[4]) {
+    const bool up = threadIdx.x & 16, odd = threadIdx.x & 8;
+    const double a = (up ? t[2] : t[0]) + __shfl_xor_sync(0xffffffffu, up ? t[0] : t[2], 16);
+    const double b = (up ? t[3] : t[1]) + __shfl_xor_sync(0xffffffffu, up ? t[1] : t[3], 16);
+    double r = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
+    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    return r;
+}
+
+// The block's sums of four totals of each thread, in out[0..3], in a fixed order.
+// Every thread of the THREADS-thread block calls it.
 template <int THREADS>
-__device__ __forceinline__ void block_field_sums(float (&hi)[4], float (&lo)[4], double *out) {
+__device__ __forceinline__ void block_field_sums(const double (&t)[4], double *out) {
     __shared__ double red[4][THREADS / 32];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        for (int o = 16; o > 0; o >>= 1) {
-            const float h = __shfl_down_sync(0xffffffffu, hi[q], o);
-            const float l = __shfl_down_sync(0xffffffffu, lo[q], o);
-            ff_add(hi[q], lo[q], h);
-            lo[q] = __fadd_rn(lo[q], l);
-        }
-        if (lane == 0) red[q][wid] = (double)hi[q] + (double)lo[q];
-    }
+    const double w4 = warp_sums(t);
+    if ((lane & 7) == 0) red[lane >> 3][wid] = w4;
     __syncthreads();
     if (threadIdx.x < 4) {
-        double t = 0.0;
-        for (int w = 0; w < THREADS / 32; ++w) t += red[threadIdx.x][w];
-        out[threadIdx.x] = t;
+        double s = 0.0;
+        for (int w = 0; w < THREADS / 32; ++w) s += red[threadIdx.x][w];
+        out[threadIdx.x] = s;
     }
+}
+// ... given as pairs
+template <int THREADS>
+__device__ __forceinline__ void block_field_sums(const float (&hi)[4], const float (&lo)[4], double *out) {
+    double t[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) t[q] = widen(hi[q]) + widen(lo[q]);
+    block_field_sums<THREADS>(t, out);
+}
+// s += the squares of e's components and the density r
+__device__ __forceinline__ void add_field(double (&s)[4], const float4 &e, float r) {
+    const double x = widen(e.x), y = widen(e.y), z = widen(e.z);
+    s[0] = fma(x, x, s[0]);
+    s[1] = fma(y, y, s[1]);
+    s[2] = fma(z, z, s[2]);
+    s[3] += widen(r);
 }
 
 // A factor and what a product with it and 2^52 + q is off by

@@ -380,10 +380,9 @@ __global__ void k_b_green(const InstDesc *__restrict__ desc, int first, int m, i
 }
 
 // Field energies and charge: block (i, b) leaves the partial sums of nodes
-// [b, b + 1) * per of instance i, in FP32 (hi, lo) pairs per thread
-// and FP64 across threads, in a fixed order.  One block per instance with FP64
-// sums kept 24 of 152 SMs busy for 0.29 ms a step on 24 instances of up to
-// 48^3 nodes; 4096 nodes a block take 19.2 us.
+// [b, b + 1) * per of instance i, in FP64 and a fixed order.  One block per
+// instance kept 24 of 152 SMs busy for 0.29 ms a step on 24 instances of up to
+// 48^3 nodes; 4096 nodes a block take 22 us (in FP32 pairs 13).
 __global__ void __launch_bounds__(256) k_b_diag_field(const InstDesc *__restrict__ desc,
                                                       const float *__restrict__ rho,
                                                       const float4 *__restrict__ E4,
@@ -394,16 +393,10 @@ __global__ void __launch_bounds__(256) k_b_diag_field(const InstDesc *__restrict
     const int64_t ng = (int64_t)D.g.n[0] * D.g.n[1] * D.g.n[2];
     const int64_t per = (ng + nb - 1) / nb;
     const int64_t q1 = D.g0 + ((blockIdx.y + 1) * per < ng ? (blockIdx.y + 1) * per : ng);
-    float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int64_t q = D.g0 + blockIdx.y * per + threadIdx.x; q < q1; q += blockDim.x) {
-        const float4 e = E4[q];
-        ff_add_sq(hi[0], lo[0], e.x);
-        ff_add_sq(hi[1], lo[1], e.y);
-        ff_add_sq(hi[2], lo[2], e.z);
-        ff_add(hi[3], lo[3], rho[q]);
-    }
-    block_field_sums<256>(hi, lo,
-                          fpart + 4 * ((int64_t)blockIdx.x * fstride + blockIdx.y));
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int64_t q = D.g0 + blockIdx.y * per + threadIdx.x; q < q1; q += blockDim.x)
+        add_field(s, E4[q], rho[q]);
+    block_field_sums<256>(s, fpart + 4 * ((int64_t)blockIdx.x * fstride + blockIdx.y));
 }
 
 // One record per instance, one block each: the instance's items are

@@ -23,7 +23,9 @@ __device__ __forceinline__ void advance_cells(const Geom &g, float sx, float sy,
 // particles (as many as a tile takes without a fold, or one loop iteration), those
 // sums in (hi, lo) pairs that carry their rounding errors, and the threads in
 // FP64.  (With FP64 totals per thread the folds kept the scarce FP64 units busy:
-// 134M particles with records 2.31 ms a push, now 2.28.)
+// 134M particles with records 2.31 ms a push, now 2.28.  The kinetic energy of 33
+// thousand to 134M particles is off by 1e-11 to 4e-10 of the FP64 sum of the same
+// velocities, with FP64 totals by 1e-11 to 3e-9: the FP32 sums decide.)
 struct Moments {
     float a[4] = {0.f, 0.f, 0.f, 0.f};
     float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
@@ -43,18 +45,12 @@ struct Moments {
     __device__ __forceinline__ double total(int q) const { return widen(hi[q]) + widen(lo[q]); }
 };
 
-// The warp's sums of the four totals: lane 8 q returns the q-th.  The lanes trade
-// halves of the four values first (2 + 1 + 3 FP64 additions and 4 for the totals
-// instead of 24 and 8 conversions at about two lanes per clock and SM: the push of
-// 4.2M particles 90.3 -> 88.6 us).
+// The warp's sums of the four totals: lane 8 q returns the q-th (each lane's four
+// summed over the warp by themselves took 24 FP64 additions and 8 conversions: the push
+// of 4.2M particles 90.3 us, so 88.6)
 __device__ __forceinline__ double warp_total(const Moments &mo) {
-    const bool up = threadIdx.x & 16, odd = threadIdx.x & 8;
-    const double t0 = mo.total(0), t1 = mo.total(1), t2 = mo.total(2), t3 = mo.total(3);
-    const double a = (up ? t2 : t0) + __shfl_xor_sync(0xffffffffu, up ? t0 : t2, 16);
-    const double b = (up ? t3 : t1) + __shfl_xor_sync(0xffffffffu, up ? t1 : t3, 16);
-    double r = (odd ? b : a) + __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
-    for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-    return r;
+    const double t[4] = {mo.total(0), mo.total(1), mo.total(2), mo.total(3)};
+    return warp_sums(t);
 }
 
 // One (y, z) row of a stencil: Ex and Ey at its two x corners, and the two Ez

@@ -17,6 +17,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():  # pragma: no cover - CPU-only machines
     pytest.skip("needs a CUDA device", allow_module_level=True)
 
+from paper_2205_11052_gb300 import capi  # noqa: E402
 from paper_2205_11052_gb300.build import build  # noqa: E402
 from paper_2205_11052_gb300.sim import Simulation  # noqa: E402
 
@@ -62,3 +63,38 @@ def test_sums_and_mode_of_a_record(n):
     scale = np.sqrt(np.mean(E[1].astype(np.float64) ** 2))
     assert abs(rec["mode"] - m) <= 1e-5 * scale
     sim.close()
+
+
+def test_field_sums_of_runs_and_ensembles():
+    """Field energies and charge against the exact sums of the same field and density:
+    within 4e-16, a few of FP64's roundings (in pairs of FP32 the squares are off by 4e-16
+    to 8e-16, their last bits not being random).  A run and an ensemble's instance of one grid have
+    the same field."""
+    import math
+
+    from paper_2205_11052_gb300.batch import Ensemble
+
+    rng = np.random.default_rng(61)
+    L = 12.0
+    members = [(n, L, rng.random((N, 3)) * L, rng.standard_normal((N, 3)), -L ** 3)
+               for n, N in ((16, 40_000), (32, 500_001), (48, 600_003), (60, 900_000))]
+    ens = Ensemble(members, dt=0.01, options=capi.PIC_OPT_FIXED_DEPOSIT, diag_every=1)
+    ens.step(1)
+    records = ens.diagnostics()[-1]
+    ens.close()
+    for (n, _, x, v, Q), rec in zip(members, records):
+        sim = Simulation(n=(n,) * 3, L=(L,) * 3, n_particles=len(x), dt=0.01, Q=Q, diag_every=1,
+                         options=capi.PIC_OPT_FIXED_DEPOSIT)
+        sim.load(x, v)
+        sim.deposit()
+        sim.field_solve()
+        rho, E = sim.field()
+        sim.step(1)
+        own = sim.diagnostics()[-1]
+        sim.close()
+        dV = (L / n) ** 3
+        for key, a in (("Wx", E[0].astype(np.float64) ** 2), ("Wy", E[1].astype(np.float64) ** 2),
+                       ("Wz", E[2].astype(np.float64) ** 2), ("Q", rho.astype(np.float64))):
+            exact = dV * math.fsum(a.ravel())
+            for got in (rec[key], own[key]):
+                assert abs(got - exact) <= 4e-16 * abs(exact), (n, key)
