@@ -1053,6 +1053,8 @@ def main():
 TRAFFIC_SOURCES = ["paper_2205_11052_gb300/csrc/k_particles.cu",
                    "paper_2205_11052_gb300/csrc/push.cuh",
                    "paper_2205_11052_gb300/csrc/cic.cuh",
+                   "paper_2205_11052_gb300/csrc/ffsum.cuh",
+                   "paper_2205_11052_gb300/csrc/records.cuh",
                    "paper_2205_11052_gb300/csrc/pic_internal.cuh"]
 
 

@@ -90,7 +90,7 @@ typedef struct {
                               ensembles: of the batched push + deposit, a
                               multiple of 32 in 64..256 (autotuned)          */
     int32_t chunk;         /* max particles per work item, 32..4095 (0: chosen
-                              from the particle count)                           */
+                              from the particle count; ensembles: 4095)          */
     int32_t options;       /* PIC_OPT_* bits (default 0)                         */
     uint64_t seed;         /* random stream of PIC_OPT_UNIFORM_MOVE              */
     double  stray_rebin;   /* stray-triggered re-binning in pic_step (default 0 =
@@ -325,7 +325,11 @@ int pic_read_timers(pic_handle_t h, double ms[PIC_PHASE_COUNT],
  * the multipliers are permuted back across each re-binning.  The reverse
  * deposit of the 3-vector G^T le accumulates in int32 shared tiles whose
  * scale comes from a bound on |le| carried from step to step.  FP32 particle
- * and grid arithmetic; J and the final reductions in FP64. */
+ * and grid arithmetic; J and the final reductions in FP64.
+ * The components of a particle within rounding of a cell face at the last
+ * step hang on the last bits of its position (the derivative of the deposit
+ * jumps there); the sweeps therefore solve by one and the same transforms
+ * (cuFFT's) on every grid, set up by the first pic_adjoint_forward. */
 
 /* Bytes of the caller-owned device buffer for pic_adjoint_forward/backward. */
 int pic_adjoint_buffer_bytes(pic_handle_t h, int n_steps, int checkpoint_every, size_t *bytes);

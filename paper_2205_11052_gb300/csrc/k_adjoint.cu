@@ -378,7 +378,7 @@ __global__ void __launch_bounds__(kAdjThreadsPerSM / 2, 2) k_adj_push(Geom g, bo
     if (bad) atomicOr(&ctrl_w->flags, PIC_FLAG_BAD_CELL);
     if (nonfinite) atomicOr(&ctrl_w->flags, PIC_FLAG_NONFINITE);
     if (PG) {
-        // block sums in FP64, fixed order: warp shuffles, then the 8 warps
+        // block sums in FP64, fixed order: warp shuffles, then the block's warps
         __shared__ double red[kPGradTerms][kAdjThreadsPerSM / 64];
         const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll

@@ -1,6 +1,7 @@
 // Field solve (Section 3.1 step 2, Eq. potential; Section 3.2 of
-// arXiv 2205.11052) of grids whose three axes are at most kFftMaxN long, in
-// three kernels around the line transforms of fft.cuh:
+// arXiv 2205.11052) of grids whose three axes are at most kFftMaxN long and products
+// of 2, 3, 5 and 7, with (y, z) planes of at most 96^2 nodes (fft_supported), in three
+// kernels around the line transforms of fft.cuh:
 //   k_fft_x_forward   rows of rho -> spectra over x (two real rows per complex
 //                     line), stored by x frequency: rho_hat[kx][z][y]
 //   k_fft_yz          one (y, z) plane of one x frequency and one component per
@@ -387,7 +388,6 @@ void fft_tables(const FftAxis ax[3], FftTables &t) {
                 f /= ax[d].radix[i];
             }
             t.pos[d][k] = p;
-            t.freq[d][p] = k;
         }
     }
 }
@@ -412,8 +412,8 @@ void fft_ktab(const Geom &g, const double *L_d, const FftTables &t, float *out) 
     int off = g.nh;
     for (int d = 1; d < 3; ++d) {
         const int n = g.n[d];
-        for (int p = 0; p < n; ++p) {
-            const int f = t.freq[d][p];
+        for (int f = 0; f < n; ++f) {
+            const int p = t.pos[d][f];
             o[p] = k[off + f];
             o[n + p] = (n & 1) == 0 && f == n / 2 ? 0.0f : k[off + f];
         }

@@ -7,11 +7,12 @@
 // with |k|^2 over the continuous wavenumbers (m_d in [-N_d/2, N_d/2)), the
 // k = 0 mode (the uniform ion background) set to zero and each axis' Nyquist
 // component of the gradient set to zero so E stays real.  The 1/N_g of the
-// inverse transform is folded in here.  k_pack_E interleaves the three planar
-// components as float4 (Ex, Ey, Ez, 0) so the gather reads 16-byte vectors.
+// inverse transform is folded in here.  k_pack_E turns what the transform leaves into
+// the x-paired field that the gathers read (32 bytes a node).
 //
 // Diagnostics (figures of Section 4): W_d = h^3 sum_g E_d^2, Q = h^3 sum_g rho,
-// accumulated in FP64 per block in a fixed order, then summed by one block.
+// per thread in FP32 pairs that carry their rounding errors (ffsum.cuh), from there on
+// in FP64, in a fixed order.
 #include <math.h>
 
 #include "ffsum.cuh"
@@ -105,9 +106,10 @@ namespace {
 // ES-th float) -> the x-paired E8 read by 256-bit loads (the components at q, then those at
 // its +x neighbour, periodic: Ex Ey Ex' Ey' | Ez Ez' 0 0) and, with SUMS, the
 // block's partial sums of Ex^2, Ey^2, Ez^2 and rho.  Bound by DRAM: 12 bytes read
-// and 32 written per node (16.8M nodes: 163 us; with E4 written too 246 us).  With the interleaving left to the inverse
-// transform (output stride 4: 407 us against 92 planar), a pairing pass (120)
-// and a pass for the sums (81), a 256^3 solve with sums took 0.85 ms.
+// and 32 written per node (16.8M nodes: 163 us; with E4 written too 246 us).  With
+// the interleaving left to the inverse transform, as the gradient sweeps have it
+// (output stride 4: 407 us against 92 planar), a pairing pass (120) and a pass for the
+// sums (81), a 256^3 solve with sums took 0.85 ms.
 template <int ES, bool SUMS>
 __global__ void __launch_bounds__(256) k_pack_E(int nx, int64_t rows, int64_t pitch, int64_t dist,
                                                 const float *planar,

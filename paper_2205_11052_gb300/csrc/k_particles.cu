@@ -210,12 +210,12 @@ __global__ void __launch_bounds__(kLoadThreads) k_unload(int64_t o0, int64_t m, 
 }
 
 // ---------------------------------------------------------------------------
-// gather + Boris push + drift + periodic wrap (push_one in push.cuh)
+// gather + Boris push + drift + periodic wrap (push_one_pairs in push.cuh)
 //
 // Each thread owns groups of 4 consecutive particles: the seven SoA streams
 // are read and written as 16-byte vectors with evict-first hints (they are
-// touched once per step), while the float4 field is read through the
-// read-only path so it stays cached (the whole 128^3 field is 32 MiB).
+// touched once per step), so that the x-paired field stays cached (64 MiB at
+// 128^3, of 129 MB of L2).
 // ---------------------------------------------------------------------------
 template <bool DIAG, bool EXT, bool MAG>
 __global__ void __launch_bounds__(256, 3) k_gather_push(int64_t n, Geom g, PushConst pc, Ctrl *ctrl,

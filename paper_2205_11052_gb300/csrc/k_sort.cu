@@ -12,9 +12,11 @@
 // contiguous destination range with a single atomic and the scatter writes
 // stay coalesced.  (Cell-level keys would send the 32 lanes of a warp to ~32
 // different cells after any drift, i.e. 4-byte scattered stores.)
-// Passes: histogram (warp-aggregated atomics) -> exclusive scan (in place) ->
-// scatter (the scanned offsets serve as cursors; afterwards bins[key] holds
-// the end of bin key) -> per-tile ranges -> scan of items per tile -> items.
+// Passes (sort_staged.cuh): histogram -> scatter.  The histogram's last block scans the
+// counts in place and lays out the work items, the scatter's blocks write them, with the
+// scanned offsets as cursors.  Above kFusedBins tiles the scan, the per-tile ranges (from
+// bins[key], the end of bin key after the scatter), the scan of items per tile and the
+// items are kernels of their own.
 // Order within a tile is the claim order (not deterministic).
 #include <algorithm>
 

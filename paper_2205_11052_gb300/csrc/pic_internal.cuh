@@ -432,11 +432,11 @@ struct FftAxis {
     int n, stages;
     int radix[kFftMaxStages];   // forward order
 };
-// per axis: exp(-2 pi i k / n), the position of frequency k after a forward
-// transform and the frequency at a position
+// per axis: exp(-2 pi i k / n) and the position of frequency k after a forward
+// transform
 struct FftTables {
     float2 tw[3][kFftMaxN];
-    int pos[3][kFftMaxN], freq[3][kFftMaxN];
+    int pos[3][kFftMaxN];
 };
 bool fft_axis(int n, FftAxis &a);   // false: not supported
 bool fft_supported(const Geom &g, FftAxis ax[3]);

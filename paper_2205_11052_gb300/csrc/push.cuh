@@ -128,11 +128,9 @@ __device__ __forceinline__ void gather_E_pairs(const Geom &g, const float4 *E8, 
 // E at the particle from a copy of the field on a box in shared memory (one
 // float4 per slot; s0 is the stencil base's slot, rows S0 slots apart in y,
 // planes S01 apart in z)
-template <int B = 0>
-__device__ __forceinline__ void gather_E_box(const float4 *sE, int s0, int S0r, int S01r, float fx,
+__device__ __forceinline__ void gather_E_box(const float4 *sE, int s0, int S0, int S01, float fx,
                                              float fy, float fz, float &ex, float &ey,
                                              float &ez) {
-    const int S0 = B > 0 ? B : S0r, S01 = B > 0 ? B * B : S01r;   // B > 0: a constant box
     const ERow r[4] = {row_of(sE[s0], sE[s0 + 1]), row_of(sE[s0 + S0], sE[s0 + S0 + 1]),
                        row_of(sE[s0 + S01], sE[s0 + S01 + 1]),
                        row_of(sE[s0 + S01 + S0], sE[s0 + S01 + S0 + 1])};
@@ -278,7 +276,7 @@ __device__ __forceinline__ void gather_E_pair_box(const float4 *sA, const float2
 // instead of one L1 wavefront per particle and 32-byte global read.  Other
 // particles, and every particle when sE is null, read the x-paired grid E8.
 // (i, j, k) receives the new stencil base.
-template <bool EXT, bool MAG, int B = 0>
+template <bool EXT, bool MAG>
 __device__ __forceinline__ void push_one_staged(const Geom &g, const PushConst &pc,
                                                 const float4 *E8, const float4 *sE,
                                                 const cic::Tile &t, int32_t &c, float &fx,
@@ -287,8 +285,8 @@ __device__ __forceinline__ void push_one_staged(const Geom &g, const PushConst &
     decode_base(g, c, i, j, k, bad);
     float ex, ey, ez;
     int s0;
-    if (sE != nullptr && cic::box_base<B>(t, g, i, j, k, s0))
-        gather_E_box<B>(sE, s0, t.S0, t.S01, fx, fy, fz, ex, ey, ez);
+    if (sE != nullptr && cic::box_base(t, g, i, j, k, s0))
+        gather_E_box(sE, s0, t.S0, t.S01, fx, fy, fz, ex, ey, ez);
     else
         gather_E_pairs(g, E8, i, j, k, fx, fy, fz, ex, ey, ez);
     int step[3];

@@ -84,9 +84,13 @@ def test_more_tiles_than_the_fused_passes_take():
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
 
 
-def test_histogram_of_more_keys_than_small_blocks_take():
-    """21^3 = 9261 tiles and enough particles for counters in shared memory."""
-    n, L, N = (84, 84, 84), (4.0, 4.0, 4.0), 6_000_001
+# 21^3 = 9261 tiles, 37 KB of counters; 24^3 = 13824 and 32^3 = 32768, 55 and 131 KB, above
+# what a block has without asking; each with enough particles (four times the tiles for
+# each of 152 blocks) for counters in shared memory
+@pytest.mark.parametrize("axis,N", [(84, 6_000_001), (96, 9_000_001), (128, 20_000_001)])
+def test_histogram_of_more_keys_than_small_blocks_take(axis, N):
+    assert -(-N // 152) >= 4 * (axis // 4) ** 3
+    n, L = (axis,) * 3, (4.0, 4.0, 4.0)
     r = np.random.default_rng(4)
     x, v = r.random((N, 3)) * 4.0, r.standard_normal((N, 3))
     out = []
